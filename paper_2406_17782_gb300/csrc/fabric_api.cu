@@ -96,7 +96,7 @@ static void float_run(const bool *on, int n, int pos, int *len, int *off) {
   *off = back;
 }
 
-bool build_material(const fabric_material &m, DevMaterial *d, std::string *why) {
+bool check_material(const fabric_material &m, std::string *why) {
   char buf[256];
   if (m.pattern_id < 0 || m.pattern_id >= kNumWeaves) {
     snprintf(buf, sizeof(buf), "unknown pattern_id %d (built-in weaves are 0..%d)", m.pattern_id, kNumWeaves - 1);
@@ -116,6 +116,11 @@ bool build_material(const fabric_material &m, DevMaterial *d, std::string *why) 
     *why = "gap in [0,1), w_blend in [0,1], |twist|, |incl| <= 89 required";
     return false;
   }
+  return true;
+}
+
+bool build_material(const fabric_material &m, DevMaterial *d, std::string *why) {
+  if (!check_material(m, why)) return false;
   std::memset(d, 0, sizeof(*d));
   const Weave &w = kWeaves[m.pattern_id];
   d->rows = w.rows;
@@ -128,22 +133,23 @@ bool build_material(const fabric_material &m, DevMaterial *d, std::string *why) 
   d->w_blend = m.w_blend;
   for (int y = 0; y < 2; ++y) {
     const double a = m.alpha[y];
-    d->alpha[y] = m.alpha[y];
-    d->inv_alpha2_minus1[y] = (float)(1.0 / (a * a) - 1.0);
-    d->one_minus_alpha2[y] = (float)(1.0 - a * a);
-    d->inv_pi_alpha[y] = (float)(1.0 / (M_PI * a));
-    d->slope_scale[y] = (float)(-(double)m.beta[y] * M_PI / 2.0);
+    d->yarn[y].slope = (float)(-(double)m.beta[y] * M_PI / 2.0);
+    d->yarn[y].inv_alpha2_minus1 = (float)(1.0 / (a * a) - 1.0);
+    d->yarn[y].one_minus_alpha2 = (float)(1.0 - a * a);
+    d->yarn[y].quarter_inv_pi_alpha = 0.25f * (float)(1.0 / (M_PI * a));
     for (int c = 0; c < 3; ++c) {
       d->kd[y][c] = m.kd[y][c];
       d->ks[y][c] = m.ks[y][c];
     }
   }
+  d->crest[0] = (float)((double)m.beta[0] * (1.0 - (double)m.gap) / (2.0 * w.cols));
+  d->crest[1] = (float)((double)m.beta[1] * (1.0 - (double)m.gap) / (2.0 * w.rows));
   const double incl = (double)m.incl_deg * M_PI / 180.0;
+  const double lncos = std::log(std::cos(incl));
   double rise_max = 0.0;
   for (int i = 0; i < w.rows; ++i) {
     for (int j = 0; j < w.cols; ++j) {
       const bool warp = w.cells[i][j] == '1';
-      if (warp) d->top[i] |= 1u << j;
       bool line[kMaxPatternDim];
       int len, off;
       if (warp) {
@@ -154,18 +160,30 @@ bool build_material(const fabric_material &m, DevMaterial *d, std::string *why) 
         float_run(line, w.cols, j, &len, &off);
       }
       // theta(t) = incl (1 - 2 (off + t) / len) = theta0 - theta1 t
-      d->theta[i * kMaxPatternDim + j] =
-          make_float2((float)(incl * (1.0 - 2.0 * off / len)), (float)(2.0 * incl / len));
+      WeaveCell &c = d->cell[i * kMaxPatternDim + j];
+      c.theta0 = (float)(incl * (1.0 - 2.0 * off / len));
+      c.theta1 = std::ldexp((float)(2.0 * incl / len), -32);
       // the float's rise, the integral of tan(theta) along it:
       // (ln cos theta(t) - ln cos incl) / (theta1 N_along)
       const int n_along = warp ? w.rows : w.cols;
-      d->rise[i * kMaxPatternDim + j] = incl != 0.0 ? (float)(len / (2.0 * incl * n_along)) : 0.0f;
-      if (incl > 0.0) rise_max = std::max(rise_max, len / (double)n_along * -std::log(std::cos(incl)) / (2.0 * incl));
+      c.rise = incl != 0.0 ? (float)(len / (2.0 * incl * n_along)) : 0.0f;
+      if (incl > 0.0) rise_max = std::max(rise_max, len / (double)n_along * -lncos / (2.0 * incl));
+      // the cell's largest height: the crest and the rise at its ends or at
+      // theta = 0 where that lies inside, enlarged past the rounding of the
+      // heights that the kernel computes in FP32
+      double rise_top = 0.0;
+      if (incl != 0.0) {
+        const double scale = len / (2.0 * incl * n_along), t_level = (len - 2.0 * off) / 2.0;
+        double best = std::max(scale * (std::log(std::cos(incl * (1.0 - 2.0 * off / len))) - lncos),
+                               scale * (std::log(std::cos(incl * (1.0 - 2.0 * (off + 1.0) / len))) - lncos));
+        if (t_level > 0.0 && t_level < 1.0) best = std::max(best, scale * -lncos);
+        rise_top = best + 1e-5 * std::fabs(scale * lncos) + 1e-5 * std::fabs(scale);
+      }
+      const double top = std::max(0.0, 1.00001 * (double)d->crest[warp ? 0 : 1] + rise_top);
+      c.top_bound = std::copysign((float)(top * 1.00001 + 1e-30), warp ? -1.0f : 1.0f);
     }
   }
-  d->crest[0] = (float)((double)m.beta[0] * (1.0 - (double)m.gap) / (2.0 * w.cols));
-  d->crest[1] = (float)((double)m.beta[1] * (1.0 - (double)m.gap) / (2.0 * w.rows));
-  d->lncos_incl = (float)std::log(std::cos(incl));
+  d->lncos_incl = (float)lncos;
   d->h_max = (float)(std::max((double)d->crest[0], (double)d->crest[1]) + rise_max);
   d->v_delta = (float)(1.0 / (16.0 * std::max(w.rows, w.cols)));
   return true;
@@ -411,9 +429,8 @@ fabric_status fabric_set_train_materials(fabric_ctx *ctx, const fabric_material 
   if (!m || n_mat < 1 || n_mat > 65535)
     return fail(ctx, FABRIC_ERR_INVALID_ARG, "need 1..65535 training materials (got %d)", n_mat);
   for (int k = 0; k < n_mat; ++k) {
-    DevMaterial tmp;
     std::string why;
-    if (!build_material(m[k], &tmp, &why))
+    if (!check_material(m[k], &why))
       return fail(ctx, FABRIC_ERR_INVALID_ARG, "training material %d: %s", k, why.c_str());
   }
   fabric_material *d = nullptr;
@@ -544,9 +561,8 @@ fabric_status fabric_shade_reference(fabric_ctx *ctx, const fabric_gbuffer *g, i
     return fail(ctx, FABRIC_ERR_INVALID_ARG, "comps output must be float-aligned");
   if (ctx->n_mat == 0) return fail(ctx, FABRIC_ERR_INVALID_ARG, "no materials set");
   const int spp = spp_x * spp_y;
-  // lanes per point: a whole warp for large sample counts, fewer otherwise
   const int lanes = ctx->ref_lanes > 0 ? ctx->ref_lanes
-                    : spp >= 256 ? 32 : spp >= 64 ? 16 : spp >= 16 ? 8 : spp >= 4 ? 4 : 1;
+                                       : reference_lanes(g->n, spp, ctx->visibility != 0, ctx->sm_count);
   FAB_CUDA(ctx,
            launch_reference(*g, ctx->d_mat, ctx->n_mat, spp_x, spp_y, seed, rgb_dev, comps_dev, ctx->d_status,
                             lanes, ctx->sm_count, static_cast<cudaStream_t>(stream), ctx->visibility != 0),

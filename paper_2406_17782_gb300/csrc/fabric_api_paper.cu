@@ -167,9 +167,8 @@ fabric_status fabric_paper_encode_params(fabric_ctx *ctx, const fabric_material 
   if (!m || !latents_dev || n_mat < 0 || n_mat > 65535)
     return fail(ctx, FABRIC_ERR_INVALID_ARG, "need materials, a latent buffer and 0..65535 records");
   for (int k = 0; k < n_mat; ++k) {
-    DevMaterial tmp;
     std::string why;
-    if (!build_material(m[k], &tmp, &why)) return fail(ctx, FABRIC_ERR_INVALID_ARG, "material %d: %s", k, why.c_str());
+    if (!check_material(m[k], &why)) return fail(ctx, FABRIC_ERR_INVALID_ARG, "material %d: %s", k, why.c_str());
   }
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (ctx->enc_raw_cap < n_mat) {

@@ -38,9 +38,8 @@ struct Carve {
 
 bool check_materials(fabric_ctx *ctx, const fabric_material *m, int n) {
   for (int k = 0; k < n; ++k) {
-    DevMaterial tmp;
     std::string why;
-    if (!build_material(m[k], &tmp, &why)) {
+    if (!check_material(m[k], &why)) {
       fail(ctx, FABRIC_ERR_INVALID_ARG, "material %d: %s", k, why.c_str());
       return false;
     }

@@ -116,28 +116,36 @@ constexpr float kSpecK = 100.0f;                    // g(x) = ln(100 x + 1)
 constexpr int kStatusBadMaterial = 1;
 constexpr int kStatusTimeout = 2;
 
-// Per-material record on the device: weave bits, per-cell inclination
-// (theta = theta0 - theta1 * t along the float) and shading constants.
+// Shading constants of one yarn: height-profile slope -beta pi / 2,
+// 1/alpha^2 - 1, 1 - alpha^2 and 1 / (4 pi alpha).
+struct alignas(16) YarnConst {
+  float slope, inv_alpha2_minus1, one_minus_alpha2, quarter_inv_pi_alpha;
+};
+
+// One cell of the weave: the inclination along the float through it,
+// theta = theta0 - theta1 t, t in units of 2^-32; an upper bound of the surface height over the
+// cell (>= 0), with the sign bit set where the warp lies on top; and the
+// float-rise scale len / (2 incl N_along) (0 without inclination).  A sample
+// reads the cell it falls into with one 16-byte load.
+struct alignas(16) WeaveCell {
+  float theta0, theta1, top_bound, rise;
+};
+
+// Per-material record on the device: weave cells and shading constants.
 struct alignas(16) DevMaterial {
   uint32_t rows, cols, gap_fixed, pad0;
-  uint32_t top[kMaxPatternDim];        // bit j of top[i]: warp over weft at (i, j)
   float inv_one_minus_gap;             // 1 / (1 - g)
   float cos_psi, sin_psi, w_blend;
-  float alpha[2];
-  float inv_alpha2_minus1[2];          // 1/alpha^2 - 1
-  float one_minus_alpha2[2];           // 1 - alpha^2
-  float inv_pi_alpha[2];               // 1 / (pi alpha)
-  float slope_scale[2];                // -beta pi / 2
+  YarnConst yarn[2];                   // warp, weft
   float kd[2][3];
   float ks[2][3];
-  float2 theta[kMaxPatternDim * kMaxPatternDim];
   // the proposed inter-yarn visibility model (height field and ray march)
   float crest[2];                      // beta w: cross-section height of each yarn, w its half-width
   float lncos_incl;                    // ln cos(inclination)
   float h_max;                         // largest surface height (repeat units)
   float v_delta;                       // horizontal march step: 1 / (16 max(rows, cols)) repeats
   float pad1[3];
-  float rise[kMaxPatternDim * kMaxPatternDim];   // per cell 1 / (theta1 N_along), 0 without inclination
+  WeaveCell cell[kMaxPatternDim * kMaxPatternDim];
 };
 
 // One segment of a batched draw, as the kernel reads it.
@@ -231,6 +239,7 @@ fabric_status fail(fabric_ctx *ctx, fabric_status s, const char *fmt, ...);
 fabric_status cuda_fail(fabric_ctx *ctx, cudaError_t e, const char *what);
 // Make sure the scratch arena holds `bytes`; returns nullptr on failure.
 void *scratch(fabric_ctx *ctx, size_t bytes);
+bool check_material(const fabric_material &m, std::string *why);
 bool build_material(const fabric_material &m, DevMaterial *out, std::string *why);
 bool check_gbuffer(fabric_ctx *ctx, const fabric_gbuffer *g);
 bool is_aligned16(const void *p);
@@ -241,6 +250,8 @@ void host_pipeline_release(fabric_ctx *ctx);
 void paper_release(fabric_ctx *ctx);
 
 // Launchers implemented in the kernel translation units.
+// Lanes per point of the reference kernel when the caller sets none.
+int reference_lanes(int64_t n, int spp, bool visibility, int sm_count);
 cudaError_t launch_reference(const fabric_gbuffer &g, const DevMaterial *mats, int n_mat, int spp_x, int spp_y,
                              uint64_t seed, float *rgb, float *comps, int *status, int lanes_per_point,
                              int sm_count, cudaStream_t s, bool visibility = false);

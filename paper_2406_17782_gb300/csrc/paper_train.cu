@@ -13,6 +13,7 @@
 // order) and multiplies by the latent block of S1.
 #include <cmath>
 
+#include "f32x2.h"
 #include "fabric_internal.h"
 #include "paper_net.h"
 #include "train_common.cuh"
@@ -39,23 +40,6 @@ struct Epi {
   int ld_out;
   int64_t slab;           // partial: floats per chunk slab
 };
-
-__device__ __forceinline__ uint64_t pn_pk2(float lo, float hi) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-  return r;
-}
-__device__ __forceinline__ float2 pn_upk2(uint64_t r) {
-  float2 f;
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(f.x), "=f"(f.y) : "l"(r));
-  return f;
-}
-// d = a * b + c in each 32-bit lane, rounded once (the same as two fmaf)
-__device__ __forceinline__ uint64_t pn_fma2(uint64_t a, uint64_t b, uint64_t c) {
-  uint64_t d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
-}
 
 // C(i, j) = sum_r A(i, r) B(j, r) for i < M, j < N, r in [r0, r1), with
 // A(i, r) = A[i a_i + r a_r] and B(j, r) = B[j b_j + r b_r].  AR / BR: the
@@ -151,9 +135,9 @@ __global__ void __launch_bounds__(kGemmThreads, 2) pn_gemm_kernel(const float *_
       }
 #pragma unroll
       for (int q = 0; q < RM; ++q) {
-        const uint64_t a2 = pn_pk2(av[q], av[q]);
+        const uint64_t a2 = pk2(av[q], av[q]);
 #pragma unroll
-        for (int t = 0; t < RN / 2; ++t) acc[q][t] = pn_fma2(a2, bv[t], acc[q][t]);
+        for (int t = 0; t < RN / 2; ++t) acc[q][t] = fma2(a2, bv[t], acc[q][t]);
         if (B_ONES) rsum[q] += av[q];   // = fmaf(av[q], 1, rsum[q])
       }
     }
@@ -170,8 +154,9 @@ __global__ void __launch_bounds__(kGemmThreads, 2) pn_gemm_kernel(const float *_
     for (int t = 0; t < RN; ++t) {
       const int j = j0 + 64 * (t / 4) + 4 * tx + (t % 4);
       if (j >= NB) continue;
-      const float2 pr = pn_upk2(acc[q][t / 2]);
-      float v = (t & 1) ? pr.y : pr.x;
+      float v0, v1;
+      upk2(acc[q][t / 2], v0, v1);
+      float v = (t & 1) ? v1 : v0;
       if (e.mode == 0) {
         v += e.bias[j];
         if (e.res) v += e.res[i * e.ld_res + j];

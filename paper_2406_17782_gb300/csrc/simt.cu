@@ -8,6 +8,7 @@
 
 #include <algorithm>
 
+#include "f32x2.h"
 #include "fabric_internal.h"
 #include "train_common.cuh"
 
@@ -979,34 +980,6 @@ constexpr int kErrBatch2 = 4;   // pair loads in flight per thread (eight withou
 constexpr int kErrPerSm2 = 4;   // resident CTAs per SM
 constexpr int kErrBlocks2 = 152 * kErrPerSm2;   // one wave on 152 SMs
 
-__device__ __forceinline__ uint64_t pk2(float lo, float hi) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-  return r;
-}
-__device__ __forceinline__ void upk2(uint64_t r, float &lo, float &hi) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(r));
-}
-__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
-  uint64_t d;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ uint64_t sub2(uint64_t a, uint64_t b) {
-  uint64_t d;
-  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
-  uint64_t d;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-  return d;
-}
-__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
-  uint64_t d;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-  return d;
-}
 constexpr uint64_t kSign2 = 0x8000000080000000ull;   // both lanes' sign bits
 
 // Packed DFloat: (h, l) += (x, y) per lane, as DFloat::add.

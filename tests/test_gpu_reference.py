@@ -150,3 +150,30 @@ def test_frame_ground_truth_1024spp_subset(fab, frame_mats):
     wc, wr = oracle.shade_reference(frame_mats, W.subset(g, idx), 32, 32, 0x6721, pixel_index=idx)
     assert_close(comps[idx], wc, "comps")
     assert_close(rgb[idx], wr, "rgb")
+
+
+@pytest.mark.parametrize("lanes,n", [(1, 4001), (4, 40007), (32, 45001)])
+def test_mixed_points_of_a_warp(fab, frame_mats, lanes, n):
+    """Points that take different variants of the sample loop (footprints on
+    both sides of half a repeat, nearly opposite directions, a bad material
+    index) interleaved, in grids where a warp integrates one or several
+    points per group of lanes."""
+    g = W.subset(W.frame_gbuffer(), np.arange(7000, 7000 + n))
+    g["radius"] = np.where(np.arange(n) % 3 == 0, g["radius"] * 20.0, g["radius"]).astype(np.float32)
+    opposite = np.arange(n) % 5 == 0
+    g["wi"][opposite] = [0.9, 0.1, 0.42]
+    g["wo"][opposite] = [-0.8, -0.05, 0.6]
+    g["material"] = g["material"].copy()
+    g["material"][11] = 300
+    fab.set_launch_config(0, 0, lanes)
+    try:
+        _, comps = fab.shade_reference(GBuffer.from_numpy(g), 8, 4, 21, comps=True)
+        with pytest.raises(FabricError):
+            fab.sync_status()
+    finally:
+        fab.set_launch_config()
+    c = comps.cpu().numpy()
+    assert np.isnan(c[11]).all()
+    idx = np.concatenate([np.arange(0, 11), np.arange(12, 300), np.arange(n - 200, n)])
+    wc, _ = oracle.shade_reference(frame_mats, W.subset(g, idx), 8, 4, 21, pixel_index=idx)
+    assert_close(c[idx], wc, f"lanes={lanes}")
