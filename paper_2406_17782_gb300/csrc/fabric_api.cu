@@ -123,6 +123,10 @@ bool build_material(const fabric_material &m, DevMaterial *d, std::string *why) 
   if (!check_material(m, why)) return false;
   std::memset(d, 0, sizeof(*d));
   const Weave &w = kWeaves[m.pattern_id];
+  if (w.rows * w.cols > kMaxPatternCells) {
+    *why = "weave has more cells than the material record holds";
+    return false;
+  }
   d->rows = w.rows;
   d->cols = w.cols;
   d->gap_fixed = (uint32_t)std::floor(0.5 * (double)m.gap * 4294967296.0);
@@ -146,7 +150,14 @@ bool build_material(const fabric_material &m, DevMaterial *d, std::string *why) 
   d->crest[1] = (float)((double)m.beta[1] * (1.0 - (double)m.gap) / (2.0 * w.rows));
   const double incl = (double)m.incl_deg * M_PI / 180.0;
   const double lncos = std::log(std::cos(incl));
-  double rise_max = 0.0;
+  double rise_max = 0.0, rise_scale = 0.0;
+  // ln cos(theta) k cells into a float of len cells; a weave has few floats
+  double memo[kMaxPatternDim + 1][kMaxPatternDim + 1] = {};   // 0: not computed (or the value is 0)
+  auto lncos_at = [&](int len, int k) {
+    double &v = memo[len][k];
+    if (v == 0.0) v = std::log(std::cos(incl * (1.0 - 2.0 * k / len)));
+    return v;
+  };
   for (int i = 0; i < w.rows; ++i) {
     for (int j = 0; j < w.cols; ++j) {
       const bool warp = w.cells[i][j] == '1';
@@ -160,13 +171,14 @@ bool build_material(const fabric_material &m, DevMaterial *d, std::string *why) 
         float_run(line, w.cols, j, &len, &off);
       }
       // theta(t) = incl (1 - 2 (off + t) / len) = theta0 - theta1 t
-      WeaveCell &c = d->cell[i * kMaxPatternDim + j];
+      WeaveCell &c = d->cell[i * w.cols + j];
       c.theta0 = (float)(incl * (1.0 - 2.0 * off / len));
       c.theta1 = std::ldexp((float)(2.0 * incl / len), -32);
       // the float's rise, the integral of tan(theta) along it:
       // (ln cos theta(t) - ln cos incl) / (theta1 N_along)
       const int n_along = warp ? w.rows : w.cols;
       c.rise = incl != 0.0 ? (float)(len / (2.0 * incl * n_along)) : 0.0f;
+      rise_scale = std::max(rise_scale, std::fabs((double)c.rise));
       if (incl > 0.0) rise_max = std::max(rise_max, len / (double)n_along * -lncos / (2.0 * incl));
       // the cell's largest height: the crest and the rise at its ends or at
       // theta = 0 where that lies inside, enlarged past the rounding of the
@@ -174,8 +186,7 @@ bool build_material(const fabric_material &m, DevMaterial *d, std::string *why) 
       double rise_top = 0.0;
       if (incl != 0.0) {
         const double scale = len / (2.0 * incl * n_along), t_level = (len - 2.0 * off) / 2.0;
-        double best = std::max(scale * (std::log(std::cos(incl * (1.0 - 2.0 * off / len))) - lncos),
-                               scale * (std::log(std::cos(incl * (1.0 - 2.0 * (off + 1.0) / len))) - lncos));
+        double best = std::max(scale * (lncos_at(len, off) - lncos), scale * (lncos_at(len, off + 1) - lncos));
         if (t_level > 0.0 && t_level < 1.0) best = std::max(best, scale * -lncos);
         rise_top = best + 1e-5 * std::fabs(scale * lncos) + 1e-5 * std::fabs(scale);
       }
@@ -185,6 +196,12 @@ bool build_material(const fabric_material &m, DevMaterial *d, std::string *why) 
   }
   d->lncos_incl = (float)lncos;
   d->h_max = (float)(std::max((double)d->crest[0], (double)d->crest[1]) + rise_max);
+  // The march's height against surface_height: the cosine of the profile's
+  // angle by its series (argument and series within 4e-7, as cosf's argument
+  // is), and ln cos(theta) from the hardware cosine (2^-20.5 absolute) and
+  // logarithm (about 2^-22 relative or absolute), five times over.
+  d->v_margin = (float)(4e-6 * std::max(d->crest[0], d->crest[1]) +
+                        rise_scale * (4e-6 / std::cos(incl) + 8e-6));
   d->v_delta = (float)(1.0 / (16.0 * std::max(w.rows, w.cols)));
   return true;
 }

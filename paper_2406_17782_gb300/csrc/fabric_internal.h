@@ -86,6 +86,7 @@ constexpr int kNumWeaves = 12;      // built-in weave tables
 constexpr int kEncIn = kPatternSlots + 6;
 constexpr int kEncHidden = 128;
 constexpr int kMaxPatternDim = 16;
+constexpr int kMaxPatternCells = 64;   // the 8 x 8 weaves
 
 // flat decoder parameter offsets (weights [out][in])
 constexpr int kOffW1 = 0;
@@ -144,8 +145,9 @@ struct alignas(16) DevMaterial {
   float lncos_incl;                    // ln cos(inclination)
   float h_max;                         // largest surface height (repeat units)
   float v_delta;                       // horizontal march step: 1 / (16 max(rows, cols)) repeats
-  float pad1[3];
-  WeaveCell cell[kMaxPatternDim * kMaxPatternDim];
+  float v_margin;                      // bound on |hardware-function height - surface_height| (reference.cu)
+  float pad1[2];
+  WeaveCell cell[kMaxPatternCells];    // cell (i, j) at i cols + j
 };
 
 // One segment of a batched draw, as the kernel reads it.

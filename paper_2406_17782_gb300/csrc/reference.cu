@@ -54,6 +54,16 @@ __device__ __forceinline__ float sin_half_pi(float x) {
   p = fmaf(p, x2, -1.6666666666666666e-01f);
   return fmaf(p * x2, x, x);
 }
+__device__ __forceinline__ float cos_half_pi(float x) {
+  const float x2 = x * x;
+  float p = 2.08767569878681e-09f;       // 1/12!
+  p = fmaf(p, x2, -2.755731922398589e-07f);
+  p = fmaf(p, x2, 2.48015873015873e-05f);
+  p = fmaf(p, x2, -1.388888888888889e-03f);
+  p = fmaf(p, x2, 4.1666666666666664e-02f);
+  p = fmaf(p, x2, -0.5f);
+  return fmaf(p, x2, 1.0f);
+}
 // Both of one angle: the two series side by side in the packed lanes.
 __device__ __forceinline__ void sincos_half_pi(float x, float &sn, float &cs) {
   const float x2 = x * x;
@@ -81,6 +91,16 @@ __device__ __forceinline__ float sqrt_hw(float x) {
   asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
   return r;
 }
+__device__ __forceinline__ float lg2_hw(float x) {
+  float r;
+  asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ float cos_hw(float x) {
+  float r;
+  asm("cos.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
 __device__ __forceinline__ float ex2_hw(float x) {
   float r;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
@@ -97,6 +117,7 @@ struct PointMaterial {
   const DevMaterial *m;
   uint32_t rows, cols, gap, gap_span;   // gap_span: 2^32 - 1 - 2 gap, the body's extent past the gap
   float inv_1mg, cos_psi, sin_psi;
+  float one_mg;                         // 1 - gap: the body's half width in cell units of [-1, 1]
   float across_mul, across_off;         // pi x / 2 = across_mul * (0.32 fixed point) - across_off
 };
 
@@ -131,7 +152,7 @@ struct CellHit {
 __device__ __forceinline__ CellHit locate(const PointMaterial &pm, uint32_t pu, uint32_t pv) {
   const uint32_t j = __umulhi(pu, pm.cols), su = pu * pm.cols;
   const uint32_t i = __umulhi(pv, pm.rows), sv = pv * pm.rows;
-  const float4 q = __ldg(reinterpret_cast<const float4 *>(pm.m->cell) + (i * kMaxPatternDim + j));
+  const float4 q = __ldg(reinterpret_cast<const float4 *>(pm.m->cell) + (i * pm.cols + j));
   CellHit h;
   h.c.theta0 = q.x;
   h.c.theta1 = q.y;
@@ -160,26 +181,113 @@ __device__ __forceinline__ float surface_height(const PointMaterial &pm, uint32_
   return __ldg(&pm.m->crest[q.warp_top ? 1 : 0]) * (cosf(x * (0.5f * kPi)) - 1.0f);
 }
 
-__device__ bool visible(const PointMaterial &pm, uint32_t pu, uint32_t pv, float3 w) {
-  if (!(w.z > 0.0f)) return false;
+// One direction's march, prepared once per point.  steps: -1 at or below the
+// horizon (never visible), 0 straight up (always visible), else 1.
+struct alignas(16) MarchDir {
+  uint32_t inc_u, inc_v;         // position increments, 0.32 fixed point
+  float dz;                      // height gained per step
+  float cell_u, cell_v;          // just under 1 / (local cell coordinate per step), for skipping
+  int steps;
+  int pad[2];
+};
+
+__device__ __forceinline__ MarchDir march_dir(const DevMaterial *__restrict__ m, float3 w) {
+  MarchDir d = {};
+  d.steps = -1;
+  if (!(w.z > 0.0f)) return d;
   const float rho2 = w.x * w.x + w.y * w.y;
-  if (rho2 == 0.0f) return true;
+  d.steps = 0;
+  if (rho2 == 0.0f) return d;
+  d.steps = 1;
   const float rho = sqrtf(rho2);
-  const float delta = __ldg(&pm.m->v_delta);
-  const uint32_t inc_u = (uint32_t)(unsigned long long)__float2ll_rn(w.x / rho * delta * 4294967296.0f);
-  const uint32_t inc_v = (uint32_t)(unsigned long long)__float2ll_rn(w.y / rho * delta * 4294967296.0f);
-  const float dz = delta * (w.z / rho);
-  const float h0 = surface_height(pm, pu, pv);
-  const float span = (__ldg(&pm.m->h_max) - h0) / dz;
+  const float delta = m->v_delta;
+  d.inc_u = (uint32_t)(unsigned long long)__float2ll_rn(w.x / rho * delta * 4294967296.0f);
+  d.inc_v = (uint32_t)(unsigned long long)__float2ll_rn(w.y / rho * delta * 4294967296.0f);
+  d.dz = delta * (w.z / rho);
+  // |increment| * cells <= 2^28, since delta is a sixteenth of the finer cell
+  const int du = abs((int)(d.inc_u * m->cols)), dv = abs((int)(d.inc_v * m->rows));
+  d.cell_u = du ? 0.999999f / (float)du : 3.0e38f;
+  d.cell_v = dv ? 0.999999f / (float)dv : 3.0e38f;
+  return d;
+}
+
+// The state of a march between its steps.
+struct March {
+  uint32_t qu, qv;               // position of the last step
+  int k, K;                      // steps taken, and in all
+  float h0;
+  MarchDir d;
+};
+
+__device__ __forceinline__ void march_start(March &r, const DevMaterial *__restrict__ m, const MarchDir &d, uint32_t pu,
+                                            uint32_t pv, float h0) {
+  r.qu = pu;
+  r.qv = pv;
+  r.k = 0;
+  r.h0 = h0;
+  r.d = d;
+  const float span = (__ldg(&m->h_max) - h0) / d.dz;
   int K = span < (float)kVisMaxSteps ? (int)floorf(span) + 1 : kVisMaxSteps;
   if (K < 1) K = 1;
-  uint32_t qu = pu, qv = pv;
-  for (int k = 1; k <= K; ++k) {
-    qu += inc_u;
-    qv += inc_v;
-    if (surface_height(pm, qu, qv) > h0 + (float)k * dz) return false;
+  r.K = d.steps > 0 ? K : 0;
+}
+
+// One step of a march (k < K), or several that cannot meet the surface; true
+// when the surface is above the ray there.  The decision at a step is that of
+// surface_height(q) > h0 + k dz, reached in most cases without it:
+//  - Over a cell the height is at most top_bound - crest xn^2 (xn in [-1, 1]
+//    across the yarn on top; cos(pi xn / 2) <= 1 - xn^2) and at most 0 in the
+//    gaps beyond |xn| = 1.  A ray at z >= 0 outside the band |xn| <
+//    sqrt((top_bound - z) / crest) cannot be below the surface until it
+//    enters the band, which it can only leave narrower since z rises: all
+//    steps up to there, or to the cell's edge, are skipped at once.
+//  - Inside, the height from the hardware cosine and logarithm decides, unless
+//    the ray is within v_margin of it, a bound on its error that the host
+//    computes per material; only there is surface_height evaluated.
+__device__ __forceinline__ bool march_step(March &r, const PointMaterial &pm) {
+  r.qu += r.d.inc_u;
+  r.qv += r.d.inc_v;
+  ++r.k;
+  const float z = fmaf((float)r.k, r.d.dz, r.h0);
+  const uint32_t j = __umulhi(r.qu, pm.cols), su = r.qu * pm.cols;
+  const uint32_t i = __umulhi(r.qv, pm.rows), sv = r.qv * pm.rows;
+  const float4 c = __ldg(reinterpret_cast<const float4 *>(pm.m->cell) + (i * pm.cols + j));
+  const float2 crest = __ldg(reinterpret_cast<const float2 *>(pm.m->crest));
+  const bool warp_top = __float_as_int(c.z) < 0;
+  const uint32_t s_top = warp_top ? su : sv, s_along = warp_top ? sv : su;
+  const float above = fabsf(c.z) - z, crest_top = warp_top ? crest.x : crest.y;
+  const float xs = fmaf((float)s_top, 2.0f * kTwoNeg32, -1.0f);   // [-1, 1] across the cell
+  // half width of the band in xs, enlarged past the rounding here
+  const float band = above > 0.0f
+                         ? fmaf(sqrt_hw(fminf(1.0f, above * rcp_hw(crest_top))), 1.0001f * pm.one_mg, 1e-5f)
+                         : -1.0f;
+  if (z >= 0.0f && fabsf(xs) > band) {
+    const int inc_top = (int)(warp_top ? r.d.inc_u : r.d.inc_v), inc_along = (int)(warp_top ? r.d.inc_v : r.d.inc_u);
+    // 0.32 distances to go: to the band when moving towards it, else to the cell's edge; and to the edge along the yarn
+    const bool towards = band >= 0.0f && (xs > 0.0f) == (inc_top < 0);
+    const float to_edge = (float)(inc_top < 0 ? s_top : ~s_top);
+    const float go_top = towards ? (fabsf(xs) - band) * 2147483648.0f : to_edge;
+    const float go_along = (float)(inc_along < 0 ? s_along : ~s_along);
+    const int n = min(min(__float2int_rz(go_top * (warp_top ? r.d.cell_u : r.d.cell_v)),
+                          __float2int_rz(go_along * (warp_top ? r.d.cell_v : r.d.cell_u))), r.K - r.k);
+    r.qu += (uint32_t)n * r.d.inc_u;
+    r.qv += (uint32_t)n * r.d.inc_v;
+    r.k += n;
+    return false;
   }
-  return true;
+  const bool body = s_top - pm.gap <= pm.gap_span;
+  if (!body && z >= 0.0f) return false;
+  const float xh = fminf(0.5f * kPi, fmaxf(-0.5f * kPi, fmaf((float)(body ? s_top : s_along), pm.across_mul, -pm.across_off)));
+  float h = cos_half_pi(xh);
+  if (body) {
+    h = fmaf(c.w, fmaf(lg2_hw(cos_hw(fmaf(-c.y, (float)s_along, c.x))), 0.6931471805599453f, -__ldg(&pm.m->lncos_incl)),
+             h * crest_top);
+  } else {
+    h = (h - 1.0f) * (warp_top ? crest.y : crest.x);
+  }
+  const float d = h - z;
+  if (fabsf(d) > __ldg(&pm.m->v_margin)) return d > 0.0f;
+  return surface_height(pm, r.qu, r.qv) > z;
 }
 
 // The integrand of Eq. 3-5 at one sample.  With hc the height profile's
@@ -260,21 +368,6 @@ __device__ __forceinline__ void accumulate(const Shaded &r, Sums &acc) {
   }
 }
 
-template <bool VIS, bool OPPOSITE>
-__device__ __forceinline__ void shade_sample(const PointMaterial &pm, const PointDirs &d, uint32_t pu, uint32_t pv,
-                                             Sums &acc) {
-  const Shaded r = shade<OPPOSITE>(pm, d, pu, pv);
-  if (VIS && r.coJ > 0.0f) {
-    // V(x_p, wo) weighs A and the numerators; V(x_p, wi) only matters with <wi.n_p> > 0
-    if (!visible(pm, pu, pv, d.wo)) return;
-    acc.a += r.coJ;
-    if (r.ci_pos && !visible(pm, pu, pv, d.wi)) return;
-  } else {
-    acc.a += r.coJ;                                    // A of Eq. 4
-  }
-  accumulate(r, acc);
-}
-
 struct RefArgs {
   const float *u, *v, *radius, *wi, *wo;
   const uint16_t *material;
@@ -283,6 +376,7 @@ struct RefArgs {
   int n_mat;
   int nx, ny;
   int rounds;          // points per group of L lanes
+  int split;           // visibility, L = 32: warps of a CTA that share each point
   float two_over_nx, two_over_ny;
   uint64_t seed;
   float *rgb, *comps;
@@ -337,55 +431,65 @@ __device__ __forceinline__ PointRecord load_point(const RefArgs &a, int64_t p) {
 }
 
 // Stratum (ix, iy) of sample k = iy nx + ix as a packed pair of floats (both
-// below 2^13, exact), stepped by the group's L samples at a time.
+// below 2^13, exact), stepped by the group's `stride` samples at a time.
 struct SamplePlan {
-  int spp;
+  int spp, stride;
   uint64_t first, step, wrap, two_over_n;
   float nx;
 };
 
-// Lane lane_g's samples of one point.  WIDE: footprints of any size (64-bit
-// conversions); OPPOSITE: directions that may be nearly opposite.
-template <int L, bool VIS, bool WIDE, bool OPPOSITE>
-__device__ __forceinline__ void integrate(const RefArgs &a, const PointRecord &R, const SamplePlan &sp, int lane_g,
-                                          Sums &acc) {
+// One point as its samples read it, and lane lane_g's place in its sequence.
+// WIDE: footprints of any size (64-bit conversions).
+template <bool WIDE>
+struct PointSampler {
   PointMaterial pm;
-  pm.m = a.mats + R.mat;
-  const uint4 m0 = __ldg(reinterpret_cast<const uint4 *>(pm.m));
-  const float4 m1 = __ldg(reinterpret_cast<const float4 *>(pm.m) + 1);
-  pm.rows = m0.x;
-  pm.cols = m0.y;
-  pm.gap = m0.z;
-  pm.gap_span = 0xFFFFFFFFu - 2u * pm.gap;
-  pm.inv_1mg = m1.x;
-  pm.cos_psi = m1.y;
-  pm.sin_psi = m1.z;
-  pm.across_off = 0.5f * kPi * m1.x;
-  pm.across_mul = pm.across_off * (2.0f * kTwoNeg32);
   PointDirs d;
-  d.wi = make_float3(R.wi_x, R.wi_y, R.wi_z);
-  d.wo = make_float3(R.wo_x, R.wo_y, R.wo_z);
-  d.h_inv = R.h_inv;
-  d.diff_k = R.diff_k;
-  d.diff_c = R.diff_c;
-  const float r32 = WIDE ? R.r : R.r * 4294967296.0f;   // a power of two: exact
-  const uint64_t hp = R.hash, rr = pk2(r32, r32);
-  const uint32_t cu = R.cu, cv = R.cv;
-  const uint64_t minus1 = pk2(-1.0f, -1.0f), xi_scale = pk2(5.9604644775390625e-08f, 5.9604644775390625e-08f);   // 2^-24
-  uint64_t strat = sp.first;
-  for (int k = lane_g; k < sp.spp; k += L) {
+  uint64_t hp, rr, strat;
+  uint32_t cu, cv;
+  int k;
+
+  __device__ __forceinline__ PointSampler(const RefArgs &a, const PointRecord &R, const SamplePlan &sp, int first) {
+    pm.m = a.mats + max(R.mat, 0);
+    const uint4 m0 = __ldg(reinterpret_cast<const uint4 *>(pm.m));
+    const float4 m1 = __ldg(reinterpret_cast<const float4 *>(pm.m) + 1);
+    pm.rows = m0.x;
+    pm.cols = m0.y;
+    pm.gap = m0.z;
+    pm.gap_span = 0xFFFFFFFFu - 2u * pm.gap;
+    pm.inv_1mg = m1.x;
+    pm.cos_psi = m1.y;
+    pm.sin_psi = m1.z;
+    pm.one_mg = 1.0f / m1.x;
+    pm.across_off = 0.5f * kPi * m1.x;
+    pm.across_mul = pm.across_off * (2.0f * kTwoNeg32);
+    d.wi = make_float3(R.wi_x, R.wi_y, R.wi_z);
+    d.wo = make_float3(R.wo_x, R.wo_y, R.wo_z);
+    d.h_inv = R.h_inv;
+    d.diff_k = R.diff_k;
+    d.diff_c = R.diff_c;
+    hp = R.hash;
+    const float r32 = WIDE ? R.r : R.r * 4294967296.0f;   // a power of two: exact
+    rr = pk2(r32, r32);
+    cu = R.cu;
+    cv = R.cv;
+    strat = sp.first;
+    k = first;
+  }
+
+  // The position of sample k; moves on to sample k + stride.
+  __device__ __forceinline__ void next(const SamplePlan &sp, uint32_t &pu, uint32_t &pv) {
     const uint64_t hk = splitmix_finalise(hp + (uint64_t)k);
     // ((k + xi) (2/n) - 1) r, rounded at every step as the oracle rounds it
     // (xi has 24 bits, so the product of the fma is exact)
     const uint64_t xi = pk2((float)(uint32_t)(hk >> 40), (float)(uint32_t)((hk >> 16) & 0xFFFFFFu));
+    const uint64_t minus1 = pk2(-1.0f, -1.0f), xi_scale = pk2(5.9604644775390625e-08f, 5.9604644775390625e-08f);   // 2^-24
     const uint64_t t = mul2(add2(mul2(fma2(xi, xi_scale, strat), sp.two_over_n), minus1), rr);
     float ou, ov;
     upk2(t, ou, ov);
-    uint32_t pu, pv;
     if (WIDE) {
       pu = cu + (uint32_t)(unsigned long long)__float2ll_rn(__fmul_rn(ou, 4294967296.0f));
       pv = cv + (uint32_t)(unsigned long long)__float2ll_rn(__fmul_rn(ov, 4294967296.0f));
-    } else {   // r32 carries the 2^32, |offset| < 2^31: one 32-bit conversion
+    } else {   // rr carries the 2^32, |offset| < 2^31: one 32-bit conversion
       pu = cu + (uint32_t)__float2int_rn(ou);
       pv = cv + (uint32_t)__float2int_rn(ov);
     }
@@ -393,7 +497,81 @@ __device__ __forceinline__ void integrate(const RefArgs &a, const PointRecord &R
     float ix, iy;
     upk2(strat, ix, iy);
     if (ix >= sp.nx) strat = add2(strat, sp.wrap);
-    shade_sample<VIS, OPPOSITE>(pm, d, pu, pv, acc);
+    k += sp.stride;
+  }
+};
+
+// Lane lane_g's samples of one point, V = 1.  OPPOSITE: directions that may
+// be nearly opposite.
+template <bool WIDE, bool OPPOSITE>
+__device__ __forceinline__ void integrate(const RefArgs &a, const PointRecord &R, const SamplePlan &sp, int lane_g,
+                                          Sums &acc) {
+  PointSampler<WIDE> s(a, R, sp, lane_g);
+  while (s.k < sp.spp) {
+    uint32_t pu, pv;
+    s.next(sp, pu, pv);
+    const Shaded r = shade<OPPOSITE>(s.pm, s.d, pu, pv);
+    acc.a += r.coJ;                                    // A of Eq. 4
+    accumulate(r, acc);
+  }
+}
+
+// The same with the visibility model: V(x_p, wo) weighs A and the numerators,
+// V(x_p, wi) the numerators (and is not marched with <wi.n_p> = 0).  Marches
+// differ in length from lane to lane, from one step to hundreds, so the
+// lanes are not kept in step: each takes its samples in order on its own.
+// While most lanes are marching the warp steps their marches; when kRefill of
+// them have none, those shade their next sample first.  Each lane's sums run
+// in sample order whatever the others do.  1080p frame at 256 spp: 59.8 ms
+// with the lanes in step and every height evaluated; with this loop and
+// march_step's skipping 25.6 ms at kRefill = 8 and three CTAs per SM, 21.8 ms
+// at 20 and four (starting the second march only together with the next
+// samples: 23.6 ms).
+constexpr int kRefill = 20;
+
+__device__ __forceinline__ void integrate_visible(const RefArgs &a, const PointRecord &R, const MarchDir &to_i,
+                                                  const MarchDir &to_o, const SamplePlan &sp, int first, Sums &acc) {
+  PointSampler<true> s(a, R, sp, first);
+  const int spp = R.mat >= 0 && to_o.steps >= 0 ? sp.spp : 0;   // wo below the horizon: every term is zero
+  Shaded r = {};
+  March m = {};
+  uint32_t pu = 0, pv = 0;
+  bool marching = false, on_wi = false;
+  for (;;) {
+    if (!marching && s.k < spp) {
+      s.next(sp, pu, pv);
+      r = shade<true>(s.pm, s.d, pu, pv);
+      if (r.coJ > 0.0f) {
+        march_start(m, s.pm.m, to_o, pu, pv, surface_height(s.pm, pu, pv));
+        marching = true;
+        on_wi = false;
+      }
+    }
+    const unsigned busy = __ballot_sync(0xFFFFFFFFu, marching), left = __ballot_sync(0xFFFFFFFFu, s.k < spp);
+    if (!(busy | left)) break;
+    const int enough = min(kRefill, __popc(left));
+    for (;;) {
+      if (marching) {
+        if (m.k < m.K && march_step(m, s.pm)) {
+          marching = false;                             // hidden
+        } else if (m.k >= m.K) {                        // above the surface all the way
+          marching = false;
+          if (!on_wi) {
+            acc.a += r.coJ;                             // A of Eq. 4
+            if (!r.ci_pos) {
+              accumulate(r, acc);
+            } else if (to_i.steps >= 0) {
+              march_start(m, s.pm.m, to_i, pu, pv, m.h0);
+              marching = on_wi = true;
+            }
+          } else {
+            accumulate(r, acc);
+          }
+        }
+      }
+      const unsigned now = __ballot_sync(0xFFFFFFFFu, marching);
+      if (now == 0 || (left && __popc(left & ~now) >= enough)) break;
+    }
   }
 }
 
@@ -412,24 +590,40 @@ __global__ void __launch_bounds__(kRefThreads, 4) reference_kernel(const RefArgs
   // a lane that integrates its own point keeps everything in registers
   constexpr bool kStaged = L > 1;
   __shared__ PointRecord recs[kStaged ? kRefWarps : 1][kStaged ? 32 : 1];
+  __shared__ MarchDir dirs[2][VIS && kStaged ? kRefWarps : 1][VIS && kStaged ? 32 : 1];
   __shared__ float sums[kStaged ? kRefWarps : 1][5][kStaged ? 32 : 1];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int lane_g = lane & (L - 1), group = lane / L;
   const int n_pts = G * a.rounds;
-  const int64_t p0 = ((int64_t)blockIdx.x * kRefWarps + warp) * n_pts;
+  // warps part, part + 1, ... of `split` share their points, each taking every split-th 32 samples
+  const int split = VIS && L == 32 ? a.split : 1, part = warp % split;
+  const int64_t p0 = ((int64_t)blockIdx.x * (kRefWarps / split) + warp / split) * n_pts;
   PointRecord own;
   own.mat = -1;
   own.r = own.h_inv = 0.0f;
   if (lane < n_pts && p0 + lane < a.n) own = load_point(a, p0 + lane);
+  MarchDir own_i = {}, own_o = {};
+  if (VIS && own.mat >= 0) {
+    own_i = march_dir(a.mats + own.mat, make_float3(own.wi_x, own.wi_y, own.wi_z));
+    own_o = march_dir(a.mats + own.mat, make_float3(own.wo_x, own.wo_y, own.wo_z));
+  }
   if (kStaged) {
-    if (lane < n_pts) recs[warp][lane] = own;
+    if (lane < n_pts) {
+      recs[warp][lane] = own;
+      if (VIS) {
+        dirs[0][warp][lane] = own_i;
+        dirs[1][warp][lane] = own_o;
+      }
+    }
     __syncwarp();
   }
   SamplePlan sp;
   sp.spp = a.nx * a.ny;
-  sp.step = pk2((float)(L % a.nx), (float)(L / a.nx));
+  sp.stride = L * split;
+  sp.step = pk2((float)(sp.stride % a.nx), (float)(sp.stride / a.nx));
   sp.wrap = pk2(-(float)a.nx, 1.0f);
-  sp.first = pk2((float)(lane_g % a.nx), (float)(lane_g / a.nx));
+  const int first = lane_g + L * part;
+  sp.first = pk2((float)(first % a.nx), (float)(first / a.nx));
   sp.two_over_n = pk2(a.two_over_nx, a.two_over_ny);
   sp.nx = (float)a.nx;
   Sums total = {0.f, 0.f, 0.f, 0.f, 0.f};
@@ -437,16 +631,18 @@ __global__ void __launch_bounds__(kRefThreads, 4) reference_kernel(const RefArgs
     const int pt = round * G + group;
     Sums acc = {0.f, 0.f, 0.f, 0.f, 0.f};
     const PointRecord &R = kStaged ? recs[warp][pt] : own;
-    // The loop's variant is chosen for the whole warp, so that its groups stay
+    // V = 1: the loop's variant is chosen for the whole warp, so that its groups stay
     // together: with one point per warp both tests are taken out of the
     // loop (about six instructions a sample), with several only the width
     // (points with |wi + wo| < 1 are a few in a hundred, so most warps of
     // eight or more points hold one).
-    const bool narrow = R.mat < 0 || fabsf(R.r) < kSmallRadius;
-    if (__all_sync(0xFFFFFFFFu, narrow && (L < 32 || R.mat < 0 || R.h_inv <= 1.0f))) {
-      if (R.mat >= 0) integrate<L, VIS, false, (L < 32)>(a, R, sp, lane_g, acc);
+    if (VIS) {
+      if (kStaged) integrate_visible(a, R, dirs[0][warp][pt], dirs[1][warp][pt], sp, first, acc);
+      else integrate_visible(a, R, own_i, own_o, sp, first, acc);
+    } else if (__all_sync(0xFFFFFFFFu, R.mat < 0 || (fabsf(R.r) < kSmallRadius && (L < 32 || R.h_inv <= 1.0f)))) {
+      if (R.mat >= 0) integrate<false, (L < 32)>(a, R, sp, lane_g, acc);
     } else {
-      if (R.mat >= 0) integrate<L, VIS, true, true>(a, R, sp, lane_g, acc);
+      if (R.mat >= 0) integrate<true, true>(a, R, sp, lane_g, acc);
     }
     __syncwarp();
     // reduction inside each group of L lanes
@@ -469,10 +665,19 @@ __global__ void __launch_bounds__(kRefThreads, 4) reference_kernel(const RefArgs
     }
   }
   const int64_t p = p0 + lane;
-  if (kStaged) __syncwarp();
-  if (lane >= n_pts || p >= a.n) return;
+  if (split > 1) __syncthreads();
+  else if (kStaged) __syncwarp();
+  if (lane >= n_pts || p >= a.n || part != 0) return;
   const int mat = own.mat;
-  if (kStaged) total = {sums[warp][0][lane], sums[warp][1][lane], sums[warp][2][lane], sums[warp][3][lane], sums[warp][4][lane]};
+  if (kStaged) {
+    for (int w = warp; w < warp + split; ++w) {
+      total.c0 += sums[w][0][lane];
+      total.c1 += sums[w][1][lane];
+      total.s0 += sums[w][2][lane];
+      total.s1 += sums[w][3][lane];
+      total.a += sums[w][4][lane];
+    }
+  }
   float c[4], rgb[3];
   if (mat < 0) {
     c[0] = c[1] = c[2] = c[3] = rgb[0] = rgb[1] = rgb[2] = __int_as_float(0x7FC00000);
@@ -510,7 +715,14 @@ void launch_lanes(const RefArgs &a, unsigned blocks, bool visibility, cudaStream
 // 0.105 with 4).  Small G-buffers take more lanes, until the resident
 // threads (1024 per SM) are used twice.
 int reference_lanes(int64_t n, int spp, bool visibility, int sm_count) {
-  if (visibility) return spp >= 256 ? 32 : spp >= 64 ? 16 : spp >= 16 ? 8 : spp >= 4 ? 4 : 1;
+  if (visibility) {
+    // as many lanes as there are samples: the marches' lengths vary most from
+    // point to point, and a warp with several points waits for the longest
+    // (1080p, 64 spp: 5.7 ms with 32 lanes, 8.2 with 16, 13.5 with 4)
+    int L = 1;
+    while (L < 32 && 2 * L <= spp) L *= 2;
+    return L;
+  }
   int L = spp >= 256 ? 32 : spp >= 32 ? 4 : 1;
   const int64_t threads = (int64_t)(sm_count > 0 ? sm_count : 148) * 2048;
   while (L < 32 && 2 * L <= spp && n * L < threads) L *= 2;
@@ -543,7 +755,19 @@ cudaError_t launch_reference(const fabric_gbuffer &g, const DevMaterial *mats, i
   const int L = lanes_per_point, G = 32 / L;
   const int64_t groups = (g.n + G - 1) / G, resident = (int64_t)(sm_count > 0 ? sm_count : 148) * 32;
   a.rounds = (int)std::max<int64_t>(1, std::min<int64_t>(L, groups / (2 * resident)));
-  const int64_t per_cta = (int64_t)kRefWarps * G * a.rounds;
+  // With the visibility model one point's marches can outlast the rest of the
+  // grid (grazing directions over wide footprints), so several warps share a
+  // point once each lane still has a few samples: 8190 queries at 2048 spp
+  // 2.9 ms with one warp a point, 1.6 with 4, 1.3 with 8; 4000 points at 1024
+  // spp 0.95, 0.35, 0.27 ms; 30 000 at 256 spp 1.15, 0.79, 0.79 ms.  Large grids
+  // at 256 spp hide the long points and keep one warp (2.07 M points 21.8 ms,
+  // 27.5 with 4; 300 000 points the same with either), as 64 spp does (60 000
+  // points 0.30 ms, 0.49 with 4); at 1024 spp 8 warps cost a large grid nothing
+  // (2.07 M points 84.1 and 85.6 ms; 100 000 points 8.5 and 7.0 ms).
+  const int spp = spp_x * spp_y;
+  a.split = !visibility || L < 32 ? 1 : spp >= 1024 ? 8 : spp >= 256 && g.n < 64 * resident ? 4 : 1;
+  if (a.split > 1) a.rounds = 1;
+  const int64_t per_cta = (int64_t)(kRefWarps / a.split) * G * a.rounds;
   const unsigned blocks = (unsigned)((g.n + per_cta - 1) / per_cta);
   switch (L) {
     case 1: launch_lanes<1>(a, blocks, visibility, s); break;

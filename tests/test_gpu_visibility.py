@@ -96,3 +96,33 @@ def test_visibility_on_degenerate_inputs(fab):
         check(rgb, wr, amb, "degenerate rgb", max_amb=0.05)
     finally:
         fab.set_materials(W.frame_materials())
+
+
+@pytest.mark.parametrize("sx,sy,n,lanes", [(1, 1, 700, 0), (3, 3, 300, 0), (5, 7, 200, 16), (16, 16, 90, 0), (32, 32, 40, 0),
+                                           (33, 32, 37, 8)])
+def test_visibility_lane_groupings(fab, sx, sy, n, lanes):
+    """Every split of a point's samples over lanes and warps (one lane, a
+    group, a warp, four and eight warps), ragged counts, a bad material index
+    and directions at and below the horizon and straight up."""
+    mats = W.frame_materials()
+    fab.set_materials(mats)
+    g = W.subset(W.multiscale_gbuffer(), W.sample_indices(1920 * 1080, n, stream=f"vis-lanes-{sx}-{sy}"))
+    g["wo"][3] = [0.6, 0.0, -0.8]
+    g["wi"][4] = [1.0, 0.0, 0.0]
+    g["wi"][5] = [0.0, 0.0, 1.0]
+    g["material"] = g["material"].copy()
+    g["material"][7] = 99
+    fab.set_launch_config(0, 0, lanes)
+    fab.set_visibility(True)
+    try:
+        _, comps = fab.shade_reference(GBuffer.from_numpy(g), sx, sy, 5, comps=True)
+        with pytest.raises(FabricError):
+            fab.sync_status()
+    finally:
+        fab.set_visibility(False)
+        fab.set_launch_config()
+    c = comps.cpu().numpy()
+    assert np.isnan(c[7]).all()
+    idx = np.delete(np.arange(n), 7)
+    wc, _, amb = oracle.shade_reference(mats, W.subset(g, idx), sx, sy, 5, pixel_index=idx, visibility=True)
+    check(c[idx], wc, amb, f"{sx}x{sy}")
