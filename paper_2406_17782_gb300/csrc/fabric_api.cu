@@ -625,7 +625,7 @@ fabric_status fabric_shade_neural_prepared(fabric_ctx *ctx, const fabric_gbuffer
   if (prec == FABRIC_PREC_FP32) {
     FAB_CUDA(ctx,
              launch_decoder_fp32(*g, ctx->d_mat, ctx->n_mat, ctx->prepared_latents, ctx->d_dec, rgb_dev, comps_dev,
-                                 nullptr, ctx->d_status, s),
+                                 nullptr, ctx->d_status, ctx->sm_count, s),
              "fp32 decoder launch");
     return FABRIC_OK;
   }

@@ -258,7 +258,7 @@ cudaError_t launch_reference(const fabric_gbuffer &g, const DevMaterial *mats, i
                              uint64_t seed, float *rgb, float *comps, int *status, int lanes_per_point,
                              int sm_count, cudaStream_t s, bool visibility = false);
 cudaError_t launch_decoder_fp32(const fabric_gbuffer &g, const DevMaterial *mats, int n_mat, const float *latents,
-                                const float *dec, float *rgb, float *comps, float *y_raw, int *status,
+                                const float *dec, float *rgb, float *comps, float *y_raw, int *status, int sm_count,
                                 cudaStream_t s);
 size_t tc_blob_bytes(int n_mat);
 int tc_k1(int n_mat);
@@ -298,7 +298,7 @@ size_t encoder_backward_work_floats(int n);
 cudaError_t launch_encoder_raw(const fabric_material *raw, int n, const float *enc, float *feats_out, float *z,
                                float *acts, cudaStream_t s);
 cudaError_t launch_decoder_raw(const fabric_gbuffer &g, const float *latents, int n_lat, const float *dec,
-                               float *y_raw, int *status, cudaStream_t s);
+                               float *y_raw, int *status, int sm_count, cudaStream_t s);
 cudaError_t launch_decoder_backward(const fabric_gbuffer &g, const float *latents, int n_lat, const float *dec,
                                     const float *dy, const float *target, int loss_mode, float *ddec, float *dlat,
                                     double *loss, void *work, int sm_count, int *status, cudaStream_t s);

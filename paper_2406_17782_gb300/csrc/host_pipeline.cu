@@ -119,7 +119,7 @@ extern "C" fabric_status fabric_shade_neural_host(fabric_ctx *ctx, const fabric_
     if (d.u && d.v && d.radius && d.wi && d.wo && d.material && rgb && (comps || !comps_host)) {
       if (prec == FABRIC_PREC_FP32)
         e = launch_decoder_fp32(d, ctx->d_mat, ctx->n_mat, ctx->prepared_latents, ctx->d_dec, rgb, comps, nullptr,
-                                ctx->d_status, caller);
+                                ctx->d_status, ctx->sm_count, caller);
       else
         e = launch_decoder_tc(d, ctx->d_blob, ctx->n_mat, (int)prec, rgb, comps, ctx->d_status, ctx->sm_count,
                               ctx->tc_ctas_per_sm, ctx->tc_warpgroups, ctx->tc_tile_wgs, caller);
@@ -166,7 +166,7 @@ extern "C" fabric_status fabric_shade_neural_host(fabric_ctx *ctx, const fabric_
       return cuda_fail(ctx, e, "host-to-device copy");
     if (prec == FABRIC_PREC_FP32)
       e = launch_decoder_fp32(d, ctx->d_mat, ctx->n_mat, ctx->prepared_latents, ctx->d_dec, rgb, comps, nullptr,
-                              ctx->d_status, s);
+                              ctx->d_status, ctx->sm_count, s);
     else
       e = launch_decoder_tc(d, ctx->d_blob, ctx->n_mat, (int)prec, rgb, comps, ctx->d_status, ctx->sm_count,
                             ctx->tc_ctas_per_sm, ctx->tc_warpgroups, ctx->tc_tile_wgs, s);

@@ -1,6 +1,7 @@
-// simt.cu -- FP32 SIMT kernels: the decoder used as the accuracy anchor, the
-// training forward/backward passes of decoder and encoder (Sec. 4.2-4.3,
-// loss of Eq. 9-11), Adam, and FP64 image-wide error reductions.
+// simt.cu -- FP32 kernels on the CUDA cores: the encoder's forward and
+// backward (Sec. 4.2), the sums over per-CTA gradient partials and per-row
+// latent gradients, Adam, FP64 image-wide error reductions and the dataset
+// shuffle.
 //
 // All reductions run in a fixed order (owner-computes partial sums per CTA,
 // then a fixed-order sum over CTAs), so repeated runs are bitwise identical.
@@ -10,282 +11,11 @@
 
 #include "f32x2.h"
 #include "fabric_internal.h"
-#include "train_common.cuh"
 
 namespace fab {
 namespace {
 
 constexpr float kLeaky = 0.01f;       // encoder residual-block activation slope
-
-// Writes the 71 decoder inputs of point p into x[i * stride + r].
-__device__ __forceinline__ void build_inputs(const fabric_gbuffer &g, int64_t p, const float *lat, float *x,
-                                             int stride, int r) {
-  for (int i = 0; i < kLatent; ++i) x[i * stride + r] = lat[i];
-  float f[16];
-  octaves_accurate(g.u[p], f);
-  for (int i = 0; i < 16; ++i) x[(32 + i) * stride + r] = f[i];
-  octaves_accurate(g.v[p], f);
-  for (int i = 0; i < 16; ++i) x[(48 + i) * stride + r] = f[i];
-  x[64 * stride + r] = (logf(fmaxf(g.radius[p], kRFloor)) - kLogRC0) * kLogRInvC1;
-  for (int i = 0; i < 3; ++i) {
-    x[(65 + i) * stride + r] = g.wi[3 * p + i];
-    x[(68 + i) * stride + r] = g.wo[3 * p + i];
-  }
-}
-
-// ---------------------------------------------------------------------------
-// FP32 decoder forward: one point per thread, weights in shared memory,
-// activations feature-major in shared memory (each thread owns a column).
-// ---------------------------------------------------------------------------
-constexpr int kFwdThreads = 64;
-
-struct FwdArgs {
-  fabric_gbuffer g;
-  const DevMaterial *mats;
-  int n_mat;
-  const float *latents;
-  int n_lat;
-  const float *dec;
-  float *rgb, *comps, *y_raw;
-  int *status;
-};
-
-__device__ __forceinline__ void dense_col(const float *W, const float *b, int n_out, int n_in, const float *in,
-                                          float *out, int t, bool relu) {
-  for (int o = 0; o < n_out; ++o) {
-    float acc = b[o];
-    const float *w = W + o * n_in;
-#pragma unroll 8
-    for (int i = 0; i < n_in; ++i) acc = fmaf(w[i], in[i * kFwdThreads + t], acc);
-    out[o * kFwdThreads + t] = relu ? fmaxf(acc, 0.0f) : acc;
-  }
-}
-
-__global__ void __launch_bounds__(kFwdThreads) decoder_fp32_kernel(const FwdArgs a) {
-  extern __shared__ float sm[];
-  float *W = sm;
-  float *bufA = W + ((kDecParams + 3) & ~3);
-  float *bufB = bufA + kDecIn * kFwdThreads;
-  for (int i = threadIdx.x; i < kDecParams; i += blockDim.x) W[i] = a.dec[i];
-  __syncthreads();
-  const int t = threadIdx.x;
-  const int64_t p = (int64_t)blockIdx.x * kFwdThreads + t;
-  if (p >= a.g.n) return;
-  const int mat = a.g.material[p];
-  const bool need_mat = a.rgb != nullptr;
-  if (mat >= a.n_lat || (need_mat && mat >= a.n_mat)) {
-    atomicOr(a.status, kStatusBadMaterial);
-    const float nan = __int_as_float(0x7FC00000);
-    if (a.y_raw) store_row4(a.y_raw, p, nan, nan, nan, nan);
-    if (a.comps) store_row4(a.comps, p, nan, nan, nan, nan);
-    if (a.rgb)
-      for (int ch = 0; ch < 3; ++ch) a.rgb[3 * p + ch] = nan;
-    return;
-  }
-  build_inputs(a.g, p, a.latents + (int64_t)mat * kLatent, bufA, kFwdThreads, t);
-  dense_col(W + kOffW1, W + kOffB1, kHidden, kDecIn, bufA, bufB, t, true);
-  dense_col(W + kOffW2, W + kOffB2, kHidden, kHidden, bufB, bufA, t, true);
-  dense_col(W + kOffW3, W + kOffB3, kHidden, kHidden, bufA, bufB, t, true);
-  float y[4];
-  for (int k = 0; k < kOut; ++k) {
-    float acc = W[kOffB4 + k];
-    for (int i = 0; i < kHidden; ++i) acc = fmaf(W[kOffW4 + k * kHidden + i], bufB[i * kFwdThreads + t], acc);
-    y[k] = acc;
-  }
-  if (a.y_raw) store_row4(a.y_raw, p, y[0], y[1], y[2], y[3]);
-  const float c0 = fmaxf(0.0f, y[0]), c1 = fmaxf(0.0f, y[1]);
-  const float s0 = fmaxf(0.0f, expm1f(y[2]) / kSpecK), s1 = fmaxf(0.0f, expm1f(y[3]) / kSpecK);
-  if (a.comps) store_row4(a.comps, p, c0, c1, s0, s1);
-  if (a.rgb) {
-    const DevMaterial &m = a.mats[mat];
-    for (int ch = 0; ch < 3; ++ch)
-      a.rgb[3 * p + ch] = m.kd[0][ch] * c0 + m.kd[1][ch] * c1 + m.ks[0][ch] * s0 + m.ks[1][ch] * s1;
-  }
-}
-
-// ---------------------------------------------------------------------------
-// Decoder forward + backward over tiles of kTR rows (kBwdThreads per CTA).
-// Either dy is given, or it comes from the Eq. 11 loss against `target`.
-// Per-CTA parameter-gradient partials stay in shared memory and are written
-// out once; dlat_rows receives each row's gradient w.r.t. its latent.
-// ---------------------------------------------------------------------------
-constexpr int kTR = 32;
-constexpr int kBwdThreads = 256;
-constexpr int kBwdWarps = kBwdThreads / 32;
-constexpr int kRS = kTR + 1;   // row stride (bank-conflict padding)
-
-struct BwdArgs {
-  fabric_gbuffer g;
-  const float *latents;
-  int n_lat;
-  const float *dec;
-  const float *dy;       // [n][4] or null
-  const float *target;   // [n][4] or null
-  int loss_mode;         // FABRIC_LOSS_EQ11 or FABRIC_LOSS_RENDERED
-  float inv_batch;       // 1/B for the loss
-  float *partial;        // [grid][kDecParams]
-  double *loss_partial;  // [grid]
-  float *dlat_rows;      // [n][32]
-  int *status;
-};
-
-__device__ __forceinline__ void layer_fwd(const float *W, const float *b, int n_out, int n_in, const float *in,
-                                          bool relu_in, float *out) {
-  // thread -> (output group, row): row r = lane, outputs o = og, og + kBwdWarps, ...
-  const int r = threadIdx.x & 31, og = threadIdx.x >> 5;
-  for (int o = og; o < n_out; o += kBwdWarps) {
-    float acc = b[o];
-    const float *w = W + o * n_in;
-    for (int i = 0; i < n_in; ++i) {
-      float v = in[i * kRS + r];
-      if (relu_in) v = fmaxf(v, 0.0f);
-      acc = fmaf(w[i], v, acc);
-    }
-    out[o * kRS + r] = acc;
-  }
-}
-
-// din[i][r] = (sum_o W[o][i] dout[o][r]) * (mask ? (pre[i][r] > 0) : 1)
-__device__ __forceinline__ void layer_bwd_input(const float *W, int n_out, int n_in, const float *dout,
-                                                const float *pre, float *din, int i_limit) {
-  const int r = threadIdx.x & 31, ig = threadIdx.x >> 5;
-  for (int i = ig; i < i_limit; i += kBwdWarps) {
-    float acc = 0.0f;
-    for (int o = 0; o < n_out; ++o) acc = fmaf(W[o * n_in + i], dout[o * kRS + r], acc);
-    if (pre) acc = pre[i * kRS + r] > 0.0f ? acc : 0.0f;
-    din[i * kRS + r] = acc;
-  }
-}
-
-// dW[o][i] += sum_r dout[o][r] * act(in[i][r]); db[o] += sum_r dout[o][r].
-// Owner computes: thread t owns 4x4 blocks (o0..o0+3, i0..i0+3).
-__device__ __forceinline__ void layer_bwd_weights(float *dW, float *db, int n_out, int n_in, const float *dout,
-                                                  const float *in, bool relu_in) {
-  const int ob = (n_out + 3) / 4, ib = (n_in + 3) / 4;
-  for (int blk = threadIdx.x; blk < ob * ib; blk += kBwdThreads) {
-    const int o0 = (blk / ib) * 4, i0 = (blk % ib) * 4;
-    float acc[4][4] = {};
-    for (int r = 0; r < kTR; ++r) {
-      float d[4], x[4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        d[q] = (o0 + q < n_out) ? dout[(o0 + q) * kRS + r] : 0.0f;
-        float v = (i0 + q < n_in) ? in[(i0 + q) * kRS + r] : 0.0f;
-        x[q] = relu_in ? fmaxf(v, 0.0f) : v;
-      }
-#pragma unroll
-      for (int q = 0; q < 4; ++q)
-#pragma unroll
-        for (int s = 0; s < 4; ++s) acc[q][s] = fmaf(d[q], x[s], acc[q][s]);
-    }
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
-#pragma unroll
-      for (int s = 0; s < 4; ++s)
-        if (o0 + q < n_out && i0 + s < n_in) dW[(o0 + q) * n_in + i0 + s] += acc[q][s];
-  }
-  for (int o = threadIdx.x; o < n_out; o += kBwdThreads) {
-    float acc = 0.0f;
-    for (int r = 0; r < kTR; ++r) acc += dout[o * kRS + r];
-    db[o] += acc;
-  }
-}
-
-__global__ void __launch_bounds__(kBwdThreads) decoder_bwd_kernel(const BwdArgs a) {
-  extern __shared__ float sm[];
-  float *W = sm;
-  float *dW = W + ((kDecParams + 3) & ~3);
-  float *X = dW + ((kDecParams + 3) & ~3);   // [72][kRS]
-  float *A1 = X + 72 * kRS;                   // pre-activations [64][kRS]
-  float *A2 = A1 + 64 * kRS;
-  float *A3 = A2 + 64 * kRS;
-  float *Y = A3 + 64 * kRS;                   // [4][kRS] head, then dy
-  float *D1 = Y + 4 * kRS;                    // [64][kRS]
-  float *D2 = D1 + 64 * kRS;
-  __shared__ double loss_red[kBwdThreads];
-  for (int i = threadIdx.x; i < kDecParams; i += blockDim.x) {
-    W[i] = a.dec[i];
-    dW[i] = 0.0f;
-  }
-  double loss_acc = 0.0;
-  const int64_t n_tiles = (a.g.n + kTR - 1) / kTR;
-  const int t = threadIdx.x;
-  for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
-    __syncthreads();
-    // ---- inputs
-    if (t < kTR) {
-      const int64_t p = tile * kTR + t;
-      int mat = p < a.g.n ? (int)a.g.material[p] : -1;
-      if (mat >= a.n_lat) {
-        atomicOr(a.status, kStatusBadMaterial);
-        mat = -1;
-      }
-      if (mat >= 0) {
-        build_inputs(a.g, p, a.latents + (int64_t)mat * kLatent, X, kRS, t);
-      } else {
-        for (int i = 0; i < kDecIn; ++i) X[i * kRS + t] = 0.0f;
-      }
-      X[kDecIn * kRS + t] = mat >= 0 ? 1.0f : 0.0f;   // row-valid flag
-    }
-    __syncthreads();
-    layer_fwd(W + kOffW1, W + kOffB1, kHidden, kDecIn, X, false, A1);
-    __syncthreads();
-    layer_fwd(W + kOffW2, W + kOffB2, kHidden, kHidden, A1, true, A2);
-    __syncthreads();
-    layer_fwd(W + kOffW3, W + kOffB3, kHidden, kHidden, A2, true, A3);
-    __syncthreads();
-    layer_fwd(W + kOffW4, W + kOffB4, kOut, kHidden, A3, true, Y);
-    __syncthreads();
-    // ---- output gradient
-    if (t < kTR * kOut) {
-      const int r = t % kTR, k = t / kTR;
-      const int64_t p = tile * kTR + r;
-      const bool valid = X[kDecIn * kRS + r] > 0.0f;
-      float d = 0.0f;
-      if (valid) {
-        if (a.target) {
-          d = loss_grad(k, Y[k * kRS + r], a.target[4 * p + k], a.g.wi[3 * p + 2], a.loss_mode, a.inv_batch,
-                        &loss_acc);
-        } else {
-          d = a.dy[4 * p + k];
-        }
-      }
-      Y[k * kRS + r] = d;
-    }
-    __syncthreads();
-    // ---- backward
-    layer_bwd_weights(dW + kOffW4, dW + kOffB4, kOut, kHidden, Y, A3, true);
-    layer_bwd_input(W + kOffW4, kOut, kHidden, Y, A3, D1, kHidden);        // dA3
-    __syncthreads();
-    layer_bwd_weights(dW + kOffW3, dW + kOffB3, kHidden, kHidden, D1, A2, true);
-    layer_bwd_input(W + kOffW3, kHidden, kHidden, D1, A2, D2, kHidden);    // dA2
-    __syncthreads();
-    layer_bwd_weights(dW + kOffW2, dW + kOffB2, kHidden, kHidden, D2, A1, true);
-    layer_bwd_input(W + kOffW2, kHidden, kHidden, D2, A1, D1, kHidden);    // dA1
-    __syncthreads();
-    layer_bwd_weights(dW + kOffW1, dW + kOffB1, kHidden, kDecIn, D1, X, false);
-    if (a.dlat_rows) {
-      // d x[0:32] = W1[:, 0:32]^T dA1
-      layer_bwd_input(W + kOffW1, kHidden, kDecIn, D1, nullptr, D2, kLatent);
-      __syncthreads();
-      for (int e = t; e < kTR * kLatent; e += kBwdThreads) {
-        const int r = e / kLatent, i = e % kLatent;
-        const int64_t p = tile * kTR + r;
-        if (p < a.g.n) a.dlat_rows[p * kLatent + i] = D2[i * kRS + r];
-      }
-    }
-  }
-  __syncthreads();
-  float *out = a.partial + (int64_t)blockIdx.x * kDecParams;
-  for (int i = t; i < kDecParams; i += blockDim.x) out[i] = dW[i];
-  loss_red[t] = loss_acc;
-  __syncthreads();
-  if (t == 0) {
-    double s = 0.0;
-    for (int k = 0; k < kBwdThreads; ++k) s += loss_red[k];
-    a.loss_partial[blockIdx.x] = s;
-  }
-}
 
 // Column sums out[j] = sum_c partial[c][j].  A CTA takes 32 consecutive
 // columns; its kSumSegs warps sum consecutive ranges of rows (in row order),
@@ -351,69 +81,96 @@ __device__ void reduce_loss_warp(const double *__restrict__ part, int n, double 
 }
 
 // dlat[m][i] = sum over rows with material m of dlat_rows[row][i]; one CTA
-// per material scans every id.  Thread t takes the rows of id groups t,
-// t + 256, ... in row order (V: groups of eight ids read as one 16-byte
-// load, four groups in flight; otherwise single ids), then the 256 thread
-// sums are added in thread order, so the result is the same on every run.
-__device__ __forceinline__ void add_row(float *acc, const float *__restrict__ rows, int64_t r) {
-  const float4 *src = reinterpret_cast<const float4 *>(rows + r * kLatent);
-#pragma unroll
-  for (int k = 0; k < kLatent / 4; ++k) {
-    const float4 v = src[k];
-    acc[4 * k] += v.x;
-    acc[4 * k + 1] += v.y;
-    acc[4 * k + 2] += v.z;
-    acc[4 * k + 3] += v.w;
-  }
-}
+// per material.  Warp w looks through the w-th eighth of the ids (32 groups of
+// eight at a time, read as 16-byte loads where V), lists the rows that match in
+// shared memory, and adds the listed rows with one lane per column and
+// eight rows' loads in flight (a row at a time as it is found costs a trip to
+// memory each: 32 us for 65 536 rows of 256 materials).  The list's order,
+// the warp's sum and the sum over warps are fixed, so the result is the same
+// on every run.
+constexpr int kSegWarps = 8;
+constexpr int kSegList = 512;    // listed rows per warp, emptied when a group of 256 might not fit
 
 template <bool V>
-__global__ void __launch_bounds__(256) latent_segment_kernel(const uint16_t *__restrict__ mat, int64_t n,
-                                                             const float *__restrict__ rows,
-                                                             float *__restrict__ dlat) {
+__global__ void __launch_bounds__(32 * kSegWarps) latent_segment_kernel(const uint16_t *__restrict__ mat, int64_t n,
+                                                                        const float *__restrict__ rows,
+                                                                        float *__restrict__ dlat) {
   grid_dependency_wait();
   grid_dependents_launch();
-  const int m = blockIdx.x;
-  __shared__ float red[256][kLatent + 1];
-  float acc[kLatent];
+  __shared__ int list[kSegWarps][kSegList];
+  __shared__ float red[kSegWarps][kLatent];
+  const uint32_t m = blockIdx.x, mm = m * 0x10001u;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t per = (((n + kSegWarps - 1) / kSegWarps) + 255) & ~int64_t(255);
+  const int64_t first = warp * per, last = first + per < n ? first + per : n;
+  const uint32_t below = (1u << lane) - 1u;
+  float acc = 0.0f;
+  int count = 0;
+  auto add_listed = [&]() {
+    __syncwarp();
+    const float *src = rows + first * kLatent + lane;
+    int e = 0;
+    for (; e + 8 <= count; e += 8) {
+      float v[8];
 #pragma unroll
-  for (int i = 0; i < kLatent; ++i) acc[i] = 0.0f;
-  const int64_t step = blockDim.x;
-  int64_t tail = 0;
-  if (V) {
-    const uint4 *ids8 = reinterpret_cast<const uint4 *>(mat);
-    const int64_t groups = n / 8;
-    tail = groups * 8;
-    for (int64_t g = threadIdx.x; g < groups; g += 4 * step) {
-      uint4 w[4];
+      for (int q = 0; q < 8; ++q) v[q] = src[(int64_t)list[warp][e + q] * kLatent];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) w[q] = g + q * step < groups ? ids8[g + q * step] : make_uint4(0u, 0u, 0u, 0u);
+      for (int q = 0; q < 8; ++q) acc += v[q];
+    }
+    for (; e < count; ++e) acc += src[(int64_t)list[warp][e] * kLatent];
+    count = 0;
+    __syncwarp();
+  };
+  // the ids of one group of 256 rows as eight bits per lane: row base + 8 lane + k
+  auto matches = [&](const uint4 &w) {
+    const uint32_t word[4] = {w.x ^ mm, w.y ^ mm, w.z ^ mm, w.w ^ mm};
+    uint32_t bits = 0;
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        if (g + q * step >= groups) break;
-        const uint32_t word[4] = {w[q].x, w[q].y, w[q].z, w[q].w};
+    for (int k = 0; k < 4; ++k) {
+      if ((word[k] & 0xFFFFu) == 0) bits |= 1u << (2 * k);
+      if ((word[k] >> 16) == 0) bits |= 2u << (2 * k);
+    }
+    return bits;
+  };
+  constexpr int kInFlight = 4;
+  for (int64_t base0 = first; base0 < last; base0 += 256 * kInFlight) {
+    uint32_t bits[kInFlight];
+    if (V) {
+      uint4 w[kInFlight];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          if ((int)((word[k >> 1] >> (16 * (k & 1))) & 0xFFFFu) == m) add_row(acc, rows, 8 * (g + q * step) + k);
-        }
+      for (int q = 0; q < kInFlight; ++q) {
+        const int64_t r = base0 + 256 * q + 8 * lane;
+        w[q] = r + 8 <= last ? *reinterpret_cast<const uint4 *>(mat + r) : make_uint4(~mm, ~mm, ~mm, ~mm);
       }
+#pragma unroll
+      for (int q = 0; q < kInFlight; ++q) bits[q] = matches(w[q]);
+    }
+#pragma unroll
+    for (int q = 0; q < kInFlight; ++q) {
+      const int64_t base = base0 + 256 * q, r = base + 8 * lane;
+      if (!V || (r < last && r + 8 > last)) {   // single ids: an unaligned array, or the last n % 8
+        bits[q] = 0;
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+          if (r + k < last && mat[r + k] == m) bits[q] |= 1u << k;
+      }
+      if (!__any_sync(0xFFFFFFFFu, bits[q] != 0)) continue;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const uint32_t hit = __ballot_sync(0xFFFFFFFFu, (bits[q] >> k) & 1u);
+        if ((bits[q] >> k) & 1u) list[warp][count + __popc(hit & below)] = (int)(r + k - first);
+        count += __popc(hit);
+      }
+      if (count > kSegList - 256) add_listed();
     }
   }
-  // single ids: every row (V = false), or the last n % 8 rows
-  for (int64_t r = tail + threadIdx.x; r < n; r += 8 * step) {
-    int ids[8];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) ids[q] = r + q * step < n ? (int)mat[r + q * step] : -1;
-#pragma unroll
-    for (int q = 0; q < 8; ++q)
-      if (ids[q] == m) add_row(acc, rows, r + q * step);
-  }
-#pragma unroll
-  for (int i = 0; i < kLatent; ++i) red[threadIdx.x][i] = acc[i];
+  add_listed();
+  red[warp][lane] = acc;
   __syncthreads();
   if (threadIdx.x < kLatent) {
-    float s = 0.0f;
-    for (int k = 0; k < 256; ++k) s += red[k][threadIdx.x];
+    float s = red[0][threadIdx.x];
+#pragma unroll
+    for (int k = 1; k < kSegWarps; ++k) s += red[k][threadIdx.x];
     dlat[m * kLatent + threadIdx.x] = s;
   }
 }
@@ -1145,77 +902,7 @@ __global__ void err_final_kernel(const double *__restrict__ part, int n_parts, d
   }
 }
 
-size_t fwd_smem_bytes() { return (((kDecParams + 3) & ~3) + (size_t)(kDecIn + kHidden) * kFwdThreads) * 4; }
-size_t bwd_smem_bytes() {
-  return (2 * (size_t)((kDecParams + 3) & ~3) + (size_t)(72 + 64 * 3 + 4 + 64 * 2) * kRS) * 4;
-}
-
 }  // namespace
-
-cudaError_t launch_decoder_fp32(const fabric_gbuffer &g, const DevMaterial *mats, int n_mat, const float *latents,
-                                const float *dec, float *rgb, float *comps, float *y_raw, int *status,
-                                cudaStream_t s) {
-  {
-    const cudaError_t e = ensure_max_dyn_smem(reinterpret_cast<const void *>(decoder_fp32_kernel),
-                                              (int)fwd_smem_bytes());
-    if (e != cudaSuccess) return e;
-  }
-  FwdArgs a;
-  a.g = g;
-  a.mats = mats;
-  a.n_mat = n_mat;
-  a.latents = latents;
-  a.n_lat = mats ? n_mat : 0;
-  a.dec = dec;
-  a.rgb = rgb;
-  a.comps = comps;
-  a.y_raw = y_raw;
-  a.status = status;
-  const unsigned blocks = (unsigned)((g.n + kFwdThreads - 1) / kFwdThreads);
-  decoder_fp32_kernel<<<blocks, kFwdThreads, fwd_smem_bytes(), s>>>(a);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_decoder_raw(const fabric_gbuffer &g, const float *latents, int n_lat, const float *dec,
-                               float *y_raw, int *status, cudaStream_t s) {
-  {
-    const cudaError_t e = ensure_max_dyn_smem(reinterpret_cast<const void *>(decoder_fp32_kernel),
-                                              (int)fwd_smem_bytes());
-    if (e != cudaSuccess) return e;
-  }
-  FwdArgs a;
-  a.g = g;
-  a.mats = nullptr;
-  a.n_mat = 0;
-  a.latents = latents;
-  a.n_lat = n_lat;
-  a.dec = dec;
-  a.rgb = nullptr;
-  a.comps = nullptr;
-  a.y_raw = y_raw;
-  a.status = status;
-  const unsigned blocks = (unsigned)((g.n + kFwdThreads - 1) / kFwdThreads);
-  decoder_fp32_kernel<<<blocks, kFwdThreads, fwd_smem_bytes(), s>>>(a);
-  return cudaGetLastError();
-}
-
-// Work layout: [grid][kDecParams] floats | [grid] doubles | [n][32] floats.
-static int bwd_grid(int64_t n, int sm_count) {
-  const int64_t tiles = (n + kTR - 1) / kTR;
-  int64_t g = sm_count > 0 ? sm_count : 148;
-  if (g > tiles) g = tiles;
-  return (int)(g < 1 ? 1 : g);
-}
-
-size_t decoder_backward_work_bytes(int64_t n, int sm_count) {
-  const int grid = bwd_grid(n, sm_count);
-  size_t bytes = (size_t)grid * kDecParams * 4;
-  bytes = (bytes + 15) & ~size_t(15);
-  bytes += (size_t)grid * 8;
-  bytes = (bytes + 15) & ~size_t(15);
-  bytes += (size_t)n * kLatent * 4;
-  return bytes + 64;
-}
 
 namespace {
 void latent_sums(const fabric_gbuffer &g, int n_lat, const float *rows, float *dlat, cudaStream_t s) {
@@ -1225,43 +912,6 @@ void latent_sums(const fabric_gbuffer &g, int n_lat, const float *rows, float *d
     launch_dependent(latent_segment_kernel<false>, n_lat, 256, 0, s, g.material, g.n, rows, dlat);
 }
 }  // namespace
-
-cudaError_t launch_decoder_backward(const fabric_gbuffer &g, const float *latents, int n_lat, const float *dec,
-                                    const float *dy, const float *target, int loss_mode, float *ddec, float *dlat,
-                                    double *loss, void *work, int sm_count, int *status, cudaStream_t s) {
-  {
-    const cudaError_t e = ensure_max_dyn_smem(reinterpret_cast<const void *>(decoder_bwd_kernel),
-                                              (int)bwd_smem_bytes());
-    if (e != cudaSuccess) return e;
-  }
-  const int grid = bwd_grid(g.n, sm_count);
-  uint8_t *w = static_cast<uint8_t *>(work);
-  float *partial = reinterpret_cast<float *>(w);
-  size_t off = ((size_t)grid * kDecParams * 4 + 15) & ~size_t(15);
-  double *loss_part = reinterpret_cast<double *>(w + off);
-  off = (off + (size_t)grid * 8 + 15) & ~size_t(15);
-  float *rows = reinterpret_cast<float *>(w + off);
-  BwdArgs a;
-  a.g = g;
-  a.latents = latents;
-  a.n_lat = n_lat;
-  a.dec = dec;
-  a.dy = dy;
-  a.target = target;
-  a.loss_mode = loss_mode;
-  a.inv_batch = 1.0f / (float)(g.n > 0 ? g.n : 1);
-  a.partial = partial;
-  a.loss_partial = loss_part;
-  a.dlat_rows = dlat ? rows : nullptr;
-  a.status = status;
-  decoder_bwd_kernel<<<grid, kBwdThreads, bwd_smem_bytes(), s>>>(a);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  launch_dependent(reduce_partials_kernel, (kDecParams + 31) / 32 + (loss ? 1 : 0), 32 * kSumSegs, 0, s, partial, grid,
-                   kDecParams, kDecParams, kDecParams, ddec, nullptr, loss_part, loss);
-  if (dlat) latent_sums(g, n_lat, rows, dlat, s);
-  return cudaGetLastError();
-}
 
 cudaError_t launch_decoder_grad_finish(const fabric_gbuffer &g, int n_lat, const float *partial, int grid, int width,
                                       const double *loss_part, const float *rows, float *ddec, double *loss,
