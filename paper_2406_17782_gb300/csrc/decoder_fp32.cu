@@ -20,7 +20,7 @@
 namespace fab {
 namespace {
 
-constexpr int kThreads = 256;
+constexpr int kThreads = 256;      // forward
 // Row strides of the weights in shared memory, [out][in] as in the flat
 // parameters: multiples of four floats (16-byte reads along the inputs)
 // whose consecutive rows start in different banks.
@@ -37,39 +37,42 @@ constexpr int kSB = kSW4 + kOut * kLdH;             // b1 b2 b3 b4
 constexpr int kSParams = kSB + 3 * kHidden + kOut;
 static_assert(kSParams % 4 == 0, "what follows the parameters stays 16-byte aligned");
 
-// The flat parameters (float-aligned) into shared memory.
+// The flat parameters (float-aligned) into shared memory, by NT threads.
+template <int NT>
 __device__ __forceinline__ void stage_params(const float *__restrict__ dec, float *W) {
-  for (int e = threadIdx.x; e < kHidden * kLd1; e += kThreads) {
+  for (int e = threadIdx.x; e < kHidden * kLd1; e += NT) {
     const int o = e / kLd1, i = e % kLd1;
     W[kSW1 + e] = i < kDecIn ? dec[kOffW1 + o * kDecIn + i] : 0.0f;
   }
-  for (int e = threadIdx.x; e < kHidden * kHidden; e += kThreads) {
+  for (int e = threadIdx.x; e < kHidden * kHidden; e += NT) {
     const int o = e / kHidden, i = e % kHidden;
     W[kSW2 + o * kLdH + i] = dec[kOffW2 + e];
     W[kSW3 + o * kLdH + i] = dec[kOffW3 + e];
   }
-  for (int e = threadIdx.x; e < kOut * kHidden; e += kThreads)
+  for (int e = threadIdx.x; e < kOut * kHidden; e += NT)
     W[kSW4 + (e / kHidden) * kLdH + e % kHidden] = dec[kOffW4 + e];
-  for (int e = threadIdx.x; e < 3 * kHidden + kOut; e += kThreads)
+  for (int e = threadIdx.x; e < 3 * kHidden + kOut; e += NT)
     W[kSB + e] = e < kHidden       ? dec[kOffB1 + e]
                  : e < 2 * kHidden ? dec[kOffB2 + e - kHidden]
                  : e < 3 * kHidden ? dec[kOffB3 + e - 2 * kHidden]
                                    : dec[kOffB4 + e - 3 * kHidden];
 }
 
-// Thread t's place in a layer: point group pg (points 4 pg .. 4 pg + 3 of every
-// 64) and output group og of 16 (outputs og, og + 16, ...).  A warp holds
-// eight point groups (one 128-byte read) and four output groups (rows in
-// different banks).
-__device__ __forceinline__ int point_group() { return (threadIdx.x & 7) | ((threadIdx.x >> 2) & 8); }
-__device__ __forceinline__ int output_group() { return ((threadIdx.x >> 3) & 3) | ((threadIdx.x >> 6) << 2); }
+// A thread's place in a layer: point group pg (points 4 pg .. 4 pg + 3) and
+// output group og of 16 (outputs og, og + 16, ...).  A warp holds eight point
+// groups (one 128-byte read) and four output groups (rows in different
+// banks): warp w takes points 32 (w mod PB) .. and output groups 4 (w / PB) ...
+template <int PB>
+__device__ __forceinline__ int point_group() { return (threadIdx.x & 7) + 8 * ((threadIdx.x >> 5) % PB); }
+template <int PB>
+__device__ __forceinline__ int output_group() { return ((threadIdx.x >> 3) & 3) + 4 * ((threadIdx.x >> 5) / PB % 4); }
 
 // out[o][p] = relu(b[o] + sum_k W[o][k] in[k][p]) for this thread's outputs of
-// RP = 4 or 8 points; K a multiple of four.  SYNC: `out` may be `in` (a CTA
+// RP = 4 or 8 points (8: 4 pg .. and 64 + 4 pg ..); K a multiple of four.  SYNC: `out` may be `in` (a CTA
 // barrier between the last read and the first write).
-template <int RP, int K, int LDW, int LDX, bool SYNC>
+template <int RP, int PB, int K, int LDW, int LDX, bool SYNC>
 __device__ __forceinline__ void layer_relu(const float *W, const float *b, const float *in, float *out) {
-  const int pg = point_group(), og = output_group();
+  const int pg = point_group<PB>(), og = output_group<PB>();
   uint64_t acc[4][RP / 2];
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
@@ -77,7 +80,7 @@ __device__ __forceinline__ void layer_relu(const float *W, const float *b, const
 #pragma unroll
     for (int p = 0; p < RP / 2; ++p) acc[q][p] = pk2(bias, bias);
   }
-#pragma unroll 2
+#pragma unroll 8
   for (int k0 = 0; k0 < K; k0 += 4) {
     float4 w[4];
 #pragma unroll
@@ -185,7 +188,7 @@ __global__ void __launch_bounds__(kThreads, 2) decoder_fp32_kernel(const FwdArgs
   constexpr int TILE = 16 * RP, PARTS = kThreads / TILE;
   extern __shared__ __align__(16) float sm[];
   float *W = sm, *X = sm + kSParams, *Y = X + kInRows * TILE;
-  stage_params(a.dec, W);
+  stage_params<kThreads>(a.dec, W);
   const int t = threadIdx.x, r = t % TILE, part = t / TILE;
   const int64_t n_tiles = (a.g.n + TILE - 1) / TILE;
   const int mat_limit = a.rgb ? min(a.n_lat, a.n_mat) : a.n_lat;
@@ -198,11 +201,11 @@ __global__ void __launch_bounds__(kThreads, 2) decoder_fp32_kernel(const FwdArgs
     // query's) network with latent 0; nothing of it is stored
     build_inputs<PARTS, TILE>(a.g, in ? p : 0, a.latents + (int64_t)(ok ? mat : 0) * kLatent, part, X, r);
     __syncthreads();
-    layer_relu<RP, kInRows, kLd1, TILE, true>(W + kSW1, W + kSB, X, X);
+    layer_relu<RP, 2, kInRows, kLd1, TILE, true>(W + kSW1, W + kSB, X, X);
     __syncthreads();
-    layer_relu<RP, kHidden, kLdH, TILE, true>(W + kSW2, W + kSB + kHidden, X, X);
+    layer_relu<RP, 2, kHidden, kLdH, TILE, true>(W + kSW2, W + kSB + kHidden, X, X);
     __syncthreads();
-    layer_relu<RP, kHidden, kLdH, TILE, true>(W + kSW3, W + kSB + 2 * kHidden, X, X);
+    layer_relu<RP, 2, kHidden, kLdH, TILE, true>(W + kSW3, W + kSB + 2 * kHidden, X, X);
     __syncthreads();
     // the head: kOut / PARTS outputs of one point per thread
 #pragma unroll
@@ -252,8 +255,10 @@ __global__ void __launch_bounds__(kThreads, 2) decoder_fp32_kernel(const FwdArgs
 // ---------------------------------------------------------------------------
 // Forward and backward
 // ---------------------------------------------------------------------------
-constexpr int kTR = 64;          // rows per tile
-constexpr int kLdR = kTR + 4;    // row stride: rows in different banks for 16-byte reads along the rows
+constexpr int kBwdThreads = 512;
+constexpr int kBlock = 32;         // rows a warp's eight point groups cover
+constexpr int kTR = 4 * kBlock;    // rows per tile
+constexpr int kLdR = kTR + 4;      // row stride: rows in different banks for 16-byte reads along the rows
 
 struct BwdArgs {
   fabric_gbuffer g;
@@ -270,17 +275,18 @@ struct BwdArgs {
   int *status;
 };
 
-constexpr size_t kBwdSmem = (size_t)(kSParams + (kInRows + 3 * kHidden + 2 * kHidden + kOut) * kLdR) * 4;
+constexpr size_t kBwdSmem = (size_t)(kSParams + (kInRows + 4 * kHidden + kOut) * kLdR) * 4;
+static_assert(kBwdSmem <= 232448, "one CTA per SM");
 
 // din[i][r] = (sum_o W[o][i] dout[o][r]) (pre[i][r] > 0) for this thread's
 // points 4 pg .. and inputs NI ig .. NI ig + NI - 1 (NI = 4 or 2).
 template <int NI, int K, int LDW>
 __device__ __forceinline__ void layer_input_grad(const float *W, const float *dout, const float *pre, float *din) {
-  const int pg = point_group(), ig = output_group();
+  const int pg = point_group<4>(), ig = output_group<4>();
   uint64_t acc[NI][2];
 #pragma unroll
   for (int q = 0; q < NI; ++q) acc[q][0] = acc[q][1] = 0ull;
-#pragma unroll 4
+#pragma unroll 8
   for (int o = 0; o < K; ++o) {
     float w[NI];
     if (NI == 4) {
@@ -319,78 +325,85 @@ __device__ __forceinline__ void layer_input_grad(const float *W, const float *do
   }
 }
 
-// Weight gradients live in registers for all of the CTA's tiles: thread
-// (og, ig) owns outputs og + 16 q and inputs ig + 16 s.  dW[q][s] += sum_r
-// dout[o][r] in[i][r] over one tile: even and odd rows in the two packed
-// lanes, added to the running sum per tile.
+// Weight gradients live in registers for all of the CTA's tiles.  Each half
+// of the threads sums over half of the tile's rows; in a half, thread (og,
+// ig) owns outputs og + 16 q and inputs ig + 16 s: dW[q][s] += sum_r
+// dout[o][r] in[i][r], r in [r0, r0 + rows), a tile's sum at a time.
 template <int NS>
-__device__ __forceinline__ void layer_weight_grad(const float *dout, const float *in, float (*dW)[NS]) {
-  const int og = output_group(), ig = point_group();
-  uint64_t acc[4][NS];
+__device__ __forceinline__ void layer_weight_grad(const float *dout, const float *in, int r0, int rows, float (*dW)[NS]) {
+  const int og = output_group<2>(), ig = point_group<2>();
+  float acc[4][NS];
 #pragma unroll
   for (int q = 0; q < 4; ++q)
 #pragma unroll
-    for (int s = 0; s < NS; ++s) acc[q][s] = 0ull;
+    for (int s = 0; s < NS; ++s) acc[q][s] = 0.0f;
 #pragma unroll 2
-  for (int r = 0; r < kTR; r += 4) {
-    ulonglong2 d[4], x[NS];
+  for (int r = r0; r < r0 + rows; r += 4) {
+    float4 d[4];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) d[q] = *reinterpret_cast<const ulonglong2 *>(dout + (og + 16 * q) * kLdR + r);
+    for (int q = 0; q < 4; ++q) d[q] = *reinterpret_cast<const float4 *>(dout + (og + 16 * q) * kLdR + r);
 #pragma unroll
-    for (int s = 0; s < NS; ++s)   // a fifth group covers inputs 64..71 only
-      x[s] = *reinterpret_cast<const ulonglong2 *>(in + (16 * s + (s == 4 ? ig & 7 : ig)) * kLdR + r);
+    for (int s = 0; s < NS; ++s) {   // a fifth group covers inputs 64..71 only
+      const float4 x = *reinterpret_cast<const float4 *>(in + (16 * s + (s == 4 ? ig & 7 : ig)) * kLdR + r);
 #pragma unroll
-    for (int q = 0; q < 4; ++q)
-#pragma unroll
-      for (int s = 0; s < NS; ++s) {
-        acc[q][s] = fma2(d[q].x, x[s].x, acc[q][s]);
-        acc[q][s] = fma2(d[q].y, x[s].y, acc[q][s]);
+      for (int q = 0; q < 4; ++q) {
+        acc[q][s] = fmaf(d[q].x, x.x, acc[q][s]);
+        acc[q][s] = fmaf(d[q].y, x.y, acc[q][s]);
+        acc[q][s] = fmaf(d[q].z, x.z, acc[q][s]);
+        acc[q][s] = fmaf(d[q].w, x.w, acc[q][s]);
       }
+    }
   }
 #pragma unroll
   for (int q = 0; q < 4; ++q)
 #pragma unroll
-    for (int s = 0; s < NS; ++s) {
-      float e, o;
-      upk2(acc[q][s], e, o);
-      dW[q][s] += e + o;
-    }
+    for (int s = 0; s < NS; ++s) dW[q][s] += acc[q][s];
 }
 
-// Thread t's share of a layer's bias gradient: rows 16 (t & 3) .. of output t / 4.
-__device__ __forceinline__ float bias_share(const float *dout) {
-  const float *d = dout + (threadIdx.x >> 2) * kLdR + 16 * (threadIdx.x & 3);
+// Thread t's share of a layer's bias gradient: an eighth of the rows of output t / 8.
+__device__ __forceinline__ float bias_share(const float *dout, int rows) {
+  const float *d = dout + (threadIdx.x >> 3) * kLdR + (rows / 8) * (threadIdx.x & 7);
   float s = 0.0f;
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const float4 v = reinterpret_cast<const float4 *>(d)[k];
+  for (int k = 0; k < rows / 8; k += 4) {
+    const float4 v = *reinterpret_cast<const float4 *>(d + k);
     s += (v.x + v.y) + (v.z + v.w);
   }
   return s;
 }
 
-// Persistent CTAs, one per SM (the parameters, a tile's inputs, activations
-// and two gradient buffers take 165 KB of shared memory).
-__global__ void __launch_bounds__(kThreads, 1) decoder_bwd_kernel(const BwdArgs a) {
+// One CTA of 16 warps per SM.  The batch is cut into blocks of 32 rows, dealt
+// to the CTAs in consecutive ranges of nearly equal length, and a CTA takes
+// up to four blocks at a time (its warps without a block wait), so that the
+// last tile of a CTA costs what it holds: 65 536 rows are 13 or 14 blocks a
+// CTA.  The parameters, a tile's inputs, activations and gradients fill the
+// shared memory (226 KB: dA2 takes H3's place, dA1 dA3's, the latent gradient
+// H2's).  Bound by shared-memory latency and bandwidth: with eight warps on
+// 64-row tiles (165 KB) the kernel took 180 us for 65 536 rows.
+__global__ void __launch_bounds__(kBwdThreads, 1) decoder_bwd_kernel(const BwdArgs a) {
   extern __shared__ __align__(16) float sm[];
   float *W = sm;
   float *X = W + kSParams;               // [72][kLdR]
   float *H1 = X + kInRows * kLdR;        // activations [64][kLdR]
   float *H2 = H1 + kHidden * kLdR;
   float *H3 = H2 + kHidden * kLdR;
-  float *D1 = H3 + kHidden * kLdR;       // [64][kLdR]
-  float *D2 = D1 + kHidden * kLdR;
-  float *DY = D2 + kHidden * kLdR;       // [4][kLdR]
-  __shared__ double loss_red[kThreads];
-  stage_params(a.dec, W);
+  float *D = H3 + kHidden * kLdR;        // [64][kLdR]
+  float *DY = D + kHidden * kLdR;        // [4][kLdR]
+  grid_dependency_wait();
+  grid_dependents_launch();
+  stage_params<kBwdThreads>(a.dec, W);
   const int t = threadIdx.x, r = t % kTR, part = t / kTR;
+  const int half = t >> 8, t2 = t & 255, rb = (t >> 5) & 3;
   float dW1[4][5] = {}, dW2[4][4] = {}, dW3[4][4] = {}, dW4 = 0.0f;
   float db1 = 0.0f, db2 = 0.0f, db3 = 0.0f, db4 = 0.0f;
   double loss_acc = 0.0;
-  const int64_t n_tiles = (a.g.n + kTR - 1) / kTR;
-  for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
-    const int64_t p = tile * kTR + r;
-    const int mat = p < a.g.n ? (int)a.g.material[p] : -1;
+  const int64_t n_blocks = (a.g.n + kBlock - 1) / kBlock;
+  const int64_t b_end = n_blocks * (blockIdx.x + 1) / gridDim.x;
+  for (int64_t b0 = n_blocks * blockIdx.x / gridDim.x; b0 < b_end; b0 += 4) {
+    const int nb = (int)(b_end - b0 < 4 ? b_end - b0 : 4), rows = nb * kBlock;
+    const bool busy = rb < nb;             // this warp's row block exists (layers)
+    const int64_t p = b0 * kBlock + r;
+    const bool in = r < rows;
+    const int mat = in && p < a.g.n ? (int)a.g.material[p] : -1;
     bool ok = mat >= 0;
     if (mat >= a.n_lat) {
       if (part == 0) atomicOr(a.status, kStatusBadMaterial);
@@ -398,18 +411,18 @@ __global__ void __launch_bounds__(kThreads, 1) decoder_bwd_kernel(const BwdArgs 
     }
     if (ok) {
       build_inputs<4, kLdR>(a.g, p, a.latents + (int64_t)mat * kLatent, part, X, r);
-    } else {
+    } else if (in) {
       for (int i = part * 18; i < part * 18 + 18; ++i) X[i * kLdR + r] = 0.0f;
     }
     __syncthreads();
-    layer_relu<4, kInRows, kLd1, kLdR, false>(W + kSW1, W + kSB, X, H1);
+    if (busy) layer_relu<4, 4, kInRows, kLd1, kLdR, false>(W + kSW1, W + kSB, X, H1);
     __syncthreads();
-    layer_relu<4, kHidden, kLdH, kLdR, false>(W + kSW2, W + kSB + kHidden, H1, H2);
+    if (busy) layer_relu<4, 4, kHidden, kLdH, kLdR, false>(W + kSW2, W + kSB + kHidden, H1, H2);
     __syncthreads();
-    layer_relu<4, kHidden, kLdH, kLdR, false>(W + kSW3, W + kSB + 2 * kHidden, H2, H3);
+    if (busy) layer_relu<4, 4, kHidden, kLdH, kLdR, false>(W + kSW3, W + kSB + 2 * kHidden, H2, H3);
     __syncthreads();
     // ---- head and output gradient: output `part` of row r
-    {
+    if (in) {
       float y = W[kSB + 3 * kHidden + part];
       const float *w = W + kSW4 + part * kLdH;
 #pragma unroll 4
@@ -428,12 +441,13 @@ __global__ void __launch_bounds__(kThreads, 1) decoder_bwd_kernel(const BwdArgs 
     }
     __syncthreads();
     // ---- backward
-    layer_input_grad<4, kOut, kLdH>(W + kSW4, DY, H3, D1);                 // dA3
+    const int hr = rows / 2, r0 = half * hr;
+    if (busy) layer_input_grad<4, kOut, kLdH>(W + kSW4, DY, H3, D);        // dA3
     {
-      const float *d = DY + (t >> 6) * kLdR, *h = H3 + (t & 63) * kLdR;     // dW4[t / 64][t % 64]
+      const float *d = DY + (t2 >> 6) * kLdR + r0, *h = H3 + (t2 & 63) * kLdR + r0;   // dW4[t2 / 64][t2 % 64]
       float s = 0.0f;
 #pragma unroll 4
-      for (int k = 0; k < kTR; k += 4) {
+      for (int k = 0; k < hr; k += 4) {
         const float4 u = *reinterpret_cast<const float4 *>(d + k), v = *reinterpret_cast<const float4 *>(h + k);
         s = fmaf(u.x, v.x, s);
         s = fmaf(u.y, v.y, s);
@@ -441,74 +455,93 @@ __global__ void __launch_bounds__(kThreads, 1) decoder_bwd_kernel(const BwdArgs 
         s = fmaf(u.w, v.w, s);
       }
       dW4 += s;
-      if (t < 4 * kOut) db4 += bias_share(DY);
+      if (t < 8 * kOut) db4 += bias_share(DY, rows);
     }
     __syncthreads();
-    layer_weight_grad<4>(D1, H2, dW3);
-    db3 += bias_share(D1);
-    layer_input_grad<4, kHidden, kLdH>(W + kSW3, D1, H2, D2);              // dA2
+    layer_weight_grad<4>(D, H2, r0, hr, dW3);
+    db3 += bias_share(D, rows);
+    if (busy) layer_input_grad<4, kHidden, kLdH>(W + kSW3, D, H2, H3);     // dA2, over H3
     __syncthreads();
-    layer_weight_grad<4>(D2, H1, dW2);
-    db2 += bias_share(D2);
-    layer_input_grad<4, kHidden, kLdH>(W + kSW2, D2, H1, D1);              // dA1
+    layer_weight_grad<4>(H3, H1, r0, hr, dW2);
+    db2 += bias_share(H3, rows);
+    if (busy) layer_input_grad<4, kHidden, kLdH>(W + kSW2, H3, H1, D);     // dA1, over dA3
     __syncthreads();
-    layer_weight_grad<5>(D1, X, dW1);
-    db1 += bias_share(D1);
+    layer_weight_grad<5>(D, X, r0, hr, dW1);
+    db1 += bias_share(D, rows);
     if (a.dlat_rows) {
-      // d x[0:32] = W1[:, 0:32]^T dA1
-      layer_input_grad<2, kHidden, kLd1>(W + kSW1, D1, nullptr, D2);
+      // d x[0:32] = W1[:, 0:32]^T dA1, over H2; then row by row, eight floats of one row per thread
+      if (busy) layer_input_grad<2, kHidden, kLd1>(W + kSW1, D, nullptr, H2);
       __syncthreads();
-      // row by row through D2 [32][rows]: eight floats of one row per thread
       const int row = t >> 2, c0 = 8 * (t & 3);
-      const int64_t q = tile * kTR + row;
-      if (q < a.g.n) {
+      const int64_t q = b0 * kBlock + row;
+      if (row < rows && q < a.g.n) {
         float4 *dst = reinterpret_cast<float4 *>(a.dlat_rows + q * kLatent + c0);
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
-          const float *s = D2 + (c0 + 4 * k) * kLdR + row;
+          const float *s = H2 + (c0 + 4 * k) * kLdR + row;
           dst[k] = make_float4(s[0], s[kLdR], s[2 * kLdR], s[3 * kLdR]);
         }
       }
     }
     __syncthreads();
   }
-  float *out = a.partial + (int64_t)blockIdx.x * kDecParams;
-  const int og = output_group(), ig = point_group();
+  // the second half's weight sums through shared memory, added to the first half's
+  float *xs = X + t2;
+  if (half == 1) {
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const int o = og + 16 * q;
+    for (int q = 0; q < 4; ++q) {
 #pragma unroll
-    for (int s = 0; s < 5; ++s) {
-      const int i = 16 * s + ig;
-      if (i < kDecIn) out[kOffW1 + o * kDecIn + i] = dW1[q][s];
+      for (int s = 0; s < 5; ++s) xs[256 * (5 * q + s)] = dW1[q][s];
+#pragma unroll
+      for (int s = 0; s < 4; ++s) {
+        xs[256 * (20 + 4 * q + s)] = dW2[q][s];
+        xs[256 * (36 + 4 * q + s)] = dW3[q][s];
+      }
     }
+    xs[256 * 52] = dW4;
+  }
+  // loss: lanes by a fixed tree, then the 16 warps in order
+  double *loss_red = reinterpret_cast<double *>(W);
 #pragma unroll
-    for (int s = 0; s < 4; ++s) {
-      out[kOffW2 + o * kHidden + 16 * s + ig] = dW2[q][s];
-      out[kOffW3 + o * kHidden + 16 * s + ig] = dW3[q][s];
-    }
-  }
-  out[kOffW4 + t] = dW4;
-  // biases: the four row shares of an output sit in neighbouring lanes
-  db1 += __shfl_xor_sync(0xFFFFFFFFu, db1, 1);
-  db2 += __shfl_xor_sync(0xFFFFFFFFu, db2, 1);
-  db3 += __shfl_xor_sync(0xFFFFFFFFu, db3, 1);
-  db4 += __shfl_xor_sync(0xFFFFFFFFu, db4, 1);
-  db1 += __shfl_xor_sync(0xFFFFFFFFu, db1, 2);
-  db2 += __shfl_xor_sync(0xFFFFFFFFu, db2, 2);
-  db3 += __shfl_xor_sync(0xFFFFFFFFu, db3, 2);
-  db4 += __shfl_xor_sync(0xFFFFFFFFu, db4, 2);
-  if ((t & 3) == 0) {
-    out[kOffB1 + t / 4] = db1;
-    out[kOffB2 + t / 4] = db2;
-    out[kOffB3 + t / 4] = db3;
-    if (t < 4 * kOut) out[kOffB4 + t / 4] = db4;
-  }
-  loss_red[t] = loss_acc;
+  for (int off = 16; off > 0; off >>= 1) loss_acc += __shfl_down_sync(0xFFFFFFFFu, loss_acc, off);
+  if ((t & 31) == 0) loss_red[t >> 5] = loss_acc;
   __syncthreads();
+  float *out = a.partial + (int64_t)blockIdx.x * kDecParams;
+  if (half == 0) {
+    const int og = output_group<2>(), ig = point_group<2>();
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int o = og + 16 * q;
+#pragma unroll
+      for (int s = 0; s < 5; ++s) {
+        const int i = 16 * s + ig;
+        if (i < kDecIn) out[kOffW1 + o * kDecIn + i] = dW1[q][s] + xs[256 * (5 * q + s)];
+      }
+#pragma unroll
+      for (int s = 0; s < 4; ++s) {
+        out[kOffW2 + o * kHidden + 16 * s + ig] = dW2[q][s] + xs[256 * (20 + 4 * q + s)];
+        out[kOffW3 + o * kHidden + 16 * s + ig] = dW3[q][s] + xs[256 * (36 + 4 * q + s)];
+      }
+    }
+    out[kOffW4 + t2] = dW4 + xs[256 * 52];
+  }
+  // biases: the eight row shares of an output sit in neighbouring lanes
+#pragma unroll
+  for (int off = 1; off < 8; off <<= 1) {
+    db1 += __shfl_xor_sync(0xFFFFFFFFu, db1, off);
+    db2 += __shfl_xor_sync(0xFFFFFFFFu, db2, off);
+    db3 += __shfl_xor_sync(0xFFFFFFFFu, db3, off);
+    db4 += __shfl_xor_sync(0xFFFFFFFFu, db4, off);
+  }
+  if ((t & 7) == 0) {
+    out[kOffB1 + t / 8] = db1;
+    out[kOffB2 + t / 8] = db2;
+    out[kOffB3 + t / 8] = db3;
+    if (t < 8 * kOut) out[kOffB4 + t / 8] = db4;
+  }
   if (t == 0) {
-    double s = 0.0;
-    for (int k = 0; k < kThreads; ++k) s += loss_red[k];
+    double s = loss_red[0];
+    for (int k = 1; k < kBwdThreads / 32; ++k) s += loss_red[k];
     a.loss_partial[blockIdx.x] = s;
   }
 }
@@ -529,8 +562,8 @@ cudaError_t launch_fwd(const FwdArgs &a, int sm_count, cudaStream_t s) {
 }
 
 int bwd_grid(int64_t n, int sm_count) {
-  const int64_t tiles = (n + kTR - 1) / kTR;
-  return (int)std::max<int64_t>(1, std::min<int64_t>(tiles, sm_count > 0 ? sm_count : 148));
+  const int64_t blocks = (n + kBlock - 1) / kBlock;
+  return (int)std::max<int64_t>(1, std::min<int64_t>(blocks, sm_count > 0 ? sm_count : 148));
 }
 
 }  // namespace
@@ -582,8 +615,7 @@ cudaError_t launch_decoder_backward(const fabric_gbuffer &g, const float *latent
   a.loss_partial = loss_part;
   a.dlat_rows = dlat ? rows : nullptr;
   a.status = status;
-  decoder_bwd_kernel<<<grid, kThreads, kBwdSmem, s>>>(a);
-  e = cudaGetLastError();
+  e = launch_dependent(decoder_bwd_kernel, grid, kBwdThreads, kBwdSmem, s, a);
   if (e != cudaSuccess) return e;
   return launch_decoder_grad_finish(g, n_lat, partial, grid, kDecParams, loss_part, rows, ddec, loss, dlat, s);
 }
