@@ -72,91 +72,104 @@ __device__ __forceinline__ uint8_t to_e4m3(float v) {
 }
 
 // Fold the latents into the first layer and pack every operand into the
-// canonical shared-memory layout.  16-bit layers 2-4 get their biases as an
-// extra input column; E4M3 layers 2-4 get the per-layer power-of-two scale
-// 2^(8 - E), amax = m 2^E with m in [0.5, 1), and an FP32 epilogue block.
-// One CTA.
+// canonical shared-memory layout, one packed value per thread (a single CTA
+// took 19 us: its loads and the fold's sums ran one after the other).  16-bit
+// layers 2-4 get their biases as an extra input column; E4M3 layers 2-4 get
+// the per-layer power-of-two scale 2^(8 - E), amax = m 2^E with m in
+// [0.5, 1), and an FP32 epilogue block; every CTA forms the three maxima for
+// itself.
+constexpr int kPackThreads = 256;
+
+// Packed values: W1', layers 2-4, the FP32 epilogue block (E4M3) and the albedos.
+__host__ __device__ constexpr int pack_items(int n_mat, int k1, bool f8) {
+  const int kk = f8 ? kHidden : kKH;
+  return kHidden * k1 + 2 * kHidden * kk + 16 * kk + (f8 ? 4 * 64 + 4 : 0) + n_mat * 12;
+}
+
 template <int PR>
-__global__ void __launch_bounds__(256) pack_kernel(const float *__restrict__ dec, const float *__restrict__ lat,
-                                                   const DevMaterial *__restrict__ mats, int n_mat, int k1,
-                                                   uint8_t *__restrict__ blob) {
+__global__ void __launch_bounds__(kPackThreads) pack_kernel(const float *__restrict__ dec, const float *__restrict__ lat,
+                                                            const DevMaterial *__restrict__ mats, int n_mat, int k1,
+                                                            uint8_t *__restrict__ blob) {
   constexpr bool H16 = PR != kPrBF16, F8 = PR == kPrE4M3;
-  extern __shared__ float fold[];   // [n_mat][64]
-  __shared__ unsigned amax_bits[3];
+  constexpr int KK = F8 ? kHidden : kKH;
+  grid_dependency_wait();
+  grid_dependents_launch();
   const BlobLayout L = blob_layout(n_mat, k1, F8);
   const float *W1 = dec + kOffW1;
-  if (threadIdx.x < 3) amax_bits[threadIdx.x] = 0u;
-  for (int e = threadIdx.x; e < n_mat * kHidden; e += blockDim.x) {
-    const int m = e / kHidden, o = e % kHidden;
-    float acc = dec[kOffB1 + o];
-    for (int j = 0; j < kLatent; ++j) acc = fmaf(W1[o * kDecIn + j], lat[m * kLatent + j], acc);
-    fold[m * kHidden + o] = acc;
-  }
-  __syncthreads();
-  for (int e = threadIdx.x; e < kHidden * k1; e += blockDim.x) {
-    const int o = e / k1, c = e % k1;
-    float v = 0.0f;
-    if (c < kQueryFeat)
-      v = W1[o * kDecIn + kLatent + c];
-    else if (c < kQueryFeat + n_mat)
-      v = fold[(c - kQueryFeat) * kHidden + o];
-    put_op<H16>(blob, L.w1 + tc::core_offset(o, c, k1), v);
-  }
-  if (!F8) {
-    for (int e = threadIdx.x; e < kHidden * kKH; e += blockDim.x) {
-      const int o = e / kKH, c = e % kKH;
-      const float v2 = c < kHidden ? dec[kOffW2 + o * kHidden + c] : (c == kHidden ? dec[kOffB2 + o] : 0.0f);
-      const float v3 = c < kHidden ? dec[kOffW3 + o * kHidden + c] : (c == kHidden ? dec[kOffB3 + o] : 0.0f);
-      put_op<H16>(blob, L.w2 + tc::core_offset(o, c, kKH), v2);
-      put_op<H16>(blob, L.w3 + tc::core_offset(o, c, kKH), v3);
-    }
-    for (int e = threadIdx.x; e < 16 * kKH; e += blockDim.x) {
-      const int o = e / kKH, c = e % kKH;
-      float v = 0.0f;
-      if (o < kOut) v = c < kHidden ? dec[kOffW4 + o * kHidden + c] : (c == kHidden ? dec[kOffB4 + o] : 0.0f);
-      put_op<H16>(blob, L.w4 + tc::core_offset(o, c, kKH), v);
-    }
-  } else {
+  float scale[3] = {1.0f, 1.0f, 1.0f}, unscale[3] = {1.0f, 1.0f, 1.0f};
+  if (F8) {
     // per-layer amax (non-negative floats order like their bit patterns)
+    __shared__ unsigned amax_bits[3];
+    if (threadIdx.x < 3) amax_bits[threadIdx.x] = 0u;
+    __syncthreads();
     float m2 = 0.0f, m3 = 0.0f, m4 = 0.0f;
-    for (int e = threadIdx.x; e < kHidden * kHidden; e += blockDim.x) {
+#pragma unroll 16
+    for (int e = threadIdx.x; e < kHidden * kHidden; e += kPackThreads) {
       m2 = fmaxf(m2, fabsf(dec[kOffW2 + e]));
       m3 = fmaxf(m3, fabsf(dec[kOffW3 + e]));
-      if (e < kOut * kHidden) m4 = fmaxf(m4, fabsf(dec[kOffW4 + e]));
     }
+    if (threadIdx.x < kOut * kHidden) m4 = fabsf(dec[kOffW4 + threadIdx.x]);
     atomicMax(&amax_bits[0], __float_as_uint(m2));
     atomicMax(&amax_bits[1], __float_as_uint(m3));
     atomicMax(&amax_bits[2], __float_as_uint(m4));
     __syncthreads();
-    float scale[3];
-    float *epi = reinterpret_cast<float *>(blob + L.epi);
 #pragma unroll
     for (int l = 0; l < 3; ++l) {
       int ex = 0;
       frexpf(__uint_as_float(amax_bits[l]), &ex);
       scale[l] = ldexpf(1.0f, 8 - ex);
-      if (threadIdx.x == 0) epi[kF8Inv + 1 + l] = ldexpf(1.0f, ex - 8);
-    }
-    if (threadIdx.x == 0) epi[kF8Inv] = 1.0f;
-    for (int e = threadIdx.x; e < 4 * 64; e += blockDim.x) {
-      const int l = e / 64, o = e % 64;
-      epi[kF8Bias + e] = l == 1 ? dec[kOffB2 + o] : l == 2 ? dec[kOffB3 + o] : (l == 3 && o < kOut) ? dec[kOffB4 + o] : 0.0f;
-    }
-    for (int e = threadIdx.x; e < kHidden * kHidden; e += blockDim.x) {
-      const int o = e / kHidden, c = e % kHidden;
-      blob[L.w2 + tc::core_offset8(o, c, 64)] = to_e4m3(dec[kOffW2 + e] * scale[0]);
-      blob[L.w3 + tc::core_offset8(o, c, 64)] = to_e4m3(dec[kOffW3 + e] * scale[1]);
-    }
-    for (int e = threadIdx.x; e < 16 * kHidden; e += blockDim.x) {
-      const int o = e / kHidden, c = e % kHidden;
-      blob[L.w4 + tc::core_offset8(o, c, 64)] = o < kOut ? to_e4m3(dec[kOffW4 + e] * scale[2]) : (uint8_t)0;
+      unscale[l] = ldexpf(1.0f, ex - 8);
     }
   }
-  float *alb = reinterpret_cast<float *>(blob + L.alb);
-  for (int e = threadIdx.x; e < n_mat * 12; e += blockDim.x) {
-    const int m = e / 12, q = e % 12;
+  const int total = pack_items(n_mat, k1, F8);
+  for (int e = blockIdx.x * kPackThreads + threadIdx.x; e < total; e += gridDim.x * kPackThreads) {
+    int i = e;
+    if (i < kHidden * k1) {   // W1' with the folded latents
+      const int o = i / k1, c = i % k1;
+      float v = 0.0f;
+      if (c < kQueryFeat) {
+        v = W1[o * kDecIn + kLatent + c];
+      } else if (c < kQueryFeat + n_mat) {
+        const float *z = lat + (c - kQueryFeat) * kLatent;
+        v = dec[kOffB1 + o];
+#pragma unroll
+        for (int j = 0; j < kLatent; ++j) v = fmaf(W1[o * kDecIn + j], z[j], v);
+      }
+      put_op<H16>(blob, L.w1 + tc::core_offset(o, c, k1), v);
+      continue;
+    }
+    i -= kHidden * k1;
+    if (i < 2 * kHidden * KK + 16 * KK) {   // layers 2, 3 and 4 (padded to 16 rows)
+      const int l = i < kHidden * KK ? 0 : i < 2 * kHidden * KK ? 1 : 2;
+      i -= l * kHidden * KK;
+      const int o = i / KK, c = i % KK;
+      const float *W = dec + (l == 0 ? kOffW2 : l == 1 ? kOffW3 : kOffW4);
+      const float *b = dec + (l == 0 ? kOffB2 : l == 1 ? kOffB3 : kOffB4);
+      float v = 0.0f;
+      if (l < 2 || o < kOut) v = c < kHidden ? W[o * kHidden + c] : c == kHidden ? b[o] : 0.0f;
+      const uint32_t base = l == 0 ? L.w2 : l == 1 ? L.w3 : L.w4;
+      if (F8)
+        blob[base + tc::core_offset8(o, c, 64)] = l < 2 || o < kOut ? to_e4m3(v * scale[l]) : (uint8_t)0;
+      else
+        put_op<H16>(blob, base + tc::core_offset(o, c, KK), v);
+      continue;
+    }
+    i -= 2 * kHidden * KK + 16 * KK;
+    if (F8) {
+      if (i < 4 * 64 + 4) {
+        float *epi = reinterpret_cast<float *>(blob + L.epi);
+        const int l = i / 64, o = i % 64;
+        if (i < 4 * 64)
+          epi[kF8Bias + i] = l == 1 ? dec[kOffB2 + o] : l == 2 ? dec[kOffB3 + o] : l == 3 && o < kOut ? dec[kOffB4 + o] : 0.0f;
+        else
+          epi[kF8Inv + o] = o == 0 ? 1.0f : unscale[o - 1];
+        continue;
+      }
+      i -= 4 * 64 + 4;
+    }
+    const int m = i / 12, q = i % 12;
     const DevMaterial &M = mats[m];
-    alb[e] = q < 3 ? M.kd[0][q] : q < 6 ? M.kd[1][q - 3] : q < 9 ? M.ks[0][q - 6] : M.ks[1][q - 9];
+    reinterpret_cast<float *>(blob + L.alb)[i] = q < 3 ? M.kd[0][q] : q < 6 ? M.kd[1][q - 3] : q < 9 ? M.ks[0][q - 6] : M.ks[1][q - 9];
   }
 }
 
@@ -342,6 +355,9 @@ __global__ void __launch_bounds__(kTile * H * WG, 4 / WG) decoder_tc_kernel(cons
     tc::fence_mbar_init();
   }
   if (warp == 0) tc::tmem_alloc(tmem_slot, kColsPerTile * WG);
+  // nothing above reads what an earlier kernel wrote
+  grid_dependency_wait();
+  grid_dependents_launch();
   // batched launches: the segment table (prefix sums of tile counts) in the
   // shared memory past the weights, when the launch gave room for it
   const int64_t *seg_t0 = a.seg_tile0;
@@ -806,14 +822,14 @@ cudaError_t launch_tc_pack(const float *dec, const float *latents, const DevMate
                            void *blob, cudaStream_t s) {
   const int k1 = tc_k1(n_mat);
   if (k1 < 0) return cudaErrorInvalidValue;
-  const size_t smem = (size_t)n_mat * kHidden * sizeof(float);
   uint8_t *out = static_cast<uint8_t *>(blob);
-  switch (prec_code(precision)) {
-    case kPrF16: pack_kernel<kPrF16><<<1, 256, smem, s>>>(dec, latents, mats, n_mat, k1, out); break;
-    case kPrE4M3: pack_kernel<kPrE4M3><<<1, 256, smem, s>>>(dec, latents, mats, n_mat, k1, out); break;
-    default: pack_kernel<kPrBF16><<<1, 256, smem, s>>>(dec, latents, mats, n_mat, k1, out); break;
+  const int pr = prec_code(precision);
+  const dim3 grid((unsigned)((pack_items(n_mat, k1, pr == kPrE4M3) + kPackThreads - 1) / kPackThreads));
+  switch (pr) {
+    case kPrF16: return launch_dependent(pack_kernel<kPrF16>, grid, kPackThreads, 0, s, dec, latents, mats, n_mat, k1, out);
+    case kPrE4M3: return launch_dependent(pack_kernel<kPrE4M3>, grid, kPackThreads, 0, s, dec, latents, mats, n_mat, k1, out);
+    default: return launch_dependent(pack_kernel<kPrBF16>, grid, kPackThreads, 0, s, dec, latents, mats, n_mat, k1, out);
   }
-  return cudaGetLastError();
 }
 
 int tc_default_ctas_per_sm(int n_mat, int precision) {
@@ -868,8 +884,8 @@ static cudaError_t launch_tc(TcArgs &a, bool multi, int precision, int sm_count,
       }
     }
   }
-  void *args[] = {&a};
-  return cudaLaunchKernel(fn, dim3((unsigned)grid), dim3(kTile * wg * h), args, launch_smem, s);
+  return launch_dependent(reinterpret_cast<void (*)(TcArgs)>(const_cast<void *>(fn)), dim3((unsigned)grid), dim3(kTile * wg * h),
+                          launch_smem, s, a);
 }
 
 cudaError_t launch_decoder_tc(const fabric_gbuffer &g, const void *blob, int n_mat, int precision, float *rgb,

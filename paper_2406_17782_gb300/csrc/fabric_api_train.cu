@@ -59,6 +59,10 @@ fabric_status fabric_encode_params(fabric_ctx *ctx, const fabric_material *m, in
     return fail(ctx, FABRIC_ERR_INVALID_ARG, "need materials, a latent buffer and 0..65535 records");
   if (!check_materials(ctx, m, n_mat)) return FABRIC_ERR_INVALID_ARG;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
+  if (encoder_takes_inline(n_mat)) {
+    FAB_CUDA(ctx, launch_encoder_inline(m, n_mat, ctx->d_enc, latents_dev, s), "encoder");
+    return FABRIC_OK;
+  }
   if (ctx->enc_raw_cap < n_mat) {
     FAB_CUDA(ctx, cudaStreamSynchronize(s), "encode staging");
     cudaFree(ctx->d_enc_raw);

@@ -274,7 +274,9 @@ cudaError_t launch_decoder_tc_segments(const SegDesc *segs, const int64_t *seg_t
                                        int ctas_per_sm, int warpgroups, int tile_wgs, cudaStream_t s);
 cudaError_t launch_selftest_mma(const float *a, const float *b, int n, int k, int a_in_tmem, float *d, int *status,
                                 cudaStream_t s);
-cudaError_t launch_encoder_raw(const fabric_material *raw, int n, const float *enc, float *z, cudaStream_t s);
+// Encoder forward from host records passed with the launch (few records).
+bool encoder_takes_inline(int n);
+cudaError_t launch_encoder_inline(const fabric_material *host, int n, const float *enc, float *z, cudaStream_t s);
 cudaError_t launch_encoder_feats(const float *feats, int n, const float *enc, float *z, float *acts,
                                  cudaStream_t s);
 // The decoder's gradient summed from per-CTA partials and its Adam update,

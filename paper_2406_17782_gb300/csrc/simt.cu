@@ -6,6 +6,8 @@
 // All reductions run in a fixed order (owner-computes partial sums per CTA,
 // then a fixed-order sum over CTAs), so repeated runs are bitwise identical.
 #include <cmath>
+#include <cstring>
+#include <type_traits>
 
 #include <algorithm>
 
@@ -251,12 +253,24 @@ __device__ __forceinline__ void enc_dot_s(const float *w, const float (*x)[LD], 
   }
 }
 
-template <bool V>
+// Records of a material edit, passed with the launch instead of copied to the
+// device first (a copy from pageable memory costs the edit an extra operation
+// on the stream and its staging on the host).
+constexpr int kInlineRecords = 32;
+struct InlineRecords {
+  fabric_material m[kInlineRecords];
+};
+struct NoRecords {};
+
+// The input features come from `recs` when REC is InlineRecords, else from
+// `raw` records on the device, or (raw null) from `feats`.
+template <bool V, typename REC>
 __global__ void __launch_bounds__(kEncHidden) encoder_fwd_kernel(const float *__restrict__ feats,
                                                                  const fabric_material *__restrict__ raw,
                                                                  float *__restrict__ feats_out, int n,
                                                                  const float *__restrict__ enc,
-                                                                 float *__restrict__ z, float *__restrict__ acts) {
+                                                                 float *__restrict__ z, float *__restrict__ acts,
+                                                                 const __grid_constant__ REC recs) {
   grid_dependency_wait();
   grid_dependents_launch();
   extern __shared__ __align__(16) float enc_smem[];
@@ -272,11 +286,12 @@ __global__ void __launch_bounds__(kEncHidden) encoder_fwd_kernel(const float *__
   __shared__ __align__(16) float h2[kEncGroup][kEncHidden];
   const int m0 = blockIdx.x * kEncGroup, j = threadIdx.x;
   const int nm = min(kEncGroup, n - m0);
-  if (raw) {
+  if (std::is_same<REC, InlineRecords>::value || raw) {
     if (j < kEncGroup) {
       float t[kEncIn];
       if (j < nm) {
-        material_features(raw[m0 + j], t);
+        if constexpr (std::is_same<REC, InlineRecords>::value) material_features(recs.m[m0 + j], t);
+        else material_features(raw[m0 + j], t);
       } else {
 #pragma unroll
         for (int i = 0; i < kEncIn; ++i) t[i] = 0.0f;
@@ -935,32 +950,34 @@ cudaError_t launch_decoder_grad_finish(const fabric_gbuffer &g, int n_lat, const
 }
 
 namespace {
+template <typename REC>
 cudaError_t encoder_fwd(const float *feats, const fabric_material *raw, float *feats_out, int n, const float *enc,
-                        float *z, float *acts, cudaStream_t s) {
+                        float *z, float *acts, const REC &recs, cudaStream_t s) {
   const int grid = (n + kEncGroup - 1) / kEncGroup;
-  const bool v = (reinterpret_cast<uintptr_t>(enc) & 15) == 0;
-  const void *k = v ? reinterpret_cast<const void *>(encoder_fwd_kernel<true>)
-                    : reinterpret_cast<const void *>(encoder_fwd_kernel<false>);
-  const cudaError_t e = ensure_max_dyn_smem(k, (int)kEncFwdSmem);
+  const auto k = (reinterpret_cast<uintptr_t>(enc) & 15) == 0 ? encoder_fwd_kernel<true, REC> : encoder_fwd_kernel<false, REC>;
+  const cudaError_t e = ensure_max_dyn_smem(reinterpret_cast<const void *>(k), (int)kEncFwdSmem);
   if (e != cudaSuccess) return e;
-  if (v)
-    launch_dependent(encoder_fwd_kernel<true>, grid, kEncHidden, kEncFwdSmem, s, feats, raw, feats_out, n, enc, z,
-                     acts);
-  else
-    launch_dependent(encoder_fwd_kernel<false>, grid, kEncHidden, kEncFwdSmem, s, feats, raw, feats_out, n, enc, z,
-                     acts);
-  return cudaGetLastError();
+  return launch_dependent(k, grid, kEncHidden, kEncFwdSmem, s, feats, raw, feats_out, n, enc, z, acts, recs);
 }
 }  // namespace
 
+bool encoder_takes_inline(int n) { return n <= kInlineRecords; }
+
+cudaError_t launch_encoder_inline(const fabric_material *host, int n, const float *enc, float *z, cudaStream_t s) {
+  InlineRecords recs;
+  std::memcpy(recs.m, host, (size_t)n * sizeof(fabric_material));
+  std::memset(recs.m + n, 0, (size_t)(kInlineRecords - n) * sizeof(fabric_material));
+  return encoder_fwd(nullptr, nullptr, nullptr, n, enc, z, nullptr, recs, s);
+}
+
 cudaError_t launch_encoder_feats(const float *feats, int n, const float *enc, float *z, float *acts,
                                  cudaStream_t s) {
-  return encoder_fwd(feats, nullptr, nullptr, n, enc, z, acts, s);
+  return encoder_fwd(feats, nullptr, nullptr, n, enc, z, acts, NoRecords{}, s);
 }
 
 cudaError_t launch_encoder_raw(const fabric_material *raw, int n, const float *enc, float *feats_out, float *z,
                                float *acts, cudaStream_t s) {
-  return encoder_fwd(nullptr, raw, feats_out, n, enc, z, acts, s);
+  return encoder_fwd(nullptr, raw, feats_out, n, enc, z, acts, NoRecords{}, s);
 }
 
 size_t encoder_backward_work_floats(int n) { return (size_t)n * 2 * kEncHidden + (size_t)n * 4 * kEncHidden; }
@@ -973,7 +990,7 @@ cudaError_t launch_encoder_backward(const float *feats, int n, const float *enc,
   float *vec = work + (size_t)n * 2 * kEncHidden;
   if (!acts_in) {
     // recompute the forward pass to obtain the pre-activations (z discarded into vec)
-    const cudaError_t e = encoder_fwd(feats, nullptr, nullptr, n, enc, vec, acts, s);
+    const cudaError_t e = encoder_fwd(feats, nullptr, nullptr, n, enc, vec, acts, NoRecords{}, s);
     if (e != cudaSuccess) return e;
     acts_in = acts;
   }

@@ -65,3 +65,12 @@ def test_batched_kernel_with_two_warpgroups_per_tile(fab, frame, h):
         fab.sync_status()
         assert torch.equal(rgb, want_rgb) and torch.equal(comps, want_c)
     plan.close()
+
+
+@pytest.mark.parametrize("n_mat", [1, 4, 5, 31, 32])
+def test_encoder_of_records_passed_with_the_launch(fab, n_mat):
+    """Few records travel with the launch, more through device memory: the
+    same latents bit for bit."""
+    mats = W.training_materials(8)[:64]
+    fab.set_params(W.decoder_init(), W.encoder_init())
+    assert torch.equal(fab.encode_params(mats[:n_mat]), fab.encode_params(mats)[:n_mat])
