@@ -647,13 +647,102 @@ __device__ __forceinline__ bool err_pairs(float ai, float bi, float wv, float &d
   return err_fast(dh) && err_fast(bh) && (!W || err_fast(wv));
 }
 
+// i / group for 0 <= i < 2^31: one multiplication (group = 1: mul 0, shift 0).
+// mul = ceil(2^p / group) < 2^32 with p = 31 + ceil(log2 group), so mul group
+// exceeds 2^p by less than 2^(p - 31) and the quotient is exact below 2^31.
+// The weights' index takes two divisions per pair of elements, which the
+// general division (about 25 instructions) dominated.
+struct GroupDiv {
+  int group;
+  uint32_t mul, shift;
+  __device__ __forceinline__ int64_t operator()(int i) const {
+    return mul ? (int64_t)(__umulhi((uint32_t)i, mul) >> shift) : (int64_t)i;
+  }
+  __device__ __forceinline__ int64_t operator()(int64_t i) const { return i / group; }
+};
+GroupDiv group_div(int group) {
+  GroupDiv d{group, 0u, 0u};
+  if (group > 1) {
+    int lg = 1;
+    while ((1ll << lg) < group) ++lg;
+    const int p = 31 + lg;
+    d.mul = (uint32_t)(((1ull << p) + (uint64_t)group - 1) / (uint64_t)group);
+    d.shift = (uint32_t)(p - 32);
+  }
+  return d;
+}
+
+// CTA totals in thread 0 through shared memory: a fixed tree, halving the
+// threads that add (the largest value compares as an integer, since it is
+// non-negative).
+__device__ __forceinline__ void err_reduce(double (*s)[kErrThreads], double &e2, double &b2, double &mx) {
+  const int t = threadIdx.x;
+  s[0][t] = e2;
+  s[1][t] = b2;
+  s[2][t] = mx;
+  __syncthreads();
+  auto larger = [](double x, double y) {
+    return __double_as_longlong(x) > __double_as_longlong(y) ? x : y;
+  };
+#pragma unroll
+  for (int off = kErrThreads / 2; off >= 32; off >>= 1) {
+    if (t < off) {
+      s[0][t] = e2 = e2 + s[0][t + off];
+      s[1][t] = b2 = b2 + s[1][t + off];
+      s[2][t] = mx = larger(mx, s[2][t + off]);
+    }
+    __syncthreads();
+  }
+  if (t < 32) {
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+      e2 += __shfl_down_sync(0xFFFFFFFFu, e2, off);
+      b2 += __shfl_down_sync(0xFFFFFFFFu, b2, off);
+      mx = larger(mx, __shfl_down_sync(0xFFFFFFFFu, mx, off));
+    }
+  }
+}
+
+// The partials summed by the last CTA to finish: thread t takes partials t,
+// t + 256, ... in order, then the fixed tree.  `done` counts the finished CTAs
+// and wraps to zero with the last one.
+__device__ void err_finish(double e2, double b2, double mx, double *__restrict__ part, unsigned *__restrict__ done,
+                           double *__restrict__ out) {
+  __shared__ double s[3][kErrThreads];
+  __shared__ bool last;
+  err_reduce(s, e2, b2, mx);
+  if (threadIdx.x == 0) {
+    part[3 * blockIdx.x] = e2;
+    part[3 * blockIdx.x + 1] = b2;
+    part[3 * blockIdx.x + 2] = mx;
+    __threadfence();
+    last = atomicInc(done, gridDim.x - 1) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  e2 = b2 = mx = 0.0;
+  for (int k = threadIdx.x; k < gridDim.x; k += kErrThreads) {
+    e2 += __ldcg(part + 3 * k);
+    b2 += __ldcg(part + 3 * k + 1);
+    mx = fmax(mx, __ldcg(part + 3 * k + 2));
+  }
+  err_reduce(s, e2, b2, mx);
+  if (threadIdx.x == 0) {
+    out[0] = e2;
+    out[1] = b2;
+    out[2] = mx;
+  }
+}
+
 // W: weights present; Idx: index type (32-bit when n and the strides fit).
 template <bool W, typename Idx>
 __global__ void __launch_bounds__(kErrThreads) err_partial_kernel(const float *__restrict__ a,
                                                                   const float *__restrict__ b, int64_t n_,
-                                                                  const float *__restrict__ w, int group,
-                                                                  int w_stride, double *__restrict__ part) {
-  __shared__ double s0[kErrThreads], s1[kErrThreads], s2[kErrThreads];
+                                                                  const float *__restrict__ w, GroupDiv group,
+                                                                  int w_stride, double *__restrict__ part,
+                                                                  unsigned *__restrict__ done,
+                                                                  double *__restrict__ out) {
   const Idx n = (Idx)n_;
   const Idx stride = (Idx)gridDim.x * kErrThreads;
   const Idx start = (Idx)blockIdx.x * kErrThreads + threadIdx.x;
@@ -672,7 +761,7 @@ __global__ void __launch_bounds__(kErrThreads) err_partial_kernel(const float *_
         const bool in = i < n;
         av[q] = in ? a[i] : 0.0f;
         bv[q] = in ? b[i] : 0.0f;
-        wv[q] = W && in ? w[(int64_t)(i / group) * w_stride] : 1.0f;
+        wv[q] = W && in ? w[group(i) * w_stride] : 1.0f;
       }
 #pragma unroll
       for (int q = 0; q < kErrBatch; ++q) {
@@ -703,7 +792,7 @@ __global__ void __launch_bounds__(kErrThreads) err_partial_kernel(const float *_
   if (slow) {
     for (Idx i = start; i < n; i += stride) {
       const float ai = a[i], bi = b[i];
-      const float wv = W ? w[(int64_t)(i / group) * w_stride] : 1.0f;
+      const float wv = W ? w[group(i) * w_stride] : 1.0f;
       float dh, dl, bh, bl;
       if (err_pairs<W>(ai, bi, wv, dh, dl, bh, bl)) continue;
       const double wi = (double)wv;
@@ -714,23 +803,7 @@ __global__ void __launch_bounds__(kErrThreads) err_partial_kernel(const float *_
       mx = fmax(mx, fabs(d));
     }
   }
-  s0[threadIdx.x] = e2;
-  s1[threadIdx.x] = b2;
-  s2[threadIdx.x] = mx;
-  __syncthreads();
-  for (int off = kErrThreads / 2; off > 0; off >>= 1) {
-    if (threadIdx.x < off) {
-      s0[threadIdx.x] += s0[threadIdx.x + off];
-      s1[threadIdx.x] += s1[threadIdx.x + off];
-      s2[threadIdx.x] = fmax(s2[threadIdx.x], s2[threadIdx.x + off]);
-    }
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    part[3 * blockIdx.x] = s0[0];
-    part[3 * blockIdx.x + 1] = s1[0];
-    part[3 * blockIdx.x + 2] = s2[0];
-  }
+  err_finish(e2, b2, mx, part, done, out);
 }
 
 // ---- the same reduction on pairs of elements with packed FP32x2
@@ -765,12 +838,27 @@ __device__ __forceinline__ void dadd2(uint64_t &h, uint64_t &l, uint64_t x, uint
   l = sub2(e, sub2(h, t));
 }
 
+// Both lanes of a run's packed sums in FP64: the high parts added exactly in
+// FP32, so that one FP64 addition is left (FP64 instructions issue at about a
+// fifteenth of a cycle each per SM, and at frame sizes a thread has only one
+// or two runs: with four per run, an FP64 square root in the range test
+// and FP64 shuffles the kernel took 36 us for a weighted 1080p RGB frame).
+__device__ __forceinline__ double lanes_sum(uint64_t h, uint64_t l) {
+  float h0, h1, l0, l1, s, e;
+  upk2(h, h0, h1);
+  upk2(l, l0, l1);
+  two_sum(h0, h1, s, e);
+  return (double)s + (double)__fadd_rn(e, __fadd_rn(l0, l1));
+}
+__device__ __forceinline__ bool finite64(double x) { return (__double2hiint(x) & 0x7FF00000) != 0x7FF00000; }
+
 template <bool W, typename Idx>
 __global__ void __launch_bounds__(kErrThreads, kErrPerSm2) err_partial2_kernel(const float *__restrict__ a,
                                                                    const float *__restrict__ b, int64_t n_,
-                                                                   const float *__restrict__ w, int group,
-                                                                   int w_stride, double *__restrict__ part) {
-  __shared__ double s0[kErrThreads], s1[kErrThreads], s2[kErrThreads];
+                                                                   const float *__restrict__ w, GroupDiv group,
+                                                                   int w_stride, double *__restrict__ part,
+                                                                   unsigned *__restrict__ done,
+                                                                   double *__restrict__ out) {
   const uint64_t *a2 = reinterpret_cast<const uint64_t *>(a);
   const uint64_t *b2 = reinterpret_cast<const uint64_t *>(b);
   const Idx n = (Idx)n_;
@@ -782,9 +870,9 @@ __global__ void __launch_bounds__(kErrThreads, kErrPerSm2) err_partial2_kernel(c
   float mh = -1.0f, ml = 0.0f, bmax = 0.0f;
   for (Idx j0 = start; j0 < np; j0 += kErrRun2 * stride) {
     uint64_t EH = 0, EL = 0, BH = 0, BL = 0;
-#pragma unroll 1
     constexpr int NB = W ? kErrBatch2 : 2 * kErrBatch2;
-    for (int r0 = 0; r0 < kErrRun2; r0 += NB) {
+#pragma unroll 1
+    for (int r0 = 0; r0 < kErrRun2 && j0 + (Idx)r0 * stride < np; r0 += NB) {
       uint64_t av[NB], bv[NB], wv[NB];
 #pragma unroll
       for (int q = 0; q < NB; ++q) {
@@ -793,8 +881,8 @@ __global__ void __launch_bounds__(kErrThreads, kErrPerSm2) err_partial2_kernel(c
         av[q] = in ? __ldg(a2 + j) : 0ull;
         bv[q] = in ? __ldg(b2 + j) : 0ull;
         if (W) {
-          const float w0 = in ? w[(int64_t)((2 * j) / group) * w_stride] : 1.0f;
-          const float w1 = in ? w[(int64_t)((2 * j + 1) / group) * w_stride] : 1.0f;
+          const float w0 = in ? w[group((Idx)(2 * j)) * w_stride] : 1.0f;
+          const float w1 = in ? w[group((Idx)(2 * j + 1)) * w_stride] : 1.0f;
           wv[q] = pk2(w0, w1);
         }
       }
@@ -840,20 +928,14 @@ __global__ void __launch_bounds__(kErrThreads, kErrPerSm2) err_partial2_kernel(c
         }
       }
     }
-    float h0, h1, l0, l1;
-    upk2(EH, h0, h1);
-    upk2(EL, l0, l1);
-    e2 += ((double)h0 + (double)l0) + ((double)h1 + (double)l1);
-    upk2(BH, h0, h1);
-    upk2(BL, l0, l1);
-    b2s += ((double)h0 + (double)l0) + ((double)h1 + (double)l1);
+    e2 += lanes_sum(EH, EL);
+    b2s += lanes_sum(BH, BL);
   }
   double mx = mh < 0.0f ? 0.0 : (double)mh + (double)ml;
   {
-    const double pairs = (double)((np - (start < np ? start : np) + stride - 1) / stride);   // this thread's pairs
-    const double floor_v = sqrt(2.0 * pairs) * 0x1p-50;
-    const bool slow = !isfinite(e2) || !isfinite(b2s) || (mh > 0.0f && (double)mh < floor_v) ||
-                      (bmax > 0.0f && (double)bmax < floor_v);
+    const float pairs = (float)((np - (start < np ? start : np) + stride - 1) / stride);   // this thread's pairs
+    const float floor_v = 1.001f * sqrtf(2.0f * pairs) * 0x1p-50f;
+    const bool slow = !finite64(e2) || !finite64(b2s) || (mh > 0.0f && mh < floor_v) || (bmax > 0.0f && bmax < floor_v);
     if (slow) {   // the thread's whole share again, in FP64
       e2 = 0.0;
       b2s = 0.0;
@@ -861,7 +943,7 @@ __global__ void __launch_bounds__(kErrThreads, kErrPerSm2) err_partial2_kernel(c
     }
     auto fp64 = [&](Idx i) {
       const float ai = a[i], bi = b[i];
-      const double wi = W ? (double)w[(int64_t)(i / group) * w_stride] : 1.0;
+      const double wi = W ? (double)w[group(i) * w_stride] : 1.0;
       const double d = ((double)ai - (double)bi) * wi;
       const double bb = (double)bi * wi;
       e2 += d * d;
@@ -875,46 +957,7 @@ __global__ void __launch_bounds__(kErrThreads, kErrPerSm2) err_partial2_kernel(c
       }
     if ((n & 1) && blockIdx.x == 0 && threadIdx.x == 0) fp64(n - 1);   // the odd last element
   }
-  s0[threadIdx.x] = e2;
-  s1[threadIdx.x] = b2s;
-  s2[threadIdx.x] = mx;
-  __syncthreads();
-  for (int off = kErrThreads / 2; off > 0; off >>= 1) {
-    if (threadIdx.x < off) {
-      s0[threadIdx.x] += s0[threadIdx.x + off];
-      s1[threadIdx.x] += s1[threadIdx.x + off];
-      s2[threadIdx.x] = fmax(s2[threadIdx.x], s2[threadIdx.x + off]);
-    }
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    part[3 * blockIdx.x] = s0[0];
-    part[3 * blockIdx.x + 1] = s1[0];
-    part[3 * blockIdx.x + 2] = s2[0];
-  }
-}
-
-// One warp: lane l sums the partials l, l + 32, ... in order, then the 32
-// lane sums are added in lane order.
-__global__ void err_final_kernel(const double *__restrict__ part, int n_parts, double *__restrict__ out) {
-  const int lane = threadIdx.x & 31;
-  double e2 = 0.0, b2 = 0.0, mx = 0.0;
-  for (int k = lane; k < n_parts; k += 32) {
-    e2 += part[3 * k];
-    b2 += part[3 * k + 1];
-    mx = fmax(mx, part[3 * k + 2]);
-  }
-  double t0 = 0.0, t1 = 0.0, t2 = 0.0;
-  for (int k = 0; k < 32; ++k) {
-    t0 += __shfl_sync(0xFFFFFFFFu, e2, k);
-    t1 += __shfl_sync(0xFFFFFFFFu, b2, k);
-    t2 = fmax(t2, __shfl_sync(0xFFFFFFFFu, mx, k));
-  }
-  if (lane == 0) {
-    out[0] = t0;
-    out[1] = t1;
-    out[2] = t2;
-  }
+  err_finish(e2, b2s, mx, part, done, out);
 }
 
 }  // namespace
@@ -1090,24 +1133,23 @@ cudaError_t launch_shuffle_dataset(const fabric_train_batch &src, const fabric_d
   return cudaGetLastError();
 }
 
-size_t error_stats_work_bytes(int64_t) { return (size_t)kErrBlocks * 3 * sizeof(double); }
+// [blocks][3] partials, then the count of finished CTAs (zero between calls)
+size_t error_stats_work_bytes(int64_t) { return (size_t)kErrBlocks * 3 * sizeof(double) + sizeof(unsigned); }
 
 cudaError_t launch_error_stats(const float *a, const float *b, int64_t n, const float *w, int group, int w_stride,
                                double *out, void *work, cudaStream_t s) {
   double *part = static_cast<double *>(work);
+  unsigned *done = reinterpret_cast<unsigned *>(part + (size_t)kErrBlocks * 3);
   const bool small = n + (int64_t)kErrRun * kErrBlocks * kErrThreads < ((int64_t)1 << 31);
   const bool packed = ((reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(b)) & 7u) == 0;
-  const int blocks = packed ? kErrBlocks2 : kErrBlocks;
-  if (packed) {
-    if (w && small) err_partial2_kernel<true, int><<<blocks, kErrThreads, 0, s>>>(a, b, n, w, group, w_stride, part);
-    else if (w) err_partial2_kernel<true, int64_t><<<blocks, kErrThreads, 0, s>>>(a, b, n, w, group, w_stride, part);
-    else if (small) err_partial2_kernel<false, int><<<blocks, kErrThreads, 0, s>>>(a, b, n, w, group, w_stride, part);
-    else err_partial2_kernel<false, int64_t><<<blocks, kErrThreads, 0, s>>>(a, b, n, w, group, w_stride, part);
-  } else if (w && small) err_partial_kernel<true, int><<<blocks, kErrThreads, 0, s>>>(a, b, n, w, group, w_stride, part);
-  else if (w) err_partial_kernel<true, int64_t><<<blocks, kErrThreads, 0, s>>>(a, b, n, w, group, w_stride, part);
-  else if (small) err_partial_kernel<false, int><<<blocks, kErrThreads, 0, s>>>(a, b, n, w, group, w_stride, part);
-  else err_partial_kernel<false, int64_t><<<blocks, kErrThreads, 0, s>>>(a, b, n, w, group, w_stride, part);
-  err_final_kernel<<<1, 32, 0, s>>>(part, blocks, out);
+  const auto kernel = packed ? (w ? (small ? err_partial2_kernel<true, int> : err_partial2_kernel<true, int64_t>)
+                                  : (small ? err_partial2_kernel<false, int> : err_partial2_kernel<false, int64_t>))
+                             : (w ? (small ? err_partial_kernel<true, int> : err_partial_kernel<true, int64_t>)
+                                  : (small ? err_partial_kernel<false, int> : err_partial_kernel<false, int64_t>));
+  // one wave of CTAs, or as many as give each thread two elements or pairs
+  const int64_t items = packed ? n / 2 : n, wave = packed ? kErrBlocks2 : kErrBlocks;
+  const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>(wave, (items + 2 * kErrThreads - 1) / (2 * kErrThreads)));
+  kernel<<<blocks, kErrThreads, 0, s>>>(a, b, n, w, group_div(group), w_stride, part, done, out);
   return cudaGetLastError();
 }
 

@@ -1,0 +1,31 @@
+"""The FP64 error reduction over its index arithmetic and launch sizes: group
+divisors, ragged and unaligned lengths, runs of one and of many CTAs, against
+numpy FP64 (1e-12 relative for the sums, the exact maximum without weights)."""
+import numpy as np
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+def expected(a, b, w, group, stride):
+    a, b = a.astype(np.float64), b.astype(np.float64)
+    k = 1.0 if w is None else w.astype(np.float64)[(np.arange(len(a)) // group) * stride]
+    d, e = k * (a - b), k * b
+    return np.array([np.sum(d * d), np.sum(e * e), np.max(np.abs(d))])
+
+
+@pytest.mark.parametrize("group,stride", [(1, 1), (2, 1), (3, 3), (5, 2), (7, 1), (64, 1), (1000, 1), (65537, 1)])
+@pytest.mark.parametrize("n,offset", [(1, 0), (2, 0), (777, 0), (311297, 0), (1245185, 1), (2500001, 0)])
+def test_group_divisors_and_sizes(fab, group, stride, n, offset):
+    r = np.random.default_rng([group, n])
+    a = r.standard_normal(n + offset).astype(np.float32)
+    b = (a + 0.1 * r.standard_normal(n + offset)).astype(np.float32)
+    w = r.uniform(0.1, 1.0, ((n - 1) // group) * stride + 1).astype(np.float32)
+    da, db, dw = (torch.from_numpy(x).cuda() for x in (a, b, w))
+    got = fab.error_stats(da[offset:], db[offset:], weights=dw, group=group, weight_stride=stride).cpu().numpy()
+    want = expected(a[offset:], b[offset:], w, group, stride)
+    assert np.all(np.abs(got - want) <= 1e-12 * want)
+    got = fab.error_stats(da[offset:], db[offset:]).cpu().numpy()
+    want = expected(a[offset:], b[offset:], None, 1, 1)
+    assert np.all(np.abs(got[:2] - want[:2]) <= 1e-12 * want[:2]) and got[2] == want[2]
