@@ -82,99 +82,157 @@ __device__ void reduce_loss_warp(const double *__restrict__ part, int n, double 
   if (lane == 0) *out = t;
 }
 
-// dlat[m][i] = sum over rows with material m of dlat_rows[row][i]; one CTA
-// per material.  Warp w looks through the w-th eighth of the ids (32 groups of
-// eight at a time, read as 16-byte loads where V), lists the rows that match in
-// shared memory, and adds the listed rows with one lane per column and
-// eight rows' loads in flight (a row at a time as it is found costs a trip to
-// memory each: 32 us for 65 536 rows of 256 materials).  The list's order,
-// the warp's sum and the sum over warps are fixed, so the result is the same
-// on every run.
+// out[m][i] = sum over rows with material m of rows[row][i], i < 32 NF; one CTA
+// per material.  The rows are summed in row order within segments of 512, and
+// the segments' sums in order: a fixed order.  The CTA goes over 128 segments
+// at a time, a warp over 16 of them: it looks through the ids 256 at a time
+// (read as 16-byte loads where V), lists the rows that match in shared
+// memory, and adds the listed rows with NF columns per lane and eight rows'
+// loads in flight (a row at a time as it is found costs a trip to memory
+// each: 32 us for 65 536 rows of 256 materials and 32 columns).
 constexpr int kSegWarps = 8;
 constexpr int kSegList = 512;    // listed rows per warp, emptied when a group of 256 might not fit
+constexpr int kSegRows = 512;    // rows per segment
+constexpr int kSegPerWarp = 16;
 
-template <bool V>
+template <int NF>
+struct Columns {
+  float v[NF];
+  __device__ __forceinline__ static Columns load(const float *p) {
+    Columns c;
+    if constexpr (NF == 4) {
+      const float4 t = *reinterpret_cast<const float4 *>(p);
+      c.v[0] = t.x;
+      c.v[1] = t.y;
+      c.v[2] = t.z;
+      c.v[3] = t.w;
+    } else if constexpr (NF == 2) {
+      const float2 t = *reinterpret_cast<const float2 *>(p);
+      c.v[0] = t.x;
+      c.v[1] = t.y;
+    } else {
+      c.v[0] = *p;
+    }
+    return c;
+  }
+  __device__ __forceinline__ void add(const Columns &o) {
+#pragma unroll
+    for (int k = 0; k < NF; ++k) v[k] += o.v[k];
+  }
+};
+
+template <bool V, int NF>
 __global__ void __launch_bounds__(32 * kSegWarps) latent_segment_kernel(const uint16_t *__restrict__ mat, int64_t n,
                                                                         const float *__restrict__ rows,
-                                                                        float *__restrict__ dlat) {
+                                                                        float *__restrict__ out) {
+  constexpr int COLS = 32 * NF;
+  extern __shared__ __align__(16) float seg_sum[];   // [kSegWarps * kSegPerWarp][COLS]
+  __shared__ int list[kSegWarps][kSegList];
+  __shared__ uint32_t present[kSegWarps];            // a warp's segments that have rows of the material
   grid_dependency_wait();
   grid_dependents_launch();
-  __shared__ int list[kSegWarps][kSegList];
-  __shared__ float red[kSegWarps][kLatent];
   const uint32_t m = blockIdx.x, mm = m * 0x10001u;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t per = (((n + kSegWarps - 1) / kSegWarps) + 255) & ~int64_t(255);
-  const int64_t first = warp * per, last = first + per < n ? first + per : n;
   const uint32_t below = (1u << lane) - 1u;
-  float acc = 0.0f;
-  int count = 0;
-  auto add_listed = [&]() {
-    __syncwarp();
-    const float *src = rows + first * kLatent + lane;
-    int e = 0;
-    for (; e + 8 <= count; e += 8) {
-      float v[8];
+  constexpr int kWarpRows = kSegPerWarp * kSegRows;
+  float total = 0.0f;
+  for (int64_t batch = 0; batch < n; batch += (int64_t)kSegWarps * kWarpRows) {
+    const int64_t first = batch + warp * kWarpRows;
+    const int last = first >= n ? 0 : (int)(n - first < kWarpRows ? n - first : kWarpRows);   // this warp's rows
+    Columns<NF> acc = {};
+    int count = 0, seg = 0;
+    uint32_t mask = 0;
+    auto close = [&](int s) {   // the sum of the current segment is complete
+      if ((mask >> seg) & 1u) {
 #pragma unroll
-      for (int q = 0; q < 8; ++q) v[q] = src[(int64_t)list[warp][e + q] * kLatent];
+        for (int k = 0; k < NF; ++k) seg_sum[(warp * kSegPerWarp + seg) * COLS + NF * lane + k] = acc.v[k];
+      }
+      seg = s;
+      acc = Columns<NF>{};
+    };
+    auto add = [&](int row, const Columns<NF> &v) {
+      if (row / kSegRows != seg) close(row / kSegRows);
+      mask |= 1u << seg;
+      acc.add(v);
+    };
+    auto add_listed = [&]() {
+      __syncwarp();
+      const float *src = rows + first * COLS + NF * lane;
+      int e = 0;
+      for (; e + 8 <= count; e += 8) {
+        int r[8];
+        Columns<NF> v[8];
 #pragma unroll
-      for (int q = 0; q < 8; ++q) acc += v[q];
-    }
-    for (; e < count; ++e) acc += src[(int64_t)list[warp][e] * kLatent];
-    count = 0;
-    __syncwarp();
-  };
-  // the ids of one group of 256 rows as eight bits per lane: row base + 8 lane + k
-  auto matches = [&](const uint4 &w) {
-    const uint32_t word[4] = {w.x ^ mm, w.y ^ mm, w.z ^ mm, w.w ^ mm};
-    uint32_t bits = 0;
+        for (int q = 0; q < 8; ++q) r[q] = list[warp][e + q];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      if ((word[k] & 0xFFFFu) == 0) bits |= 1u << (2 * k);
-      if ((word[k] >> 16) == 0) bits |= 2u << (2 * k);
-    }
-    return bits;
-  };
-  constexpr int kInFlight = 4;
-  for (int64_t base0 = first; base0 < last; base0 += 256 * kInFlight) {
-    uint32_t bits[kInFlight];
-    if (V) {
+        for (int q = 0; q < 8; ++q) v[q] = Columns<NF>::load(src + r[q] * COLS);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) add(r[q], v[q]);
+      }
+      for (; e < count; ++e) {
+        const int r = list[warp][e];
+        add(r, Columns<NF>::load(src + r * COLS));
+      }
+      count = 0;
+      __syncwarp();
+    };
+    constexpr int kInFlight = 4;
+    for (int base0 = 0; base0 < last; base0 += 256 * kInFlight) {
       uint4 w[kInFlight];
 #pragma unroll
       for (int q = 0; q < kInFlight; ++q) {
-        const int64_t r = base0 + 256 * q + 8 * lane;
-        w[q] = r + 8 <= last ? *reinterpret_cast<const uint4 *>(mat + r) : make_uint4(~mm, ~mm, ~mm, ~mm);
+        const int r = base0 + 256 * q + 8 * lane;
+        w[q] = V && r + 8 <= last ? *reinterpret_cast<const uint4 *>(mat + first + r) : make_uint4(~mm, ~mm, ~mm, ~mm);
       }
 #pragma unroll
-      for (int q = 0; q < kInFlight; ++q) bits[q] = matches(w[q]);
-    }
+      for (int q = 0; q < kInFlight; ++q) {
+        // rows r .. r + 7 that match, as bits
+        const int r = base0 + 256 * q + 8 * lane;
+        const uint32_t word[4] = {w[q].x ^ mm, w[q].y ^ mm, w[q].z ^ mm, w[q].w ^ mm};
+        uint32_t bits = 0;
 #pragma unroll
-    for (int q = 0; q < kInFlight; ++q) {
-      const int64_t base = base0 + 256 * q, r = base + 8 * lane;
-      if (!V || (r < last && r + 8 > last)) {   // single ids: an unaligned array, or the last n % 8
-        bits[q] = 0;
+        for (int k = 0; k < 4; ++k) {
+          if ((word[k] & 0xFFFFu) == 0) bits |= 1u << (2 * k);
+          if ((word[k] >> 16) == 0) bits |= 2u << (2 * k);
+        }
+        if (!V || (r < last && r + 8 > last)) {   // single ids: an unaligned array, or the last n % 8
+          bits = 0;
+#pragma unroll
+          for (int k = 0; k < 8; ++k)
+            if (r + k < last && mat[first + r + k] == m) bits |= 1u << k;
+        }
+        if (!__any_sync(0xFFFFFFFFu, bits != 0)) continue;
+        int before = 0, hits = 0;   // matches of lower lanes, and of all
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          const uint32_t hit = __ballot_sync(0xFFFFFFFFu, (bits >> k) & 1u);
+          before += __popc(hit & below);
+          hits += __popc(hit);
+        }
 #pragma unroll
         for (int k = 0; k < 8; ++k)
-          if (r + k < last && mat[r + k] == m) bits[q] |= 1u << k;
+          if ((bits >> k) & 1u) list[warp][count + before + __popc(bits & ((1u << k) - 1u))] = r + k;
+        count += hits;
+        if (count > kSegList - 256) add_listed();
       }
-      if (!__any_sync(0xFFFFFFFFu, bits[q] != 0)) continue;
-#pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        const uint32_t hit = __ballot_sync(0xFFFFFFFFu, (bits[q] >> k) & 1u);
-        if ((bits[q] >> k) & 1u) list[warp][count + __popc(hit & below)] = (int)(r + k - first);
-        count += __popc(hit);
-      }
-      if (count > kSegList - 256) add_listed();
     }
+    add_listed();
+    close(0);
+    if (lane == 0) present[warp] = mask;
+    __syncthreads();
+    if (threadIdx.x < COLS) {
+      for (int w = 0; w < kSegWarps; ++w) {
+        uint32_t p = present[w];
+        while (p) {
+          const int s = __ffs(p) - 1;
+          p &= p - 1;
+          total += seg_sum[(w * kSegPerWarp + s) * COLS + threadIdx.x];
+        }
+      }
+    }
+    __syncthreads();
   }
-  add_listed();
-  red[warp][lane] = acc;
-  __syncthreads();
-  if (threadIdx.x < kLatent) {
-    float s = red[0][threadIdx.x];
-#pragma unroll
-    for (int k = 1; k < kSegWarps; ++k) s += red[k][threadIdx.x];
-    dlat[m * kLatent + threadIdx.x] = s;
-  }
+  if (threadIdx.x < COLS) out[(int64_t)m * COLS + threadIdx.x] = total;
 }
 
 // ---------------------------------------------------------------------------
@@ -962,14 +1020,17 @@ __global__ void __launch_bounds__(kErrThreads, kErrPerSm2) err_partial2_kernel(c
 
 }  // namespace
 
-namespace {
-void latent_sums(const fabric_gbuffer &g, int n_lat, const float *rows, float *dlat, cudaStream_t s) {
-  if ((reinterpret_cast<uintptr_t>(g.material) & 15) == 0)
-    launch_dependent(latent_segment_kernel<true>, n_lat, 256, 0, s, g.material, g.n, rows, dlat);
-  else
-    launch_dependent(latent_segment_kernel<false>, n_lat, 256, 0, s, g.material, g.n, rows, dlat);
+cudaError_t launch_material_row_sums(const uint16_t *material, int64_t n, int n_mat, const float *rows, int cols,
+                                     float *out, cudaStream_t s) {
+  const bool v = (reinterpret_cast<uintptr_t>(material) & 15) == 0;
+  const auto k = cols == 128  ? (v ? latent_segment_kernel<true, 4> : latent_segment_kernel<false, 4>)
+                 : cols == 64 ? (v ? latent_segment_kernel<true, 2> : latent_segment_kernel<false, 2>)
+                              : (v ? latent_segment_kernel<true, 1> : latent_segment_kernel<false, 1>);
+  const size_t smem = (size_t)kSegWarps * kSegPerWarp * cols * sizeof(float);
+  const cudaError_t e = ensure_max_dyn_smem(reinterpret_cast<const void *>(k), (int)smem);
+  if (e != cudaSuccess) return e;
+  return launch_dependent(k, n_mat, 32 * kSegWarps, smem, s, material, n, rows, out);
 }
-}  // namespace
 
 cudaError_t launch_decoder_grad_finish(const fabric_gbuffer &g, int n_lat, const float *partial, int grid, int width,
                                       const double *loss_part, const float *rows, float *ddec, double *loss,
@@ -988,7 +1049,7 @@ cudaError_t launch_decoder_grad_finish(const fabric_gbuffer &g, int n_lat, const
                        partial + kDecParams, grid, width, cols, 0, static_cast<float *>(nullptr), dlat, loss_part,
                        loss);
   }
-  if (dlat && !folded) latent_sums(g, n_lat, rows, dlat, s);
+  if (dlat && !folded) launch_material_row_sums(g.material, g.n, n_lat, rows, kLatent, dlat, s);
   return cudaGetLastError();
 }
 
