@@ -325,60 +325,97 @@ __device__ __forceinline__ void layer_input_grad(const float *W, const float *do
   }
 }
 
-// Weight gradients live in registers for all of the CTA's tiles.  Each half
-// of the threads sums over half of the tile's rows; in a half, thread (og,
-// ig) owns outputs og + 16 q and inputs ig + 16 s: dW[q][s] += sum_r
-// dout[o][r] in[i][r], r in [r0, r0 + rows), a tile's sum at a time.
+// Weight gradients live in registers for all of the CTA's blocks.  A thread's
+// place is (og, ig): outputs og + 16 q, inputs ig + 16 s; the two halves of a
+// warp share it and take the blocks 0, 1 and 2, 3 of a tile.  Each block's
+// sum is a chain over its 32 rows in order, and the running sums add the
+// blocks in order: half h keeps those of q = 2h, 2h + 1, and the halves
+// exchange the others by shuffles.
+__device__ __forceinline__ int grad_half() { return (threadIdx.x >> 4) & 1; }
+__device__ __forceinline__ int grad_og() { return ((threadIdx.x >> 3) & 1) + 2 * ((threadIdx.x >> 5) & 7); }
+__device__ __forceinline__ int grad_ig() { return (threadIdx.x & 7) + 8 * (threadIdx.x >> 8); }
+
 template <int NS>
-__device__ __forceinline__ void layer_weight_grad(const float *dout, const float *in, int r0, int rows, float (*dW)[NS]) {
-  const int og = output_group<2>(), ig = point_group<2>();
-  float acc[4][NS];
+__device__ __forceinline__ void layer_weight_grad(const float *dout, const float *in, int nb, float (*dW)[NS]) {
+  const int og = grad_og(), ig = grad_ig(), half = grad_half();
+  float sum[2][4][NS];
 #pragma unroll
-  for (int q = 0; q < 4; ++q)
+  for (int j = 0; j < 2; ++j) {
 #pragma unroll
-    for (int s = 0; s < NS; ++s) acc[q][s] = 0.0f;
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+      for (int s = 0; s < NS; ++s) sum[j][q][s] = 0.0f;
+    if (j >= nb) break;
+    const int r0 = kBlock * (2 * half + j);
 #pragma unroll 2
-  for (int r = r0; r < r0 + rows; r += 4) {
-    float4 d[4];
+    for (int r = r0; r < r0 + kBlock; r += 4) {
+      float4 d[4];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) d[q] = *reinterpret_cast<const float4 *>(dout + (og + 16 * q) * kLdR + r);
+      for (int q = 0; q < 4; ++q) d[q] = *reinterpret_cast<const float4 *>(dout + (og + 16 * q) * kLdR + r);
 #pragma unroll
-    for (int s = 0; s < NS; ++s) {   // a fifth group covers inputs 64..71 only
-      const float4 x = *reinterpret_cast<const float4 *>(in + (16 * s + (s == 4 ? ig & 7 : ig)) * kLdR + r);
+      for (int s = 0; s < NS; ++s) {   // a fifth group covers inputs 64..71 only
+        const float4 x = *reinterpret_cast<const float4 *>(in + (16 * s + (s == 4 ? ig & 7 : ig)) * kLdR + r);
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        acc[q][s] = fmaf(d[q].x, x.x, acc[q][s]);
-        acc[q][s] = fmaf(d[q].y, x.y, acc[q][s]);
-        acc[q][s] = fmaf(d[q].z, x.z, acc[q][s]);
-        acc[q][s] = fmaf(d[q].w, x.w, acc[q][s]);
+        for (int q = 0; q < 4; ++q) {
+          sum[j][q][s] = fmaf(d[q].x, x.x, sum[j][q][s]);
+          sum[j][q][s] = fmaf(d[q].y, x.y, sum[j][q][s]);
+          sum[j][q][s] = fmaf(d[q].z, x.z, sum[j][q][s]);
+          sum[j][q][s] = fmaf(d[q].w, x.w, sum[j][q][s]);
+        }
       }
     }
   }
 #pragma unroll
-  for (int q = 0; q < 4; ++q)
+  for (int q = 0; q < 2; ++q)
 #pragma unroll
-    for (int s = 0; s < NS; ++s) dW[q][s] += acc[q][s];
+    for (int s = 0; s < NS; ++s) {
+      float lo[2], hi[2];   // blocks 0, 1 and 2, 3 of output og + 16 (2 half + q)
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const float keep = half ? sum[j][q + 2][s] : sum[j][q][s];
+        const float got = __shfl_xor_sync(0xFFFFFFFFu, half ? sum[j][q][s] : sum[j][q + 2][s], 16);
+        lo[j] = half ? got : keep;
+        hi[j] = half ? keep : got;
+      }
+      float w = dW[q][s] + lo[0];
+      if (nb > 1) w += lo[1];
+      if (nb > 2) w += hi[0];
+      if (nb > 3) w += hi[1];
+      dW[q][s] = w;
+    }
 }
 
-// Thread t's share of a layer's bias gradient: an eighth of the rows of output t / 8.
-__device__ __forceinline__ float bias_share(const float *dout, int rows) {
-  const float *d = dout + (threadIdx.x >> 3) * kLdR + (rows / 8) * (threadIdx.x & 7);
+// Bias gradients: thread (o, blk) = (t / 4, t % 4) of the first 4 n_out threads
+// adds block blk's rows of output o in order; the blocks' sums are added in
+// order in the lane of block 0.
+__device__ __forceinline__ void bias_grad(const float *dout, int n_out, int nb, float &db) {
+  const int t = threadIdx.x, blk = t & 3;
+  if ((t & ~31) >= 4 * n_out) return;            // whole warps
+  const float *d = dout + min(t >> 2, n_out - 1) * kLdR + kBlock * blk;
   float s = 0.0f;
-  for (int k = 0; k < rows / 8; k += 4) {
+#pragma unroll
+  for (int k = 0; k < kBlock; k += 4) {
     const float4 v = *reinterpret_cast<const float4 *>(d + k);
-    s += (v.x + v.y) + (v.z + v.w);
+    s += v.x;
+    s += v.y;
+    s += v.z;
+    s += v.w;
   }
-  return s;
+  db += s;
+#pragma unroll
+  for (int k = 1; k < 4; ++k) {
+    const float o = __shfl_down_sync(0xFFFFFFFFu, s, k);
+    if (k < nb) db += o;
+  }
 }
 
-// One CTA of 16 warps per SM.  The batch is cut into blocks of 32 rows, dealt
-// to the CTAs in consecutive ranges of nearly equal length, and a CTA takes
-// up to four blocks at a time (its warps without a block wait), so that the
-// last tile of a CTA costs what it holds: 65 536 rows are 13 or 14 blocks a
-// CTA.  The parameters, a tile's inputs, activations and gradients fill the
-// shared memory (226 KB: dA2 takes H3's place, dA1 dA3's, the latent gradient
-// H2's).  Bound by shared-memory latency and bandwidth: with eight warps on
-// 64-row tiles (165 KB) the kernel took 180 us for 65 536 rows.
+// One CTA of 16 warps per SM.  The batch is cut into blocks of 32 rows; CTA c
+// takes blocks c, c + grid, ..., four of them at a time as one tile (warps
+// without a block wait), so that 65 536 rows are 13 or 14 blocks a CTA.  The
+// parameters, a tile's inputs, activations and gradients fill the shared
+// memory (226 KB: dA2 takes H3's place, dA1 dA3's, the latent gradient H2's).
+// Bound by shared-memory latency and bandwidth: with eight warps on 64-row
+// tiles (165 KB) the kernel took 180 us for 65 536 rows.
 __global__ void __launch_bounds__(kBwdThreads, 1) decoder_bwd_kernel(const BwdArgs a) {
   extern __shared__ __align__(16) float sm[];
   float *W = sm;
@@ -392,16 +429,16 @@ __global__ void __launch_bounds__(kBwdThreads, 1) decoder_bwd_kernel(const BwdAr
   grid_dependents_launch();
   stage_params<kBwdThreads>(a.dec, W);
   const int t = threadIdx.x, r = t % kTR, part = t / kTR;
-  const int half = t >> 8, t2 = t & 255, rb = (t >> 5) & 3;
-  float dW1[4][5] = {}, dW2[4][4] = {}, dW3[4][4] = {}, dW4 = 0.0f;
+  const int rb = (t >> 5) & 3;
+  float dW1[2][5] = {}, dW2[2][4] = {}, dW3[2][4] = {}, dW4 = 0.0f;
   float db1 = 0.0f, db2 = 0.0f, db3 = 0.0f, db4 = 0.0f;
   double loss_acc = 0.0;
-  const int64_t n_blocks = (a.g.n + kBlock - 1) / kBlock;
-  const int64_t b_end = n_blocks * (blockIdx.x + 1) / gridDim.x;
-  for (int64_t b0 = n_blocks * blockIdx.x / gridDim.x; b0 < b_end; b0 += 4) {
-    const int nb = (int)(b_end - b0 < 4 ? b_end - b0 : 4), rows = nb * kBlock;
+  const int64_t n_blocks = (a.g.n + kBlock - 1) / kBlock, stride = gridDim.x;
+  for (int64_t b0 = blockIdx.x; b0 < n_blocks; b0 += 4 * stride) {
+    const int nb = (int)min((int64_t)4, (n_blocks - b0 + stride - 1) / stride), rows = nb * kBlock;
     const bool busy = rb < nb;             // this warp's row block exists (layers)
-    const int64_t p = b0 * kBlock + r;
+    auto point = [&](int row) { return (b0 + (row / kBlock) * stride) * kBlock + row % kBlock; };
+    const int64_t p = point(r);
     const bool in = r < rows;
     const int mat = in && p < a.g.n ? (int)a.g.material[p] : -1;
     bool ok = mat >= 0;
@@ -441,39 +478,40 @@ __global__ void __launch_bounds__(kBwdThreads, 1) decoder_bwd_kernel(const BwdAr
     }
     __syncthreads();
     // ---- backward
-    const int hr = rows / 2, r0 = half * hr;
     if (busy) layer_input_grad<4, kOut, kLdH>(W + kSW4, DY, H3, D);        // dA3
-    {
-      const float *d = DY + (t2 >> 6) * kLdR + r0, *h = H3 + (t2 & 63) * kLdR + r0;   // dW4[t2 / 64][t2 % 64]
-      float s = 0.0f;
-#pragma unroll 4
-      for (int k = 0; k < hr; k += 4) {
-        const float4 u = *reinterpret_cast<const float4 *>(d + k), v = *reinterpret_cast<const float4 *>(h + k);
-        s = fmaf(u.x, v.x, s);
-        s = fmaf(u.y, v.y, s);
-        s = fmaf(u.z, v.z, s);
-        s = fmaf(u.w, v.w, s);
+    if (t < kOut * kHidden) {
+      const float *d = DY + (t >> 6) * kLdR, *h = H3 + (t & 63) * kLdR;     // dW4[t / 64][t % 64]
+      for (int blk = 0; blk < nb; ++blk, d += kBlock, h += kBlock) {
+        float s = 0.0f;
+#pragma unroll
+        for (int k = 0; k < kBlock; k += 4) {
+          const float4 u = *reinterpret_cast<const float4 *>(d + k), v = *reinterpret_cast<const float4 *>(h + k);
+          s = fmaf(u.x, v.x, s);
+          s = fmaf(u.y, v.y, s);
+          s = fmaf(u.z, v.z, s);
+          s = fmaf(u.w, v.w, s);
+        }
+        dW4 += s;
       }
-      dW4 += s;
-      if (t < 8 * kOut) db4 += bias_share(DY, rows);
     }
+    bias_grad(DY, kOut, nb, db4);
     __syncthreads();
-    layer_weight_grad<4>(D, H2, r0, hr, dW3);
-    db3 += bias_share(D, rows);
+    layer_weight_grad<4>(D, H2, nb, dW3);
+    bias_grad(D, kHidden, nb, db3);
     if (busy) layer_input_grad<4, kHidden, kLdH>(W + kSW3, D, H2, H3);     // dA2, over H3
     __syncthreads();
-    layer_weight_grad<4>(H3, H1, r0, hr, dW2);
-    db2 += bias_share(H3, rows);
+    layer_weight_grad<4>(H3, H1, nb, dW2);
+    bias_grad(H3, kHidden, nb, db2);
     if (busy) layer_input_grad<4, kHidden, kLdH>(W + kSW2, H3, H1, D);     // dA1, over dA3
     __syncthreads();
-    layer_weight_grad<5>(D, X, r0, hr, dW1);
-    db1 += bias_share(D, rows);
+    layer_weight_grad<5>(D, X, nb, dW1);
+    bias_grad(D, kHidden, nb, db1);
     if (a.dlat_rows) {
       // d x[0:32] = W1[:, 0:32]^T dA1, over H2; then row by row, eight floats of one row per thread
       if (busy) layer_input_grad<2, kHidden, kLd1>(W + kSW1, D, nullptr, H2);
       __syncthreads();
       const int row = t >> 2, c0 = 8 * (t & 3);
-      const int64_t q = b0 * kBlock + row;
+      const int64_t q = point(row);
       if (row < rows && q < a.g.n) {
         float4 *dst = reinterpret_cast<float4 *>(a.dlat_rows + q * kLatent + c0);
 #pragma unroll
@@ -485,60 +523,35 @@ __global__ void __launch_bounds__(kBwdThreads, 1) decoder_bwd_kernel(const BwdAr
     }
     __syncthreads();
   }
-  // the second half's weight sums through shared memory, added to the first half's
-  float *xs = X + t2;
-  if (half == 1) {
+  float *out = a.partial + (int64_t)blockIdx.x * kDecParams;
+  const int og = grad_og(), ig = grad_ig(), half = grad_half();
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
+  for (int q = 0; q < 2; ++q) {
+    const int o = og + 16 * (2 * half + q);
 #pragma unroll
-      for (int s = 0; s < 5; ++s) xs[256 * (5 * q + s)] = dW1[q][s];
-#pragma unroll
-      for (int s = 0; s < 4; ++s) {
-        xs[256 * (20 + 4 * q + s)] = dW2[q][s];
-        xs[256 * (36 + 4 * q + s)] = dW3[q][s];
-      }
+    for (int s = 0; s < 5; ++s) {
+      const int i = 16 * s + ig;
+      if (i < kDecIn) out[kOffW1 + o * kDecIn + i] = dW1[q][s];
     }
-    xs[256 * 52] = dW4;
+#pragma unroll
+    for (int s = 0; s < 4; ++s) {
+      out[kOffW2 + o * kHidden + 16 * s + ig] = dW2[q][s];
+      out[kOffW3 + o * kHidden + 16 * s + ig] = dW3[q][s];
+    }
+  }
+  if (t < kOut * kHidden) out[kOffW4 + t] = dW4;
+  if (t < 4 * kHidden && (t & 3) == 0) {
+    out[kOffB1 + t / 4] = db1;
+    out[kOffB2 + t / 4] = db2;
+    out[kOffB3 + t / 4] = db3;
+    if (t < 4 * kOut) out[kOffB4 + t / 4] = db4;
   }
   // loss: lanes by a fixed tree, then the 16 warps in order
-  double *loss_red = reinterpret_cast<double *>(W);
+  double *loss_red = reinterpret_cast<double *>(X);
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) loss_acc += __shfl_down_sync(0xFFFFFFFFu, loss_acc, off);
   if ((t & 31) == 0) loss_red[t >> 5] = loss_acc;
   __syncthreads();
-  float *out = a.partial + (int64_t)blockIdx.x * kDecParams;
-  if (half == 0) {
-    const int og = output_group<2>(), ig = point_group<2>();
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int o = og + 16 * q;
-#pragma unroll
-      for (int s = 0; s < 5; ++s) {
-        const int i = 16 * s + ig;
-        if (i < kDecIn) out[kOffW1 + o * kDecIn + i] = dW1[q][s] + xs[256 * (5 * q + s)];
-      }
-#pragma unroll
-      for (int s = 0; s < 4; ++s) {
-        out[kOffW2 + o * kHidden + 16 * s + ig] = dW2[q][s] + xs[256 * (20 + 4 * q + s)];
-        out[kOffW3 + o * kHidden + 16 * s + ig] = dW3[q][s] + xs[256 * (36 + 4 * q + s)];
-      }
-    }
-    out[kOffW4 + t2] = dW4 + xs[256 * 52];
-  }
-  // biases: the eight row shares of an output sit in neighbouring lanes
-#pragma unroll
-  for (int off = 1; off < 8; off <<= 1) {
-    db1 += __shfl_xor_sync(0xFFFFFFFFu, db1, off);
-    db2 += __shfl_xor_sync(0xFFFFFFFFu, db2, off);
-    db3 += __shfl_xor_sync(0xFFFFFFFFu, db3, off);
-    db4 += __shfl_xor_sync(0xFFFFFFFFu, db4, off);
-  }
-  if ((t & 7) == 0) {
-    out[kOffB1 + t / 8] = db1;
-    out[kOffB2 + t / 8] = db2;
-    out[kOffB3 + t / 8] = db3;
-    if (t < 8 * kOut) out[kOffB4 + t / 8] = db4;
-  }
   if (t == 0) {
     double s = loss_red[0];
     for (int k = 1; k < kBwdThreads / 32; ++k) s += loss_red[k];

@@ -82,16 +82,121 @@ __device__ void reduce_loss_warp(const double *__restrict__ part, int n, double 
   if (lane == 0) *out = t;
 }
 
+// dlat[m][i] = sum over rows with material m of rows[row][i], i < 32; one CTA per
+// material.  The sums are those of 256 bins added in order, a bin's rows in
+// row order: with V (ids read as 16-byte groups of eight) bin (row / 8) mod
+// 256, the last n mod 8 rows going to bins 0..7, else bin row mod 256.  Warp w
+// owns bins 32 w .. 32 w + 31: it looks through their ids 256 rows at a time
+// (lane l those of bin 32 w + l), lists the rows that match, and adds the
+// listed rows to their bins in shared memory with one lane per column and
+// eight rows' loads in flight (a row at a time as it is found costs a trip to
+// memory each: 32 us for 65 536 rows of 256 materials, 20 us so).
+constexpr int kSegWarps = 8;
+constexpr int kSegList = 512;    // listed rows per warp, emptied when a group of 256 might not fit
+
+template <bool V>
+__global__ void __launch_bounds__(32 * kSegWarps) latent_sums_kernel(const uint16_t *__restrict__ mat, int64_t n,
+                                                                     const float *__restrict__ rows,
+                                                                     float *__restrict__ dlat) {
+  __shared__ float bins[32 * kSegWarps][kLatent];
+  __shared__ uint32_t list[kSegWarps][kSegList];   // rows (fewer than 2^32: they are 128 bytes each)
+  grid_dependency_wait();
+  grid_dependents_launch();
+  const uint32_t m = blockIdx.x, mm = m * 0x10001u;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t below = (1u << lane) - 1u;
+  for (int k = 0; k < 32; ++k) bins[32 * warp + k][lane] = 0.0f;
+  const int64_t whole = V ? n & ~int64_t(7) : n;
+  int count = 0;
+  auto bin_of = [&](uint32_t r) { return 32 * warp + (int)(V ? (r < whole ? (r >> 3) & 31u : (uint32_t)(r - whole)) : r & 31u); };
+  auto add_listed = [&]() {
+    __syncwarp();
+    int e = 0;
+    for (; e + 8 <= count; e += 8) {
+      uint32_t r[8];
+      float v[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) r[q] = list[warp][e + q];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) v[q] = rows[(int64_t)r[q] * kLatent + lane];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) bins[bin_of(r[q])][lane] += v[q];
+    }
+    for (; e < count; ++e) {
+      const uint32_t r = list[warp][e];
+      bins[bin_of(r)][lane] += rows[(int64_t)r * kLatent + lane];
+    }
+    count = 0;
+    __syncwarp();
+  };
+  // row of bit k of this lane in the group at `base`, and the groups' stride
+  constexpr int64_t kGroup = 8 * 32 * kSegWarps;
+  auto row_of = [&](int64_t base, int k) {
+    return V ? base + 256 * warp + 8 * lane + k : base + 256 * k + 32 * warp + lane;
+  };
+  constexpr int kInFlight = 4;
+  for (int64_t base0 = 0; base0 < whole; base0 += kInFlight * kGroup) {
+    uint4 w[kInFlight];
+    uint32_t bits[kInFlight];
+#pragma unroll
+    for (int q = 0; q < kInFlight; ++q) {
+      const int64_t r = row_of(base0 + q * kGroup, 0);
+      w[q] = V && r + 8 <= whole ? *reinterpret_cast<const uint4 *>(mat + r) : make_uint4(~mm, ~mm, ~mm, ~mm);
+    }
+#pragma unroll
+    for (int q = 0; q < kInFlight; ++q) {
+      bits[q] = 0;
+      if (V) {
+        const uint32_t word[4] = {w[q].x ^ mm, w[q].y ^ mm, w[q].z ^ mm, w[q].w ^ mm};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          if ((word[k] & 0xFFFFu) == 0) bits[q] |= 1u << (2 * k);
+          if ((word[k] >> 16) == 0) bits[q] |= 2u << (2 * k);
+        }
+      } else {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          const int64_t r = row_of(base0 + q * kGroup, k);
+          if (r < n && mat[r] == m) bits[q] |= 1u << k;
+        }
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < kInFlight; ++q) {
+      if (!__any_sync(0xFFFFFFFFu, bits[q] != 0)) continue;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) {
+        const uint32_t hit = __ballot_sync(0xFFFFFFFFu, (bits[q] >> k) & 1u);
+        if ((bits[q] >> k) & 1u) list[warp][count + __popc(hit & below)] = (uint32_t)row_of(base0 + q * kGroup, k);
+        count += __popc(hit);
+      }
+      if (count > kSegList - 256) add_listed();
+    }
+  }
+  if (V && warp == 0) {   // the last n mod 8 rows
+    const int64_t r = whole + lane;
+    const bool match = r < n && mat[r] == m;
+    const uint32_t hit = __ballot_sync(0xFFFFFFFFu, match);
+    if (match) list[warp][count + __popc(hit & below)] = (uint32_t)r;
+    count += __popc(hit);
+  }
+  add_listed();
+  __syncthreads();
+  if (threadIdx.x < kLatent) {
+    float s = 0.0f;
+#pragma unroll 16
+    for (int k = 0; k < 32 * kSegWarps; ++k) s += bins[k][threadIdx.x];
+    dlat[(int64_t)m * kLatent + threadIdx.x] = s;
+  }
+}
+
 // out[m][i] = sum over rows with material m of rows[row][i], i < 32 NF; one CTA
 // per material.  The rows are summed in row order within segments of 512, and
 // the segments' sums in order: a fixed order.  The CTA goes over 128 segments
 // at a time, a warp over 16 of them: it looks through the ids 256 at a time
 // (read as 16-byte loads where V), lists the rows that match in shared
 // memory, and adds the listed rows with NF columns per lane and eight rows'
-// loads in flight (a row at a time as it is found costs a trip to memory
-// each: 32 us for 65 536 rows of 256 materials and 32 columns).
-constexpr int kSegWarps = 8;
-constexpr int kSegList = 512;    // listed rows per warp, emptied when a group of 256 might not fit
+// loads in flight.
 constexpr int kSegRows = 512;    // rows per segment
 constexpr int kSegPerWarp = 16;
 
@@ -122,7 +227,7 @@ struct Columns {
 };
 
 template <bool V, int NF>
-__global__ void __launch_bounds__(32 * kSegWarps) latent_segment_kernel(const uint16_t *__restrict__ mat, int64_t n,
+__global__ void __launch_bounds__(32 * kSegWarps) segment_sums_kernel(const uint16_t *__restrict__ mat, int64_t n,
                                                                         const float *__restrict__ rows,
                                                                         float *__restrict__ out) {
   constexpr int COLS = 32 * NF;
@@ -1023,14 +1128,20 @@ __global__ void __launch_bounds__(kErrThreads, kErrPerSm2) err_partial2_kernel(c
 cudaError_t launch_material_row_sums(const uint16_t *material, int64_t n, int n_mat, const float *rows, int cols,
                                      float *out, cudaStream_t s) {
   const bool v = (reinterpret_cast<uintptr_t>(material) & 15) == 0;
-  const auto k = cols == 128  ? (v ? latent_segment_kernel<true, 4> : latent_segment_kernel<false, 4>)
-                 : cols == 64 ? (v ? latent_segment_kernel<true, 2> : latent_segment_kernel<false, 2>)
-                              : (v ? latent_segment_kernel<true, 1> : latent_segment_kernel<false, 1>);
+  const auto k = cols == 128 ? (v ? segment_sums_kernel<true, 4> : segment_sums_kernel<false, 4>)
+                             : (v ? segment_sums_kernel<true, 2> : segment_sums_kernel<false, 2>);
   const size_t smem = (size_t)kSegWarps * kSegPerWarp * cols * sizeof(float);
   const cudaError_t e = ensure_max_dyn_smem(reinterpret_cast<const void *>(k), (int)smem);
   if (e != cudaSuccess) return e;
   return launch_dependent(k, n_mat, 32 * kSegWarps, smem, s, material, n, rows, out);
 }
+
+namespace {
+cudaError_t latent_sums(const fabric_gbuffer &g, int n_lat, const float *rows, float *dlat, cudaStream_t s) {
+  const auto k = (reinterpret_cast<uintptr_t>(g.material) & 15) == 0 ? latent_sums_kernel<true> : latent_sums_kernel<false>;
+  return launch_dependent(k, n_lat, 32 * kSegWarps, 0, s, g.material, g.n, rows, dlat);
+}
+}  // namespace
 
 cudaError_t launch_decoder_grad_finish(const fabric_gbuffer &g, int n_lat, const float *partial, int grid, int width,
                                       const double *loss_part, const float *rows, float *ddec, double *loss,
@@ -1049,7 +1160,7 @@ cudaError_t launch_decoder_grad_finish(const fabric_gbuffer &g, int n_lat, const
                        partial + kDecParams, grid, width, cols, 0, static_cast<float *>(nullptr), dlat, loss_part,
                        loss);
   }
-  if (dlat && !folded) launch_material_row_sums(g.material, g.n, n_lat, rows, kLatent, dlat, s);
+  if (dlat && !folded) latent_sums(g, n_lat, rows, dlat, s);
   return cudaGetLastError();
 }
 
