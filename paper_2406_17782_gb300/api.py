@@ -17,13 +17,16 @@ from ._abi import PAPER_STRUCTURES, FabricDatasetOut, FabricGBuffer, FabricMater
 LATENT = 32
 
 
-def _stream_handle(stream) -> ctypes.c_void_p:
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+def _stream_handle(stream) -> int:
+    """The stream's cudaStream_t; the current device's current stream when
+    None (read without building a torch.cuda.Stream, 0.2 instead of 3 us)."""
+    if stream is not None:
+        return stream.cuda_stream
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _ptr(t):
-    return ctypes.c_void_p(t.data_ptr()) if t is not None else None
+    return t.data_ptr() if t is not None else None
 
 
 def material_array(materials) -> ctypes.Array:
@@ -77,13 +80,14 @@ class GBuffer:
                    for k in ("u", "v", "radius", "wi", "wo", "material"))
 
     def struct(self, host: bool = False) -> FabricGBuffer:
-        for k in ("u", "v", "radius", "wi", "wo", "material"):
-            t = getattr(self, k)
+        u, v, radius, wi, wo, material = fields = (self.u, self.v, self.radius, self.wi, self.wo, self.material)
+        for k, t in enumerate(fields):
             if t.is_cuda == host or not t.is_contiguous():
+                name = ("u", "v", "radius", "wi", "wo", "material")[k]
                 where = "host" if host else "CUDA"
-                raise ValueError(f"G-buffer field {k} must be a contiguous {where} tensor")
-        return FabricGBuffer(self.u.data_ptr(), self.v.data_ptr(), self.radius.data_ptr(), self.wi.data_ptr(),
-                             self.wo.data_ptr(), self.material.data_ptr(), self.n)
+                raise ValueError(f"G-buffer field {name} must be a contiguous {where} tensor")
+        return FabricGBuffer(u.data_ptr(), v.data_ptr(), radius.data_ptr(), wi.data_ptr(), wo.data_ptr(),
+                             material.data_ptr(), u.shape[0])
 
 
 class Fabric:
