@@ -346,7 +346,7 @@ __global__ void __launch_bounds__(kTile * H * WG, 4 / WG) decoder_tc_kernel(cons
   const int h = H == 1 ? 0 : tp >> 7;   // which half of the row's columns
   const int row = tp & (kTile - 1);     // tile row owned by this thread
   const int warp = tid >> 5;
-  const bool lead = tp == 0;            // issues the MMAs
+  const bool lead_warp = __shfl_sync(0xFFFFFFFFu, warp, 0) % (PT / 32) == 0;   // issues the MMAs
   uint64_t *my_bar = bar_mma + wg;
 
   if (tid == 0) {
@@ -459,7 +459,7 @@ __global__ void __launch_bounds__(kTile * H * WG, 4 / WG) decoder_tc_kernel(cons
         ok = false;
         goto teardown;
       }
-      if (lead) {
+      if (lead_warp && tc::elect_one()) {
         tc::tc_fence_after();
         const uint32_t w_addr = layer == 0 ? w1_addr : layer == 1 ? w2_addr : layer == 2 ? w3_addr : w4_addr;
         if (F8 && layer > 0) {

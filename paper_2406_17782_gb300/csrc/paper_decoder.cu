@@ -8,8 +8,8 @@
 //
 // Same execution scheme as the workload's decoder (decoder_tc.cu): a
 // persistent CTA holds one copy of the packed 16-bit weights in shared memory
-// (one bulk copy), and WG tile pipelines of one warpgroup each stream
-// 128-point tiles, one point per thread.  Per pipeline, tensor memory holds the
+// (one bulk copy), and WG tile pipelines of H warpgroups each stream
+// 128-point tiles, H threads per point.  Per pipeline, tensor memory holds the
 // FP32 accumulator D (W columns) and the 16-bit A operand of the next layer
 // (two values per 32-bit column).  Seven MMA chains per tile:
 //   L0  S1': [one-blob (24) | one-hot material] -> W     (latent folded: the
@@ -136,20 +136,27 @@ struct PnPoint {
   int mat;   // -1: beyond the end
 };
 
-__device__ __forceinline__ PnPoint pn_load(const PnArgs &a, int64_t p) {
+// What thread h of the point's H threads needs: the first u and the radius,
+// the last v and the angular inputs.
+template <int H>
+__device__ __forceinline__ PnPoint pn_load(const PnArgs &a, int64_t p, int h) {
   PnPoint q;
   q.u = q.v = q.r = q.wi0 = q.wi1 = q.wi2 = q.wo0 = q.wo1 = 0.0f;
   q.mat = -1;
   if (p < a.n) {
     q.mat = __ldg(a.material + p);
-    q.u = __ldg(a.u + p);
-    q.v = __ldg(a.v + p);
-    q.r = __ldg(a.radius + p);
-    q.wi0 = __ldg(a.wi + 3 * p);
-    q.wi1 = __ldg(a.wi + 3 * p + 1);
-    q.wi2 = __ldg(a.wi + 3 * p + 2);
-    q.wo0 = __ldg(a.wo + 3 * p);
-    q.wo1 = __ldg(a.wo + 3 * p + 1);
+    if (H == 1 || h == 0) {
+      q.u = __ldg(a.u + p);
+      q.r = __ldg(a.radius + p);
+    }
+    if (H == 1 || h == 1) {
+      q.v = __ldg(a.v + p);
+      q.wi0 = __ldg(a.wi + 3 * p);
+      q.wi1 = __ldg(a.wi + 3 * p + 1);
+      q.wi2 = __ldg(a.wi + 3 * p + 2);
+      q.wo0 = __ldg(a.wo + 3 * p);
+      q.wo1 = __ldg(a.wo + 3 * p + 1);
+    }
   }
   return q;
 }
@@ -219,10 +226,12 @@ __device__ __forceinline__ float2 unpack2(uint32_t w) {
 }
 
 // W: network width; F16: FP16 (else BF16) operands; WG tile pipelines per CTA;
-// LDR: 32-column tensor-memory loads in flight per wait in the epilogues.
-template <int W, bool F16, int WG, int LDR>
-__global__ void __launch_bounds__(kTile * WG, (W == 64 && WG == 2) ? 2 : 1) pn_decoder_kernel(const PnArgs a) {
-  constexpr int PT = kTile;
+// H threads per point (each takes W / H accumulator columns); LDR: 32-column
+// tensor-memory loads in flight per wait in the epilogues.
+template <int W, bool F16, int WG, int H, int LDR>
+__global__ void __launch_bounds__(kTile * WG * H, (W == 64 && WG == 2) ? 2 : 1) pn_decoder_kernel(const PnArgs a) {
+  constexpr int PT = kTile * H;
+  constexpr int CH = W / 32 / H;   // 32-column chunks per thread
   constexpr uint32_t COLS = pn_cols(W);
   constexpr uint32_t COL_A = W;
   constexpr int KH = W + 16;
@@ -235,9 +244,11 @@ __global__ void __launch_bounds__(kTile * WG, (W == 64 && WG == 2) ? 2 : 1) pn_d
   uint8_t *wts = smem + 1024;
   const int tid = threadIdx.x;
   const int wg = tid / PT;
-  const int row = tid % PT;
+  const int row = tid % kTile;
+  const int h = H == 1 ? 0 : (tid % PT) / kTile;
   const int warp = tid >> 5;
-  const bool lead = row == 0;
+  const bool lead = tid % PT == 0;
+  const bool lead_warp = __shfl_sync(0xFFFFFFFFu, warp, 0) % (PT / 32) == 0;
   uint64_t *my_bar = bar_mma + wg;
 
   if (tid == 0) {
@@ -259,7 +270,7 @@ __global__ void __launch_bounds__(kTile * WG, (W == 64 && WG == 2) ? 2 : 1) pn_d
   }
   const int64_t stride = (int64_t)gridDim.x * WG;
   int64_t tile = (int64_t)blockIdx.x * WG + wg;
-  PnPoint pt = pn_load(a, tile * kTile + row);
+  PnPoint pt = pn_load<H>(a, tile * kTile + row, h);
   bool ok = tc::mbar_wait_sleep(bar_w, 0, kWaitCycles);
   const float *alb = reinterpret_cast<const float *>(wts + B.alb);
   uint32_t wl[7];
@@ -274,36 +285,42 @@ __global__ void __launch_bounds__(kTile * WG, (W == 64 && WG == 2) ? 2 : 1) pn_d
     const int64_t p = tile * kTile + row;
     int mat = pt.mat;
     if (mat >= a.n_mat) {
-      atomicOr(a.status, kStatusBadMaterial);
+      if (h == 0) atomicOr(a.status, kStatusBadMaterial);
       mat = -2;
     }
     const float wi0 = pt.wi0, wi1 = pt.wi1, wi2 = pt.wi2, wo0 = pt.wo0, wo1 = pt.wo1;
     // ---- layer-0 A operand: one-blob (24 channels) and the one-hot material
     {
-      uint32_t w[16];
-      if (mat >= 0) {
-        blob_periodic<F16>(pt.u, w);
-        blob_periodic<F16>(pt.v, w + 4);
-        const float t = (__logf(fmaxf(pt.r, kRFloor)) - kPnLnRLo) * kPnInvLnSpan;
-        blob_plain<F16>(t, w + 8);
-      } else {
-#pragma unroll
-        for (int k = 0; k < 12; ++k) w[k] = 0u;
-      }
       const int hot = kPnBlob + mat;   // feature index of the material's bias column
+      if (H == 1 || h == 0) {
+        uint32_t wu[4] = {0u, 0u, 0u, 0u}, wr[4] = {0u, 0u, 0u, 0u};
+        if (mat >= 0) {
+          blob_periodic<F16>(pt.u, wu);
+          const float t = (__logf(fmaxf(pt.r, kRFloor)) - kPnLnRLo) * kPnInvLnSpan;
+          blob_plain<F16>(t, wr);
+        }
+        tc::tmem_st4(t_a, wu);
+        tc::tmem_st4(t_a + 8, wr);
+      }
+      if (H == 1 || h == 1) {
+        uint32_t wv[4] = {0u, 0u, 0u, 0u}, w[4];
+        if (mat >= 0) blob_periodic<F16>(pt.v, wv);
+        tc::tmem_st4(t_a + 4, wv);
 #pragma unroll
-      for (int k = 12; k < 16; ++k) w[k] = (hot == 2 * k ? one16 : 0u) | (hot == 2 * k + 1 ? one16 << 16 : 0u);
-      tc::tmem_st16(t_a, w);           // features 0..31
-      for (int c = 2; c < B.k1 / 16; ++c) {
-        uint32_t h8[8];
+        for (int k = 0; k < 4; ++k)
+          w[k] = (hot == 24 + 2 * k ? one16 : 0u) | (hot == 25 + 2 * k ? one16 << 16 : 0u);
+        tc::tmem_st4(t_a + 12, w);       // features 24..31
+        for (int c = 2; c < B.k1 / 16; ++c) {
+          uint32_t h8[8];
 #pragma unroll
-        for (int k = 0; k < 8; ++k)
-          h8[k] = (hot == 16 * c + 2 * k ? one16 : 0u) | (hot == 16 * c + 2 * k + 1 ? one16 << 16 : 0u);
-        tc::tmem_st8(t_a + 8 * c, h8);
+          for (int k = 0; k < 8; ++k)
+            h8[k] = (hot == 16 * c + 2 * k ? one16 : 0u) | (hot == 16 * c + 2 * k + 1 ? one16 << 16 : 0u);
+          tc::tmem_st8(t_a + 8 * c, h8);
+        }
       }
       tc::tmem_st_wait();
     }
-    uint32_t skip[W / 2];   // k1 as 16-bit operand pairs, for the residual block
+    uint32_t skip[16 * CH];   // k1 as 16-bit operand pairs, for the residual block
 #pragma unroll
     for (int layer = 0; layer < 7; ++layer) {
       tc::tc_fence_before();
@@ -311,7 +328,7 @@ __global__ void __launch_bounds__(kTile * WG, (W == 64 && WG == 2) ? 2 : 1) pn_d
         ok = false;
         goto teardown;
       }
-      if (lead) {
+      if (lead_warp && tc::elect_one()) {
         tc::tc_fence_after();
         const int K = layer == 0 ? B.k1 : KH;
         const uint32_t sbo = (uint32_t)K * 16u;
@@ -321,16 +338,17 @@ __global__ void __launch_bounds__(kTile * WG, (W == 64 && WG == 2) ? 2 : 1) pn_d
         }
         tc::mma_commit(my_bar);
       }
-      if (layer == 0) pt = pn_load(a, (tile + stride) * kTile + row);   // next tile's inputs in flight
+      if (layer == 0) pt = pn_load<H>(a, (tile + stride) * kTile + row, h);   // next tile's inputs in flight
       ok = tc::mbar_wait_sleep(my_bar, phase, kWaitCycles) && ok;
       phase ^= 1u;
       tc::tc_fence_after();
       if (layer < 6) {
 #pragma unroll
-        for (int c0 = 0; c0 < W / 32; c0 += LDR) {
+        for (int c0 = 0; c0 < CH; c0 += LDR) {
+          const int col0 = CH * h + c0;   // chunk of D
           float acc[32 * LDR];
 #pragma unroll
-          for (int r = 0; r < LDR; ++r) tc::tmem_ld32(t_d + 32 * (c0 + r), acc + 32 * r);
+          for (int r = 0; r < LDR; ++r) tc::tmem_ld32(t_d + 32 * (col0 + r), acc + 32 * r);
           tc::tmem_ld_wait();
 #pragma unroll
           for (int r = 0; r < LDR; ++r) {
@@ -346,20 +364,22 @@ __global__ void __launch_bounds__(kTile * WG, (W == 64 && WG == 2) ? 2 : 1) pn_d
               w[k] = tc::pack2<F16>(lrelu(x0), lrelu(x1));
               if (layer == 2) skip[(c0 + r) * 16 + k] = w[k];
             }
-            tc::tmem_st16(t_a + 16 * (c0 + r), w);
+            tc::tmem_st16(t_a + 16 * (col0 + r), w);
           }
         }
         // input columns W..W+15: the angular inputs and the constant one of
         // A1's bias after the spatial fusion, else the constant-one bias column
-        uint32_t w8[8] = {one16, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
-        if (layer == 1) {
-          w8[0] = tc::pack2<F16>(wi0, wi1);
-          w8[1] = tc::pack2<F16>(wi2, wo0);
-          w8[2] = tc::pack2<F16>(wo1, 1.0f);
+        if (H == 1 || h == 1) {
+          uint32_t w8[8] = {one16, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
+          if (layer == 1) {
+            w8[0] = tc::pack2<F16>(wi0, wi1);
+            w8[1] = tc::pack2<F16>(wi2, wo0);
+            w8[2] = tc::pack2<F16>(wo1, 1.0f);
+          }
+          tc::tmem_st8(t_a + W / 2, w8);
         }
-        tc::tmem_st8(t_a + W / 2, w8);
         tc::tmem_st_wait();
-      } else {
+      } else if (H == 1 || h == 0) {
         float y[4];
         tc::tmem_ld4(t_d, y);
         tc::tmem_ld_wait();
@@ -387,7 +407,7 @@ __global__ void __launch_bounds__(kTile * WG, (W == 64 && WG == 2) ? 2 : 1) pn_d
   ok = !pn_bar_or<PT>(wg, !ok);
 teardown:
   if (!ok) {
-    if (tid == 0) atomicOr(a.status, kStatusTimeout);
+    if (lead) atomicOr(a.status, kStatusTimeout);
     tc::mbar_wait(bar_w, 0, kWaitCycles);
     tc::mbar_wait(my_bar, phase ^ 1u, kWaitCycles);
   }
@@ -399,14 +419,21 @@ teardown:
   }
 }
 
+constexpr int kPnWG = 2;
+// Threads per point.  Width 128: two, each with half of the 128 accumulator
+// columns (1080p, 8 materials: 371 us, against 425 with one and 754 with four
+// of 64 registers).  Width 64: one; two would leave 64 registers a thread at
+// two CTAs per SM, and spill (167 us against 209).
+constexpr int pn_threads(int w) { return w == 64 ? 1 : 2; }
+
 // W = 64: two pipelines of 128 columns per CTA, two CTAs per SM (four CTAs
 // of one pipeline would need four copies of the 57 KB of weights); W = 128:
 // one CTA of two pipelines of 256 columns.  Either way the SM's 512
 // tensor-memory columns are taken.
 template <int W, bool F16>
 const void *pn_kernel() {
-  if (W == 64) return reinterpret_cast<const void *>(pn_decoder_kernel<64, F16, 2, 1>);
-  return reinterpret_cast<const void *>(pn_decoder_kernel<128, F16, 2, 2>);
+  if (W == 64) return reinterpret_cast<const void *>(pn_decoder_kernel<64, F16, kPnWG, pn_threads(64), 1>);
+  return reinterpret_cast<const void *>(pn_decoder_kernel<128, F16, kPnWG, pn_threads(128), 2>);
 }
 
 }  // namespace
@@ -440,7 +467,7 @@ cudaError_t launch_paper_decoder(int w, int precision, const fabric_gbuffer &g, 
   const bool f16 = precision == FABRIC_PREC_FP16;
   const void *fn = w == 64 ? (f16 ? pn_kernel<64, true>() : pn_kernel<64, false>())
                            : (f16 ? pn_kernel<128, true>() : pn_kernel<128, false>());
-  const int wg = 2;
+  const int wg = kPnWG;
   PnArgs a = {};
   a.u = g.u;
   a.v = g.v;
@@ -470,7 +497,7 @@ cudaError_t launch_paper_decoder(int w, int precision, const fabric_gbuffer &g, 
   if (grid > need) grid = need;
   if (grid < 1) grid = 1;
   void *args[] = {&a};
-  return cudaLaunchKernel(fn, dim3((unsigned)grid), dim3(kTile * wg), args, smem, s);
+  return cudaLaunchKernel(fn, dim3((unsigned)grid), dim3(kTile * wg * pn_threads(w)), args, smem, s);
 }
 
 }  // namespace fab

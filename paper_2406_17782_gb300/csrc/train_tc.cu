@@ -16,7 +16,7 @@
 //             all of the CTA's tiles in tensor memory; the bias gradients
 //             come out as the row of the constant-one input.
 //   latent    dz rows = da_1 W1[:, :32] (FP32, for the per-material sums).
-// Thread 0 issues the products an epilogue reads and thread 128 the weight-
+// Warp 0 issues the products an epilogue reads and warp 4 the weight-
 // gradient products, which nothing reads until the tile loop ends: each dW
 // chain is waited for only before the shared-memory operand it reads is
 // rewritten (the da operands alternate between two buffers for this).
@@ -76,9 +76,9 @@ constexpr uint32_t kColDz = 336;
 constexpr int kDzTiles = 5;
 static_assert(kColDz + 32 * kDzTiles <= 512, "latent-gradient rows inside the allocation");
 
-// Thread 0 issues the products the epilogues read; thread 128 (the first
-// thread of half 1) issues the weight-gradient products.
-constexpr int kDwIssuer = 128;
+// Warp 0's elected thread issues the products the epilogues read; that of warp
+// 4 (the first of half 1) issues the weight-gradient products.
+constexpr int kDwIssuer = 4;
 
 // Instruction-descriptor bits: A and B read MN-major (transposed).
 constexpr uint32_t kTransA = 1u << 15, kTransB = 1u << 16;
@@ -188,7 +188,7 @@ __global__ void __launch_bounds__(kThreads, 1) train_tc_kernel(const TrainTcArgs
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t *bar_w = reinterpret_cast<uint64_t *>(smem);
-  uint64_t *bar_mma = bar_w + 1;     // thread 0's products
+  uint64_t *bar_mma = bar_w + 1;     // warp 0's products
   uint64_t *bar_dw = bar_w + 2;      // [3]: dW4, dW3 and dW1 (each once per tile)
   uint64_t *bar_drain = bar_w + 5;   // both issuers' products, after a failed wait
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bar_w + 6);
@@ -198,6 +198,7 @@ __global__ void __launch_bounds__(kThreads, 1) train_tc_kernel(const TrainTcArgs
   uint8_t *daA = sm + kSmDaA, *daB = sm + kSmDaB;
   const int tid = threadIdx.x;
   const int warp = tid >> 5;
+  const int warp_u = __shfl_sync(0xFFFFFFFFu, warp, 0);   // uniform to the compiler (see round())
   const int hf = warp >> 2;                      // which half of every epilogue's columns
   const int r = ((warp & 3) << 5) | (tid & 31);  // tile row (query) = tensor-memory lane
   const bool lead = tid == 0;
@@ -253,9 +254,9 @@ __global__ void __launch_bounds__(kThreads, 1) train_tc_kernel(const TrainTcArgs
       tc::mma_bf16(tmem + d_col, ad, bd, tc::idesc_bf16(128, N) | kTransA | kTransB, (acc || kk > 0) ? 1u : 0u);
     }
   };
-  // All threads make their stores visible and meet.  Then thread 0 issues
+  // All threads make their stores visible and meet.  Then warp 0 issues
   // `issue` (the products the epilogue reads) and commits it to bar_mma, and
-  // thread 128 issues `issue_dw` (weight-gradient products, read only after
+  // warp 4 issues `issue_dw` (weight-gradient products, read only after
   // the tile loop) and commits it to dw_bar where one is given; a dW chain
   // is waited for only before the shared-memory operands it reads are
   // overwritten.  Every thread then runs `overlap` (half 1's share of the
@@ -267,14 +268,18 @@ __global__ void __launch_bounds__(kThreads, 1) train_tc_kernel(const TrainTcArgs
     tc::fence_proxy_async_smem();
     tc::tc_fence_before();
     if (!__syncthreads_and(ok)) return false;
-    if (lead) {
-      tc::tc_fence_after();
-      issue();
-      tc::mma_commit(bar_mma);
-    } else if (tid == kDwIssuer) {
-      tc::tc_fence_after();
-      issue_dw();
-      if (dw_bar != nullptr) tc::mma_commit(dw_bar);
+    if (warp_u == 0) {
+      if (tc::elect_one()) {
+        tc::tc_fence_after();
+        issue();
+        tc::mma_commit(bar_mma);
+      }
+    } else if (warp_u == kDwIssuer) {
+      if (tc::elect_one()) {
+        tc::tc_fence_after();
+        issue_dw();
+        if (dw_bar != nullptr) tc::mma_commit(dw_bar);
+      }
     }
     overlap();
     ok = tc::mbar_wait(bar_mma, phase, kWaitCycles);   // spin: one CTA per SM, nothing else to run
@@ -681,7 +686,7 @@ __global__ void __launch_bounds__(kThreads, 1) train_tc_kernel(const TrainTcArgs
   }
   if (!ok) {   // after an expired wait: let the weights' copy and both issuers' products finish
     tc::mbar_wait(bar_w, 0, kWaitCycles);
-    if (lead || tid == kDwIssuer) tc::mma_commit(bar_drain);
+    if ((warp_u == 0 || warp_u == kDwIssuer) && tc::elect_one()) tc::mma_commit(bar_drain);
     tc::mbar_wait(bar_drain, 0, kWaitCycles);
   }
   tc::tc_fence_before();
