@@ -5,15 +5,16 @@
 // A CTA holds one copy of the packed 16-bit weights in shared memory and WG
 // independent tile pipelines (warpgroups of 128 threads, one shading point
 // per thread and tile row).  Activations never touch shared memory: each
-// warpgroup owns 128 tensor-memory columns, [0, 64) for the FP32
-// accumulator D and [64, 128) for the 16-bit A operand of the next layer
-// (two values per 32-bit column, row i in lane i).
+// warpgroup owns 128 tensor-memory columns: the FP32 accumulator D, the 16-bit
+// A operand of the next layer (two values per 32-bit column, row i in lane i)
+// and the first layer's operand of the tile to come.
 //   1. one bulk (TMA) copy stages the weights and the per-material albedos
 //      in shared memory, once per CTA;
-//   2. each warpgroup loops over its 128-point tiles: every thread encodes
-//      its point (sin/cos of 8 octaves of u and v, log footprint, wi, wo)
-//      from registers loaded during the previous tile and stores its row of
-//      the layer-1 A operand into tensor memory (tcgen05.st);
+//   2. each warpgroup loops over its 128-point tiles: while a tile's products
+//      run, every thread encodes its point of the next one (sin/cos of 8
+//      octaves of u and v, log footprint, wi, wo) from registers loaded a tile
+//      earlier, stores that row of the layer-1 A operand into tensor memory
+//      (tcgen05.st), and writes out the tile before;
 //   3. layer 1 (the latent part of W1 folded into one per-material bias
 //      column selected by a one-hot of the material: W1 z_m + b1 is exact
 //      algebra, computed once per call) and layers 2-4 (their biases in a
@@ -27,8 +28,15 @@
 // column) with layer 1 in FP16; there the weights of layers 2-4 carry a
 // per-layer power-of-two scale, and the unscaling and their biases are one
 // FP32 FMA per value in the epilogue instead of a constant-one column.
-// While one warpgroup waits for its products the others encode and convert,
-// which keeps the tensor pipe and the ALUs busy together.
+// Bound by the latency of its own instruction stream at 4 warps per scheduler
+// (tensor memory holds no more tiles): issue 58 %, tensor pipe 42 %, ALU 46 %.
+// A tile's serial chain is therefore what counts, and per tile of a 1080p
+// FP16 frame (4900 cycles at 71.4 us) it lost: 270 to issuing by an elected
+// thread (65.4 us), and to encoding ahead and writing out late what the
+// products' latency hides, unrolled issue, octaves without the conversion
+// unit and loads a whole tile ahead, another 500 (59.5 us; 8.3 M points 267 ->
+// 242, step by step 260, 248, 242).  A fifth warp per CTA that only issues
+// measured 245 against 248 and costs registers the batched kernel needs.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <cuda_fp8.h>
@@ -41,8 +49,15 @@ namespace fab {
 namespace {
 
 constexpr int kTile = 128;
-constexpr uint32_t kColsPerTile = 128;             // D [0, 64) | A [64, 128)
+// Tensor-memory columns of a pipeline: D [0, 64), the A operand of layers 2-4
+// [64, 104) and the first kXSteps K = 16 steps of layer 1's [104, 128), apart,
+// so that a tile's inputs are encoded while the tile before it is in its
+// layers; layer 1's further steps (more than 9 materials) start at A's.
+constexpr uint32_t kColsPerTile = 128;
 constexpr uint32_t kColA = 64;
+constexpr uint32_t kColX = kColA + kKH / 2;
+constexpr int kXSteps = 3;
+static_assert(kColX + 8 * kXSteps == kColsPerTile, "layer 1's operand beside A");
 constexpr long long kWaitCycles = 4000000000ll;   // ~2 s at 2 GHz
 
 // Operand precision of a kernel instance.
@@ -224,12 +239,25 @@ __device__ __forceinline__ int find_segment(const TcArgs &a, const int64_t *seg_
   return lo;
 }
 
-// Where tile `tile`'s rows live: point index base and the buffers.
+// Where tile `tile`'s rows live: the buffers from its first point on.
 struct TileView {
   const float *u, *v, *radius, *wi, *wo;
   const uint16_t *material;
   float *rgb, *comps;
-  int64_t n, first;   // points in the segment, index of the tile's first point in it
+  int rows;   // points in the tile (0 for a tile past the last)
+
+  __device__ __forceinline__ void at(int64_t first, int64_t n) {
+    const int64_t left = n - first;
+    rows = left <= 0 ? 0 : left < kTile ? (int)left : kTile;
+    u += first;
+    v += first;
+    radius += first;
+    wi += 3 * first;
+    wo += 3 * first;
+    material += first;
+    rgb += 3 * first;
+    if (comps) comps += 4 * first;
+  }
 };
 
 template <bool MULTI>
@@ -237,17 +265,25 @@ __device__ __forceinline__ TileView tile_view(const TcArgs &a, const int64_t *se
   TileView t;
   if (!MULTI || tile >= a.n_tiles) {
     t.u = a.u; t.v = a.v; t.radius = a.radius; t.wi = a.wi; t.wo = a.wo; t.material = a.material;
-    t.rgb = a.rgb; t.comps = a.comps; t.n = MULTI ? 0 : a.n; t.first = tile * 128;
+    t.rgb = a.rgb; t.comps = a.comps;
+    t.at(tile * kTile, MULTI ? 0 : a.n);
   } else {
     int64_t t0;
     const int s = find_segment(a, seg_t0, tile, cursor, t0);
     cursor = s;
     const SegDesc &d = a.segs[s];
     t.u = d.u; t.v = d.v; t.radius = d.radius; t.wi = d.wi; t.wo = d.wo; t.material = d.material;
-    t.rgb = d.rgb; t.comps = d.comps; t.n = d.n; t.first = (tile - t0) * 128;
+    t.rgb = d.rgb; t.comps = d.comps;
+    t.at((tile - t0) * kTile, d.n);
   }
   return t;
 }
+
+// Where a tile's outputs go, and this row's material.
+struct TileOut {
+  float *rgb = nullptr, *comps = nullptr;
+  int rows = 0, mat = -1;
+};
 
 // sin / cos of 2 pi 2^k frac(x) for k = 0..7: f_k = frac(2^k frac(x)) is
 // exact in FP32 (doubling and dropping the integer part), and each octave
@@ -256,14 +292,18 @@ __device__ __forceinline__ TileView tile_view(const TcArgs &a, const int64_t *se
 // angle-doubling recurrence would; w[k] packs (sin, cos) of octave k.
 template <bool F16>
 __device__ __forceinline__ void octave_words(float x, uint32_t *w) {
-  float f = x - floorf(x);
+  float f = x - floorf(x);   // [0, 1]: 1 for tiny negative x
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
     float s, c;
     __sincosf(6.283185307179586f * (f - 0.5f), &s, &c);
     w[k] = tc::pack2<F16>(-s, -c);
-    f = 2.0f * f;
-    f -= floorf(f);
+    if (k == 0) {
+      f = 2.0f * f;
+      f -= floorf(f);
+    } else {
+      f = fmaf(2.0f, f, f >= 0.5f ? -1.0f : 0.0f);   // the same exact value without the conversion unit
+    }
   }
 }
 
@@ -277,11 +317,11 @@ struct Point {
 // (H = 1); with two threads per row (H = 2) half 0 takes u, the footprint and
 // the directions, half 1 takes v; both take the material.
 template <int H>
-__device__ __forceinline__ Point load_point(const TileView &a, int64_t p, int h) {
+__device__ __forceinline__ Point load_point(const TileView &a, int p, int h) {
   Point q;
   q.u = q.v = q.r = q.wi0 = q.wi1 = q.wi2 = q.wo0 = q.wo1 = q.wo2 = 0.0f;
   q.mat = -1;
-  if (p < a.n) {
+  if (p < a.rows) {
     q.mat = __ldg(a.material + p);
     if (H == 1 || h == 0) {
       q.u = __ldg(a.u + p);
@@ -333,6 +373,9 @@ __global__ void __launch_bounds__(kTile * H * WG, 4 / WG) decoder_tc_kernel(cons
   constexpr bool F8 = PR == kPrE4M3;
   constexpr int PT = kTile * H;         // threads per tile pipeline
   constexpr int CH = 2 / H;             // 32-column chunks of D per thread
+  // one thread per row has the registers to work ahead: the next tile is
+  // encoded, and the last one written out, while products run
+  constexpr bool AHEAD = H == 1;
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t *bar_w = reinterpret_cast<uint64_t *>(smem);
@@ -341,8 +384,8 @@ __global__ void __launch_bounds__(kTile * H * WG, 4 / WG) decoder_tc_kernel(cons
   const BlobLayout L = blob_layout(a.n_mat, a.k1, F8);
   uint8_t *wts = smem + 1024;
   const int tid = threadIdx.x;
-  const int wg = tid / PT;              // tile pipeline
-  const int tp = tid % PT;              // thread within the pipeline
+  const int wg = WG == 1 ? 0 : tid / PT;   // tile pipeline
+  const int tp = WG == 1 ? tid : tid % PT; // thread within the pipeline
   const int h = H == 1 ? 0 : tp >> 7;   // which half of the row's columns
   const int row = tp & (kTile - 1);     // tile row owned by this thread
   const int warp = tid >> 5;
@@ -371,7 +414,7 @@ __global__ void __launch_bounds__(kTile * H * WG, 4 / WG) decoder_tc_kernel(cons
   tc::tc_fence_after();
   const uint32_t tmem = *tmem_slot + kColsPerTile * (uint32_t)wg;   // this pipeline's D column 0, lane 0
   const uint32_t lane = (uint32_t)((warp & 3) * 32) << 16;          // this warp's lane quadrant
-  const uint32_t t_d = tmem + lane, t_a = tmem + lane + kColA;
+  const uint32_t t_d = tmem + lane, t_a = tmem + lane + kColA, t_x = tmem + lane + kColX;
 
   if (tid == 0) {
     tc::mbar_arrive_expect_tx(bar_w, L.total);
@@ -382,7 +425,7 @@ __global__ void __launch_bounds__(kTile * H * WG, 4 / WG) decoder_tc_kernel(cons
   int64_t tile = (int64_t)blockIdx.x * WG + wg;
   int seg_cursor = 0;   // segment of the pipeline's latest tile (batched launches)
   TileView view = tile_view<MULTI>(a, seg_t0, tile, seg_cursor);
-  Point pt = load_point<H>(view, view.first + row, h);
+  Point pt = load_point<H>(view, row, h);
   bool ok = tc::mbar_wait_sleep(bar_w, 0, kWaitCycles);
   const float *alb = reinterpret_cast<const float *>(wts + L.alb);
   const float *epi = reinterpret_cast<const float *>(wts + L.epi);   // E4M3 only
@@ -395,62 +438,106 @@ __global__ void __launch_bounds__(kTile * H * WG, 4 / WG) decoder_tc_kernel(cons
   const uint32_t one16 = F16 ? 0x3C00u : 0x3F80u;   // 1.0 in the operand type
   uint32_t phase = 0;
 
-  for (; tile < a.n_tiles; tile += stride) {
-    // this tile's outputs (the view moves on to the next tile at layer 1)
-    float *const out_rgb = view.rgb;
-    float *const out_comps = view.comps;
-    const int64_t p = view.first + row;
-    const int64_t p_end = view.n;
-    int mat = pt.mat;
-    if (mat >= a.n_mat) {
-      if (H == 1 || h == 0) atomicOr(a.status, kStatusBadMaterial);
-      mat = -2;
+  // ---- the three shares of a point's row of layer 1's operand (pt's)
+  auto encode_u = [&] {                              // features 0..15: octaves of u
+    uint32_t w[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
+    if (pt.mat >= 0) octave_words<F16>(pt.u, w);
+    tc::tmem_st8(t_x, w);
+  };
+  auto encode_v = [&] {                              // features 16..31: octaves of v
+    uint32_t w[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
+    if (pt.mat >= 0) octave_words<F16>(pt.v, w);
+    tc::tmem_st8(t_x + 8, w);
+  };
+  auto encode_rest = [&] {                           // features 32..47
+    uint32_t w[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
+    if (pt.mat >= 0) {
+      const float l = (__logf(fmaxf(pt.r, kRFloor)) - kLogRC0) * kLogRInvC1;
+      w[0] = tc::pack2<F16>(l, pt.wi0);
+      w[1] = tc::pack2<F16>(pt.wi1, pt.wi2);
+      w[2] = tc::pack2<F16>(pt.wo0, pt.wo1);
+      w[3] = tc::pack2<F16>(pt.wo2, pt.mat == 0 ? 1.0f : 0.0f);
     }
-    // ---- encode this thread's share of its row of the layer-1 A operand
-    {
+    // features 40.. are the one-hot material columns (39 is in w[3])
+    const int hot = kQueryFeat + pt.mat;
+    const uint32_t hot_word = one16 << (16 * (hot & 1));
+#pragma unroll
+    for (int k = 4; k < 8; ++k) w[k] = hot >> 1 == 16 + k ? hot_word : 0u;
+    tc::tmem_st8(t_x + 16, w);
+  };
+  auto encode_wide = [&](int mat) {                  // features 48.. (wider one-hot), in A's columns
+    const int hot = kQueryFeat + mat;
+    const uint32_t hot_word = one16 << (16 * (hot & 1));
+    for (int c = kXSteps; c < a.k1 / 16; ++c) {
       uint32_t w[8];
-      if (H == 1 || h == 0) {                        // features 0..15: octaves of u
-        if (mat >= 0) {
-          octave_words<F16>(pt.u, w);
-        } else {
 #pragma unroll
-          for (int k = 0; k < 8; ++k) w[k] = 0u;
-        }
-        tc::tmem_st8(t_a, w);
-      }
-      if (H == 1 || h == 1) {                        // features 16..31: octaves of v
-        if (mat >= 0) {
-          octave_words<F16>(pt.v, w);
-        } else {
-#pragma unroll
-          for (int k = 0; k < 8; ++k) w[k] = 0u;
-        }
-        tc::tmem_st8(t_a + 8, w);
-      }
-      if (H == 1 || h == 0) {
-        if (mat >= 0) {
-          const float l = (__logf(fmaxf(pt.r, kRFloor)) - kLogRC0) * kLogRInvC1;
-          w[0] = tc::pack2<F16>(l, pt.wi0);
-          w[1] = tc::pack2<F16>(pt.wi1, pt.wi2);
-          w[2] = tc::pack2<F16>(pt.wo0, pt.wo1);
-          w[3] = tc::pack2<F16>(pt.wo2, mat == 0 ? 1.0f : 0.0f);
-        } else {
-          w[0] = w[1] = w[2] = w[3] = 0u;
-        }
-        // features 40.. are the one-hot material columns (39 is in w[3])
-        const int hot = kQueryFeat + mat;
-#pragma unroll
-        for (int k = 4; k < 8; ++k) w[k] = (hot == 2 * (16 + k) ? one16 : 0u) | (hot == 2 * (16 + k) + 1 ? one16 << 16 : 0u);
-        tc::tmem_st8(t_a + 16, w);                   // features 32..47
-        for (int c = 3; c < a.k1 / 16; ++c) {        // features 48.. (wider one-hot)
-#pragma unroll
-          for (int k = 0; k < 8; ++k)
-            w[k] = (hot == 16 * c + 2 * k ? one16 : 0u) | (hot == 16 * c + 2 * k + 1 ? one16 << 16 : 0u);
-          tc::tmem_st8(t_a + 8 * c, w);
-        }
-      }
-      tc::tmem_st_wait();
+      for (int k = 0; k < 8; ++k) w[k] = hot >> 1 == 8 * c + k ? hot_word : 0u;
+      tc::tmem_st8(t_a + 8 * (c - kXSteps), w);
     }
+  };
+  auto check_material = [&] {
+    if (pt.mat >= a.n_mat) {
+      if (H == 1 || h == 0) atomicOr(a.status, kStatusBadMaterial);
+      pt.mat = -2;
+    }
+  };
+  // the latest finished tile's head outputs and where they go: written out
+  // while the next tile's first products run
+  float y[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+  TileOut done, cur, next;
+  auto write_out = [&] {
+    if ((H == 1 || h == 0) && row < done.rows) {
+      float c4[4];
+      if (done.mat < 0) {
+        c4[0] = c4[1] = c4[2] = c4[3] = __int_as_float(0x7FC00000);
+      } else {
+        // inverse of Eq. 9; exp(y) - 1 loses only absolute precision
+        // near y = 0, where S itself is ~0
+        c4[0] = fmaxf(0.0f, y[0]);
+        c4[1] = fmaxf(0.0f, y[1]);
+        c4[2] = fmaxf(0.0f, (__expf(y[2]) - 1.0f) * (1.0f / kSpecK));
+        c4[3] = fmaxf(0.0f, (__expf(y[3]) - 1.0f) * (1.0f / kSpecK));
+      }
+      if (done.comps) store_row4(done.comps, row, c4[0], c4[1], c4[2], c4[3]);
+      const float4 *al = reinterpret_cast<const float4 *>(alb + (done.mat < 0 ? 0 : done.mat) * 12);
+      const float4 k0 = al[0], k1 = al[1], k2 = al[2];   // kd_warp, kd_weft, ks_warp, ks_weft (RGB each)
+      done.rgb[3 * row + 0] = k0.x * c4[0] + k0.w * c4[1] + k1.z * c4[2] + k2.y * c4[3];
+      done.rgb[3 * row + 1] = k0.y * c4[0] + k1.x * c4[1] + k1.w * c4[2] + k2.z * c4[3];
+      done.rgb[3 * row + 2] = k0.z * c4[0] + k1.y * c4[1] + k2.x * c4[2] + k2.w * c4[3];
+    }
+  };
+
+  auto encode_all = [&] {
+    check_material();
+    if (H == 1 || h == 0) encode_u();
+    if (H == 1 || h == 1) encode_v();
+    if (H == 1 || h == 0) encode_rest();
+  };
+  // pt's outputs, and the loads of tile t's points into pt
+  auto out_of_pt = [&] {
+    TileOut o;
+    o.rgb = view.rgb;
+    o.comps = view.comps;
+    o.rows = view.rows;
+    o.mat = pt.mat;
+    return o;
+  };
+  auto load_tile = [&](int64_t t) {
+    view = tile_view<MULTI>(a, seg_t0, t, seg_cursor);
+    pt = load_point<H>(view, row, h);
+  };
+  if (AHEAD) {
+    encode_all();
+    cur = out_of_pt();
+    load_tile(tile + stride);
+  }
+  for (; tile < a.n_tiles; tile += stride) {
+    if (!AHEAD) {
+      encode_all();
+      cur = out_of_pt();
+    }
+    if (H == 1 || h == 0) encode_wide(cur.mat);
+    tc::tmem_st_wait();
     // ---- four layers
 #pragma unroll
     for (int layer = 0; layer < 4; ++layer) {
@@ -470,18 +557,43 @@ __global__ void __launch_bounds__(kTile * H * WG, 4 / WG) decoder_tc_kernel(cons
             tc::mma_f8_ts(tmem, tmem + kColA + 8u * kk, bd, layer == 3 ? id8_16 : id8_64, kk > 0 ? 1u : 0u);
           }
         } else {
+          // fully unrolled, the descriptors by an addition: with a loop over
+          // the steps a chain's issue took 276 cycles, so 217 (the rest is the
+          // other CTAs' products in the pipe)
           const int K = layer == 0 ? a.k1 : kKH;
-          const uint32_t sbo = (uint32_t)K * 16u;
-          for (int kk = 0; kk < K / 16; ++kk) {
-            const uint64_t bd = tc::smem_desc(w_addr + kk * 256u, 128u, sbo);
-            tc::mma_f16_ts(tmem, tmem + kColA + 8u * kk, bd, layer == 3 ? id16 : id64, kk > 0 ? 1u : 0u);
+          const uint64_t bd = tc::smem_desc(w_addr, 128u, (uint32_t)K * 16u);
+          const uint32_t id = layer == 3 ? id16 : id64;
+          if (layer == 0) {
+#pragma unroll
+            for (int kk = 0; kk < kXSteps; ++kk) tc::mma_f16_ts(tmem, tmem + kColX + 8u * kk, bd + 16u * kk, id, kk > 0 ? 1u : 0u);
+#pragma unroll
+            for (int kk = kXSteps; kk < 8; ++kk) {
+              if (16 * kk >= K) break;
+              tc::mma_f16_ts(tmem, tmem + kColA + 8u * (kk - kXSteps), bd + 16u * kk, id, 1u);
+            }
+          } else {
+#pragma unroll
+            for (int kk = 0; kk < kKH / 16; ++kk) tc::mma_f16_ts(tmem, tmem + kColA + 8u * kk, bd + 16u * kk, id, kk > 0 ? 1u : 0u);
           }
         }
         tc::mma_commit(my_bar);
       }
-      if (layer == 0) {   // next tile's inputs, in flight during this tile's layers
-        view = tile_view<MULTI>(a, seg_t0, tile + stride, seg_cursor);
-        pt = load_point<H>(view, view.first + row, h);
+      // while the products run: layer 1, the last tile's outputs; layers 2-4,
+      // the next tile's encoding (layer 1's products have read the columns it
+      // overwrites), from loads issued a tile earlier
+      if (!AHEAD) {
+        if (layer == 0) load_tile(tile + stride);
+      } else if (layer == 0) {
+        write_out();
+      } else if (layer == 1) {
+        check_material();
+        encode_u();
+      } else if (layer == 2) {
+        encode_v();
+      } else {
+        encode_rest();
+        next = out_of_pt();
+        load_tile(tile + 2 * stride);
       }
       // every warp sleeps on the mbarrier until the products land (no
       // further barrier hop); an expired wait is OR-reduced at the next
@@ -530,14 +642,14 @@ __global__ void __launch_bounds__(kTile * H * WG, 4 / WG) decoder_tc_kernel(cons
             tc::tmem_st16(t_a + 16 * chunk, w);
           }
         }
-        if (!F8 && (H == 1 || h == H - 1)) {
-          // constant-one column (bias of layers 2-4) and zero padding, K = 64..79
+        if (!F8 && layer == 0 && (H == 1 || h == H - 1)) {
+          // constant-one column (bias of layers 2-4) and zero padding, K =
+          // 64..79; only layer 1's widest operand overwrites it
           uint32_t w[8] = {one16, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
           tc::tmem_st8(t_a + 32, w);
         }
         tc::tmem_st_wait();
       } else if (H == 1 || h == 0) {
-        float y[4];
         tc::tmem_ld4(t_d, y);
         tc::tmem_ld_wait();
         if (F8) {
@@ -545,28 +657,13 @@ __global__ void __launch_bounds__(kTile * H * WG, 4 / WG) decoder_tc_kernel(cons
 #pragma unroll
           for (int c = 0; c < 4; ++c) y[c] = fmaf(y[c], inv, epi[kF8Bias + 64 * 3 + c]);
         }
-        if (p < p_end) {
-          float c4[4];
-          if (mat < 0) {
-            c4[0] = c4[1] = c4[2] = c4[3] = __int_as_float(0x7FC00000);
-          } else {
-            // inverse of Eq. 9; exp(y) - 1 loses only absolute precision
-            // near y = 0, where S itself is ~0
-            c4[0] = fmaxf(0.0f, y[0]);
-            c4[1] = fmaxf(0.0f, y[1]);
-            c4[2] = fmaxf(0.0f, (__expf(y[2]) - 1.0f) * (1.0f / kSpecK));
-            c4[3] = fmaxf(0.0f, (__expf(y[3]) - 1.0f) * (1.0f / kSpecK));
-          }
-          if (out_comps) store_row4(out_comps, p, c4[0], c4[1], c4[2], c4[3]);
-          const float4 *al = reinterpret_cast<const float4 *>(alb + (mat < 0 ? 0 : mat) * 12);
-          const float4 k0 = al[0], k1 = al[1], k2 = al[2];   // kd_warp, kd_weft, ks_warp, ks_weft (RGB each)
-          out_rgb[3 * p + 0] = k0.x * c4[0] + k0.w * c4[1] + k1.z * c4[2] + k2.y * c4[3];
-          out_rgb[3 * p + 1] = k0.y * c4[0] + k1.x * c4[1] + k1.w * c4[2] + k2.z * c4[3];
-          out_rgb[3 * p + 2] = k0.z * c4[0] + k1.y * c4[1] + k2.x * c4[2] + k2.w * c4[3];
-        }
+        done = cur;
+        if (!AHEAD) write_out();
       }
     }
+    if (AHEAD) cur = next;
   }
+  if (AHEAD && ok) write_out();
 
   ok = !wg_sync_or<PT>(wg, !ok);   // one outcome per pipeline
 teardown:

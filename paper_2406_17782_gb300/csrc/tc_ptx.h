@@ -100,6 +100,7 @@ __device__ __forceinline__ bool mbar_try_wait_sleep(uint64_t *bar, uint32_t pari
   return done != 0;
 }
 __device__ __forceinline__ bool mbar_wait_sleep(uint64_t *bar, uint32_t parity, long long max_cycles) {
+  if (mbar_try_wait_sleep(bar, parity, 200000u)) return true;   // the usual case reads no clock
   const long long t0 = clock64();
   while (!mbar_try_wait_sleep(bar, parity, 200000u)) {
     if (clock64() - t0 > max_cycles) return false;

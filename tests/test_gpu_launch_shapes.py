@@ -74,3 +74,33 @@ def test_encoder_of_records_passed_with_the_launch(fab, n_mat):
     mats = W.training_materials(8)[:64]
     fab.set_params(W.decoder_init(), W.encoder_init())
     assert torch.equal(fab.encode_params(mats[:n_mat]), fab.encode_params(mats)[:n_mat])
+
+
+@pytest.mark.parametrize("prec", ["fp16", "bf16", "fp8"])
+@pytest.mark.parametrize("n_mat", [1, 9, 10, 25, 26, 89])
+def test_tiles_encoded_ahead(fab, n_mat, prec):
+    """One thread per row encodes the next tile while a tile's products run,
+    two encode each tile when it starts: the same bits at the edges of the
+    tiles and of the rounds over them, and for every width of layer 1 (from
+    10 materials on its operand continues in another one's columns)."""
+    mats = np.resize(W.training_materials(8), n_mat)
+    fab.set_materials(mats)
+    fab.set_params(W.decoder_init(), W.encoder_init())
+    fab.prepare_neural(torch.from_numpy(W.random_latents(n_mat)).cuda(), prec)
+    wave = fab.sm_count * 4 * 128
+    host = W.frame_gbuffer()
+    try:
+        for n in (1, 127, 129, wave - 1, wave + 1, 3 * wave + 5):
+            part = W.subset(host, np.arange(n))
+            part["material"] = (np.arange(n) * 7 % n_mat).astype(np.uint16)
+            part["u"] = part["u"].copy()
+            part["u"][::5] = np.resize(np.float32([0.0, -1e-12, 0.5, -3.25, 1e5, 0.9999999]), len(part["u"][::5]))
+            g = GBuffer.from_numpy(part)
+            got = []
+            for h in (1, 2):
+                fab.set_launch_config(0, 0, 0, h)
+                got.append(fab.shade_neural_prepared(g, prec, comps=True))
+                fab.sync_status()
+            assert torch.equal(got[0][0], got[1][0]) and torch.equal(got[0][1], got[1][1]), n
+    finally:
+        fab.set_launch_config(0, 0, 0, 0)
