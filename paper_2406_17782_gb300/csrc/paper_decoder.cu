@@ -9,9 +9,10 @@
 // Same execution scheme as the workload's decoder (decoder_tc.cu): a
 // persistent CTA holds one copy of the packed 16-bit weights in shared memory
 // (one bulk copy), and WG tile pipelines of H warpgroups each stream
-// 128-point tiles, H threads per point.  Per pipeline, tensor memory holds the
-// FP32 accumulator D (W columns) and the 16-bit A operand of the next layer
-// (two values per 32-bit column).  Seven MMA chains per tile:
+// 128-point tiles, H threads per point.  Per pipeline, tensor memory holds two
+// regions of W columns: a layer's FP32 accumulator D in one, its 16-bit A
+// operand (two values per 32-bit column) in the other.  Seven MMA chains per
+// tile:
 //   L0  S1': [one-blob (24) | one-hot material] -> W     (latent folded: the
 //       per-material column holds S1[:, :64] z_m + s1, exact algebra)
 //   L1  S2 : h1 -> h                                    (bias in a constant-one column)
@@ -27,6 +28,7 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include "f32x2.h"
 #include "fabric_internal.h"
 #include "paper_net.h"
 #include "tc_ptx.h"
@@ -35,6 +37,10 @@ namespace fab {
 namespace {
 
 constexpr int kTile = 128;
+// A layer's operand begins kColBias columns of its region after the packed
+// values of the first 32 inputs: its K step W / 16, the bias input (and after
+// the spatial fusion the angular ones).  Layer 0's operand begins there too.
+constexpr uint32_t kColBias = 16;
 constexpr long long kWaitCycles = 4000000000ll;   // ~2 s at 2 GHz
 constexpr int kPnMaxK1 = 128;                     // layer-0 K: 24 + materials, padded to 16
 
@@ -136,8 +142,8 @@ struct PnPoint {
   int mat;   // -1: beyond the end
 };
 
-// What thread h of the point's H threads needs: the first u and the radius,
-// the last v and the angular inputs.
+// What thread h of the point's H threads needs: the first u, the radius and
+// the angular inputs, the last v.
 template <int H>
 __device__ __forceinline__ PnPoint pn_load(const PnArgs &a, int64_t p, int h) {
   PnPoint q;
@@ -148,15 +154,13 @@ __device__ __forceinline__ PnPoint pn_load(const PnArgs &a, int64_t p, int h) {
     if (H == 1 || h == 0) {
       q.u = __ldg(a.u + p);
       q.r = __ldg(a.radius + p);
-    }
-    if (H == 1 || h == 1) {
-      q.v = __ldg(a.v + p);
       q.wi0 = __ldg(a.wi + 3 * p);
       q.wi1 = __ldg(a.wi + 3 * p + 1);
       q.wi2 = __ldg(a.wi + 3 * p + 2);
       q.wo0 = __ldg(a.wo + 3 * p);
       q.wo1 = __ldg(a.wo + 3 * p + 1);
     }
+    if (H == 1 || h == 1) q.v = __ldg(a.v + p);
   }
   return q;
 }
@@ -199,22 +203,29 @@ __device__ __forceinline__ void blob_plain(float t, uint32_t *w) {
   for (int k = 0; k < 4; ++k) w[k] = tc::pack2<F16>(b[2 * k], b[2 * k + 1]);
 }
 
-template <int PT>
-__device__ __forceinline__ bool pn_bar_or(int wg, bool pred) {
+// Named barriers over the N threads of a pipeline: OR-reducing `pred`, and
+// split into the waiting side (the issuing warp) and the arriving one.
+template <int N>
+__device__ __forceinline__ bool pn_bar_or(int id, bool pred) {
   int r;
-  const int id = 1 + wg;
   asm volatile(
       "{\n\t.reg .pred p, q;\n\t"
       "setp.ne.b32 p, %1, 0;\n\t"
       "bar.red.or.pred q, %2, %3, p;\n\t"
       "selp.s32 %0, 1, 0, q;\n\t}"
       : "=r"(r)
-      : "r"((int)pred), "r"(id), "n"(PT)
+      : "r"((int)pred), "r"(id), "n"(N)
       : "memory");
   return r != 0;
 }
-
-__device__ __forceinline__ float lrelu(float x) { return fmaxf(x, kPnSlope * x); }
+template <int N>
+__device__ __forceinline__ void pn_bar_sync(int id) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(N) : "memory");
+}
+template <int N>
+__device__ __forceinline__ void pn_bar_arrive(int id) {
+  asm volatile("bar.arrive %0, %1;" ::"r"(id), "n"(N) : "memory");
+}
 
 template <bool F16>
 __device__ __forceinline__ float2 unpack2(uint32_t w) {
@@ -226,34 +237,49 @@ __device__ __forceinline__ float2 unpack2(uint32_t w) {
 }
 
 // W: network width; F16: FP16 (else BF16) operands; WG tile pipelines per CTA;
-// H threads per point (each takes W / H accumulator columns); LDR: 32-column
-// tensor-memory loads in flight per wait in the epilogues.
-template <int W, bool F16, int WG, int H, int LDR>
-__global__ void __launch_bounds__(kTile * WG * H, (W == 64 && WG == 2) ? 2 : 1) pn_decoder_kernel(const PnArgs a) {
+// H threads per point, each with two of the 32-column chunks of the
+// accumulator (chunk c H + h in turn c, so that the chunks are done in order).
+// Bound by the chain of a tile's seven layers, of which tensor memory holds two
+// tiles per SM at width 128.  With one accumulator and one operand column set
+// a layer's conversion (665 cycles) and its products (1090 with their issue)
+// took turns; with the next layer's first products under the second half of
+// the conversion, the next tile's encoding under the head and packed
+// multiplies for the leaky ReLU: 1080p, 8 materials, width 128 363 -> 302 us
+// (tensor pipe 43 -> 60 %, issue 60 %), width 64 158 -> 155 us (issue-bound).
+template <int W, bool F16, int WG, int H>
+__global__ void __launch_bounds__(kTile * WG * H, W == 64 ? 2 : 1) pn_decoder_kernel(const PnArgs a) {
+  static_assert(W == 64 * H, "two chunks per thread");
   constexpr int PT = kTile * H;
-  constexpr int CH = W / 32 / H;   // 32-column chunks per thread
   constexpr uint32_t COLS = pn_cols(W);
-  constexpr uint32_t COL_A = W;
+  static_assert(COLS == 2 * W, "two regions");
   constexpr int KH = W + 16;
+  constexpr int HALF = W / 32;      // K steps of the first turn's chunks
+  constexpr int FIT = (W - (int)kColBias) / 8;   // K steps of layer 0 beside D of layer 6
+  static_assert(H == 1 || FIT >= kPnMaxK1 / 16, "further steps overwrite the head's columns, which h = 0 reads");
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t *bar_w = reinterpret_cast<uint64_t *>(smem);
-  uint64_t *bar_mma = bar_w + 1;
-  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bar_w + 1 + WG);
+  uint64_t *bar_mma = bar_w + 1;         // one per pipeline
+  uint64_t *bar_drain = bar_mma + WG;    // one per pipeline: its products, after a failed wait
+  uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bar_drain + WG);
   const PnBlob B = pn_blob(W, a.n_mat);
   uint8_t *wts = smem + 1024;
   const int tid = threadIdx.x;
-  const int wg = tid / PT;
-  const int row = tid % kTile;
-  const int h = H == 1 ? 0 : (tid % PT) / kTile;
   const int warp = tid >> 5;
-  const bool lead = tid % PT == 0;
-  const bool lead_warp = __shfl_sync(0xFFFFFFFFu, warp, 0) % (PT / 32) == 0;
+  const int warp_u = __shfl_sync(0xFFFFFFFFu, warp, 0);   // uniform to the compiler (see elect_one)
+  const int wg = warp_u / (PT / 32);
+  const int row = tid % kTile;
+  const int h = H == 1 ? 0 : warp_u / (kTile / 32) % H;
+  const bool lead = warp_u % (PT / 32) == 0;   // the warp that issues the pipeline's products
   uint64_t *my_bar = bar_mma + wg;
+  const int bar0 = 1 + 2 * wg;   // named barriers of the two turns
 
   if (tid == 0) {
     tc::mbar_init(bar_w, 1);
-    for (int g = 0; g < WG; ++g) tc::mbar_init(bar_mma + g, 1);
+    for (int g = 0; g < WG; ++g) {
+      tc::mbar_init(bar_mma + g, 1);
+      tc::mbar_init(bar_drain + g, 1);
+    }
     tc::fence_mbar_init();
   }
   if (warp == 0) tc::tmem_alloc(tmem_slot, COLS * WG);
@@ -262,7 +288,6 @@ __global__ void __launch_bounds__(kTile * WG * H, (W == 64 && WG == 2) ? 2 : 1) 
   tc::tc_fence_after();
   const uint32_t tmem = *tmem_slot + COLS * (uint32_t)wg;
   const uint32_t lane = (uint32_t)((warp & 3) * 32) << 16;
-  const uint32_t t_d = tmem + lane, t_a = tmem + lane + COL_A;
 
   if (tid == 0) {
     tc::mbar_arrive_expect_tx(bar_w, B.total);
@@ -271,145 +296,202 @@ __global__ void __launch_bounds__(kTile * WG * H, (W == 64 && WG == 2) ? 2 : 1) 
   const int64_t stride = (int64_t)gridDim.x * WG;
   int64_t tile = (int64_t)blockIdx.x * WG + wg;
   PnPoint pt = pn_load<H>(a, tile * kTile + row, h);
-  bool ok = tc::mbar_wait_sleep(bar_w, 0, kWaitCycles);
+  bool ok = __all_sync(0xFFFFFFFFu, tc::mbar_wait_sleep(bar_w, 0, kWaitCycles));   // one outcome per warp
   const float *alb = reinterpret_cast<const float *>(wts + B.alb);
-  uint32_t wl[7];
-#pragma unroll
-  for (int l = 0; l < 7; ++l) wl[l] = tc::smem_addr(wts + B.l[l]);
+  const uint32_t w_base = tc::smem_addr(wts);
   const uint32_t idW = F16 ? tc::idesc_f16(128, W) : tc::idesc_bf16(128, W);
   const uint32_t id16 = F16 ? tc::idesc_f16(128, 16) : tc::idesc_bf16(128, 16);
   const uint32_t one16 = F16 ? 0x3C00u : 0x3F80u;
+  const uint64_t slope = pk2(kPnSlope, kPnSlope);
   uint32_t phase = 0;
+  uint32_t par = 0;   // 0 or W: the region of this tile's even accumulators
 
-  for (; tile < a.n_tiles; tile += stride) {
-    const int64_t p = tile * kTile + row;
-    int mat = pt.mat;
-    if (mat >= a.n_mat) {
+  // Layer l's accumulator is in region R(l), its operand in the other one, on
+  // top of the accumulator it was made from: the values of chunk j in columns
+  // 32 j .. 32 j + 15, the bias step in 16 .. 23.  So the products of a
+  // layer's first inputs run while its last ones are still being converted.
+  // Layer 0's operand lies in R(6), past the head's 16 columns; K steps that
+  // do not fit are written into those once the head has been read.
+  auto issue = [&](int layer, int turn) {
+    if (tc::elect_one() && ok) {
+      tc::tc_fence_after();
+      const uint32_t rd = tmem + ((layer & 1) ? W - par : par), ra = tmem + ((layer & 1) ? par : W - par);
+      const uint32_t id = layer == 6 ? id16 : idW;
+      if (layer == 0) {
+        const uint64_t bd = tc::smem_desc(w_base + B.l[0], 128u, (uint32_t)B.k1 * 16u);
+#pragma unroll
+        for (int kk = 0; kk < kPnMaxK1 / 16; ++kk) {
+          if (16 * kk >= B.k1) break;
+          tc::mma_f16_ts(rd, ra + (kk < FIT ? kColBias + 8u * kk : 8u * (kk - FIT)), bd + 16u * kk, id, kk > 0 ? 1u : 0u);
+        }
+      } else {
+        const uint64_t bd = tc::smem_desc(w_base + B.l[layer], 128u, KH * 16u);
+#pragma unroll
+        for (int kk = turn * HALF; kk < (turn == 0 ? HALF : KH / 16); ++kk)
+          tc::mma_f16_ts(rd, ra + (kk < W / 16 ? 16u * (kk & ~1) + 8u * (kk & 1) : kColBias), bd + 16u * kk, id, kk > 0 ? 1u : 0u);
+      }
+      if (turn == 1) tc::mma_commit(my_bar);
+    }
+    __syncwarp();
+  };
+  // This warp's stores of a turn are done: the issuing warp waits for the
+  // others and issues, the others go on.  They cannot arrive twice in a turn:
+  // the next one follows the wait for this layer's products, or, once such a
+  // wait has expired, everybody waits here until the tile's end.
+  auto hand_over = [&](int layer, int turn) {
+    tc::tmem_st_wait();
+    tc::tc_fence_before();
+    if (lead) {
+      pn_bar_sync<PT>(bar0 + turn);
+      issue(layer, turn);
+    } else if (ok) {
+      pn_bar_arrive<PT>(bar0 + turn);
+    } else {
+      pn_bar_sync<PT>(bar0 + turn);
+    }
+  };
+  // layer 0's operand of pt's point: one-blob (24 channels), one-hot material
+  auto hot_words = [&](int c, int mat, uint32_t *w8) {   // K step c (16 features) of the one-hot part
+    const int hot = kPnBlob + mat;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) w8[k] = hot >> 1 == 8 * c + k ? one16 << (16 * (hot & 1)) : 0u;
+  };
+  auto encode = [&](uint32_t t_x) {
+    if (pt.mat >= a.n_mat) {
       if (h == 0) atomicOr(a.status, kStatusBadMaterial);
-      mat = -2;
+      pt.mat = -2;
     }
-    const float wi0 = pt.wi0, wi1 = pt.wi1, wi2 = pt.wi2, wo0 = pt.wo0, wo1 = pt.wo1;
-    // ---- layer-0 A operand: one-blob (24 channels) and the one-hot material
-    {
-      const int hot = kPnBlob + mat;   // feature index of the material's bias column
-      if (H == 1 || h == 0) {
-        uint32_t wu[4] = {0u, 0u, 0u, 0u}, wr[4] = {0u, 0u, 0u, 0u};
-        if (mat >= 0) {
-          blob_periodic<F16>(pt.u, wu);
-          const float t = (__logf(fmaxf(pt.r, kRFloor)) - kPnLnRLo) * kPnInvLnSpan;
-          blob_plain<F16>(t, wr);
-        }
-        tc::tmem_st4(t_a, wu);
-        tc::tmem_st4(t_a + 8, wr);
+    if (H == 1 || h == 0) {
+      uint32_t wu[4] = {0u, 0u, 0u, 0u}, wr[4] = {0u, 0u, 0u, 0u};
+      if (pt.mat >= 0) {
+        blob_periodic<F16>(pt.u, wu);
+        const float t = (__logf(fmaxf(pt.r, kRFloor)) - kPnLnRLo) * kPnInvLnSpan;
+        blob_plain<F16>(t, wr);
       }
-      if (H == 1 || h == 1) {
-        uint32_t wv[4] = {0u, 0u, 0u, 0u}, w[4];
-        if (mat >= 0) blob_periodic<F16>(pt.v, wv);
-        tc::tmem_st4(t_a + 4, wv);
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-          w[k] = (hot == 24 + 2 * k ? one16 : 0u) | (hot == 25 + 2 * k ? one16 << 16 : 0u);
-        tc::tmem_st4(t_a + 12, w);       // features 24..31
-        for (int c = 2; c < B.k1 / 16; ++c) {
-          uint32_t h8[8];
-#pragma unroll
-          for (int k = 0; k < 8; ++k)
-            h8[k] = (hot == 16 * c + 2 * k ? one16 : 0u) | (hot == 16 * c + 2 * k + 1 ? one16 << 16 : 0u);
-          tc::tmem_st8(t_a + 8 * c, h8);
-        }
-      }
-      tc::tmem_st_wait();
+      tc::tmem_st4(t_x, wu);
+      tc::tmem_st4(t_x + 8, wr);
     }
-    uint32_t skip[16 * CH];   // k1 as 16-bit operand pairs, for the residual block
+    if (H == 1 || h == 1) {
+      uint32_t wv[4] = {0u, 0u, 0u, 0u}, w8[8];
+      if (pt.mat >= 0) blob_periodic<F16>(pt.v, wv);
+      tc::tmem_st4(t_x + 4, wv);
+      hot_words(1, pt.mat, w8);
+      tc::tmem_st4(t_x + 12, w8 + 4);       // features 24..31
+      for (int c = 2; c < B.k1 / 16 && c < FIT; ++c) {
+        hot_words(c, pt.mat, w8);
+        tc::tmem_st8(t_x + 8 * c, w8);
+      }
+    }
+  };
+  // a tile's head outputs, written while the next tile's first products run
+  float y[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+  int64_t done_p = a.n;
+  int done_mat = -1, cur_mat = -1;
+  auto write_out = [&] {
+    if ((H == 1 || h == 0) && done_p < a.n) {
+      float c4[4];
+      if (done_mat < 0) {
+        c4[0] = c4[1] = c4[2] = c4[3] = __int_as_float(0x7FC00000);
+      } else {
+        c4[0] = fmaxf(0.0f, y[0]);
+        c4[1] = fmaxf(0.0f, y[1]);
+        c4[2] = fmaxf(0.0f, (__expf(y[2]) - 1.0f) * (1.0f / kSpecK));
+        c4[3] = fmaxf(0.0f, (__expf(y[3]) - 1.0f) * (1.0f / kSpecK));
+      }
+      if (a.comps) store_row4(a.comps, done_p, c4[0], c4[1], c4[2], c4[3]);
+      const float4 *al = reinterpret_cast<const float4 *>(alb + (done_mat < 0 ? 0 : done_mat) * 12);
+      const float4 k0 = al[0], k1 = al[1], k2 = al[2];
+      a.rgb[3 * done_p + 0] = k0.x * c4[0] + k0.w * c4[1] + k1.z * c4[2] + k2.y * c4[3];
+      a.rgb[3 * done_p + 1] = k0.y * c4[0] + k1.x * c4[1] + k1.w * c4[2] + k2.z * c4[3];
+      a.rgb[3 * done_p + 2] = k0.z * c4[0] + k1.y * c4[1] + k2.x * c4[2] + k2.w * c4[3];
+    }
+  };
+
+  encode(tmem + lane + W - par + kColBias);
+  for (; tile < a.n_tiles; tile += stride) {
+    cur_mat = pt.mat;
+    // the angular inputs, with the constant one of A1's bias after them
+    const uint32_t ang0 = tc::pack2<F16>(pt.wi0, pt.wi1), ang1 = tc::pack2<F16>(pt.wi2, pt.wo0);
+    const uint32_t ang2 = tc::pack2<F16>(pt.wo1, 1.0f);
+    if (H == 1 || h == 1) {
+      for (int c = FIT; c < B.k1 / 16; ++c) {
+        uint32_t w8[8];
+        hot_words(c, cur_mat, w8);
+        tc::tmem_st8(tmem + lane + W - par + 8 * (c - FIT), w8);
+      }
+    }
+    tc::tmem_st_wait();
+    tc::tc_fence_before();
+    if (pn_bar_or<PT>(bar0, !ok)) {
+      ok = false;
+      goto teardown;
+    }
+    if (lead) issue(0, 1);
+    pt = pn_load<H>(a, (tile + stride) * kTile + row, h);
+    write_out();
+    uint32_t skip[32];   // k1 as 16-bit operand pairs, for the residual block
 #pragma unroll
-    for (int layer = 0; layer < 7; ++layer) {
-      tc::tc_fence_before();
-      if (pn_bar_or<PT>(wg, !ok)) {
-        ok = false;
-        goto teardown;
-      }
-      if (lead_warp && tc::elect_one()) {
-        tc::tc_fence_after();
-        const int K = layer == 0 ? B.k1 : KH;
-        const uint32_t sbo = (uint32_t)K * 16u;
-        for (int kk = 0; kk < K / 16; ++kk) {
-          const uint64_t bd = tc::smem_desc(wl[layer] + kk * 256u, 128u, sbo);
-          tc::mma_f16_ts(tmem, tmem + COL_A + 8u * kk, bd, layer == 6 ? id16 : idW, kk > 0 ? 1u : 0u);
-        }
-        tc::mma_commit(my_bar);
-      }
-      if (layer == 0) pt = pn_load<H>(a, (tile + stride) * kTile + row, h);   // next tile's inputs in flight
-      ok = tc::mbar_wait_sleep(my_bar, phase, kWaitCycles) && ok;
+    for (int layer = 0; layer < 6; ++layer) {
+      ok = __all_sync(0xFFFFFFFFu, ok && tc::mbar_wait_sleep(my_bar, phase, kWaitCycles));
       phase ^= 1u;
       tc::tc_fence_after();
-      if (layer < 6) {
+      const uint32_t t_d = tmem + lane + ((layer & 1) ? W - par : par);   // and the next operand
+      float acc[2][32];
+      tc::tmem_ld32(t_d + 32 * h, acc[0]);
+      tc::tmem_ld_wait32(acc[0]);
+      tc::tmem_ld32(t_d + 32 * (H + h), acc[1]);
 #pragma unroll
-        for (int c0 = 0; c0 < CH; c0 += LDR) {
-          const int col0 = CH * h + c0;   // chunk of D
-          float acc[32 * LDR];
+      for (int c = 0; c < 2; ++c) {
+        if (c == 1) tc::tmem_ld_wait32(acc[1]);
+        uint32_t w[16];
 #pragma unroll
-          for (int r = 0; r < LDR; ++r) tc::tmem_ld32(t_d + 32 * (col0 + r), acc + 32 * r);
-          tc::tmem_ld_wait();
-#pragma unroll
-          for (int r = 0; r < LDR; ++r) {
-            uint32_t w[16];
-#pragma unroll
-            for (int k = 0; k < 16; ++k) {
-              float x0 = acc[32 * r + 2 * k], x1 = acc[32 * r + 2 * k + 1];
-              if (layer == 4) {
-                const float2 s = unpack2<F16>(skip[(c0 + r) * 16 + k]);
-                x0 += s.x;
-                x1 += s.y;
-              }
-              w[k] = tc::pack2<F16>(lrelu(x0), lrelu(x1));
-              if (layer == 2) skip[(c0 + r) * 16 + k] = w[k];
-            }
-            tc::tmem_st16(t_a + 16 * (col0 + r), w);
+        for (int k = 0; k < 16; ++k) {
+          uint64_t x = pk2(acc[c][2 * k], acc[c][2 * k + 1]);
+          if (layer == 4) {
+            const float2 s = unpack2<F16>(skip[16 * c + k]);
+            x = add2(x, pk2(s.x, s.y));
           }
+          float x0, x1, l0, l1;
+          upk2(x, x0, x1);
+          upk2(mul2(x, slope), l0, l1);
+          w[k] = tc::pack2<F16>(fmaxf(x0, l0), fmaxf(x1, l1));   // leaky ReLU
+          if (layer == 2) skip[16 * c + k] = w[k];
         }
-        // input columns W..W+15: the angular inputs and the constant one of
-        // A1's bias after the spatial fusion, else the constant-one bias column
-        if (H == 1 || h == 1) {
+        tc::tmem_st16(t_d + 32 * (c * H + h), w);
+        if (c == 0 && h == 0) {
           uint32_t w8[8] = {one16, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
           if (layer == 1) {
-            w8[0] = tc::pack2<F16>(wi0, wi1);
-            w8[1] = tc::pack2<F16>(wi2, wo0);
-            w8[2] = tc::pack2<F16>(wo1, 1.0f);
+            w8[0] = ang0;
+            w8[1] = ang1;
+            w8[2] = ang2;
           }
-          tc::tmem_st8(t_a + W / 2, w8);
+          tc::tmem_st8(t_d + kColBias, w8);
         }
-        tc::tmem_st_wait();
-      } else if (H == 1 || h == 0) {
-        float y[4];
-        tc::tmem_ld4(t_d, y);
-        tc::tmem_ld_wait();
-        if (p < a.n) {
-          float c4[4];
-          if (mat < 0) {
-            c4[0] = c4[1] = c4[2] = c4[3] = __int_as_float(0x7FC00000);
-          } else {
-            c4[0] = fmaxf(0.0f, y[0]);
-            c4[1] = fmaxf(0.0f, y[1]);
-            c4[2] = fmaxf(0.0f, (__expf(y[2]) - 1.0f) * (1.0f / kSpecK));
-            c4[3] = fmaxf(0.0f, (__expf(y[3]) - 1.0f) * (1.0f / kSpecK));
-          }
-          if (a.comps) store_row4(a.comps, p, c4[0], c4[1], c4[2], c4[3]);
-          const float4 *al = reinterpret_cast<const float4 *>(alb + (mat < 0 ? 0 : mat) * 12);
-          const float4 k0 = al[0], k1 = al[1], k2 = al[2];
-          a.rgb[3 * p + 0] = k0.x * c4[0] + k0.w * c4[1] + k1.z * c4[2] + k2.y * c4[3];
-          a.rgb[3 * p + 1] = k0.y * c4[0] + k1.x * c4[1] + k1.w * c4[2] + k2.z * c4[3];
-          a.rgb[3 * p + 2] = k0.z * c4[0] + k1.y * c4[1] + k2.x * c4[2] + k2.w * c4[3];
-        }
+        hand_over(layer + 1, c);
       }
     }
+    // under the head's products: the next tile's layer 0 operand
+    encode(tmem + lane + par + kColBias);
+    ok = __all_sync(0xFFFFFFFFu, ok && tc::mbar_wait_sleep(my_bar, phase, kWaitCycles));
+    phase ^= 1u;
+    tc::tc_fence_after();
+    if (H == 1 || h == 0) {
+      tc::tmem_ld4(tmem + lane + par, y);
+      tc::tmem_ld_wait();
+      done_p = tile * kTile + row;
+      done_mat = cur_mat;
+    }
+    par = W - par;
   }
+  if (ok) write_out();
 
-  ok = !pn_bar_or<PT>(wg, !ok);
+  ok = !pn_bar_or<PT>(bar0, !ok);
 teardown:
-  if (!ok) {
-    if (lead) atomicOr(a.status, kStatusTimeout);
+  if (!ok) {   // let the weights' copy and the pipeline's products land before the memory goes away
+    if ((tid & 31) == 0) atomicOr(a.status, kStatusTimeout);
+    if (lead && tc::elect_one()) tc::mma_commit(bar_drain + wg);
     tc::mbar_wait(bar_w, 0, kWaitCycles);
-    tc::mbar_wait(my_bar, phase ^ 1u, kWaitCycles);
+    tc::mbar_wait(bar_drain + wg, 0, kWaitCycles);
   }
   tc::tc_fence_before();
   __syncthreads();
@@ -432,8 +514,8 @@ constexpr int pn_threads(int w) { return w == 64 ? 1 : 2; }
 // tensor-memory columns are taken.
 template <int W, bool F16>
 const void *pn_kernel() {
-  if (W == 64) return reinterpret_cast<const void *>(pn_decoder_kernel<64, F16, kPnWG, pn_threads(64), 1>);
-  return reinterpret_cast<const void *>(pn_decoder_kernel<128, F16, kPnWG, pn_threads(128), 2>);
+  if (W == 64) return reinterpret_cast<const void *>(pn_decoder_kernel<64, F16, kPnWG, pn_threads(64)>);
+  return reinterpret_cast<const void *>(pn_decoder_kernel<128, F16, kPnWG, pn_threads(128)>);
 }
 
 }  // namespace

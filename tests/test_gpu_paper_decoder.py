@@ -139,3 +139,31 @@ def test_paper_decoder_bad_material_index(fab, net):
     assert e.value.status == 7
     c = comps.cpu().numpy()
     assert np.isnan(c[40]).all() and np.isfinite(np.delete(c, 40, 0)).all()
+
+
+@pytest.mark.parametrize("n_mat", [1, 8, 9, 72, 73, 104])
+def test_paper_tiles_of_a_long_call_match_short_ones(fab, net, n_mat):
+    """A pipeline works several tiles ahead and behind, in tensor-memory
+    regions that swap from tile to tile: each point comes out bit for bit as in
+    a call of one round of tiles, where every tile is the first of its
+    pipeline.  From 9, 73 materials on layer 0 has a further K step, and at
+    width 64 one that waits for the head."""
+    w, mats, dec, z = net
+    fab.set_materials(np.resize(mats, n_mat))
+    try:
+        round_ = fab.sm_count * (4 if w == 64 else 2) * 128
+        n = 3 * round_ + 129
+        host = W.subset(W.frame_gbuffer(), np.arange(n))
+        host["material"] = (np.arange(n) * 7 % n_mat).astype(np.uint16)
+        lat = torch.from_numpy(W.random_latents(n_mat, seed=33, dim=64)).cuda()
+        for prec in ("fp16", "bf16"):
+            fab.paper_prepare(lat, prec)
+            rgb, comps = fab.paper_shade_prepared(GBuffer.from_numpy(host), prec, comps=True)
+            for first in range(0, n, round_):
+                part = slice(first, min(first + round_, n))
+                g = GBuffer.from_numpy(W.subset(host, np.arange(part.start, part.stop)))
+                got_rgb, got_c = fab.paper_shade_prepared(g, prec, comps=True)
+                fab.sync_status()
+                assert torch.equal(got_rgb, rgb[part]) and torch.equal(got_c, comps[part]), (prec, first)
+    finally:
+        fab.set_materials(mats)
