@@ -377,7 +377,7 @@ __global__ void __launch_bounds__(kTile * H * WG, 4 / WG) decoder_tc_kernel(cons
   // encoded, and the last one written out, while products run
   constexpr bool AHEAD = H == 1;
   extern __shared__ uint8_t smem_raw[];
-  uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t *smem = smem_raw + (-tc::smem_addr(smem_raw) & 1023u);   // an offset: a rounded address would be generic
   uint64_t *bar_w = reinterpret_cast<uint64_t *>(smem);
   uint64_t *bar_mma = bar_w + 1;                         // one per pipeline
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bar_w + 1 + WG);

@@ -257,7 +257,7 @@ __global__ void __launch_bounds__(kTile * WG * H, W == 64 ? 2 : 1) pn_decoder_ke
   constexpr int FIT = (W - (int)kColBias) / 8;   // K steps of layer 0 beside D of layer 6
   static_assert(H == 1 || FIT >= kPnMaxK1 / 16, "further steps overwrite the head's columns, which h = 0 reads");
   extern __shared__ uint8_t smem_raw[];
-  uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t *smem = smem_raw + (-tc::smem_addr(smem_raw) & 1023u);   // an offset: a rounded address would be generic
   uint64_t *bar_w = reinterpret_cast<uint64_t *>(smem);
   uint64_t *bar_mma = bar_w + 1;         // one per pipeline
   uint64_t *bar_drain = bar_mma + WG;    // one per pipeline: its products, after a failed wait

@@ -74,6 +74,7 @@ constexpr uint32_t kColD = 0, kColA = 64, kColW1 = 128, kColW2 = 192, kColW3 = 2
 // 32 columns per tile from kColDz, for the per-material sums at the end.
 constexpr uint32_t kColDz = 336;
 constexpr int kDzTiles = 5;
+constexpr int kSumList = kRows;   // rows looked through, and at most listed, at a time by the per-material sums
 static_assert(kColDz + 32 * kDzTiles <= 512, "latent-gradient rows inside the allocation");
 
 // Warp 0's elected thread issues the products the epilogues read; that of warp
@@ -186,7 +187,7 @@ __global__ void __launch_bounds__(kThreads, 1) train_tc_kernel(const TrainTcArgs
   // the wait for them comes before the weights and latents they write.
   grid_dependents_launch();
   extern __shared__ uint8_t smem_raw[];
-  uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t *smem = smem_raw + (-tc::smem_addr(smem_raw) & 1023u);   // an offset: a rounded address would be generic
   uint64_t *bar_w = reinterpret_cast<uint64_t *>(smem);
   uint64_t *bar_mma = bar_w + 1;     // warp 0's products
   uint64_t *bar_dw = bar_w + 2;      // [3]: dW4, dW3 and dW1 (each once per tile)
@@ -239,20 +240,20 @@ __global__ void __launch_bounds__(kThreads, 1) train_tc_kernel(const TrainTcArgs
 
   // one MMA chain (K/16 steps) of A in tensor memory by B in shared memory
   auto mma_ts = [&](uint32_t d_col, uint32_t b_addr, int K, int N) {
-    for (int kk = 0; kk < K / 16; ++kk) {
-      const uint64_t bd = tc::smem_desc(b_addr + kk * 256u, 128u, (uint32_t)K * 16u);
-      tc::mma_f16_ts(tmem + d_col, tmem + kColA + 8u * kk, bd, tc::idesc_bf16(128, N), kk > 0 ? 1u : 0u);
-    }
+    const uint64_t bd = tc::smem_desc(b_addr, 128u, (uint32_t)K * 16u);
+#pragma unroll
+    for (int kk = 0; kk < K / 16; ++kk)
+      tc::mma_f16_ts(tmem + d_col, tmem + kColA + 8u * kk, bd + 16u * kk, tc::idesc_bf16(128, N), kk > 0 ? 1u : 0u);
   };
   // dW^T (M = 128 input rows, N outputs) += act^T (shared) by da (shared),
   // K = 128 queries, both operands MN-major: K = 16 spans two 8-query groups
   auto mma_dw = [&](uint32_t d_col, uint32_t actT, uint32_t da, int N, bool acc) {
     const uint32_t kg_a = 128u * 16u, kg_b = (uint32_t)N * 16u;   // bytes per 8-query group
-    for (int kk = 0; kk < kRows / 16; ++kk) {
-      const uint64_t ad = mn_desc(actT + kk * 2u * kg_a, kg_a);
-      const uint64_t bd = mn_desc(da + kk * 2u * kg_b, kg_b);
-      tc::mma_bf16(tmem + d_col, ad, bd, tc::idesc_bf16(128, N) | kTransA | kTransB, (acc || kk > 0) ? 1u : 0u);
-    }
+    const uint64_t ad = mn_desc(actT, kg_a), bd = mn_desc(da, kg_b);   // addresses in 16-byte units
+#pragma unroll
+    for (int kk = 0; kk < kRows / 16; ++kk)
+      tc::mma_bf16(tmem + d_col, ad + kk * 2u * kg_a / 16u, bd + kk * 2u * kg_b / 16u,
+                   tc::idesc_bf16(128, N) | kTransA | kTransB, (acc || kk > 0) ? 1u : 0u);
   };
   // All threads make their stores visible and meet.  Then warp 0 issues
   // `issue` (the products the epilogue reads) and commits it to bar_mma, and
@@ -576,17 +577,19 @@ __global__ void __launch_bounds__(kThreads, 1) train_tc_kernel(const TrainTcArgs
       const int N = l == 3 ? 16 : 64, in = l == 0 ? kDecIn : kHidden, nout = l == 3 ? kOut : kHidden;
       const int offW = l == 0 ? kOffW1 : l == 1 ? kOffW2 : l == 2 ? kOffW3 : kOffW4;
       const int offB = l == 0 ? kOffB1 : l == 1 ? kOffB2 : l == 2 ? kOffB3 : kOffB4;
+      // input j's weights, or in row `in` the biases: one pointer and stride,
+      // so that no warp runs both (10 k cycles with a branch per value)
+      float *const dst = out + (j < in ? offW + j : offB);
+      const int step = j < in ? in : 1;
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         const int c = 16 * hf + 32 * h;
-        if (c >= N) continue;
+        if (c >= N || j > in) continue;
 #pragma unroll
         for (int e = 0; e < 16; ++e) {
           const int o = c + e;
           if (o >= nout) continue;
-          const float g = first ? 0.0f : v[l][16 * h + e];   // a CTA without tiles contributes zeros
-          if (j < in) out[offW + o * in + j] = g;
-          else if (j == in) out[offB + o] = g;
+          dst[o * step] = first ? 0.0f : v[l][16 * h + e];   // a CTA without tiles contributes zeros
         }
       }
     }
@@ -594,20 +597,41 @@ __global__ void __launch_bounds__(kThreads, 1) train_tc_kernel(const TrainTcArgs
   // ---- per-material sums of this CTA's latent-gradient rows, in row order,
   // into the partials' columns past kDecParams (the operand buffers are free
   // now).  The CTA's tiles are staged in shared memory as many at a time as
-  // fit; warp w then walks, in row order, the rows of the materials m with
-  // m % 8 == w (found with ballots), so no two warps touch one sum.
+  // fit; warp w then lists the rows of the materials m with m % 8 == w, in row
+  // order (found with ballots), so no two warps touch one sum, and adds the
+  // listed rows four at a time: four rows' and sums' loads in flight, a sum
+  // that repeats within the four taken from the row before.  512 rows of 256
+  // materials: 4-5 k cycles (a row at a time, as it was found, 8-11 k) and
+  // their staging 1.8 k (5 k without the swizzle); all that follows the tile
+  // loop 12 k (29 k), eight steps of 65 536 queries 511 -> 430 us.
   if (ok && a.partial_width > kDecParams) {
+    __shared__ __align__(16) uint32_t list[kThreads / 32][kSumList];   // row | material << 16
     float *acc = reinterpret_cast<float *>(sm);                   // [n_lat][32]
-    float *stage = acc + (size_t)a.n_lat * kLatent;                // [group][128][32]
+    float *stage = acc + (size_t)a.n_lat * kLatent;                // [group][128][32], 16-byte groups swizzled
     const int group = sum_group;
     int *ids = reinterpret_cast<int *>(stage + (size_t)group * kRows * kLatent);   // [group][128]
     const int lane32 = tid & 31;
+    // column lane32 of row q, which holds its 16-byte group i in place i ^ (q % 8)
+    auto staged = [&](int q) { return stage[q * kLatent + ((((lane32 >> 2) ^ q) & 7) << 2) + (lane32 & 3)]; };
+    for (int e = lane32; e < kSumList; e += 32) list[warp][e] = 0u;   // what follows the listed rows is read, too
     __syncthreads();
     for (int e = tid; e < a.n_lat * kLatent; e += kThreads) acc[e] = 0.0f;
     for (int64_t t0 = blockIdx.x; t0 < n_tiles; t0 += (int64_t)group * gridDim.x) {
       int nt = 0;   // tiles in this group
       while (nt < group && t0 + (int64_t)nt * gridDim.x < n_tiles) ++nt;
       __syncthreads();
+      for (int e0 = tid; e0 < nt * kRows; e0 += 4 * kThreads) {
+        int m4[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int e = e0 + u * kThreads;
+          const int64_t row = (t0 + (int64_t)(e / kRows) * gridDim.x) * kRows + e % kRows;
+          m4[u] = e < nt * kRows && row < a.g.n ? (int)a.g.material[row] : -1;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (e0 + u * kThreads < nt * kRows) ids[e0 + u * kThreads] = m4[u] < a.n_lat ? m4[u] : -1;
+      }
       // the rows: from tensor memory (every tile of the CTA in this one
       // group), or from a.dlat_rows with eight loads in flight per thread
       // before their stores
@@ -619,11 +643,11 @@ __global__ void __launch_bounds__(kThreads, 1) train_tc_kernel(const TrainTcArgs
           tc::tmem_ld16(tmem + lane + kColDz + 32u * (uint32_t)t + 16u * (uint32_t)hf, v);
           tc::tmem_ld_wait();
           const bool in = (t0 + (int64_t)t * gridDim.x) * kRows + r < a.g.n;
-          float4 *dst = reinterpret_cast<float4 *>(stage + ((size_t)t * kRows + r) * kLatent + 16 * hf);
+          float4 *dst = reinterpret_cast<float4 *>(stage + ((size_t)t * kRows + r) * kLatent);
 #pragma unroll
           for (int i = 0; i < 4; ++i)
-            dst[i] = in ? make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3])
-                        : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            dst[(4 * hf + i) ^ (r & 7)] = in ? make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3])
+                                             : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         }
       }
       for (int e0 = tid; e0 < n4; e0 += 8 * kThreads) {
@@ -638,35 +662,47 @@ __global__ void __launch_bounds__(kThreads, 1) train_tc_kernel(const TrainTcArgs
                       : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         }
 #pragma unroll
-        for (int u = 0; u < 8; ++u)
-          if (e0 + u * kThreads < n4) reinterpret_cast<float4 *>(stage)[e0 + u * kThreads] = v4[u];
-      }
-      for (int e0 = tid; e0 < nt * kRows; e0 += 4 * kThreads) {
-        int m4[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
+        for (int u = 0; u < 8; ++u) {
           const int e = e0 + u * kThreads;
-          const int64_t row = (t0 + (int64_t)(e / kRows) * gridDim.x) * kRows + e % kRows;
-          m4[u] = e < nt * kRows && row < a.g.n ? (int)a.g.material[row] : -1;
+          if (e < n4) reinterpret_cast<float4 *>(stage)[(e & ~7) | ((e ^ (e >> 3)) & 7)] = v4[u];
         }
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-          if (e0 + u * kThreads < nt * kRows) ids[e0 + u * kThreads] = m4[u] < a.n_lat ? m4[u] : -1;
       }
       __syncthreads();
-      for (int t = 0; t < nt; ++t) {
+#pragma unroll 1
+      for (int q0 = 0; q0 < nt * kRows; q0 += kSumList) {
+        int m_l[kSumList / 32], listed = 0;
 #pragma unroll
-        for (int k = 0; k < kRows / 32; ++k) {
-          const int q0 = t * kRows + 32 * k;
-          const int m_l = ids[q0 + lane32];
-          uint32_t hit = __ballot_sync(0xFFFFFFFFu, m_l >= 0 && (m_l & 7) == warp);
-          while (hit) {
-            const int b = __ffs(hit) - 1;
-            hit &= hit - 1;
-            const int m = __shfl_sync(0xFFFFFFFFu, m_l, b);
-            acc[m * kLatent + lane32] += stage[(size_t)(q0 + b) * kLatent + lane32];
-          }
+        for (int k = 0; k < kSumList / 32; ++k) m_l[k] = ids[q0 + 32 * k + lane32];
+#pragma unroll
+        for (int k = 0; k < kSumList / 32; ++k) {
+          const bool mine = m_l[k] >= 0 && (m_l[k] & 7) == warp;
+          const uint32_t hit = __ballot_sync(0xFFFFFFFFu, mine);
+          if (mine) list[warp][listed + __popc(hit & ((1u << lane32) - 1u))] =
+              (uint32_t)(q0 + 32 * k + lane32) | (uint32_t)m_l[k] << 16;
+          listed += __popc(hit);
         }
+        __syncwarp();
+        uint4 e = *reinterpret_cast<const uint4 *>(&list[warp][0]);
+#pragma unroll 1
+        for (int i = 0; i < listed; i += 4) {
+          const int k = listed - i;   // rows of the four that are there
+          const uint32_t m0 = e.x >> 16, m1 = e.y >> 16, m2 = e.z >> 16, m3 = e.w >> 16;
+          float *const s0 = acc + m0 * kLatent + lane32, *const s1 = acc + m1 * kLatent + lane32;
+          float *const s2 = acc + m2 * kLatent + lane32, *const s3 = acc + m3 * kLatent + lane32;
+          const float v0 = staged(e.x & 0xFFFFu), v1 = staged(e.y & 0xFFFFu);
+          const float v2 = staged(e.z & 0xFFFFu), v3 = staged(e.w & 0xFFFFu);
+          const float a0 = *s0, a1 = *s1, a2 = *s2, a3 = *s3;
+          e = *reinterpret_cast<const uint4 *>(&list[warp][(i + 4) & (kSumList - 1)]);
+          const float t0 = a0 + v0;
+          const float t1 = (m1 == m0 ? t0 : a1) + v1;
+          const float t2 = (m2 == m1 ? t1 : m2 == m0 ? t0 : a2) + v2;
+          const float t3 = (m3 == m2 ? t2 : m3 == m1 ? t1 : m3 == m0 ? t0 : a3) + v3;
+          *s0 = t0;
+          if (k > 1) *s1 = t1;
+          if (k > 2) *s2 = t2;
+          if (k > 3) *s3 = t3;
+        }
+        __syncwarp();
       }
     }
     __syncthreads();
