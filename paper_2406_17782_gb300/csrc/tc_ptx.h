@@ -80,6 +80,7 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
 }
 // Wait for phase `parity` to complete; gives up after ~max_cycles SM clocks.
 __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, long long max_cycles) {
+  if (mbar_try_wait(bar, parity)) return true;   // the usual case reads no clock
   const long long t0 = clock64();
   while (!mbar_try_wait(bar, parity)) {
     if (clock64() - t0 > max_cycles) return false;

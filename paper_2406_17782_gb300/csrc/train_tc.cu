@@ -16,7 +16,7 @@
 //             all of the CTA's tiles in tensor memory; the bias gradients
 //             come out as the row of the constant-one input.
 //   latent    dz rows = da_1 W1[:, :32] (FP32, for the per-material sums).
-// Warp 0 issues the products an epilogue reads and warp 4 the weight-
+// Warp 0 issues the products an epilogue reads and after them the weight-
 // gradient products, which nothing reads until the tile loop ends: each dW
 // chain is waited for only before the shared-memory operand it reads is
 // rewritten (the da operands alternate between two buffers for this).
@@ -76,10 +76,6 @@ constexpr uint32_t kColDz = 336;
 constexpr int kDzTiles = 5;
 constexpr int kSumList = kRows;   // rows looked through, and at most listed, at a time by the per-material sums
 static_assert(kColDz + 32 * kDzTiles <= 512, "latent-gradient rows inside the allocation");
-
-// Warp 0's elected thread issues the products the epilogues read; that of warp
-// 4 (the first of half 1) issues the weight-gradient products.
-constexpr int kDwIssuer = 4;
 
 // Instruction-descriptor bits: A and B read MN-major (transposed).
 constexpr uint32_t kTransA = 1u << 15, kTransB = 1u << 16;
@@ -191,7 +187,7 @@ __global__ void __launch_bounds__(kThreads, 1) train_tc_kernel(const TrainTcArgs
   uint64_t *bar_w = reinterpret_cast<uint64_t *>(smem);
   uint64_t *bar_mma = bar_w + 1;     // warp 0's products
   uint64_t *bar_dw = bar_w + 2;      // [3]: dW4, dW3 and dW1 (each once per tile)
-  uint64_t *bar_drain = bar_w + 5;   // both issuers' products, after a failed wait
+  uint64_t *bar_drain = bar_w + 5;   // all products, after a failed wait
   uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bar_w + 6);
   __shared__ double loss_red[4];
   uint8_t *sm = smem + 1024;
@@ -208,7 +204,7 @@ __global__ void __launch_bounds__(kThreads, 1) train_tc_kernel(const TrainTcArgs
     tc::mbar_init(bar_w, 1);
     tc::mbar_init(bar_mma, 1);
     for (int k = 0; k < 3; ++k) tc::mbar_init(bar_dw + k, 1);
-    tc::mbar_init(bar_drain, 2);
+    tc::mbar_init(bar_drain, 1);
     tc::fence_mbar_init();
   }
   if (warp == 0) tc::tmem_alloc(tmem_slot, 512);
@@ -257,8 +253,10 @@ __global__ void __launch_bounds__(kThreads, 1) train_tc_kernel(const TrainTcArgs
   };
   // All threads make their stores visible and meet.  Then warp 0 issues
   // `issue` (the products the epilogue reads) and commits it to bar_mma, and
-  // warp 4 issues `issue_dw` (weight-gradient products, read only after
-  // the tile loop) and commits it to dw_bar where one is given; a dW chain
+  // after it `issue_dw` (weight-gradient products, read only after the tile
+  // loop; from a warp of their own they took the pipe in turn with the others
+  // and a tile 10.9 k cycles, so 10.0 k) and commits it to dw_bar where one is
+  // given; a dW chain
   // is waited for only before the shared-memory operands it reads are
   // overwritten.  Every thread then runs `overlap` (half 1's share of the
   // next tile's inputs) and waits for bar_mma.  The outcome of each wait
@@ -274,10 +272,6 @@ __global__ void __launch_bounds__(kThreads, 1) train_tc_kernel(const TrainTcArgs
         tc::tc_fence_after();
         issue();
         tc::mma_commit(bar_mma);
-      }
-    } else if (warp_u == kDwIssuer) {
-      if (tc::elect_one()) {
-        tc::tc_fence_after();
         issue_dw();
         if (dw_bar != nullptr) tc::mma_commit(dw_bar);
       }
@@ -343,10 +337,11 @@ __global__ void __launch_bounds__(kThreads, 1) train_tc_kernel(const TrainTcArgs
     }
   };
   // half 1, step s of encoding the next tile's record into [q | 1 | 0], in
-  // pieces that fit the waits they fill: 1 and 2 the octaves 0-3 and 4-7 of
-  // u, 3 and 4 those of v, and with 4 also log r, the directions, the
-  // constant one and the padding, and all zeros where there is no query.
-  // Each octave is the one octaves_accurate() computes.
+  // pieces that fit the waits they fill (two octaves take about 350 cycles, a
+  // round's products 420; four at a time held up the next round by as much):
+  // 1 to 4 the octaves of u, 5 to 8 those of v, with 4 also log r, the
+  // directions, the constant one and the padding, and with 8 all zeros where
+  // there is no query.  Each octave is the one octaves_accurate() computes.
   auto octave = [&](float x, int k) -> uint32_t {
     const float f0 = x - floorf(x);
     const float sc = f0 * (float)(1 << k);
@@ -357,9 +352,9 @@ __global__ void __launch_bounds__(kThreads, 1) train_tc_kernel(const TrainTcArgs
   };
   auto encode_step = [&](int s) {
     if (hf != 1 || s < 1) return;
-    const int c = (s - 1) >> 1, k0 = 4 * ((s - 1) & 1);   // coordinate (u, v) and first octave
+    const int c = (s - 1) >> 2, k0 = 2 * ((s - 1) & 3);   // coordinate (u, v) and first octave
 #pragma unroll
-    for (int k = 0; k < 4; ++k) in_x[8 * c + k0 + k] = octave(in_v[c], k0 + k);
+    for (int k = 0; k < 2; ++k) in_x[8 * c + k0 + k] = octave(in_v[c], k0 + k);
     if (s == 4) {
       resolve();
       static_assert(kDecIn - kLatent - 32 == 7, "inputs 32..79: 32 octave values, log r, 6 directions, one");
@@ -372,10 +367,10 @@ __global__ void __launch_bounds__(kThreads, 1) train_tc_kernel(const TrainTcArgs
       for (int i = 8; i < 16; ++i) x[i] = 0.0f;
 #pragma unroll
       for (int k = 0; k < 8; ++k) in_x[16 + k] = tc::pack_bf16(x[2 * k], x[2 * k + 1]);
-      if (nxt_mat < 0) {
+    }
+    if (s == 8 && nxt_mat < 0) {
 #pragma unroll
-        for (int k = 0; k < 24; ++k) in_x[k] = 0u;
-      }
+      for (int k = 0; k < 24; ++k) in_x[k] = 0u;
     }
   };
   // half 0: latent row (16-byte loads: the rows of different queries are
@@ -415,7 +410,7 @@ __global__ void __launch_bounds__(kThreads, 1) train_tc_kernel(const TrainTcArgs
   load_early(blockIdx.x);
   resolve();
   if (hf == 1) {
-    for (int k = 1; k <= 4; ++k) encode_step(k);
+    for (int k = 1; k <= 8; ++k) encode_step(k);
   }
   grid_dependency_wait();
   if (lead) {
@@ -425,6 +420,7 @@ __global__ void __launch_bounds__(kThreads, 1) train_tc_kernel(const TrainTcArgs
   if (hf == 0) load_late(blockIdx.x);
   ok = tc::mbar_wait_sleep(bar_w, 0, kWaitCycles);
 
+  bool ones = false;   // whether this row's constant-one inputs of h1..h3 are set (all zero at first)
   bool fail = false;   // CTA-uniform: a round found an expired wait
   for (int64_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
     // the previous tile's dW1 (and with it every earlier dW chain) has read
@@ -476,12 +472,12 @@ __global__ void __launch_bounds__(kThreads, 1) train_tc_kernel(const TrainTcArgs
       put_half(acc, hT[l], 128, 32 * hf);
       if (hf == 1) {   // constant-one input of the next layer and padding, K = 64..79
         uint32_t w[8] = {valid ? tc::pack_bf16(1.0f, 0.0f) : 0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
-        tc::tmem_st8(t_a + 32, w);
-        st_row8(hT[l], 64, r, 128, w);
-        st_row8(hT[l], 72, r, 128, w + 4);
+        if (l == 0) tc::tmem_st8(t_a + 32, w);   // stays there until the next tile's inputs
+        if (valid != ones) st_row8(hT[l], 64, r, 128, w);   // stays there; 72..79 are never written
       }
     }
     if (fail) break;
+    ones = valid;
     if (!round([&] { mma_ts(kColD, s_w + kW4f, kKH, 16); }, none, nullptr, [&] { encode_step(3); })) {
       fail = true;
       break;
@@ -522,7 +518,7 @@ __global__ void __launch_bounds__(kThreads, 1) train_tc_kernel(const TrainTcArgs
       // layer l+2 (1-based) produced h_{l+1}: dh_{l+1} = da W_{l+2}, dW_{l+2}^T += h_{l+1}^T da
       const int Kin = l == 2 ? 16 : 64, Nw = l == 2 ? 16 : 64;
       if (!round([&] { mma_ts(kColD, wt[l], Kin, 64); }, [&] { mma_dw(cdw[l], hTa[l], da_in[l], Nw, !first); },
-                 dw_commit[l], none)) { fail = true; break; }
+                 dw_commit[l], [&] { encode_step(7 - l); })) { fail = true; break; }
       float acc[32];
       tc::tmem_ld32(t_d + 32 * hf, acc);
       tc::tmem_ld_wait();
@@ -535,7 +531,7 @@ __global__ void __launch_bounds__(kThreads, 1) train_tc_kernel(const TrainTcArgs
     // ---- dz rows = da1 W1[:, :32] (16 columns per half); dW1^T += x^T da1
     const uint32_t dz_col = dz_tmem ? kColDz + 32u * (uint32_t)ti : kColD;
     if (!round([&] { mma_ts(dz_col, s_w + kW1t, 64, 32); }, [&] { mma_dw(kColW1, s_xT, s_daB, 64, !first); },
-               bar_dw + 2, none)) { fail = true; break; }
+               bar_dw + 2, [&] { encode_step(8); })) { fail = true; break; }
     if (!dz_tmem) {
       float dz[16];
       tc::tmem_ld16(t_d + 16 * hf, dz);
@@ -720,9 +716,9 @@ __global__ void __launch_bounds__(kThreads, 1) train_tc_kernel(const TrainTcArgs
     a.loss_partial[blockIdx.x] = (loss_red[0] + loss_red[1]) + (loss_red[2] + loss_red[3]);
     if (!ok) atomicOr(a.status, kStatusTimeout);
   }
-  if (!ok) {   // after an expired wait: let the weights' copy and both issuers' products finish
+  if (!ok) {   // after an expired wait: let the weights' copy and all products finish
     tc::mbar_wait(bar_w, 0, kWaitCycles);
-    if ((warp_u == 0 || warp_u == kDwIssuer) && tc::elect_one()) tc::mma_commit(bar_drain);
+    if (warp_u == 0 && tc::elect_one()) tc::mma_commit(bar_drain);
     tc::mbar_wait(bar_drain, 0, kWaitCycles);
   }
   tc::tc_fence_before();

@@ -121,6 +121,26 @@ def test_tensor_core_gradient_large_batch(fab, tmp_path, n):
     assert rel_l2(g_bf[:ND], want[:ND]) <= TOL_DEC_BF16 and rel_l2(g_bf[ND:], want[ND:]) <= TOL_ENC_BF16
 
 
+@pytest.mark.parametrize("layout", ["one", "same_warp", "runs", "last"])
+@pytest.mark.parametrize("n", [1000, 2 * 152 * 128 + 5])
+def test_tensor_core_gradient_material_layouts(fab, tmp_path, n, layout):
+    """The per-material sums take their rows four at a time from lists per
+    warp (materials m with m % 8 in common): every row of one material, two
+    materials of one list in turn, runs of equal rows, and rows of other lists
+    only but for the last."""
+    mats = W.training_materials(2)
+    g = W.training_queries(n, len(mats), stream=f"tc-grad-layout-{n}")
+    i = np.arange(n)
+    g["material"] = {"one": np.full(n, 5), "same_warp": 3 + 8 * (i % 2), "runs": i // 7 % len(mats),
+                     "last": np.where(i == n - 1, 9, 2)}[layout].astype(np.uint16)
+    target = np.abs(np.random.default_rng(14).standard_normal((n, 4)) * 0.2).astype(np.float32)
+    gd, tt = GBuffer.from_numpy(g), torch.from_numpy(target).cuda()
+    dec, enc = W.decoder_init(weight_bound="small"), W.encoder_init(weight_bound="small")
+    _, want = oracle_gradient(mats, g, target, dec, enc, "eq11")
+    _, got = one_step_gradient(fab, tmp_path, "bf16", "eq11", mats, gd, tt, dec, enc)
+    assert rel_l2(got[:ND], want[:ND]) <= TOL_DEC_BF16 and rel_l2(got[ND:], want[ND:]) <= TOL_ENC_BF16
+
+
 def test_tensor_core_training_is_repeatable_and_learns(fab):
     mats = W.training_materials(2)
     g = W.training_queries(8192, len(mats), stream="tc-learn")
