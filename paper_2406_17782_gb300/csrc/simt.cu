@@ -361,6 +361,15 @@ __device__ __forceinline__ void material_features(const fabric_material &m, floa
 // them and keeps one accumulator per material (each sum still runs over the
 // inputs in order, as for a single material).
 constexpr int kEncGroup = 4;
+// Threads per unit, each with half of the group's materials: the kernels run
+// one CTA per SM and wait on their own latencies (256 materials: forward 6.3
+// -> 6.1 us, backward 4.9 us either way).  What more they gain comes from
+// starting under the kernel before: the backward's weights and the forward's
+// features are on their way before the wait (with the decoder's sums and
+// Adam's operands, which do the same, eight BF16 steps 405 -> 384 us).
+constexpr int kEncSplit = 2;
+constexpr int kEncEach = kEncGroup / kEncSplit;
+constexpr int kEncThreads = kEncHidden * kEncSplit;
 
 // The encoder kernels stage the weights they read in shared memory with
 // asynchronous copies issued at once, so that all of them are one round trip
@@ -399,15 +408,15 @@ __device__ __forceinline__ void stage_rows(float *dst, int ld, const float *src,
   }
 }
 
-// dot of a shared-memory weight row w (LEN floats; 16-byte aligned) with the
-// group's vectors x[g][0..LEN), one accumulator per material, inputs in order
+// dot of a shared-memory weight row w (LEN floats; 16-byte aligned) with
+// kEncEach vectors x[g][0..LEN), one accumulator per material, inputs in order
 template <int LEN, int LD>
 __device__ __forceinline__ void enc_dot_s(const float *w, const float (*x)[LD], float *acc) {
 #pragma unroll 8
   for (int i4 = 0; i4 < LEN / 4; ++i4) {
     const float4 c = reinterpret_cast<const float4 *>(w)[i4];
 #pragma unroll
-    for (int g = 0; g < kEncGroup; ++g) {
+    for (int g = 0; g < kEncEach; ++g) {
       acc[g] = fmaf(c.x, x[g][4 * i4], acc[g]);
       acc[g] = fmaf(c.y, x[g][4 * i4 + 1], acc[g]);
       acc[g] = fmaf(c.z, x[g][4 * i4 + 2], acc[g]);
@@ -428,45 +437,49 @@ struct NoRecords {};
 // The input features come from `recs` when REC is InlineRecords, else from
 // `raw` records on the device, or (raw null) from `feats`.
 template <bool V, typename REC>
-__global__ void __launch_bounds__(kEncHidden) encoder_fwd_kernel(const float *__restrict__ feats,
+__global__ void __launch_bounds__(kEncThreads) encoder_fwd_kernel(const float *__restrict__ feats,
                                                                  const fabric_material *__restrict__ raw,
                                                                  float *__restrict__ feats_out, int n,
                                                                  const float *__restrict__ enc,
                                                                  float *__restrict__ z, float *__restrict__ acts,
                                                                  const __grid_constant__ REC recs) {
-  grid_dependency_wait();
-  grid_dependents_launch();
   extern __shared__ __align__(16) float enc_smem[];
   float *e1 = enc_smem;                             // [128][kE1Ld]
   float *e2 = e1 + kEncHidden * kE1Ld;              // [128][kERowLd]
   float *e3 = e2 + kEncHidden * kERowLd;            // [32][kERowLd]
   static_assert((kEncHidden * kE1Ld) % 4 == 0, "E2 rows 16-byte aligned in shared memory");
-  stage_rows<false>(e1, kE1Ld, enc + kOffE1, kEncHidden, kEncIn);
-  stage_rows<V>(e2, kERowLd, enc + kOffE2, kEncHidden, kEncHidden);
-  stage_rows<V>(e3, kERowLd, enc + kOffE3, kLatent, kEncHidden);
   __shared__ float f[kEncGroup][kEncIn];
   __shared__ __align__(16) float h1[kEncGroup][kEncHidden];
   __shared__ __align__(16) float h2[kEncGroup][kEncHidden];
-  const int m0 = blockIdx.x * kEncGroup, j = threadIdx.x;
+  const int m0 = blockIdx.x * kEncGroup, tid = threadIdx.x;
+  const int j = tid % kEncHidden, g0 = tid / kEncHidden * kEncEach;   // unit, first material of the group
   const int nm = min(kEncGroup, n - m0);
-  if (std::is_same<REC, InlineRecords>::value || raw) {
-    if (j < kEncGroup) {
-      float t[kEncIn];
-      if (j < nm) {
-        if constexpr (std::is_same<REC, InlineRecords>::value) material_features(recs.m[m0 + j], t);
-        else material_features(raw[m0 + j], t);
-      } else {
+  // the records' features, before the wait: no kernel writes records
+  const bool records = std::is_same<REC, InlineRecords>::value || raw;
+  if (records && tid < kEncGroup) {
+    float t[kEncIn];
+    if (tid < nm) {
+      if constexpr (std::is_same<REC, InlineRecords>::value) material_features(recs.m[m0 + tid], t);
+      else material_features(raw[m0 + tid], t);
+    } else {
 #pragma unroll
-        for (int i = 0; i < kEncIn; ++i) t[i] = 0.0f;
-      }
+      for (int i = 0; i < kEncIn; ++i) t[i] = 0.0f;
+    }
 #pragma unroll
-      for (int i = 0; i < kEncIn; ++i) {
-        f[j][i] = t[i];
-        if (j < nm && feats_out) feats_out[(int64_t)(m0 + j) * kEncIn + i] = t[i];
-      }
+    for (int i = 0; i < kEncIn; ++i) f[tid][i] = t[i];
+  }
+  grid_dependency_wait();
+  grid_dependents_launch();
+  stage_rows<false>(e1, kE1Ld, enc + kOffE1, kEncHidden, kEncIn);
+  stage_rows<V>(e2, kERowLd, enc + kOffE2, kEncHidden, kEncHidden);
+  stage_rows<V>(e3, kERowLd, enc + kOffE3, kLatent, kEncHidden);
+  if (records) {
+    if (tid < nm && feats_out) {
+#pragma unroll
+      for (int i = 0; i < kEncIn; ++i) feats_out[(int64_t)(m0 + tid) * kEncIn + i] = f[tid][i];
     }
   } else {
-    for (int t = j; t < kEncGroup * kEncIn; t += kEncHidden) {
+    for (int t = tid; t < kEncGroup * kEncIn; t += kEncThreads) {
       const int g = t / kEncIn, i = t % kEncIn;
       f[g][i] = g < nm ? feats[(int64_t)(m0 + g) * kEncIn + i] : 0.0f;
     }
@@ -474,32 +487,33 @@ __global__ void __launch_bounds__(kEncHidden) encoder_fwd_kernel(const float *__
   const float b1 = enc[kOffEb1 + j], b2 = enc[kOffEb2 + j], b3 = enc[kOffEb3 + j % kLatent];
   cp_async_wait_all();
   __syncthreads();
-  float a1[kEncGroup], a2[kEncGroup];
+  float a1[kEncEach], a2[kEncEach];
 #pragma unroll
-  for (int g = 0; g < kEncGroup; ++g) a1[g] = b1;
+  for (int g = 0; g < kEncEach; ++g) a1[g] = b1;
 #pragma unroll
   for (int i = 0; i < kEncIn; ++i) {
     const float c = e1[j * kE1Ld + i];
 #pragma unroll
-    for (int g = 0; g < kEncGroup; ++g) a1[g] = fmaf(c, f[g][i], a1[g]);
+    for (int g = 0; g < kEncEach; ++g) a1[g] = fmaf(c, f[g0 + g][i], a1[g]);
   }
 #pragma unroll
-  for (int g = 0; g < kEncGroup; ++g) h1[g][j] = lrelu(a1[g]);
+  for (int g = 0; g < kEncEach; ++g) h1[g0 + g][j] = lrelu(a1[g]);
   __syncthreads();
 #pragma unroll
-  for (int g = 0; g < kEncGroup; ++g) a2[g] = b2 + h1[g][j];   // skip connection before the last activation
-  enc_dot_s<kEncHidden, kEncHidden>(e2 + j * kERowLd, h1, a2);
+  for (int g = 0; g < kEncEach; ++g) a2[g] = b2 + h1[g0 + g][j];   // skip connection before the last activation
+  enc_dot_s<kEncHidden, kEncHidden>(e2 + j * kERowLd, h1 + g0, a2);
 #pragma unroll
-  for (int g = 0; g < kEncGroup; ++g) {
-    h2[g][j] = lrelu(a2[g]);
-    if (acts && g < nm) {
-      acts[(int64_t)(m0 + g) * 2 * kEncHidden + j] = a1[g];
-      acts[(int64_t)(m0 + g) * 2 * kEncHidden + kEncHidden + j] = a2[g];
+  for (int g = 0; g < kEncEach; ++g) {
+    h2[g0 + g][j] = lrelu(a2[g]);
+    if (acts && g0 + g < nm) {
+      acts[(int64_t)(m0 + g0 + g) * 2 * kEncHidden + j] = a1[g];
+      acts[(int64_t)(m0 + g0 + g) * 2 * kEncHidden + kEncHidden + j] = a2[g];
     }
   }
   __syncthreads();
-  // layer 3: thread j computes latent output k = j % 32 of material j / 32
+  // layer 3: thread j < 128 computes latent output k = j % 32 of material j / 32
   static_assert(kEncGroup * kLatent == kEncHidden, "one layer-3 output per thread");
+  if (tid >= kEncHidden) return;
   const int k = j % kLatent, g = j / kLatent;
   float acc = b3;
   const float *w3 = e3 + k * kERowLd;
@@ -517,48 +531,51 @@ __global__ void __launch_bounds__(kEncHidden) encoder_fwd_kernel(const float *__
 // Per material: back-propagated pre-activation gradients da1, da2 and the
 // activations h1, h2 into work [n][4][128]; kEncGroup materials per CTA.
 template <bool V>
-__global__ void __launch_bounds__(kEncHidden) encoder_bwd_vec_kernel(const float *__restrict__ enc, int n,
+__global__ void __launch_bounds__(kEncThreads) encoder_bwd_vec_kernel(const float *__restrict__ enc, int n,
                                                                      const float *__restrict__ acts,
                                                                      const float *__restrict__ dz,
                                                                      float *__restrict__ work) {
-  grid_dependency_wait();
-  grid_dependents_launch();
   // E2 and E3 staged as they are (thread j reads their column j: a warp's
-  // reads are consecutive words)
+  // reads are consecutive words), on their way before the kernel before this
+  // one has finished: it never writes them (the sums of a training step, or
+  // the encoder's forward pass)
   extern __shared__ __align__(16) float enc_smem[];
   float *e2 = enc_smem;                          // [128][128]
   float *e3 = e2 + kEncHidden * kEncHidden;      // [32][128]
   stage_rows<V>(e2, kEncHidden, enc + kOffE2, kEncHidden, kEncHidden);
   stage_rows<V>(e3, kEncHidden, enc + kOffE3, kLatent, kEncHidden);
+  grid_dependency_wait();
+  grid_dependents_launch();
   __shared__ float sdz[kEncGroup][kLatent], da2s[kEncGroup][kEncHidden];
-  const int m0 = blockIdx.x * kEncGroup, j = threadIdx.x;
+  const int m0 = blockIdx.x * kEncGroup, tid = threadIdx.x;
+  const int j = tid % kEncHidden, g0 = tid / kEncHidden * kEncEach;   // unit, first material of the group
   const int nm = min(kEncGroup, n - m0);
-  float a1[kEncGroup], a2[kEncGroup];
+  float a1[kEncEach], a2[kEncEach];
 #pragma unroll
-  for (int g = 0; g < kEncGroup; ++g) {
-    const int64_t m = g < nm ? m0 + g : m0;
+  for (int g = 0; g < kEncEach; ++g) {
+    const int64_t m = g0 + g < nm ? m0 + g0 + g : m0;
     a1[g] = acts[m * 2 * kEncHidden + j];
     a2[g] = acts[m * 2 * kEncHidden + kEncHidden + j];
   }
-  {
-    const int k = j % kLatent, g = j / kLatent;
+  if (tid < kEncGroup * kLatent) {
+    const int k = tid % kLatent, g = tid / kLatent;
     sdz[g][k] = g < nm ? dz[(int64_t)(m0 + g) * kLatent + k] : 0.0f;
   }
   cp_async_wait_all();
   __syncthreads();
-  float dh2[kEncGroup], dh1[kEncGroup];
+  float dh2[kEncEach], dh1[kEncEach];
 #pragma unroll
-  for (int g = 0; g < kEncGroup; ++g) dh2[g] = 0.0f;
+  for (int g = 0; g < kEncEach; ++g) dh2[g] = 0.0f;
 #pragma unroll 8
   for (int k = 0; k < kLatent; ++k) {
     const float w3 = e3[k * kEncHidden + j];
 #pragma unroll
-    for (int g = 0; g < kEncGroup; ++g) dh2[g] = fmaf(w3, sdz[g][k], dh2[g]);
+    for (int g = 0; g < kEncEach; ++g) dh2[g] = fmaf(w3, sdz[g0 + g][k], dh2[g]);
   }
 #pragma unroll
-  for (int g = 0; g < kEncGroup; ++g) {
+  for (int g = 0; g < kEncEach; ++g) {
     const float da2 = dh2[g] * (a2[g] > 0.0f ? 1.0f : kLeaky);
-    da2s[g][j] = da2;
+    da2s[g0 + g][j] = da2;
     dh1[g] = da2;   // through the skip
   }
   __syncthreads();
@@ -566,14 +583,14 @@ __global__ void __launch_bounds__(kEncHidden) encoder_bwd_vec_kernel(const float
   for (int o = 0; o < kEncHidden; ++o) {
     const float w2 = e2[o * kEncHidden + j];
 #pragma unroll
-    for (int g = 0; g < kEncGroup; ++g) dh1[g] = fmaf(w2, da2s[g][o], dh1[g]);
+    for (int g = 0; g < kEncEach; ++g) dh1[g] = fmaf(w2, da2s[g0 + g][o], dh1[g]);
   }
 #pragma unroll
-  for (int g = 0; g < kEncGroup; ++g) {
-    if (g >= nm) break;
-    float *w = work + (int64_t)(m0 + g) * 4 * kEncHidden;
+  for (int g = 0; g < kEncEach; ++g) {
+    if (g0 + g >= nm) break;
+    float *w = work + (int64_t)(m0 + g0 + g) * 4 * kEncHidden;
     w[j] = dh1[g] * (a1[g] > 0.0f ? 1.0f : kLeaky);
-    w[kEncHidden + j] = da2s[g][j];
+    w[kEncHidden + j] = da2s[g0 + g][j];
     w[2 * kEncHidden + j] = lrelu(a1[g]);
     w[3 * kEncHidden + j] = lrelu(a2[g]);
   }
@@ -581,12 +598,16 @@ __global__ void __launch_bounds__(kEncHidden) encoder_bwd_vec_kernel(const float
 
 // Encoder parameter gradients: every block is a sum over materials of outer
 // products, out[r][c] = sum_m L[m][r] R[m][c] (R = 1 for the biases).  A CTA
-// takes a 32 x 32 block of one of them with two groups of 256 threads: group
-// q sums over the q-th half of the materials, staging 64 materials' rows of L
-// and R at a time in shared memory (all of a chunk's loads in flight
-// together), thread (w, c) accumulating rows 4w..4w+3 of column c over its
-// materials in order; the block is then (first half) + (second half).
-constexpr int kGradChunk = 64;
+// takes a 16 x 16 tile of one of them with two groups of 64 threads: group q
+// sums over the q-th half of the materials, staging kGradChunk materials' rows
+// of L and R at a time in shared memory (all of a chunk's copies in flight
+// together), thread (ty, tx) accumulating rows 2 ty, 2 ty + 1 of columns 2 tx,
+// 2 tx + 1 over its materials in order; the tile is then (first half) +
+// (second half).  Bound by the shared-memory loads: four warps with two 8-byte
+// loads a step on 112 SMs, instead of sixteen with a 16-byte and a 4-byte one
+// on 33 (256 materials: 8.5 -> 5.7 us).
+constexpr int kGradChunk = 128;
+constexpr int kGradTile = 16;
 
 // Adam (Kingma and Ba 2015) with bias correction, one parameter.
 __device__ __forceinline__ void adam_update(float *p, float *m, float *v, float g, float lr, float bc1, float bc2) {
@@ -600,27 +621,30 @@ __device__ __forceinline__ void adam_update(float *p, float *m, float *v, float 
 // Block cb of the decoder's gradient: columns 32 cb .. 32 cb + 31 summed over
 // the partials exactly as reduce_partials_kernel sums them (kSumSegs
 // segments of partials in order, then the segments in order), then Adam.
-// Run by threads 0..255 of the block.
+constexpr int kGradThreads = 128;
 __device__ void dec_reduce_adam(const DecAdamArgs &d, int cb) {
   __shared__ float seg_sum[kSumSegs][32];
-  const int lane = threadIdx.x & 31, seg = threadIdx.x >> 5;
+  const int lane = threadIdx.x & 31;
   const int j = cb * 32 + lane;
   const int per = (d.n_part + kSumSegs - 1) / kSumSegs;
-  const int c0 = min(d.n_part, seg * per), c1 = min(d.n_part, c0 + per);
-  float s = 0.0f;
-  if (j < d.n) {
-    for (int c = c0; c < c1; c += kSumBatch) {
-      float t[kSumBatch];
 #pragma unroll
-      for (int q = 0; q < kSumBatch; ++q) t[q] = c + q < c1 ? d.partial[(int64_t)(c + q) * d.stride + j] : 0.0f;
+  for (int seg = threadIdx.x >> 5; seg < kSumSegs; seg += kGradThreads / 32) {
+    const int c0 = min(d.n_part, seg * per), c1 = min(d.n_part, c0 + per);
+    float s = 0.0f;
+    if (j < d.n) {
+      for (int c = c0; c < c1; c += kSumBatch) {
+        float t[kSumBatch];
 #pragma unroll
-      for (int q = 0; q < kSumBatch; ++q)
-        if (c + q < c1) s += t[q];
+        for (int q = 0; q < kSumBatch; ++q) t[q] = c + q < c1 ? d.partial[(int64_t)(c + q) * d.stride + j] : 0.0f;
+#pragma unroll
+        for (int q = 0; q < kSumBatch; ++q)
+          if (c + q < c1) s += t[q];
+      }
     }
+    seg_sum[seg][lane] = s;
   }
-  seg_sum[seg][lane] = s;
-  asm volatile("bar.sync 1, %0;" ::"n"(32 * kSumSegs) : "memory");
-  if (seg == 0 && j < d.n) {
+  __syncthreads();
+  if (threadIdx.x < 32 && j < d.n) {
     float tot = seg_sum[0][lane];
 #pragma unroll
     for (int k = 1; k < kSumSegs; ++k) tot += seg_sum[k][lane];
@@ -635,14 +659,27 @@ struct GradBlock {
   int out;                 // offset of the block in the encoder parameters
 };
 
-__constant__ GradBlock kGradBlocks[6] = {
-    {0, 0, 0, 1, kEncHidden, kEncIn, kOffE1},                              // E1[j][i] = sum da1_j f_i
-    {0, -1, 0, 0, kEncHidden, 1, kOffEb1},                                 // e1[j]
-    {kEncHidden, 2 * kEncHidden, 0, 0, kEncHidden, kEncHidden, kOffE2},    // E2[j][i] = sum da2_j h1_i
-    {kEncHidden, -1, 0, 0, kEncHidden, 1, kOffEb2},                        // e2[j]
-    {0, 3 * kEncHidden, 2, 0, kLatent, kEncHidden, kOffE3},                // E3[k][i] = sum dz_k h2_i
-    {0, -1, 2, 0, kLatent, 1, kOffEb3},                                    // e3[k]
-};
+__host__ __device__ constexpr int grad_tiles(int rows, int cols) {
+  return rows / kGradTile * ((cols + kGradTile - 1) / kGradTile);
+}
+static_assert(kEncHidden % kGradTile == 0 && kLatent % kGradTile == 0, "whole tiles of rows");
+constexpr int kGradTiles = grad_tiles(kEncHidden, kEncIn) + grad_tiles(kEncHidden, 1) +
+                           grad_tiles(kEncHidden, kEncHidden) + grad_tiles(kEncHidden, 1) +
+                           grad_tiles(kLatent, kEncHidden) + grad_tiles(kLatent, 1);
+
+// The parameter block of tile t, and t's place in it: immediate operands (the
+// table in constant memory was six dependent misses at each CTA's start).
+__device__ __forceinline__ GradBlock grad_block(int &t) {
+  constexpr int t1 = grad_tiles(kEncHidden, kEncIn), t2 = t1 + grad_tiles(kEncHidden, 1);
+  constexpr int t3 = t2 + grad_tiles(kEncHidden, kEncHidden), t4 = t3 + grad_tiles(kEncHidden, 1);
+  constexpr int t5 = t4 + grad_tiles(kLatent, kEncHidden);
+  if (t < t1) return {0, 0, 0, 1, kEncHidden, kEncIn, kOffE1};                              // E1[j][i] = sum da1_j f_i
+  if (t < t2) return t -= t1, GradBlock{0, -1, 0, 0, kEncHidden, 1, kOffEb1};               // e1[j]
+  if (t < t3) return t -= t2, GradBlock{kEncHidden, 2 * kEncHidden, 0, 0, kEncHidden, kEncHidden, kOffE2};   // E2[j][i] = sum da2_j h1_i
+  if (t < t4) return t -= t3, GradBlock{kEncHidden, -1, 0, 0, kEncHidden, 1, kOffEb2};      // e2[j]
+  if (t < t5) return t -= t4, GradBlock{0, 3 * kEncHidden, 2, 0, kLatent, kEncHidden, kOffE3};   // E3[k][i] = sum dz_k h2_i
+  return t -= t5, GradBlock{0, -1, 2, 0, kLatent, 1, kOffEb3};                              // e3[k]
+}
 
 __device__ __forceinline__ const float *grad_src(int src, const float *work, const float *feats, const float *dz,
                                                  int &ld) {
@@ -650,79 +687,81 @@ __device__ __forceinline__ const float *grad_src(int src, const float *work, con
   return src == 0 ? work : src == 1 ? feats : dz;
 }
 
-// Blocks of 32 x 32 outputs, in the order of kGradBlocks.
-__host__ __device__ constexpr int grad_tiles(int rows, int cols) { return ((rows + 31) / 32) * ((cols + 31) / 32); }
-constexpr int kGradTiles = grad_tiles(kEncHidden, kEncIn) + grad_tiles(kEncHidden, 1) +
-                           grad_tiles(kEncHidden, kEncHidden) + grad_tiles(kEncHidden, 1) +
-                           grad_tiles(kLatent, kEncHidden) + grad_tiles(kLatent, 1);
-
-constexpr int kGradThreads = 512;
-
+// dz_v: dz can be read as float4 (the work rows always can).
 __global__ void __launch_bounds__(kGradThreads) encoder_grad_kernel(const float *__restrict__ feats, int n,
-                                                                    const float *__restrict__ dz,
+                                                                    const float *__restrict__ dz, int dz_v,
                                                                     const float *__restrict__ work,
                                                                     float *__restrict__ denc, const DecAdamArgs dec) {
-  grid_dependency_wait();
-  grid_dependents_launch();
-  if (blockIdx.x >= kGradTiles) {   // the decoder's gradient sums and Adam update
-    if (threadIdx.x < 32 * kSumSegs) dec_reduce_adam(dec, blockIdx.x - kGradTiles);
+  // The decoder's gradient sums and Adam update, without a wait: the kernel
+  // that wrote the partials and the one that read the parameters had completed
+  // when the encoder's backward, the kernel before this one, passed its wait.
+  if (blockIdx.x >= kGradTiles) {
+    dec_reduce_adam(dec, blockIdx.x - kGradTiles);
     return;
   }
-  __shared__ __align__(16) float sl[2][kGradChunk][32];
-  __shared__ float sr[2][kGradChunk][32];
-  // which block, and which 32 x 32 tile of it
-  int t = blockIdx.x, b = 0;
-  while (t >= grad_tiles(kGradBlocks[b].rows, kGradBlocks[b].cols)) {
-    t -= grad_tiles(kGradBlocks[b].rows, kGradBlocks[b].cols);
-    ++b;
-  }
-  const GradBlock B = kGradBlocks[b];
-  const int ct = (B.cols + 31) / 32;
-  const int r0 = (t / ct) * 32, c0 = (t % ct) * 32;
+  grid_dependency_wait();
+  grid_dependents_launch();
+  __shared__ __align__(16) float sl[2][kGradChunk][kGradTile];
+  __shared__ __align__(16) float sr[2][kGradChunk][kGradTile];
+  // which block, and which tile of it
+  int t = blockIdx.x;
+  const GradBlock B = grad_block(t);
+  const int ct = (B.cols + kGradTile - 1) / kGradTile;
+  const int r0 = (t / ct) * kGradTile, c0 = (t % ct) * kGradTile;
   int ldl, ldr;
-  const float *L = grad_src(B.l_src, work, feats, dz, ldl);
-  const float *R = grad_src(B.r_src, work, feats, dz, ldr);
-  const int q = threadIdx.x >> 8, tid = threadIdx.x & 255, c = tid & 31, w = tid >> 5;
+  const float *L = grad_src(B.l_src, work, feats, dz, ldl) + B.l_off + r0;
+  const float *R = grad_src(B.r_src, work, feats, dz, ldr) + B.r_off + c0;
+  const int q = threadIdx.x >> 6, tid = threadIdx.x & 63, ty = tid >> 3, tx = tid & 7;
   const int half = (n + 1) / 2, m_begin = q == 0 ? 0 : half, m_end = q == 0 ? half : n;
   const int rounds = (half + kGradChunk - 1) / kGradChunk;   // the same for both groups (CTA barriers)
-  float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+  // mc rows of 16 columns, `cols` of them there, into s
+  auto stage = [&](float(*s)[kGradTile], const float *src, int ld, int mc, int cols, bool v) {
+    if (v) {
+      for (int e = tid; e < mc * (kGradTile / 4); e += 64) cp_async16(&s[e >> 2][4 * (e & 3)], src + (int64_t)(e >> 2) * ld + 4 * (e & 3));
+    } else {
+      for (int e = tid; e < mc * kGradTile; e += 64)
+        if ((e & 15) < cols) cp_async4(&s[e >> 4][e & 15], src + (int64_t)(e >> 4) * ld + (e & 15));
+    }
+  };
+  float acc[2][2] = {{0.0f, 0.0f}, {0.0f, 0.0f}};
   for (int k0 = 0; k0 < rounds; ++k0) {
     const int m0 = m_begin + k0 * kGradChunk;
     const int mc = max(0, min(kGradChunk, m_end - m0));
     __syncthreads();
-#pragma unroll
-    for (int u = 0; u < kGradChunk * 32 / 256; ++u) {
-      const int e = tid + 256 * u, mm = e >> 5, k = e & 31;
-      const bool in = mm < mc;
-      sl[q][mm][k] = in && r0 + k < B.rows ? L[(int64_t)(m0 + mm) * ldl + B.l_off + r0 + k] : 0.0f;
-      sr[q][mm][k] = !in ? 0.0f
-                         : B.r_off < 0 ? 1.0f
-                                       : (c0 + k < B.cols ? R[(int64_t)(m0 + mm) * ldr + B.r_off + c0 + k] : 0.0f);
+    stage(sl[q], L + (int64_t)m0 * ldl, ldl, mc, kGradTile, B.l_src == 0 || dz_v);
+    if (B.r_off >= 0) {
+      stage(sr[q], R + (int64_t)m0 * ldr, ldr, mc, B.cols - c0, B.r_src == 0);
+    } else {
+      for (int mm = tid; mm < mc; mm += 64) sr[q][mm][0] = 1.0f;
     }
+    cp_async_wait_all();
     __syncthreads();
+#pragma unroll 8
     for (int mm = 0; mm < mc; ++mm) {
-      const float4 a = reinterpret_cast<const float4 *>(sl[q][mm])[w];
-      const float x = sr[q][mm][c];
-      acc[0] = fmaf(a.x, x, acc[0]);
-      acc[1] = fmaf(a.y, x, acc[1]);
-      acc[2] = fmaf(a.z, x, acc[2]);
-      acc[3] = fmaf(a.w, x, acc[3]);
+      const float2 a = reinterpret_cast<const float2 *>(sl[q][mm])[ty];
+      const float2 x = reinterpret_cast<const float2 *>(sr[q][mm])[tx];
+      acc[0][0] = fmaf(a.x, x.x, acc[0][0]);
+      acc[0][1] = fmaf(a.x, x.y, acc[0][1]);
+      acc[1][0] = fmaf(a.y, x.x, acc[1][0]);
+      acc[1][1] = fmaf(a.y, x.y, acc[1][1]);
     }
   }
   // the second half's sums through shared memory, added to the first half's
   __syncthreads();
-  float(*part)[32] = sl[1];   // [32 rows][32 columns]: rows 4w..4w+3 of column c
+  float(*part)[kGradTile] = sl[0];
   if (q == 1) {
 #pragma unroll
-    for (int k = 0; k < 4; ++k) part[4 * w + k][c] = acc[k];
+    for (int i = 0; i < 2; ++i) reinterpret_cast<float2 *>(part[2 * ty + i])[tx] = make_float2(acc[i][0], acc[i][1]);
   }
   __syncthreads();
-  if (q == 0 && c0 + c < B.cols) {
+  if (q == 0) {
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const int r = r0 + 4 * w + k;
-      if (r < B.rows) denc[B.out + r * B.cols + c0 + c] = acc[k] + part[4 * w + k][c];
-    }
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const int c = c0 + 2 * tx + k;
+        if (c < B.cols) denc[B.out + (r0 + 2 * ty + i) * B.cols + c] = acc[i][k] + part[2 * ty + i][2 * tx + k];
+      }
   }
 }
 
@@ -734,12 +773,22 @@ __global__ void __launch_bounds__(kGradThreads) encoder_grad_kernel(const float 
 __global__ void adam_kernel(float *__restrict__ p0, int64_t n0, float *__restrict__ p1, int64_t n1,
                             const float *__restrict__ g, float *__restrict__ m, float *__restrict__ v, float lr,
                             float bc1, float bc2) {
+  // what is updated is read before the wait: only Adam writes it
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  float *p = i < n0 ? p0 + i : p1 + (i - n0);
+  float pi = 0.0f, mi = 0.0f, vi = 0.0f;
+  if (i < n0 + n1) {
+    pi = *p;
+    mi = m[i];
+    vi = v[i];
+  }
   grid_dependency_wait();
   grid_dependents_launch();
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n0 + n1) return;
-  float *p = i < n0 ? p0 + i : p1 + (i - n0);
-  adam_update(p, m + i, v + i, g[i], lr, bc1, bc2);
+  adam_update(&pi, &mi, &vi, g[i], lr, bc1, bc2);
+  *p = pi;
+  m[i] = mi;
+  v[i] = vi;
 }
 
 // ---------------------------------------------------------------------------
@@ -1172,7 +1221,7 @@ cudaError_t encoder_fwd(const float *feats, const fabric_material *raw, float *f
   const auto k = (reinterpret_cast<uintptr_t>(enc) & 15) == 0 ? encoder_fwd_kernel<true, REC> : encoder_fwd_kernel<false, REC>;
   const cudaError_t e = ensure_max_dyn_smem(reinterpret_cast<const void *>(k), (int)kEncFwdSmem);
   if (e != cudaSuccess) return e;
-  return launch_dependent(k, grid, kEncHidden, kEncFwdSmem, s, feats, raw, feats_out, n, enc, z, acts, recs);
+  return launch_dependent(k, grid, kEncThreads, kEncFwdSmem, s, feats, raw, feats_out, n, enc, z, acts, recs);
 }
 }  // namespace
 
@@ -1218,16 +1267,17 @@ cudaError_t launch_encoder_backward(const float *feats, int n, const float *enc,
   }
   const int grid = (n + kEncGroup - 1) / kEncGroup;
   if (v)
-    launch_dependent(encoder_bwd_vec_kernel<true>, grid, kEncHidden, kEncBwdSmem, s, enc, n, acts_in, dz, vec);
+    launch_dependent(encoder_bwd_vec_kernel<true>, grid, kEncThreads, kEncBwdSmem, s, enc, n, acts_in, dz, vec);
   else
-    launch_dependent(encoder_bwd_vec_kernel<false>, grid, kEncHidden, kEncBwdSmem, s, enc, n, acts_in, dz, vec);
+    launch_dependent(encoder_bwd_vec_kernel<false>, grid, kEncThreads, kEncBwdSmem, s, enc, n, acts_in, dz, vec);
   DecAdamArgs d{};
   int extra = 0;
   if (dec_adam) {
     d = *dec_adam;
     extra = (d.n + 31) / 32;
   }
-  launch_dependent(encoder_grad_kernel, kGradTiles + extra, kGradThreads, 0, s, feats, n, dz, vec, denc, d);
+  launch_dependent(encoder_grad_kernel, kGradTiles + extra, kGradThreads, 0, s, feats, n, dz,
+                   (int)((reinterpret_cast<uintptr_t>(dz) & 15) == 0), vec, denc, d);
   return cudaGetLastError();
 }
 
