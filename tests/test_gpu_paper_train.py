@@ -250,3 +250,35 @@ def test_paper_ablation_trains(fab):
             assert runs[0][-1] < 0.5 * runs[0][0]
     finally:
         fab.paper_set_params(64, W.paper_decoder_init(64), W.paper_encoder_init())
+
+
+@pytest.mark.parametrize("ablation", ["full", "no_fusion"])
+@pytest.mark.parametrize("w", [64, 128])
+def test_paper_gradient_at_tile_edges(fab, w, ablation):
+    """The mean gradient over a batch is that of its two parts, weighted by
+    their sizes, at sizes around the tiles of the products (64 rows), the
+    chunks of the weight gradients (256) and the per-material sums; the second
+    part's material ids start at an odd address.  Every row's own arithmetic is
+    the same in both, so only the order of FP32 sums differs (1e-4 is some 50
+    times that; a row lost or counted twice is at least 1/513)."""
+    mats = W.training_materials(2)
+    dec = W.paper_decoder_init(w, weight_bound="small", ablation=ablation)
+    fab.paper_set_params(w, dec, W.paper_encoder_init(weight_bound="small"), ablation=ablation)
+    fab.set_train_materials(mats)
+    try:
+        for n in (2, 63, 64, 65, 255, 256, 257, 513):
+            full = GBuffer.from_numpy(W.training_queries(n, len(mats), stream=f"paper-edge-{n}"))
+            target = torch.from_numpy(np.abs(np.random.default_rng(n).standard_normal((n, 4)) * 0.2)).float().cuda()
+
+            def step(a, b):
+                part = GBuffer(*[getattr(full, f)[a:b] for f in ("u", "v", "radius", "wi", "wo", "material")])
+                loss = float(fab.paper_train_step(part, target[a:b].contiguous(), 0.0).item())
+                fab.sync_status()
+                return loss * (b - a), fab.paper_gradient().astype(np.float64) * (b - a)
+
+            cut = n // 3 | 1
+            whole, first, second = step(0, n), step(0, cut), step(cut, n)
+            assert abs(whole[0] - first[0] - second[0]) <= 1e-5 * abs(whole[0]), n
+            assert rel_l2(first[1] + second[1], whole[1]) <= 1e-4, n
+    finally:
+        fab.paper_set_params(w, W.paper_decoder_init(w), W.paper_encoder_init())
