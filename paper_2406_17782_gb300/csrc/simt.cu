@@ -86,21 +86,26 @@ __device__ void reduce_loss_warp(const double *__restrict__ part, int n, double 
 // material.  The sums are those of 256 bins added in order, a bin's rows in
 // row order: with V (ids read as 16-byte groups of eight) bin (row / 8) mod
 // 256, the last n mod 8 rows going to bins 0..7, else bin row mod 256.  Warp w
-// owns bins 32 w .. 32 w + 31: it looks through their ids 256 rows at a time
-// (lane l those of bin 32 w + l), lists the rows that match, and adds the
+// owns bins 32 w .. 32 w + 31: it looks through their ids, eight groups of 256
+// rows in flight (lane l those of bin 32 w + l, so that only a lane's own order
+// counts), lists the rows that match, a row per lane at a time, and adds the
 // listed rows to their bins in shared memory with one lane per column and
-// eight rows' loads in flight (a row at a time as it is found costs a trip to
-// memory each: 32 us for 65 536 rows of 256 materials, 17.6 us so).
+// sixteen rows' loads in flight.  65 536 rows of 256 materials: 14.9 us (32 with
+// a row at a time as it is found, 17.7 with a ballot for each of a group's
+// eight rows and eight loads in flight).
 constexpr int kSegWarps = 8;
-constexpr int kSegList = 512;    // listed rows per warp, emptied when a group of 256 might not fit
+constexpr int kSegList = 512;    // listed rows per warp, emptied when 32 more might not fit
 
 template <bool V>
 __global__ void __launch_bounds__(32 * kSegWarps) latent_sums_kernel(const uint16_t *__restrict__ mat, int64_t n,
                                                                      const float *__restrict__ rows,
-                                                                     float *__restrict__ dlat) {
+                                                                     float *__restrict__ dlat, int early) {
   __shared__ float bins[32 * kSegWarps][kLatent];
   __shared__ uint32_t list[kSegWarps][kSegList];   // rows (fewer than 2^32: they are 128 bytes each)
-  grid_dependency_wait();
+  // early: the kernel before this one is the sum over the same partials'
+  // kernel, which had completed when that one let this one start; it is waited
+  // for at the end, so that this kernel's completion implies its
+  if (!early) grid_dependency_wait();
   grid_dependents_launch();
   const uint32_t m = blockIdx.x, mm = m * 0x10001u;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -109,22 +114,19 @@ __global__ void __launch_bounds__(32 * kSegWarps) latent_sums_kernel(const uint1
   const int64_t whole = V ? n & ~int64_t(7) : n;
   int count = 0;
   auto bin_of = [&](uint32_t r) { return 32 * warp + (int)(V ? (r < whole ? (r >> 3) & 31u : (uint32_t)(r - whole)) : r & 31u); };
+  constexpr int kRowsInFlight = 16;
   auto add_listed = [&]() {
     __syncwarp();
-    int e = 0;
-    for (; e + 8 <= count; e += 8) {
-      uint32_t r[8];
-      float v[8];
+    for (int e = 0; e < count; e += kRowsInFlight) {
+      uint32_t r[kRowsInFlight];
+      float v[kRowsInFlight];
 #pragma unroll
-      for (int q = 0; q < 8; ++q) r[q] = list[warp][e + q];
+      for (int q = 0; q < kRowsInFlight; ++q) r[q] = e + q < count ? list[warp][e + q] : 0u;
 #pragma unroll
-      for (int q = 0; q < 8; ++q) v[q] = rows[(int64_t)r[q] * kLatent + lane];
+      for (int q = 0; q < kRowsInFlight; ++q) v[q] = e + q < count ? rows[(int64_t)r[q] * kLatent + lane] : 0.0f;
 #pragma unroll
-      for (int q = 0; q < 8; ++q) bins[bin_of(r[q])][lane] += v[q];
-    }
-    for (; e < count; ++e) {
-      const uint32_t r = list[warp][e];
-      bins[bin_of(r)][lane] += rows[(int64_t)r * kLatent + lane];
+      for (int q = 0; q < kRowsInFlight; ++q)
+        if (e + q < count) bins[bin_of(r[q])][lane] += v[q];
     }
     count = 0;
     __syncwarp();
@@ -134,46 +136,48 @@ __global__ void __launch_bounds__(32 * kSegWarps) latent_sums_kernel(const uint1
   auto row_of = [&](int64_t base, int k) {
     return V ? base + 256 * warp + 8 * lane + k : base + 256 * k + 32 * warp + lane;
   };
-  constexpr int kInFlight = 4;
+  constexpr int kInFlight = 8;
   for (int64_t base0 = 0; base0 < whole; base0 += kInFlight * kGroup) {
     uint4 w[kInFlight];
-    uint32_t bits[kInFlight];
 #pragma unroll
     for (int q = 0; q < kInFlight; ++q) {
       const int64_t r = row_of(base0 + q * kGroup, 0);
       w[q] = V && r + 8 <= whole ? *reinterpret_cast<const uint4 *>(mat + r) : make_uint4(~mm, ~mm, ~mm, ~mm);
     }
+    uint64_t bits = 0;   // bit 8 q + k: row k of group q
 #pragma unroll
     for (int q = 0; q < kInFlight; ++q) {
-      bits[q] = 0;
+      uint32_t b8 = 0;
       if (V) {
         const uint32_t word[4] = {w[q].x ^ mm, w[q].y ^ mm, w[q].z ^ mm, w[q].w ^ mm};
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-          if ((word[k] & 0xFFFFu) == 0) bits[q] |= 1u << (2 * k);
-          if ((word[k] >> 16) == 0) bits[q] |= 2u << (2 * k);
+          if ((word[k] & 0xFFFFu) == 0) b8 |= 1u << (2 * k);
+          if ((word[k] >> 16) == 0) b8 |= 2u << (2 * k);
         }
       } else {
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
           const int64_t r = row_of(base0 + q * kGroup, k);
-          if (r < n && mat[r] == m) bits[q] |= 1u << k;
+          if (r < n && mat[r] == m) b8 |= 1u << k;
         }
       }
+      bits |= (uint64_t)b8 << (8 * q);
     }
-#pragma unroll
-    for (int q = 0; q < kInFlight; ++q) {
-      if (!__any_sync(0xFFFFFFFFu, bits[q] != 0)) continue;
-#pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        const uint32_t hit = __ballot_sync(0xFFFFFFFFu, (bits[q] >> k) & 1u);
-        if ((bits[q] >> k) & 1u) list[warp][count + __popc(hit & below)] = (uint32_t)row_of(base0 + q * kGroup, k);
-        count += __popc(hit);
+    // each lane's rows (one bin's) in row order, a row per lane at a time
+    uint32_t hit;
+    while ((hit = __ballot_sync(0xFFFFFFFFu, bits != 0)) != 0) {
+      if (count > kSegList - 32) add_listed();
+      if (bits) {
+        const int k = __ffsll(bits) - 1;
+        bits &= bits - 1;
+        list[warp][count + __popc(hit & below)] = (uint32_t)row_of(base0 + (k >> 3) * kGroup, k & 7);
       }
-      if (count > kSegList - 256) add_listed();
+      count += __popc(hit);
     }
   }
   if (V && warp == 0) {   // the last n mod 8 rows
+    if (count > kSegList - 32) add_listed();
     const int64_t r = whole + lane;
     const bool match = r < n && mat[r] == m;
     const uint32_t hit = __ballot_sync(0xFFFFFFFFu, match);
@@ -188,6 +192,7 @@ __global__ void __launch_bounds__(32 * kSegWarps) latent_sums_kernel(const uint1
     for (int k = 0; k < 32 * kSegWarps; ++k) s += bins[k][threadIdx.x];
     dlat[(int64_t)m * kLatent + threadIdx.x] = s;
   }
+  if (early) grid_dependency_wait();
 }
 
 // out[m][i] = sum over rows with material m of rows[row][i], i < 32 NF; one CTA
@@ -1186,9 +1191,9 @@ cudaError_t launch_material_row_sums(const uint16_t *material, int64_t n, int n_
 }
 
 namespace {
-cudaError_t latent_sums(const fabric_gbuffer &g, int n_lat, const float *rows, float *dlat, cudaStream_t s) {
+cudaError_t latent_sums(const fabric_gbuffer &g, int n_lat, const float *rows, float *dlat, bool early, cudaStream_t s) {
   const auto k = (reinterpret_cast<uintptr_t>(g.material) & 15) == 0 ? latent_sums_kernel<true> : latent_sums_kernel<false>;
-  return launch_dependent(k, n_lat, 32 * kSegWarps, 0, s, g.material, g.n, rows, dlat);
+  return launch_dependent(k, n_lat, 32 * kSegWarps, 0, s, g.material, g.n, rows, dlat, (int)early);
 }
 }  // namespace
 
@@ -1198,18 +1203,21 @@ cudaError_t launch_decoder_grad_finish(const fabric_gbuffer &g, int n_lat, const
   // width > kDecParams: the per-CTA partials already hold the per-material
   // latent-gradient sums after the decoder's columns
   const bool folded = width > kDecParams;
+  bool sums = false;   // the sums over the partials were launched
   if (ddec) {
+    sums = true;
     const int cols = dlat ? width : kDecParams;
     launch_dependent(reduce_partials_kernel, (cols + 31) / 32 + (loss ? 1 : 0), 32 * kSumSegs, 0, s, partial, grid,
                      width, cols, kDecParams, ddec, dlat, loss_part, loss);
   } else {   // only the latent columns (folded) and the loss
     const int cols = dlat && folded ? width - kDecParams : 0;
-    if (cols > 0 || loss)
+    sums = cols > 0 || loss;
+    if (sums)
       launch_dependent(reduce_partials_kernel, (cols + 31) / 32 + (loss ? 1 : 0), 32 * kSumSegs, 0, s,
                        partial + kDecParams, grid, width, cols, 0, static_cast<float *>(nullptr), dlat, loss_part,
                        loss);
   }
-  if (dlat && !folded) latent_sums(g, n_lat, rows, dlat, s);
+  if (dlat && !folded) latent_sums(g, n_lat, rows, dlat, sums, s);
   return cudaGetLastError();
 }
 
