@@ -306,7 +306,8 @@ cudaError_t launch_decoder_backward(const fabric_gbuffer &g, const float *latent
                                     double *loss, void *work, int sm_count, int *status, cudaStream_t s);
 size_t decoder_backward_work_bytes(int64_t n, int sm_count);
 // out[m][c] = sum of rows[r][c] over the rows r < n of material m, in a fixed
-// order; cols = 64 or 128 floats per row, 16-byte aligned.
+// order; cols = 64 or 128 floats per row, 16-byte aligned.  Starts under the
+// kernel before it, which must not write the rows.
 cudaError_t launch_material_row_sums(const uint16_t *material, int64_t n, int n_mat, const float *rows, int cols,
                                      float *out, cudaStream_t s);
 // The fixed-order sums after a backward pass that wrote per-CTA partials

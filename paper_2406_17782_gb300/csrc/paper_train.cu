@@ -79,7 +79,7 @@ __global__ void __launch_bounds__(BM *BN / 64, 3) pn_layer_kernel(const float *_
   extern __shared__ __align__(16) float lsm[];   // [kStages][kStageFloats]
   const int tid = threadIdx.x, tx = tid % TX, ty = tid / TX;
   const int64_t i0 = (int64_t)blockIdx.x * BM;
-  grid_dependency_wait();
+  if (!GRAD) grid_dependency_wait();   // GRAD: waited for at the end (see launch_paper_train)
   grid_dependents_launch();
   const int steps = (K + kDepth - 1) / kDepth;
   const int cr = tid / PA, cp = 4 * (tid % PA), br = tid / (BN / 4), bc = 4 * (tid % (BN / 4));
@@ -179,6 +179,7 @@ __global__ void __launch_bounds__(BM *BN / 64, 3) pn_layer_kernel(const float *_
       *reinterpret_cast<float4 *>(e.out + i * e.ld_out + j) = v;
     }
   }
+  if (GRAD) grid_dependency_wait();
 }
 
 // Weight-gradient partial of one chunk of kChunkRows rows: part[i][j] = sum_r
@@ -203,8 +204,7 @@ __global__ void __launch_bounds__(BM *BN / (8 * RM)) pn_wgrad_kernel(const float
   const int i0 = blockIdx.y * BM;
   const int64_t r_begin = (int64_t)blockIdx.x * kChunkRows;
   const int n = (int)(rows - r_begin < kChunkRows ? rows - r_begin : kChunkRows);
-  grid_dependency_wait();
-  grid_dependents_launch();
+  grid_dependents_launch();   // the kernel before is waited for at the end (see launch_paper_train)
   const int steps = (n + kRowDepth - 1) / kRowDepth;
   const int ra = tid / PA, ca = 4 * (tid % PA), rb = tid / PB, cb = 4 * (tid % PB);
   const float *ga = dZ + (r_begin + ra) * W + i0 + ca, *gb = X + (r_begin + rb) * ldx + cb;
@@ -320,6 +320,7 @@ __global__ void __launch_bounds__(BM *BN / (8 * RM)) pn_wgrad_kernel(const float
       for (int q = 0; q < NE; ++q) out[(int64_t)row_of(e0 + q) * N + j] = ext[q];
     }
   }
+  grid_dependency_wait();
 }
 
 // out_w[i][j] = sum_c part[c][i][j] for j < K, out_b[i] = sum_c part[c][i][K]:
@@ -714,8 +715,7 @@ __global__ void __launch_bounds__(kEH) pn_enc_bwd_kernel(const float *__restrict
                                                          float *__restrict__ DA2) {
   __shared__ float sg[128], sdz[kPnLatent], da2[kEH];
   const int m = blockIdx.x, j = threadIdx.x;
-  grid_dependency_wait();
-  grid_dependents_launch();
+  grid_dependents_launch();   // the kernel before is waited for at the end (see launch_paper_train)
   if (j < W) sg[j] = G[(int64_t)m * W + j];
   __syncthreads();
   if (j < kPnLatent) {
@@ -737,6 +737,7 @@ __global__ void __launch_bounds__(kEH) pn_enc_bwd_kernel(const float *__restrict
 #pragma unroll 16
   for (int o = 0; o < kEH; ++o) g = fmaf(enc[oE2 + o * kEH + j], da2[o], g);
   DA1[m * kEH + j] = g * (H1[m * kEH + j] > 0.0f ? 1.0f : kPnSlope);
+  grid_dependency_wait();
 }
 
 // Encoder parameter gradients as sums over materials of outer products,
@@ -887,9 +888,9 @@ cudaError_t reduce_chunks(const float *part, int chunks, int N, int K, float *dW
   return launch_dependent(pn_reduce_chunks_kernel, dim3((unsigned)((4 * tot + 255) / 256)), 256, 0, s, part, chunks, N, K, dW, db);
 }
 
-// weight and bias gradients: dW[j][k] = sum_b dZ[b][j] X[b][k] for k < K, db[j] = sum_b dZ[b][j]; X [B][ldx].
-cudaError_t wgrad(const float *dZ, int w, const float *X, int ldx, int K, int64_t B, float *part, float *dW, float *db,
-                  cudaStream_t s) {
+// Chunk sums (see reduce_chunks) of the weight and bias gradients dW[j][k] = sum_b
+// dZ[b][j] X[b][k] for k < K, db[j] = sum_b dZ[b][j]; X [B][ldx].
+cudaError_t wgrad(const float *dZ, int w, const float *X, int ldx, int K, int64_t B, float *part, cudaStream_t s) {
   cudaError_t e;
   if (w == 128)
     e = K > 128 ? wgrad_partials<128, 64, 128, 8, true>(dZ, X, ldx, K, B, part, s)
@@ -898,8 +899,7 @@ cudaError_t wgrad(const float *dZ, int w, const float *X, int ldx, int K, int64_
     e = K > 72   ? wgrad_partials<64, 64, 128, 8, false>(dZ, X, ldx, K, B, part, s)
         : K > 64 ? wgrad_partials<64, 64, 64, 4, true>(dZ, X, ldx, K, B, part, s)
                  : wgrad_partials<64, 64, 64, 4, false>(dZ, X, ldx, K, B, part, s);
-  if (e != cudaSuccess) return e;
-  return reduce_chunks(part, chunk_count(B), w, K, dW, db, s);
+  return e;
 }
 
 template <bool TRAIN>
@@ -991,7 +991,7 @@ struct Count {
 
 // Buffers of a training step after the forward pass's.
 struct PnTrain {
-  float *D1, *D2, *D3, *part, *G, *dz, *F, *EH1, *EH2, *DA1, *DA2, *z;
+  float *D1, *D2, *D3, *part[2], *G, *dz, *F, *EH1, *EH2, *DA1, *DA2, *z;
   double *lpart;
 };
 template <class Take>
@@ -1002,7 +1002,7 @@ PnTrain pn_train_buffers(int w, int ablation, int64_t B, int n_mat, Take take) {
   T.D3 = take((size_t)B * w);
   // weight-gradient partials of the widest layer
   const int k_max = std::max(paper_x0_inputs(ablation), paper_a1_inputs(w, ablation));
-  T.part = take((size_t)chunk_count(B) * w * (k_max + 1));
+  for (float *&part : T.part) part = take((size_t)chunk_count(B) * w * (k_max + 1));
   T.G = take((size_t)n_mat * w);
   T.dz = take((size_t)n_mat * kPnLatent);
   T.F = take((size_t)n_mat * kEI);
@@ -1043,7 +1043,7 @@ cudaError_t launch_paper_train(int w, int ablation, const fabric_gbuffer &q, con
   };
   const PnPass P = pn_pass_buffers(w, ablation, B, true, take);
   const PnTrain T = pn_train_buffers(w, ablation, B, n_mat, take);
-  float *D1 = T.D1, *D2 = T.D2, *D3 = T.D3, *part = T.part;
+  float *D1 = T.D1, *D2 = T.D2, *D3 = T.D3, *const *part = T.part;
   float *gd = grad, *ge = grad + o.total;
   cudaError_t e;
 #define PN_TRY(x)                     \
@@ -1065,25 +1065,40 @@ cudaError_t launch_paper_train(int w, int ablation, const fabric_gbuffer &q, con
   h.mode = loss_mode;
   h.inv_batch = 1.0f / (float)B;
   h.dq4 = D1;
-  h.part = part;
+  h.part = part[0];
   h.loss_part = T.lpart;
   PN_TRY(head<true>(w, h, s));
-  PN_TRY(reduce_chunks(part, chunk_count(B), 4, w, gd + o.A5, gd + o.a5, s));
+  PN_TRY(reduce_chunks(part[0], chunk_count(B), 4, w, gd + o.A5, gd + o.a5, s));
   PN_TRY(launch_dependent(pn_loss_final_kernel, dim3(1), 32, 0, s, T.lpart, chunk_count(B), loss));
   // ---- backward (D1..D3 rotate as dq4, dq3, dq2, dq1, dg2, dg1)
-  PN_TRY(wgrad(D1, w, P.K3, w, w, B, part, gd + o.A4, gd + o.a4, s));
+  // Three launches per layer: chunk sums of its weight gradients, input
+  // gradient, reduction of the sums.  Only the reduction waits for the kernel
+  // before it first.  The chunk sums start under the reduction of the layer
+  // before (whose own wait the input gradient they read had to pass; their
+  // buffers alternate), the input gradient under the chunk sums, filling the SMs
+  // as the last of those run, and each waits at its end for the kernel it
+  // started under, so that its completion still implies that one's: one after
+  // the other, 65 536 queries at width 128 took 1063 us a step, so 1000.
+  const int chunks = chunk_count(B);
+  PN_TRY(wgrad(D1, w, P.K3, w, w, B, part[1], s));
   PN_TRY(bwd_in(D1, dec + o.A4, w, w, B, D2, nullptr, P.K3, w, s));          // dq3
-  PN_TRY(wgrad(D2, w, P.K2, w, w, B, part, gd + o.A3, gd + o.a3, s));
+  PN_TRY(reduce_chunks(part[1], chunks, w, w, gd + o.A4, gd + o.a4, s));
+  PN_TRY(wgrad(D2, w, P.K2, w, w, B, part[0], s));
   PN_TRY(bwd_in(D2, dec + o.A3, w, w, B, D3, nullptr, P.K2, w, s));          // dq2
-  PN_TRY(wgrad(D3, w, P.K1, w, w, B, part, gd + o.A2, gd + o.a2, s));
+  PN_TRY(reduce_chunks(part[0], chunks, w, w, gd + o.A3, gd + o.a3, s));
+  PN_TRY(wgrad(D3, w, P.K1, w, w, B, part[1], s));
   PN_TRY(bwd_in(D3, dec + o.A2, w, w, B, D1, D2, P.K1, w, s));               // dq1 (+ dq3 through the skip)
-  PN_TRY(wgrad(D1, w, P.XA, P.lda, P.KA, B, part, gd + o.A1, gd + o.a1, s));
+  PN_TRY(reduce_chunks(part[1], chunks, w, w, gd + o.A2, gd + o.a2, s));
+  PN_TRY(wgrad(D1, w, P.XA, P.lda, P.KA, B, part[0], s));
   PN_TRY(bwd_in(D1, P.W.A1, P.lda, w, B, D2, nullptr, P.XA, P.lda, s));      // dg2
-  PN_TRY(wgrad(D2, w, P.H1, w, w, B, part, gd + o.S2, gd + o.s2, s));
+  PN_TRY(reduce_chunks(part[0], chunks, w, P.KA, gd + o.A1, gd + o.a1, s));
+  PN_TRY(wgrad(D2, w, P.H1, w, w, B, part[1], s));
   PN_TRY(bwd_in(D2, dec + o.S2, w, w, B, D3, nullptr, P.H1, w, s));          // dg1
-  PN_TRY(wgrad(D3, w, P.X0, P.ld0, P.KX0, B, part, gd + o.S1, gd + o.s1, s));
+  PN_TRY(reduce_chunks(part[1], chunks, w, w, gd + o.S2, gd + o.s2, s));
   // ---- latent gradient: per-material sums of dg1, times S1's latent block; encoder backward
+  PN_TRY(wgrad(D3, w, P.X0, P.ld0, P.KX0, B, part[0], s));
   PN_TRY(launch_material_row_sums(q.material, B, n_mat, D3, w, T.G, s));
+  PN_TRY(reduce_chunks(part[0], chunks, w, P.KX0, gd + o.S1, gd + o.s1, s));
   PN_TRY(launch_dependent(pn_enc_bwd_kernel, dim3(n_mat), kEH, 0, s, T.G, w, dec + o.S1, P.KX0, enc, T.EH1, T.EH2, T.dz, T.DA1, T.DA2));
   PN_TRY(launch_dependent(pn_enc_grad_kernel, dim3(kPnEncGradTiles), 256, 0, s, n_mat, T.F, T.EH1, T.EH2, T.dz, T.DA1, T.DA2, ge));
 #undef PN_TRY

@@ -239,7 +239,8 @@ __global__ void __launch_bounds__(32 * kSegWarps) segment_sums_kernel(const uint
   extern __shared__ __align__(16) float seg_sum[];   // [kSegWarps * kSegPerWarp][COLS]
   __shared__ int list[kSegWarps][kSegList];
   __shared__ uint32_t present[kSegWarps];            // a warp's segments that have rows of the material
-  grid_dependency_wait();
+  // the kernel before wrote nothing that is read here; it is waited for at the
+  // end, so that this kernel's completion implies its
   grid_dependents_launch();
   const uint32_t m = blockIdx.x, mm = m * 0x10001u;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -343,6 +344,7 @@ __global__ void __launch_bounds__(32 * kSegWarps) segment_sums_kernel(const uint
     __syncthreads();
   }
   if (threadIdx.x < COLS) out[(int64_t)m * COLS + threadIdx.x] = total;
+  grid_dependency_wait();
 }
 
 // ---------------------------------------------------------------------------
