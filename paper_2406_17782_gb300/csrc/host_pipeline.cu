@@ -105,12 +105,12 @@ extern "C" fabric_status fabric_shade_neural_host(fabric_ctx *ctx, const fabric_
   if (chunk_points == 0) {
     // Direct: when every buffer is mapped page-locked memory the decoder
     // reads the G-buffer and writes its outputs over the host link itself,
-    // in one launch and without staging copies.  By default with two threads
-    // per tile row, which encode a tile when it starts and write it out when
-    // it ends: the decoder that works ahead lets no tile finish before the
-    // next one's inputs are there, and behind the link that is a third of the
-    // outputs written after the last read (233 036 points, three tiles per
-    // pipeline: 53.8 us against 48.4; 2 073 600: 391 and 390).
+    // in one launch and without staging copies.  Always with two threads per
+    // tile row (where the pipelines per CTA allow it), which encode a tile when
+    // it starts and write it out when it ends: the decoder that works ahead lets
+    // no tile finish before the next one's inputs are there, and behind the link
+    // that is a third of the outputs written after the last read (233 036 points,
+    // three tiles per pipeline: 53.8 us against 48.4; 2 073 600: 391 and 390).
     fabric_gbuffer d;
     d.u = static_cast<const float *>(mapped(g_host->u));
     d.v = static_cast<const float *>(mapped(g_host->v));
@@ -127,7 +127,7 @@ extern "C" fabric_status fabric_shade_neural_host(fabric_ctx *ctx, const fabric_
                                 ctx->d_status, ctx->sm_count, caller);
       else
         e = launch_decoder_tc(d, ctx->d_blob, ctx->n_mat, (int)prec, rgb, comps, ctx->d_status, ctx->sm_count,
-                              ctx->tc_ctas_per_sm, ctx->tc_warpgroups, ctx->tc_tile_wgs ? ctx->tc_tile_wgs : 2, caller);
+                              ctx->tc_ctas_per_sm, ctx->tc_warpgroups, 2, caller);
       if (e != cudaSuccess) return cuda_fail(ctx, e, "decoder launch");
       return FABRIC_OK;
     }
