@@ -22,7 +22,12 @@ namespace fab {
 // kernel wrote (the wait returns once those kernels have completed and
 // their memory is visible; without a pending dependency it returns at
 // once), and grid_dependents_launch() once the next kernel may be
-// scheduled.
+// scheduled.  Two exceptions, each explained where it is made: a kernel may
+// read ahead of its wait what kernels wrote that the one before it had waited
+// for (the operands of Adam, the encoder's weights in its backward pass), and
+// a kernel that needs nothing from the one before it waits at its end, so that
+// its completion still implies that one's; what follows such a kernel and
+// reads ahead of its own wait must not need either of the two.
 #ifdef __CUDACC__
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dependents_launch() { asm volatile("griddepcontrol.launch_dependents;" :::); }

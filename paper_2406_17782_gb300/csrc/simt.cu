@@ -461,9 +461,13 @@ __global__ void __launch_bounds__(kEncThreads) encoder_fwd_kernel(const float *_
   const int m0 = blockIdx.x * kEncGroup, tid = threadIdx.x;
   const int j = tid % kEncHidden, g0 = tid / kEncHidden * kEncEach;   // unit, first material of the group
   const int nm = min(kEncGroup, n - m0);
-  // the records' features, before the wait: no kernel writes records
+  // The records' features: before the wait where the records came with the
+  // launch or are a training step's (long there; they are the ones whose
+  // features are kept), after it where a copy on the stream has just brought them.
   const bool records = std::is_same<REC, InlineRecords>::value || raw;
-  if (records && tid < kEncGroup) {
+  const bool early = std::is_same<REC, InlineRecords>::value || feats_out;
+  auto features = [&] {
+    if (tid >= kEncGroup) return;
     float t[kEncIn];
     if (tid < nm) {
       if constexpr (std::is_same<REC, InlineRecords>::value) material_features(recs.m[m0 + tid], t);
@@ -474,13 +478,15 @@ __global__ void __launch_bounds__(kEncThreads) encoder_fwd_kernel(const float *_
     }
 #pragma unroll
     for (int i = 0; i < kEncIn; ++i) f[tid][i] = t[i];
-  }
+  };
+  if (records && early) features();
   grid_dependency_wait();
   grid_dependents_launch();
   stage_rows<false>(e1, kE1Ld, enc + kOffE1, kEncHidden, kEncIn);
   stage_rows<V>(e2, kERowLd, enc + kOffE2, kEncHidden, kEncHidden);
   stage_rows<V>(e3, kERowLd, enc + kOffE3, kLatent, kEncHidden);
   if (records) {
+    if (!early) features();
     if (tid < nm && feats_out) {
 #pragma unroll
       for (int i = 0; i < kEncIn; ++i) feats_out[(int64_t)(m0 + tid) * kEncIn + i] = f[tid][i];
