@@ -390,7 +390,10 @@ fabric_status fabric_encoder_backward(fabric_ctx *ctx, const float *feats_dev, i
  * weights_dev[i / group] (one weight per group of `group` consecutive
  * floats, e.g. per RGB pixel), read with stride weight_stride floats, so
  * that for instance the z of a [n][3] direction array can weight RGB
- * (renderers multiply f_P by <wi . n_s> under direct light).  Deterministic. */
+ * (renderers multiply f_P by <wi . n_s> under direct light).  Deterministic.
+ * The calls of one context share its partial sums, so calls on different
+ * streams have to be ordered by the caller: two that run at once may both give
+ * wrong values (later ones are not affected). */
 fabric_status fabric_error_stats(fabric_ctx *ctx, const float *a_dev, const float *b_dev, int64_t n,
                                  const float *weights_dev, int group, int weight_stride, double *out_dev,
                                  void *stream);

@@ -315,7 +315,6 @@ fabric_status fabric_create(fabric_ctx **out, int device) {
   cudaMemset(ctx->d_enc, 0, kEncParams * sizeof(float));
   cudaMemset(ctx->d_adam, 0, 2 * np * sizeof(float));
   cudaMemset(ctx->d_status, 0, sizeof(int));
-  cudaMemset(ctx->d_err_work, 0, error_stats_work_bytes(0));
   if (cudaDeviceSynchronize() != cudaSuccess) {
     fabric_destroy(ctx);
     return FABRIC_ERR_CUDA;

@@ -928,29 +928,36 @@ __device__ __forceinline__ void err_reduce(double (*s)[kErrThreads], double &e2,
   }
 }
 
-// The partials summed by the last CTA to finish: thread t takes partials t,
-// t + 256, ... in order, then the fixed tree.  `done` counts the finished CTAs
-// and wraps to zero with the last one.
-__device__ void err_finish(double e2, double b2, double mx, double *__restrict__ part, unsigned *__restrict__ done,
-                           double *__restrict__ out) {
+// A CTA's totals into its place among the partials, or, when it is the only
+// one, to the output.
+__device__ __forceinline__ void err_store(double e2, double b2, double mx, double *__restrict__ part,
+                                          double *__restrict__ out) {
   __shared__ double s[3][kErrThreads];
-  __shared__ bool last;
   err_reduce(s, e2, b2, mx);
   if (threadIdx.x == 0) {
-    part[3 * blockIdx.x] = e2;
-    part[3 * blockIdx.x + 1] = b2;
-    part[3 * blockIdx.x + 2] = mx;
-    __threadfence();
-    last = atomicInc(done, gridDim.x - 1) == gridDim.x - 1;
+    double *o = gridDim.x == 1 ? out : part + 3 * blockIdx.x;
+    o[0] = e2;
+    o[1] = b2;
+    o[2] = mx;
   }
-  __syncthreads();
-  if (!last) return;
-  __threadfence();
-  e2 = b2 = mx = 0.0;
-  for (int k = threadIdx.x; k < gridDim.x; k += kErrThreads) {
-    e2 += __ldcg(part + 3 * k);
-    b2 += __ldcg(part + 3 * k + 1);
-    mx = fmax(mx, __ldcg(part + 3 * k + 2));
+}
+
+// The sum over the partials, by one CTA: thread t takes partials t, t + 256,
+// ... in order, then the fixed tree.  Launched under the kernel that writes
+// them, so that it is ready when that one ends.  (The last CTA of that kernel
+// doing it instead needs a counter that outlives the call, which two calls
+// at once on two streams left at a value from which no later call recovered,
+// and is no faster: a weighted 1080p RGB frame 24.8 us either way, 1000
+// elements, one CTA that needs no sum, 6.2 against 8.3.)
+__global__ void __launch_bounds__(kErrThreads) err_final_kernel(const double *__restrict__ part, int n,
+                                                                double *__restrict__ out) {
+  __shared__ double s[3][kErrThreads];
+  grid_dependency_wait();
+  double e2 = 0.0, b2 = 0.0, mx = 0.0;
+  for (int k = threadIdx.x; k < n; k += kErrThreads) {
+    e2 += part[3 * k];
+    b2 += part[3 * k + 1];
+    mx = fmax(mx, part[3 * k + 2]);
   }
   err_reduce(s, e2, b2, mx);
   if (threadIdx.x == 0) {
@@ -966,8 +973,8 @@ __global__ void __launch_bounds__(kErrThreads) err_partial_kernel(const float *_
                                                                   const float *__restrict__ b, int64_t n_,
                                                                   const float *__restrict__ w, GroupDiv group,
                                                                   int w_stride, double *__restrict__ part,
-                                                                  unsigned *__restrict__ done,
                                                                   double *__restrict__ out) {
+  grid_dependents_launch();   // the sum over the partials (err_final_kernel)
   const Idx n = (Idx)n_;
   const Idx stride = (Idx)gridDim.x * kErrThreads;
   const Idx start = (Idx)blockIdx.x * kErrThreads + threadIdx.x;
@@ -1028,7 +1035,7 @@ __global__ void __launch_bounds__(kErrThreads) err_partial_kernel(const float *_
       mx = fmax(mx, fabs(d));
     }
   }
-  err_finish(e2, b2, mx, part, done, out);
+  err_store(e2, b2, mx, part, out);
 }
 
 // ---- the same reduction on pairs of elements with packed FP32x2
@@ -1082,8 +1089,8 @@ __global__ void __launch_bounds__(kErrThreads, kErrPerSm2) err_partial2_kernel(c
                                                                    const float *__restrict__ b, int64_t n_,
                                                                    const float *__restrict__ w, GroupDiv group,
                                                                    int w_stride, double *__restrict__ part,
-                                                                   unsigned *__restrict__ done,
                                                                    double *__restrict__ out) {
+  grid_dependents_launch();   // the sum over the partials (err_final_kernel)
   const uint64_t *a2 = reinterpret_cast<const uint64_t *>(a);
   const uint64_t *b2 = reinterpret_cast<const uint64_t *>(b);
   const Idx n = (Idx)n_;
@@ -1182,7 +1189,7 @@ __global__ void __launch_bounds__(kErrThreads, kErrPerSm2) err_partial2_kernel(c
       }
     if ((n & 1) && blockIdx.x == 0 && threadIdx.x == 0) fp64(n - 1);   // the odd last element
   }
-  err_finish(e2, b2s, mx, part, done, out);
+  err_store(e2, b2s, mx, part, out);
 }
 
 }  // namespace
@@ -1371,13 +1378,12 @@ cudaError_t launch_shuffle_dataset(const fabric_train_batch &src, const fabric_d
   return cudaGetLastError();
 }
 
-// [blocks][3] partials, then the count of finished CTAs (zero between calls)
-size_t error_stats_work_bytes(int64_t) { return (size_t)kErrBlocks * 3 * sizeof(double) + sizeof(unsigned); }
+// [blocks][3] partials
+size_t error_stats_work_bytes(int64_t) { return (size_t)kErrBlocks * 3 * sizeof(double); }
 
 cudaError_t launch_error_stats(const float *a, const float *b, int64_t n, const float *w, int group, int w_stride,
                                double *out, void *work, cudaStream_t s) {
   double *part = static_cast<double *>(work);
-  unsigned *done = reinterpret_cast<unsigned *>(part + (size_t)kErrBlocks * 3);
   const bool small = n + (int64_t)kErrRun * kErrBlocks * kErrThreads < ((int64_t)1 << 31);
   const bool packed = ((reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(b)) & 7u) == 0;
   const auto kernel = packed ? (w ? (small ? err_partial2_kernel<true, int> : err_partial2_kernel<true, int64_t>)
@@ -1387,8 +1393,10 @@ cudaError_t launch_error_stats(const float *a, const float *b, int64_t n, const 
   // one wave of CTAs, or as many as give each thread two elements or pairs
   const int64_t items = packed ? n / 2 : n, wave = packed ? kErrBlocks2 : kErrBlocks;
   const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>(wave, (items + 2 * kErrThreads - 1) / (2 * kErrThreads)));
-  kernel<<<blocks, kErrThreads, 0, s>>>(a, b, n, w, group_div(group), w_stride, part, done, out);
-  return cudaGetLastError();
+  kernel<<<blocks, kErrThreads, 0, s>>>(a, b, n, w, group_div(group), w_stride, part, out);
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess || blocks == 1) return e;
+  return launch_dependent(err_final_kernel, dim3(1), kErrThreads, 0, s, static_cast<const double *>(part), blocks, out);
 }
 
 }  // namespace fab

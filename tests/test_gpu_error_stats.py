@@ -29,3 +29,29 @@ def test_group_divisors_and_sizes(fab, group, stride, n, offset):
     got = fab.error_stats(da[offset:], db[offset:]).cpu().numpy()
     want = expected(a[offset:], b[offset:], None, 1, 1)
     assert np.all(np.abs(got[:2] - want[:2]) <= 1e-12 * want[:2]) and got[2] == want[2]
+
+
+def test_calls_at_once_leave_nothing_behind(fab):
+    """Three sizes on three streams at once may spoil each other (they share
+    the partial sums), but a call alone afterwards, on other values, is right:
+    nothing that one call counts or leaves is read by another."""
+    r = np.random.default_rng(11)
+
+    def arrays(n):
+        a = r.standard_normal(n).astype(np.float32)
+        b = (a + 0.1 * r.standard_normal(n)).astype(np.float32)
+        return torch.from_numpy(a).cuda(), torch.from_numpy(b).cuda(), expected(a, b, None, 1, 1)
+
+    sizes = (1000, 311297, 1 << 22)
+    at_once = [arrays(n) for n in sizes]
+    alone = [arrays(n) for n in sizes]
+    streams = [torch.cuda.Stream() for _ in sizes]
+    out = torch.empty(3, dtype=torch.float64, device="cuda")
+    for _ in range(20):
+        torch.cuda.synchronize()
+        for s, (a, b, _) in list(zip(streams, at_once)) * 10:
+            fab.error_stats(a, b, out=out, stream=s)
+        torch.cuda.synchronize()
+        for a, b, want in alone:
+            got = fab.error_stats(a, b, out=torch.full((3,), float("nan"), dtype=torch.float64, device="cuda"))
+            assert np.all(np.abs(got.cpu().numpy() - want) <= 1e-12 * want)
