@@ -109,6 +109,11 @@ __global__ void __launch_bounds__(32 * kSegWarps) latent_sums_kernel(const uint1
   grid_dependents_launch();
   const uint32_t m = blockIdx.x, mm = m * 0x10001u;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (m > 0xFFFFu) {   // no 16-bit id names it (and mm has overflowed)
+    if (threadIdx.x < kLatent) dlat[(int64_t)m * kLatent + threadIdx.x] = 0.0f;
+    if (early) grid_dependency_wait();
+    return;
+  }
   const uint32_t below = (1u << lane) - 1u;
   for (int k = 0; k < 32; ++k) bins[32 * warp + k][lane] = 0.0f;
   const int64_t whole = V ? n & ~int64_t(7) : n;

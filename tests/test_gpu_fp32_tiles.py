@@ -117,3 +117,21 @@ def test_bad_material_rows_do_not_contribute(fab):
     fab.sync_status()
     for a, b in zip(got, want):
         assert rel(a.cpu().numpy(), b.cpu().numpy()) < 1e-5
+
+
+@pytest.mark.parametrize("offset", [0, 1])
+def test_latent_rows_no_id_can_name(fab, offset):
+    """Ids have 16 bits, latent tables may have more rows: those past 65 536
+    get zero gradients, the others theirs, whether the ids can be read as
+    16-byte words or not."""
+    n, n_lat = 4001, 65540
+    g, dec, _ = setup(n + offset, 8, 25)
+    full = GBuffer.from_numpy(g)
+    full.material[::2] = -1                       # 65 535, the last id there is
+    view = GBuffer(*(getattr(full, k)[offset:] for k in ("u", "v", "radius", "wi", "wo", "material")))
+    lat = torch.randn((n_lat, 32), generator=torch.Generator("cuda").manual_seed(6), device="cuda")
+    dy = torch.randn((n, 4), generator=torch.Generator("cuda").manual_seed(7), device="cuda")
+    _, dlat = fab.decoder_backward(view, lat, torch.from_numpy(dec).cuda(), dy)
+    fab.sync_status()
+    assert not dlat[65536:].any() and not dlat[8:65535].any()
+    assert dlat[65535].any() and all(dlat[m].any() for m in range(8))
