@@ -400,7 +400,6 @@ __global__ void __launch_bounds__(kTile * H * WG, 4 / WG) decoder_tc_kernel(cons
   if (warp == 0) tc::tmem_alloc(tmem_slot, kColsPerTile * WG);
   // nothing above reads what an earlier kernel wrote
   grid_dependency_wait();
-  grid_dependents_launch();
   // batched launches: the segment table (prefix sums of tile counts) in the
   // shared memory past the weights, when the launch gave room for it
   const int64_t *seg_t0 = a.seg_tile0;
@@ -412,6 +411,10 @@ __global__ void __launch_bounds__(kTile * H * WG, 4 / WG) decoder_tc_kernel(cons
   tc::tc_fence_before();
   __syncthreads();
   tc::tc_fence_after();
+  // Only now that this CTA holds its tensor memory: a dependent kernel's CTA
+  // may allocate before it waits for this grid, and columns it took first
+  // would never come free for a CTA of this grid still waiting for its own.
+  grid_dependents_launch();
   const uint32_t tmem = *tmem_slot + kColsPerTile * (uint32_t)wg;   // this pipeline's D column 0, lane 0
   const uint32_t lane = (uint32_t)((warp & 3) * 32) << 16;          // this warp's lane quadrant
   const uint32_t t_d = tmem + lane, t_a = tmem + lane + kColA, t_x = tmem + lane + kColX;

@@ -181,7 +181,6 @@ __global__ void __launch_bounds__(kThreads, 1) train_tc_kernel(const TrainTcArgs
   // The set-up and the first tile's G-buffer reads (inputs of the step, which
   // the step's first kernel waited for) overlap the kernels before this one;
   // the wait for them comes before the weights and latents they write.
-  grid_dependents_launch();
   extern __shared__ uint8_t smem_raw[];
   uint8_t *smem = smem_raw + (-tc::smem_addr(smem_raw) & 1023u);   // an offset: a rounded address would be generic
   uint64_t *bar_w = reinterpret_cast<uint64_t *>(smem);
@@ -213,6 +212,7 @@ __global__ void __launch_bounds__(kThreads, 1) train_tc_kernel(const TrainTcArgs
     reinterpret_cast<uint4 *>(xT)[e] = make_uint4(0u, 0u, 0u, 0u);
   tc::fence_proxy_async_smem();
   sync_all();
+  grid_dependents_launch();   // with the tensor memory held, as in decoder_tc_kernel
   const uint32_t tmem = *tmem_slot;
   const uint32_t lane = (uint32_t)((warp & 3) * 32) << 16;   // this warp's lane quadrant
   const uint32_t t_d = tmem + lane + kColD, t_a = tmem + lane + kColA;

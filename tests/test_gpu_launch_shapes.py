@@ -104,3 +104,19 @@ def test_tiles_encoded_ahead(fab, n_mat, prec):
             assert torch.equal(got[0][0], got[1][0]) and torch.equal(got[0][1], got[1][1]), n
     finally:
         fab.set_launch_config(0, 0, 0, 0)
+
+
+def test_launches_of_different_shapes_back_to_back(fab, frame):
+    """Each launch starts under the one before, whose CTAs are of another
+    size and hold other amounts of tensor memory."""
+    lat, g = frame
+    fab.prepare_neural(lat, "fp16")
+    want, _ = fab.shade_neural_prepared(g, "fp16")
+    outs = [torch.full_like(want, float("nan")) for _ in SHAPES]
+    for _ in range(20):
+        for out, (wg, ctas, h) in zip(outs, SHAPES):
+            fab.set_launch_config(ctas, wg, 0, h)
+            fab.shade_neural_prepared(g, "fp16", out_rgb=out)
+    fab.sync_status()
+    fab.set_launch_config(0, 0, 0, 0)
+    assert all(torch.equal(out, want) for out in outs)
