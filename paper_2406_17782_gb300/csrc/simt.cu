@@ -1055,8 +1055,10 @@ __global__ void __launch_bounds__(kErrThreads) err_partial_kernel(const float *_
 // square whose low part falls below the normal range loses at most 2^-149
 // absolutely, which is below 2^-49 of the thread's sum unless its largest
 // |w(a-b)| (or |w b|) is under sqrt(elements) 2^-50.  A thread in either
-// case redoes its whole share in FP64 instead; one whose largest value is
-// exactly zero does not, since its sums are then exact.
+// case redoes its whole share in FP64 instead.  One whose largest value is
+// exactly zero need not where its sums are then exact: without weights, and
+// with them unless it met a nonzero weight and a nonzero a - b (or b), whose
+// product may have underflowed (three ORs a pair, no difference in time).
 constexpr int kErrRun2 = 16;    // pairs per run
 constexpr int kErrBatch2 = 4;   // pair loads in flight per thread (eight without weights)
 constexpr int kErrPerSm2 = 4;   // resident CTAs per SM
@@ -1105,6 +1107,8 @@ __global__ void __launch_bounds__(kErrThreads, kErrPerSm2) err_partial2_kernel(c
   const uint64_t two = pk2(2.0f, 2.0f);
   double e2 = 0.0, b2s = 0.0;
   float mh = -1.0f, ml = 0.0f, bmax = 0.0f;
+  uint32_t any_d = 0, any_b = 0, any_w = 0;   // W: all bits of a - b, b and w
+  auto bits2 = [](uint64_t x) { return (uint32_t)x | (uint32_t)(x >> 32); };
   for (Idx j0 = start; j0 < np; j0 += kErrRun2 * stride) {
     uint64_t EH = 0, EL = 0, BH = 0, BL = 0;
     constexpr int NB = W ? kErrBatch2 : 2 * kErrBatch2;
@@ -1132,6 +1136,9 @@ __global__ void __launch_bounds__(kErrThreads, kErrPerSm2) err_partial2_kernel(c
         uint64_t E = sub2(sub2(av[q], AV), add2(bv[q], BV));
         uint64_t Bh = bv[q], Bl = 0;
         if (W) {
+          any_d |= bits2(D);
+          any_b |= bits2(bv[q]);
+          any_w |= bits2(wv[q]);
           const uint64_t P = mul2(D, wv[q]);
           const uint64_t PE = fma2(D, wv[q], P ^ kSign2);
           E = fma2(E, wv[q], PE);
@@ -1172,7 +1179,10 @@ __global__ void __launch_bounds__(kErrThreads, kErrPerSm2) err_partial2_kernel(c
   {
     const float pairs = (float)((np - (start < np ? start : np) + stride - 1) / stride);   // this thread's pairs
     const float floor_v = 1.001f * sqrtf(2.0f * pairs) * 0x1p-50f;
-    const bool slow = !finite64(e2) || !finite64(b2s) || (mh > 0.0f && mh < floor_v) || (bmax > 0.0f && bmax < floor_v);
+    const bool weighed = W && (any_w << 1) != 0;   // a nonzero weight
+    const bool slow = !finite64(e2) || !finite64(b2s) ||
+                      (mh < floor_v && (mh > 0.0f || (weighed && (any_d << 1) != 0))) ||
+                      (bmax < floor_v && (bmax > 0.0f || (weighed && (any_b << 1) != 0)));
     if (slow) {   // the thread's whole share again, in FP64
       e2 = 0.0;
       b2s = 0.0;

@@ -55,3 +55,21 @@ def test_calls_at_once_leave_nothing_behind(fab):
         for a, b, want in alone:
             got = fab.error_stats(a, b, out=torch.full((3,), float("nan"), dtype=torch.float64, device="cuda"))
             assert np.all(np.abs(got.cpu().numpy() - want) <= 1e-12 * want)
+
+
+@pytest.mark.parametrize("offset", [0, 1])
+@pytest.mark.parametrize("n", [1000, 311297])
+def test_products_below_the_fp32_range(fab, n, offset):
+    """Weights whose products with the differences, or with b, vanish in FP32
+    still count, on the packed and on the scalar path; so do zero weights and
+    equal values for nothing."""
+    r = np.random.default_rng(n)
+    b = (2.0 ** -58 * r.uniform(1.0, 2.0, n + offset)).astype(np.float32)
+    a = (b * r.uniform(1.0, 2.0, n + offset)).astype(np.float32)
+    w = (2.0 ** -100 * r.uniform(1.0, 2.0, n)).astype(np.float32)
+    w[::3] = 0.0
+    a[::4] = b[::4]
+    da, db, dw = (torch.from_numpy(x).cuda() for x in (a, b, w))
+    got = fab.error_stats(da[offset:], db[offset:], weights=dw).cpu().numpy()
+    want = expected(a[offset:], b[offset:], w, 1, 1)
+    assert np.all(want > 0.0) and np.all(np.abs(got - want) <= 1e-12 * want)
