@@ -1058,7 +1058,8 @@ __global__ void __launch_bounds__(kErrThreads) err_partial_kernel(const float *_
 // case redoes its whole share in FP64 instead.  One whose largest value is
 // exactly zero need not where its sums are then exact: without weights, and
 // with them unless it met a nonzero weight and a nonzero a - b (or b), whose
-// product may have underflowed (three ORs a pair, no difference in time).
+// product may have underflowed (three ORs a pair: a weighted 1080p RGB frame
+// 24.5 -> 24.8 us, 2^25 elements 84.3 -> 86.4).
 constexpr int kErrRun2 = 16;    // pairs per run
 constexpr int kErrBatch2 = 4;   // pair loads in flight per thread (eight without weights)
 constexpr int kErrPerSm2 = 4;   // resident CTAs per SM
@@ -1077,17 +1078,23 @@ __device__ __forceinline__ void dadd2(uint64_t &h, uint64_t &l, uint64_t x, uint
   l = sub2(e, sub2(h, t));
 }
 
-// Both lanes of a run's packed sums in FP64: the high parts added exactly in
-// FP32, so that one FP64 addition is left (FP64 instructions issue at about a
+// Both lanes of a run's packed sums in FP64, but for `rest`: the lanes' parts
+// are joined by TwoSums in FP32, whose last terms (2^-48 of the sum) collect
+// there for the whole thread, so that a run costs two FP64 conversions and
+// one addition instead of four and three (FP64 instructions issue at about a
 // fifteenth of a cycle each per SM, and at frame sizes a thread has only one
-// or two runs: with four per run, an FP64 square root in the range test
-// and FP64 shuffles the kernel took 36 us for a weighted 1080p RGB frame).
-__device__ __forceinline__ double lanes_sum(uint64_t h, uint64_t l) {
-  float h0, h1, l0, l1, s, e;
+// or two runs: a weighted 1080p RGB frame 24.8 us, 26.8 with all of it in
+// FP64 and the same error, 6.5e-16 of the exact sum; 50 001 elements 1.1e-16,
+// and 2.8e-16 without those terms).
+__device__ __forceinline__ double lanes_sum(uint64_t h, uint64_t l, float &rest) {
+  float h0, h1, l0, l1, s, e, a, r1, b, r2;
   upk2(h, h0, h1);
   upk2(l, l0, l1);
   two_sum(h0, h1, s, e);
-  return (double)s + (double)__fadd_rn(e, __fadd_rn(l0, l1));
+  two_sum(l0, l1, a, r1);
+  two_sum(e, a, b, r2);
+  rest = __fadd_rn(rest, __fadd_rn(r1, r2));
+  return (double)s + (double)b;
 }
 __device__ __forceinline__ bool finite64(double x) { return (__double2hiint(x) & 0x7FF00000) != 0x7FF00000; }
 
@@ -1106,6 +1113,7 @@ __global__ void __launch_bounds__(kErrThreads, kErrPerSm2) err_partial2_kernel(c
   const Idx start = (Idx)blockIdx.x * kErrThreads + threadIdx.x;
   const uint64_t two = pk2(2.0f, 2.0f);
   double e2 = 0.0, b2s = 0.0;
+  float e_rest = 0.0f, b_rest = 0.0f;
   float mh = -1.0f, ml = 0.0f, bmax = 0.0f;
   uint32_t any_d = 0, any_b = 0, any_w = 0;   // W: all bits of a - b, b and w
   auto bits2 = [](uint64_t x) { return (uint32_t)x | (uint32_t)(x >> 32); };
@@ -1172,9 +1180,17 @@ __global__ void __launch_bounds__(kErrThreads, kErrPerSm2) err_partial2_kernel(c
         }
       }
     }
-    e2 += lanes_sum(EH, EL);
-    b2s += lanes_sum(BH, BL);
+    const double e_run = lanes_sum(EH, EL, e_rest), b_run = lanes_sum(BH, BL, b_rest);
+    if (!W && j0 == start) {   // (2^25 elements 67.1 -> 63.9 us; weighted 87.2 -> 88.4, so not there)
+      e2 = e_run;
+      b2s = b_run;
+    } else {
+      e2 += e_run;
+      b2s += b_run;
+    }
   }
+  e2 += (double)e_rest;
+  b2s += (double)b_rest;
   double mx = mh < 0.0f ? 0.0 : (double)mh + (double)ml;
   {
     const float pairs = (float)((np - (start < np ? start : np) + stride - 1) / stride);   // this thread's pairs
@@ -1405,9 +1421,11 @@ cudaError_t launch_error_stats(const float *a, const float *b, int64_t n, const 
                                   : (small ? err_partial2_kernel<false, int> : err_partial2_kernel<false, int64_t>))
                              : (w ? (small ? err_partial_kernel<true, int> : err_partial_kernel<true, int64_t>)
                                   : (small ? err_partial_kernel<false, int> : err_partial_kernel<false, int64_t>));
-  // one wave of CTAs, or as many as give each thread two elements or pairs
+  // one wave of CTAs, or as many as give each thread an element or pair (two
+  // are added in double-float, one not at all: 50 001 elements with two 3.6e-16
+  // off the exact sum, so 1.1e-16; 300 000 10.3 us, so 14.4)
   const int64_t items = packed ? n / 2 : n, wave = packed ? kErrBlocks2 : kErrBlocks;
-  const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>(wave, (items + 2 * kErrThreads - 1) / (2 * kErrThreads)));
+  const int blocks = (int)std::max<int64_t>(1, std::min<int64_t>(wave, (items + kErrThreads - 1) / kErrThreads));
   kernel<<<blocks, kErrThreads, 0, s>>>(a, b, n, w, group_div(group), w_stride, part, out);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess || blocks == 1) return e;

@@ -1,6 +1,8 @@
 """The FP64 error reduction over its index arithmetic and launch sizes: group
 divisors, ragged and unaligned lengths, runs of one and of many CTAs, against
 numpy FP64 (1e-12 relative for the sums, the exact maximum without weights)."""
+import math
+
 import numpy as np
 import pytest
 import torch
@@ -73,3 +75,23 @@ def test_products_below_the_fp32_range(fab, n, offset):
     got = fab.error_stats(da[offset:], db[offset:], weights=dw).cpu().numpy()
     want = expected(a[offset:], b[offset:], w, 1, 1)
     assert np.all(want > 0.0) and np.all(np.abs(got - want) <= 1e-12 * want)
+
+
+def test_sums_round_only_in_fp64(fab):
+    """FP32 values with all 24 bits in use and a = -b, so that every term is
+    exact in FP64, one pair to a thread: what is left are the roundings of a
+    tree of FP64 additions, at most 22 in sequence, each at most 2^-53 of the
+    sum and to either side.  Rounded anywhere to the 48 bits of an FP32 pair
+    the sums come out low (odd squares are 1 modulo 4, so their ties all fall
+    the same way).  A call's error is then below sqrt(22 / 3) 2^-53 = 3.0e-16
+    rms, the mean over 40 calls within three standard deviations of zero below
+    1.43e-16."""
+    n, calls = 50001, 40
+    err = np.zeros(2)
+    for k in range(calls):
+        b = np.random.default_rng([5, k]).random(n).astype(np.float32)
+        got = fab.error_stats(torch.from_numpy(-b).cuda(), torch.from_numpy(b).cuda()).cpu().numpy()
+        want = math.fsum(b.astype(np.float64) ** 2)
+        for j, scale in enumerate((0.25, 1.0)):
+            err[j] += math.fsum([scale * float(got[j]), -want]) / want / calls
+    assert np.all(np.abs(err) < 1.43e-16), err
