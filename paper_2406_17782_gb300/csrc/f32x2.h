@@ -1,6 +1,6 @@
 // f32x2.h -- the packed FP32x2 instructions of sm_100-class GPUs: one
 // instruction works on two FP32 lanes, each rounded to nearest as the scalar
-// instruction rounds it.  A pair is held in 64 bits, lane 0 in the low half.
+// instruction rounds it (but see mul2_rounded).  A pair is held in 64 bits, lane 0 in the low half.
 #pragma once
 
 #include <cstdint>
@@ -30,6 +30,15 @@ __device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
   uint64_t d;
   asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
   return d;
+}
+// The same where the product's own rounding counts although it goes into an
+// add2 or sub2: the assembler may join a packed multiplication and the addition
+// that takes its result, in spite of .rn, where it leaves scalar ones alone.
+__device__ __forceinline__ uint64_t mul2_rounded(uint64_t a, uint64_t b) {
+  float a0, a1, b0, b1;
+  upk2(a, a0, a1);
+  upk2(b, b0, b1);
+  return pk2(__fmul_rn(a0, b0), __fmul_rn(a1, b1));
 }
 __device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
   uint64_t d;

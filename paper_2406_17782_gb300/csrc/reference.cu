@@ -480,10 +480,12 @@ struct PointSampler {
   __device__ __forceinline__ void next(const SamplePlan &sp, uint32_t &pu, uint32_t &pv) {
     const uint64_t hk = splitmix_finalise(hp + (uint64_t)k);
     // ((k + xi) (2/n) - 1) r, rounded at every step as the oracle rounds it
-    // (xi has 24 bits, so the product of the fma is exact)
+    // (xi has 24 bits, so the product of the fma is exact; the first product
+    // has to be kept from joining the subtraction, which moved the samples
+    // wherever 2/n is no power of two)
     const uint64_t xi = pk2((float)(uint32_t)(hk >> 40), (float)(uint32_t)((hk >> 16) & 0xFFFFFFu));
     const uint64_t minus1 = pk2(-1.0f, -1.0f), xi_scale = pk2(5.9604644775390625e-08f, 5.9604644775390625e-08f);   // 2^-24
-    const uint64_t t = mul2(add2(mul2(fma2(xi, xi_scale, strat), sp.two_over_n), minus1), rr);
+    const uint64_t t = mul2(add2(mul2_rounded(fma2(xi, xi_scale, strat), sp.two_over_n), minus1), rr);
     float ou, ov;
     upk2(t, ou, ov);
     if (WIDE) {

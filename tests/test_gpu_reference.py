@@ -177,3 +177,25 @@ def test_mixed_points_of_a_warp(fab, frame_mats, lanes, n):
     idx = np.concatenate([np.arange(0, 11), np.arange(12, 300), np.arange(n - 200, n)])
     wc, _ = oracle.shade_reference(frame_mats, W.subset(g, idx), 8, 4, 21, pixel_index=idx)
     assert_close(c[idx], wc, f"lanes={lanes}")
+
+
+@pytest.mark.parametrize("vis", [False, True])
+@pytest.mark.parametrize("sx,sy", [(5, 3), (3, 7), (6, 1), (1, 10), (12, 20)])
+def test_positions_round_at_every_step(fab, frame_mats, sx, sy, vis):
+    """Footprints of hundreds of repeats, where a rounding of a sample's offset
+    is a visible part of a cell, with stratum counts whose 2 / n is no power of
+    two: ((k + xi) (2 / n) - 1) r is rounded at each of its steps."""
+    g = W.subset(W.frame_gbuffer(), W.sample_indices(1920 * 1080, 256, stream=f"steps{sx}x{sy}"))
+    g["radius"] = np.geomspace(50.0, 1000.0, 256).astype(np.float32)
+    fab.set_visibility(vis)
+    try:
+        _, comps = run_gpu(fab, g, sx, sy, 13)
+    finally:
+        fab.set_visibility(False)
+    if vis:
+        wc, _, near_tie = oracle.shade_reference(frame_mats, g, sx, sy, 13, visibility=True)
+        assert near_tie.mean() < 0.02
+        comps, wc = comps[~near_tie], wc[~near_tie]
+    else:
+        wc, _ = oracle.shade_reference(frame_mats, g, sx, sy, 13)
+    assert_close(comps, wc, f"{sx}x{sy}")
