@@ -516,17 +516,34 @@ struct PointSampler {
 };
 
 // Lane lane_g's samples of one point, V = 1.  OPPOSITE: directions that may
-// be nearly opposite.
-template <bool WIDE, bool OPPOSITE>
+// be nearly opposite.  A lane alone with its point adds its samples in blocks,
+// so that its sums round no more often than those of several lanes do.
+constexpr int kLaneBlock = 4;
+template <bool WIDE, bool OPPOSITE, int L>
 __device__ __forceinline__ void integrate(const RefArgs &a, const PointRecord &R, const SamplePlan &sp, int lane_g,
                                           Sums &acc) {
   PointSampler<WIDE> s(a, R, sp, lane_g);
-  while (s.k < sp.spp) {
-    uint32_t pu, pv;
-    s.next(sp, pu, pv);
-    const Shaded r = shade<OPPOSITE>(s.pm, s.d, pu, pv);
-    acc.a += r.coJ;                                    // A of Eq. 4
-    accumulate(r, acc);
+  auto add_samples = [&](int end, Sums &t) {
+    do {
+      uint32_t pu, pv;
+      s.next(sp, pu, pv);
+      const Shaded r = shade<OPPOSITE>(s.pm, s.d, pu, pv);
+      t.a += r.coJ;                                    // A of Eq. 4
+      accumulate(r, t);
+    } while (s.k < end);
+  };
+  if (L == 1) {
+    while (s.k < sp.spp) {
+      Sums t = {0.f, 0.f, 0.f, 0.f, 0.f};
+      add_samples(min(sp.spp, s.k + kLaneBlock), t);
+      acc.c0 += t.c0;
+      acc.c1 += t.c1;
+      acc.s0 += t.s0;
+      acc.s1 += t.s1;
+      acc.a += t.a;
+    }
+  } else if (s.k < sp.spp) {
+    add_samples(sp.spp, acc);
   }
 }
 
@@ -654,9 +671,9 @@ __global__ void __launch_bounds__(kRefThreads, 4) reference_kernel(const RefArgs
       if (kStaged) integrate_visible(a, R, dirs[0][warp][pt], dirs[1][warp][pt], sp, first, acc);
       else integrate_visible(a, R, own_i, own_o, sp, first, acc);
     } else if (__all_sync(0xFFFFFFFFu, R.mat < 0 || (fabsf(R.r) < kSmallRadius && (L < 32 || R.h_inv <= 1.0f)))) {
-      if (R.mat >= 0) integrate<false, (L < 32)>(a, R, sp, lane_g, acc);
+      if (R.mat >= 0) integrate<false, (L < 32), L>(a, R, sp, lane_g, acc);
     } else {
-      if (R.mat >= 0) integrate<true, true>(a, R, sp, lane_g, acc);
+      if (R.mat >= 0) integrate<true, true, L>(a, R, sp, lane_g, acc);
     }
     __syncwarp();
     // reduction inside each group of L lanes
@@ -724,10 +741,15 @@ void launch_lanes(const RefArgs &a, unsigned blocks, bool visibility, cudaStream
 // strata, which mostly fall into the same cell and yarn, so the branches stay
 // together (1080p frame, 1024 spp: 10.8 ms with 32 lanes, 11.7 with 8, 12.4
 // with one; 256 spp: 2.89, 2.99, 3.11 ms).  With fewer samples the reduction and
-// the warp's rounds outweigh that (64 spp: 0.79 ms with 4 lanes, 0.84 with 16,
-// 0.92 with 32; 16 spp: 0.22 ms with one, 0.26 with 8; 4 spp: 0.076 with one,
-// 0.105 with 4).  Small G-buffers take more lanes, until the resident
-// threads (1024 per SM) are used twice.
+// the warp's rounds outweigh that (64 spp: 0.79 ms with 4 lanes, 0.80 with 8,
+// 0.84 with 16, 0.92 with 32; 16 spp: 0.22 ms with one, 0.26 with 8; 4 spp:
+// 0.076 with one, 0.105 with 4), but the lines lie where a lane's chain of
+// additions does not yet cost digits: with 4 lanes the median error of the
+// diffuse components at 64 spp is 7.0e-8 of FP64 and 7.2e-8 at 120, with 8
+// 6.6e-8 and 16 6.4e-8; one lane's 16 samples are added in blocks of four
+// (7.2e-8, with 16 lanes 6.9e-8; one chain had 0.9e-8 more; 0.22 -> 0.23 ms).
+// Small G-buffers take more lanes, until the resident threads (1024 per SM) are
+// used twice.
 int reference_lanes(int64_t n, int spp, bool visibility, int sm_count) {
   if (visibility) {
     // as many lanes as there are samples: the marches' lengths vary most from
@@ -737,7 +759,7 @@ int reference_lanes(int64_t n, int spp, bool visibility, int sm_count) {
     while (L < 32 && 2 * L <= spp) L *= 2;
     return L;
   }
-  int L = spp >= 256 ? 32 : spp >= 32 ? 4 : 1;
+  int L = spp >= 256 ? 32 : spp >= 96 ? 16 : spp >= 32 ? 8 : spp > 16 ? 4 : 1;
   const int64_t threads = (int64_t)(sm_count > 0 ? sm_count : 148) * 2048;
   while (L < 32 && 2 * L <= spp && n * L < threads) L *= 2;
   return L;

@@ -221,3 +221,27 @@ def test_errors_average_out_over_the_samples(fab, frame_mats):
     rel = np.abs(comps[:, :2] - wc[:, :2])[seen] / wc[:, :2][seen]
     print(np.median(rel), np.quantile(rel, 0.99), np.quantile(rel, 0.999))
     assert np.quantile(rel, 0.99) < 8.3e-7
+
+
+@pytest.mark.parametrize("sx,sy", [(4, 4), (5, 5), (8, 8), (10, 12)])
+def test_few_lanes_add_as_exactly_as_many(fab, frame_mats, sx, sy):
+    """Large grids give a point few lanes, whose chains of additions are long.
+    N terms of a size in one chain have an error of 2^-24 sqrt(N / 9) of the
+    sum, in chains of N / 16 over 16 lanes 2^-24 sqrt((N / 16 + 4) / 9) at
+    most; with that of the terms (two thirds of the median at 16 lanes)
+    every chain of up to 8 additions stays within 1.1 of 16 lanes."""
+    n = 320001
+    g = W.subset(W.frame_gbuffer(), np.arange(400_000, 400_000 + n))
+    errors = []
+    try:
+        for lanes in (0, 16):
+            fab.set_launch_config(0, 0, lanes)
+            errors.append(run_gpu(fab, g, sx, sy, 3)[1])
+    finally:
+        fab.set_launch_config()
+    idx = np.arange(0, n, 8)
+    wc, _ = oracle.shade_reference(frame_mats, W.subset(g, idx), sx, sy, 3, pixel_index=idx)
+    seen = wc[:, :2] > 1e-3 * wc[:, :2].mean()
+    med = [np.median(np.abs(c[idx, :2] - wc[:, :2])[seen] / wc[:, :2][seen]) for c in errors]
+    print(med)
+    assert med[0] < 1.1 * med[1]
