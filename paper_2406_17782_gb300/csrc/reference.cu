@@ -345,7 +345,8 @@ __device__ __forceinline__ Shaded shade(const PointMaterial &pm, const PointDirs
   r.ci_pos = ci > 0.0f;
   r.diff = fmaf(d.diff_k, ci, d.diff_c) * ci * r.coJ;
   r.spec = 0.0f;
-  if (ni > 0.0f && no > 0.0f && d.h_inv > 0.0f) {
+  const float cc = ni * no;
+  if (cc > 0.0f && d.h_inv > 0.0f) {   // where the product vanishes in FP32, so does the term (and 1 / X may overflow)
     const float sp = (r.weft ? pm.sin_psi : -pm.sin_psi) * inv;
     const float ti = fmaf(sp, fmaf(hct, Bi, ic), pm.cos_psi * fmaf(ct, ia, st * d.wi.z));
     const float to = fmaf(sp, fmaf(hct, Bo, oc), pm.cos_psi * fmaf(ct, oa, st * d.wo.z));
@@ -359,7 +360,6 @@ __device__ __forceinline__ Shaded shade(const PointMaterial &pm, const PointDirs
     const float si = sqrt_hw(fmaxf(0.0f, fmaf(-yc.z * ti, ti, 1.0f)));
     const float so = sqrt_hw(fmaxf(0.0f, fmaf(-yc.z * to, to, 1.0f)));
     const float X = fmaf(si, no, so * ni);
-    const float cc = ni * no;
     // Eq. 2 with T rho = 2: 1 - exp(-y).  Above y = 1 the hardware exp2's
     // error is below an ulp of the difference; below, expm1 keeps its digits
     const float y = X * rcp_hw(cc) * (2.0f * len);
@@ -714,11 +714,12 @@ __global__ void __launch_bounds__(kRefThreads, 4) reference_kernel(const RefArgs
     c[0] = c[1] = c[2] = c[3] = rgb[0] = rgb[1] = rgb[2] = __int_as_float(0x7FC00000);
   } else {
     const bool seen = total.a > 0.0f;
-    const float ia = seen ? 1.0f / total.a : 0.0f;
-    c[0] = seen ? total.c0 * ia : 0.0f;
-    c[1] = seen ? total.c1 * ia : 0.0f;
-    c[2] = seen ? total.s0 * ia : 0.0f;
-    c[3] = seen ? total.s1 * ia : 0.0f;
+    const float up = total.a < 0x1p-64f ? 0x1p64f : 1.0f;   // the reciprocal of a subnormal A overflows
+    const float ia = seen ? 1.0f / (total.a * up) : 0.0f;
+    c[0] = seen ? total.c0 * up * ia : 0.0f;
+    c[1] = seen ? total.c1 * up * ia : 0.0f;
+    c[2] = seen ? total.s0 * up * ia : 0.0f;
+    c[3] = seen ? total.s1 * up * ia : 0.0f;
     const DevMaterial *m = a.mats + mat;
 #pragma unroll
     for (int ch = 0; ch < 3; ++ch)

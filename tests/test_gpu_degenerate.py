@@ -109,3 +109,23 @@ def test_expired_wait_is_reported_and_context_survives(fab, sleep):
     rgb, _ = fab.shade_reference(GBuffer.from_numpy(g), 2, 2, 1)
     fab.sync_status()
     assert torch.isfinite(rgb).all()
+
+
+@pytest.mark.parametrize("spp", [1, 4, 16])
+def test_reference_with_subnormal_cosines(fab, spp):
+    """On a flat level weave the cosines are the directions' z: where their
+    product vanishes in FP32 the specular term is zero, not 0 times the
+    reciprocal of a subnormal."""
+    fab.set_materials(np.array([W.make_material(pattern=0, twist_deg=0.0, incl_deg=0.0, alpha=[0.3, 0.5],
+                                                beta=[0.0, 0.0], kd=np.full((2, 3), 0.5), ks=np.full((2, 3), 0.5),
+                                                gap=0.2)]))
+    z = np.float32([1e-45, 1e-42, 5e-39, 1e-38, 1e-37, 1e-30, 1e-20])
+    n = len(z) ** 2
+    g = dict(u=np.linspace(0, 1, n, dtype=np.float32), v=np.linspace(0, 1, n, dtype=np.float32),
+             radius=np.full(n, 1e-2, np.float32), wi=np.zeros((n, 3), np.float32), wo=np.zeros((n, 3), np.float32),
+             material=np.zeros(n, np.uint16))
+    g["wi"][:, 0], g["wi"][:, 2] = 1.0, np.repeat(z, len(z))
+    g["wo"][:, 1], g["wo"][:, 2] = 1.0, np.tile(z, len(z))
+    rgb, comps = fab.shade_reference(GBuffer.from_numpy(g), spp, spp, 5, comps=True)
+    fab.sync_status()
+    assert torch.isfinite(comps).all() and torch.isfinite(rgb).all() and (comps >= 0).all()
