@@ -1157,6 +1157,10 @@ __global__ void __launch_bounds__(kErrThreads, kErrPerSm2) err_partial2_kernel(c
         float dh0, dh1, bh0, bh1;
         upk2(D, dh0, dh1);
         upk2(Bh, bh0, bh1);
+        // PP and QQ go into additions (dadd2), where the assembler could join
+        // them (see mul2_rounded) and the sums would be off by 1e-8; it does
+        // not here: the same bits as with mul2_rounded, which with weights
+        // costs 2 %
         const uint64_t PP = mul2(D, D);
         const uint64_t X = fma2(mul2(D, two), E, fma2(D, D, PP ^ kSign2));
         const uint64_t QQ = mul2(Bh, Bh);
