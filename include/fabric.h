@@ -150,8 +150,8 @@ fabric_status fabric_set_launch_config(fabric_ctx *ctx, int decoder_ctas_per_sm,
 /* Warpgroups per decoder tile pipeline: 1 (0 = 1) or 2.  With 2, the two
  * threads of each tile row split the encoding and the epilogues' columns;
  * this applies with 1 or 2 pipelines per CTA (with 4 the setting is ignored).
- * fabric_shade_neural_host without staging always takes 2; every setting
- * gives the same outputs.
+ * fabric_shade_neural_host without staging always takes 2, and two CTAs of 2
+ * pipelines for each one of 4; every setting gives the same outputs.
  * FABRIC_ERR_INVALID_ARG outside 0..2. */
 fabric_status fabric_set_decoder_tile_warpgroups(fabric_ctx *ctx, int warpgroups_per_tile);
 

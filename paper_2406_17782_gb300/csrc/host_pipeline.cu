@@ -106,11 +106,14 @@ extern "C" fabric_status fabric_shade_neural_host(fabric_ctx *ctx, const fabric_
     // Direct: when every buffer is mapped page-locked memory the decoder
     // reads the G-buffer and writes its outputs over the host link itself,
     // in one launch and without staging copies.  Always with two threads per
-    // tile row (where the pipelines per CTA allow it), which encode a tile when
-    // it starts and write it out when it ends: the decoder that works ahead lets
-    // no tile finish before the next one's inputs are there, and behind the link
-    // that is a third of the outputs written after the last read (233 036 points,
-    // three tiles per pipeline: 53.8 us against 48.4; 2 073 600: 391 and 390).
+    // tile row, which encode a tile when it starts and write it out when it
+    // ends: the decoder that works ahead lets no tile finish before the next
+    // one's inputs are there, and behind the link that is a third of the outputs
+    // written after the last read.  One thread and two, FP16: 44 430 points 14.0
+    // and 13.5 us, 155 648 38.1 and 35.5, 233 036 (three tiles per pipeline) 54.1
+    // and 49.0, 400 000 82.6 and 80.2, 2 073 600 391.5 and 391.  CTAs of four
+    // pipelines, which have one thread per row only, become two of two (233 036
+    // points 55.5 -> 49.5 us).
     fabric_gbuffer d;
     d.u = static_cast<const float *>(mapped(g_host->u));
     d.v = static_cast<const float *>(mapped(g_host->v));
@@ -127,7 +130,8 @@ extern "C" fabric_status fabric_shade_neural_host(fabric_ctx *ctx, const fabric_
                                 ctx->d_status, ctx->sm_count, caller);
       else
         e = launch_decoder_tc(d, ctx->d_blob, ctx->n_mat, (int)prec, rgb, comps, ctx->d_status, ctx->sm_count,
-                              ctx->tc_ctas_per_sm, ctx->tc_warpgroups, 2, caller);
+                              ctx->tc_ctas_per_sm * (ctx->tc_warpgroups == 4 ? 2 : 1),
+                              ctx->tc_warpgroups == 4 ? 2 : ctx->tc_warpgroups, 2, caller);
       if (e != cudaSuccess) return cuda_fail(ctx, e, "decoder launch");
       return FABRIC_OK;
     }

@@ -62,3 +62,21 @@ def test_host_call_repeats_and_refuses(fab, frame):
         fab.shade_neural_host(gh, "bf16", out_rgb=a)
     with pytest.raises(ValueError):                      # a device G-buffer
         fab.shade_neural_host(GBuffer.from_numpy(host), "fp16")
+
+
+@pytest.mark.parametrize("ctas,pipelines,h", [(0, 1, 1), (0, 2, 2), (0, 4, 0), (1, 4, 2), (1, 2, 1), (2, 1, 0)])
+def test_direct_path_with_every_launch_shape(fab, frame, ctas, pipelines, h):
+    """The direct path has its own choice of threads per row and pipelines per
+    CTA; the outputs are the device call's under any setting."""
+    lat, host = frame
+    fab.prepare_neural(lat, "fp16")
+    want, _ = fab.shade_neural_prepared(GBuffer.from_numpy(host), "fp16")
+    gh = GBuffer.from_numpy(host, device="cpu", pin=True)
+    rgb = torch.full((gh.n, 3), float("nan")).pin_memory()
+    fab.set_launch_config(ctas, pipelines, 0, h)
+    try:
+        fab.shade_neural_host(gh, "fp16", out_rgb=rgb)
+        fab.sync_status()
+    finally:
+        fab.set_launch_config(0, 0, 0, 0)
+    assert torch.equal(rgb, want.cpu())
