@@ -120,3 +120,14 @@ def test_launches_of_different_shapes_back_to_back(fab, frame):
     fab.sync_status()
     fab.set_launch_config(0, 0, 0, 0)
     assert all(torch.equal(out, want) for out in outs)
+
+
+@pytest.mark.parametrize("n_mat", [1, 33, 88, 89])
+def test_encoder_of_records_from_device_memory(fab, n_mat):
+    """Up to 89 records travel with the launch, 90 and more through device
+    memory: the same latents bit for bit."""
+    mats = np.resize(W.training_materials(8), 300)
+    mats["twist_deg"] += np.arange(300, dtype=np.float32) / 100.0
+    fab.set_params(W.decoder_init(), W.encoder_init())
+    for more in (90, 300):
+        assert torch.equal(fab.encode_params(mats[:n_mat]), fab.encode_params(mats[:more])[:n_mat])
