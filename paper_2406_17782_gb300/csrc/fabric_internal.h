@@ -294,6 +294,10 @@ struct DecAdamArgs {
   float *p, *m, *v;       // the decoder's parameters and their Adam moments
   float lr, bc1, bc2;
 };
+// With acts given, the encoder's weights are read before the wait for the
+// kernel in front, and the decoder's partials, parameters and moments (dec_adam)
+// before the wait for the one after it: the kernel in front must not write any
+// of them, and must have waited for whatever did.
 cudaError_t launch_encoder_backward(const float *feats, int n, const float *enc, const float *acts,
                                     const float *dz, float *denc, float *work, cudaStream_t s,
                                     const DecAdamArgs *dec_adam = nullptr);
@@ -302,6 +306,8 @@ void adam_bias(int64_t step, float *bc1, float *bc2);
 size_t encoder_backward_work_floats(int n);
 // Encoder forward with the input features computed from the material
 // records (and written to feats_out, when not null, for the backward pass).
+// With feats_out the records are read before the wait for the kernel in front,
+// which must not write them.
 cudaError_t launch_encoder_raw(const fabric_material *raw, int n, const float *enc, float *feats_out, float *z,
                                float *acts, cudaStream_t s);
 cudaError_t launch_decoder_raw(const fabric_gbuffer &g, const float *latents, int n_lat, const float *dec,
@@ -312,7 +318,8 @@ cudaError_t launch_decoder_backward(const fabric_gbuffer &g, const float *latent
 size_t decoder_backward_work_bytes(int64_t n, int sm_count);
 // out[m][c] = sum of rows[r][c] over the rows r < n of material m, in a fixed
 // order; cols = 64 or 128 floats per row, 16-byte aligned.  Starts under the
-// kernel before it, which must not write the rows.
+// kernel before it and waits for it at its end: that kernel must not write the
+// rows, and must itself have started after whatever did had completed.
 cudaError_t launch_material_row_sums(const uint16_t *material, int64_t n, int n_mat, const float *rows, int cols,
                                      float *out, cudaStream_t s);
 // The fixed-order sums after a backward pass that wrote per-CTA partials
@@ -336,6 +343,10 @@ cudaError_t launch_train_tc(const fabric_gbuffer &g, const float *latents, int n
 // dst[p] = src[pi(p)] for the dataset's fields (fabric_shuffle_dataset).
 cudaError_t launch_shuffle_dataset(const fabric_train_batch &src, const fabric_dataset_out &dst, uint64_t seed,
                                    int sm_count, cudaStream_t s);
+// Adam over two sets of parameters.  Reads them and their moments before it
+// waits for the kernel in front of it, which therefore must not write them (and
+// must not be an Adam launch on the same parameters), and must itself have
+// waited for whatever did.
 cudaError_t launch_adam(float *p0, int64_t n0, float *p1, int64_t n1, const float *grad, float *m, float *v, float lr,
                         int64_t step, cudaStream_t s);
 // The paper's decoder structure (paper_decoder.cu): K of its first layer for

@@ -221,12 +221,11 @@ struct Columns {
       c.v[1] = t.y;
       c.v[2] = t.z;
       c.v[3] = t.w;
-    } else if constexpr (NF == 2) {
+    } else {
+      static_assert(NF == 2, "64 or 128 columns");
       const float2 t = *reinterpret_cast<const float2 *>(p);
       c.v[0] = t.x;
       c.v[1] = t.y;
-    } else {
-      c.v[0] = *p;
     }
     return c;
   }
@@ -794,7 +793,8 @@ __global__ void __launch_bounds__(kGradThreads) encoder_grad_kernel(const float 
 __global__ void adam_kernel(float *__restrict__ p0, int64_t n0, float *__restrict__ p1, int64_t n1,
                             const float *__restrict__ g, float *__restrict__ m, float *__restrict__ v, float lr,
                             float bc1, float bc2) {
-  // what is updated is read before the wait: only Adam writes it
+  // what is updated is read before the wait: the kernel before has not written
+  // it (launch_adam's condition)
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   float *p = i < n0 ? p0 + i : p1 + (i - n0);
   float pi = 0.0f, mi = 0.0f, vi = 0.0f;
