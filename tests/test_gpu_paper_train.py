@@ -282,3 +282,32 @@ def test_paper_gradient_at_tile_edges(fab, w, ablation):
             assert rel_l2(first[1] + second[1], whole[1]) <= 1e-4, n
     finally:
         fab.paper_set_params(w, W.paper_decoder_init(w), W.paper_encoder_init())
+
+
+@pytest.mark.parametrize("n", [127, 128, 129, 383, 385])
+@pytest.mark.parametrize("ablation", ["full", "no_oneblob"])
+def test_paper_gradient_at_the_narrow_layers_tiles(fab, ablation, n):
+    """At width 64 the layers' products have tiles of 128 rows (64 at width
+    128), with a copy layout of their own: batches of one and of three such tiles
+    with a row missing or a row over, against their two parts as above."""
+    mats = W.training_materials(2)
+    fab.paper_set_params(64, W.paper_decoder_init(64, weight_bound="small", ablation=ablation),
+                         W.paper_encoder_init(weight_bound="small"), ablation=ablation)
+    fab.set_train_materials(mats)
+    full = GBuffer.from_numpy(W.training_queries(n, len(mats), stream=f"paper-narrow-{n}"))
+    target = torch.from_numpy(np.abs(np.random.default_rng(n).standard_normal((n, 4)) * 0.2)).float().cuda()
+
+    def step(a, b):
+        part = GBuffer(*[getattr(full, f)[a:b] for f in ("u", "v", "radius", "wi", "wo", "material")])
+        loss = float(fab.paper_train_step(part, target[a:b].contiguous(), 0.0).item())
+        fab.sync_status()
+        return loss * (b - a), fab.paper_gradient().astype(np.float64) * (b - a)
+
+    try:
+        whole = step(0, n)
+        for cut in (1, n - 1, n // 2 + 1):
+            first, second = step(0, cut), step(cut, n)
+            assert abs(whole[0] - first[0] - second[0]) <= 1e-5 * abs(whole[0]), cut
+            assert rel_l2(first[1] + second[1], whole[1]) <= 1e-4, cut
+    finally:
+        fab.paper_set_params(64, W.paper_decoder_init(64), W.paper_encoder_init())
