@@ -81,14 +81,15 @@ __device__ __forceinline__ void sincos_half_pi(float x, float &sn, float &cs) {
 }
 
 // One hardware operation each (relative error about 2^-23), without the
-// range checks and fix-up branches of the IEEE forms.  Where an error stays
-// the same over all samples of a point, and so does not average out, the
-// result is refined: 1 / |N| and 1 / cos(theta) by a Newton step, the factor
-// of the position across a yarn by its remainder.  A 256 spp frame's diffuse
-// components lie 6.4e-8 (median) and 6.3e-7 (99 %) off FP64 so, 7.3e-8 and
-// 8.3e-7 with the IEEE forms of all of these, 7.6e-8 and 9.8e-7 without the
-// refinements, for 2.98, 4.42 and 2.91 ms; IEEE divisions, square roots or
-// expm1 in addition change none of these figures and take 6 % each.
+// range checks and fix-up branches of the IEEE forms.  What is the same in all
+// samples of a point does not average out and is kept exact instead: the
+// factor of the position across a yarn carries its remainder, and w / (pi wi.z)
+// the remainder of pi.  The diffuse components of a 256 spp frame lie 6.2e-8
+// (median) and 6.4e-7 (99 %) off FP64 so, in relative L2 8.6e-8; without the
+// two remainders 7.6e-8, 9.8e-7 and 1.18e-7; with IEEE operations throughout
+// and no remainders 7.3e-8, 8.3e-7 and 1.16e-7, for 2.94, 2.91 and 4.42 ms.
+// IEEE divisions, square roots or expm1 in addition change none of these
+// figures and take 6 % each; a Newton step on 1 / |N| 2 % for 5.9e-8.
 __device__ __forceinline__ float rsqrt_hw(float x) {
   float r;
   asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
@@ -331,9 +332,7 @@ __device__ __forceinline__ Shaded shade(const PointMaterial &pm, const PointDirs
   ct = q.body ? ct : 1.0f;
   const float hct = yc.x * sin_half_pi(xh) * ct;   // hc cos(theta)
   const float n2 = fmaf(hct, hct, 1.0f);
-  float inv = rsqrt_hw(n2);
-  const float len = n2 * inv;                             // |N|
-  inv = fmaf(inv, fmaf(-0.5f * len, inv, 0.5f), inv);     // one Newton step
+  const float inv = rsqrt_hw(n2);
   const float ia = r.weft ? d.wi.x : d.wi.y, ic = r.weft ? d.wi.y : d.wi.x;
   const float oa = r.weft ? d.wo.x : d.wo.y, oc = r.weft ? d.wo.y : d.wo.x;
   const float Bi = fmaf(ct, d.wi.z, -st * ia), Bo = fmaf(ct, d.wo.z, -st * oa);   // cos(theta) w_z - sin(theta) w_a
@@ -362,7 +361,7 @@ __device__ __forceinline__ Shaded shade(const PointMaterial &pm, const PointDirs
     const float X = fmaf(si, no, so * ni);
     // Eq. 2 with T rho = 2: 1 - exp(-y).  Above y = 1 the hardware exp2's
     // error is below an ulp of the difference; below, expm1 keeps its digits
-    const float y = X * rcp_hw(cc) * (2.0f * len);
+    const float y = X * rcp_hw(cc) * (2.0f * (n2 * inv));
     const float E = y > 1.0f ? 1.0f - ex2_hw(-1.4426950408889634f * y) : -expm1f(-y);
     r.spec = (yc.w * rct) * (cc * E) * rcp_hw(qd * qd * X);
   }
@@ -431,7 +430,11 @@ __device__ __forceinline__ PointRecord load_point(const RefArgs &a, int64_t p) {
   const float3 h = make_float3(wi.x + wo.x, wi.y + wo.y, wi.z + wo.z);
   const float hn2 = h.x * h.x + h.y * h.y + h.z * h.z;
   R.h_inv = hn2 > 0.0f ? rsqrtf(hn2) : 0.0f;
-  R.diff_k = w / (kPi * fmaxf(wi.z, 1e-3f));
+  // w / (pi wi.z) to the last bit: pi's FP32 value is 2.8e-8 too large, and
+  // this factor is in all samples of the brightest points
+  const float z = fmaxf(wi.z, 1e-3f), den = kPi * z, rest = fmaf(kPi, z, -den) + 2.0f * kHalfPiRest * z;
+  const float k = w / den;
+  R.diff_k = k + (fmaf(-k, den, w) - k * rest) / den;
   R.diff_c = (1.0f - w) / kPi;
   R.cu = centre_fixed(u);
   R.cv = centre_fixed(v);
@@ -746,11 +749,10 @@ void launch_lanes(const RefArgs &a, unsigned blocks, bool visibility, cudaStream
 // 0.84 with 16, 0.92 with 32; 16 spp: 0.22 ms with one, 0.26 with 8; 4 spp:
 // 0.076 with one, 0.105 with 4), but the lines lie where a lane's chain of
 // additions does not yet cost digits: with 4 lanes the median error of the
-// diffuse components at 64 spp is 7.0e-8 of FP64 and 7.2e-8 at 120, with 8
-// 6.6e-8 and 16 6.4e-8; one lane's 16 samples are added in blocks of four
-// (7.2e-8, with 16 lanes 6.9e-8; one chain had 0.9e-8 more; 0.22 -> 0.23 ms).
-// Small G-buffers take more lanes, until the resident threads (1024 per SM) are
-// used twice.
+// diffuse components at 64 and 120 spp is 6 and 12 % above that with 16, with 8
+// lanes 2 %; one lane's 16 samples are added in blocks of four (4 % above 16
+// lanes, one chain 15 %; 0.224 -> 0.227 ms).  Small G-buffers take more lanes,
+// until the resident threads (1024 per SM) are used twice.
 int reference_lanes(int64_t n, int spp, bool visibility, int sm_count) {
   if (visibility) {
     // as many lanes as there are samples: the marches' lengths vary most from
