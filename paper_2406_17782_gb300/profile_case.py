@@ -4,7 +4,7 @@ for profilers (ncu) and quick timing:
   python -m paper_2406_17782_gb300.profile_case reference [--spp 16] [--reps 3]
   python -m paper_2406_17782_gb300.profile_case decoder [--precision fp16] [--reps 3]
   python -m paper_2406_17782_gb300.profile_case train [--batch 65536] [--train-precision fp32|bf16] [--reps 3]
-  python -m paper_2406_17782_gb300.profile_case error [--elements 33554432] [--reps 3]
+  python -m paper_2406_17782_gb300.profile_case error [--elements 33554432] [--weighted] [--reps 3]
   python -m paper_2406_17782_gb300.profile_case batched [--precision fp16] [--reps 3]
   python -m paper_2406_17782_gb300.profile_case paper [--width 128] [--precision fp16] [--reps 3]
   python -m paper_2406_17782_gb300.profile_case paper-train [--width 128] [--batch 65536] [--reps 3]
@@ -14,7 +14,8 @@ The workload is the 1920 x 1080 G-buffer of eight weave materials (random-init
 networks); the training case uses a batch of queries over 256 training
 materials with targets from the reference kernel at 4 x 4 samples; the error
 case reduces two arrays of uniform random floats (2^25 elements each by
-default, 268 MB together: more than L2); the batched case shades the 4K
+default, 268 MB together: more than L2; with --weighted one weight for three
+elements, as the z of a direction per RGB pixel); the batched case shades the 4K
 view plus 256 ragged segments through one plan (one launch per call); the
 paper cases run the paper's decoder structure (random-init, width 64 or
 128) on the 1080p G-buffer, or its FP32 training step.  Prints the
@@ -47,6 +48,7 @@ def main(argv=None):
     ap.add_argument("--batch", type=int, default=65536)
     ap.add_argument("--train-precision", default="fp32", choices=["fp32", "bf16"])
     ap.add_argument("--elements", type=int, default=1 << 25, help="array length (error)")
+    ap.add_argument("--weighted", action="store_true", help="a weight per three elements (error)")
     ap.add_argument("--reps", type=int, default=3)
     ap.add_argument("--visibility", action="store_true", help="the reference with the proposed visibility model")
     args = ap.parse_args(argv)
@@ -67,8 +69,10 @@ def main(argv=None):
     elif args.case == "error":
         ea = torch.rand(args.elements, device=fab.device)
         eb = torch.rand(args.elements, device=fab.device)
+        ew = torch.rand((args.elements // 3 + 1, 3), device=fab.device).view(-1)[2:] if args.weighted else None
         out = torch.empty(3, dtype=torch.float64, device=fab.device)
-        fn = lambda: fab.error_stats(ea, eb, out=out)
+        fn = lambda: fab.error_stats(ea, eb, weights=ew, group=3 if args.weighted else 1,
+                                     weight_stride=3 if args.weighted else 1, out=out)
         points = args.elements
     elif args.case in ("paper", "paper-train"):
         fab.paper_set_params(args.width, W.paper_decoder_init(args.width), W.paper_encoder_init())
