@@ -9,7 +9,10 @@ frame; the latent fold and weight packing run once per material edit and are
 timed separately).  Four G-buffer copies rotate so that every step reads
 inputs that are not in L2 (4 x 79 MB > 129 MB).
 
-Also measured in the same run and reported on the JSON line:
+Also measured in the same run; the JSON line has the main figures of these, so
+that it stays short enough (below 2 900 characters) to be read whole from the
+end of a log, and everything goes to standard error as a line of its own, or
+to the file that --details names:
   * the reference integral of the same frame at 256 spp;
   * the full neural call including the fold;
   * the end-to-end path from page-locked host memory (fabric_shade_neural_host);
@@ -66,7 +69,7 @@ FLOP_PER_POINT = 2 * (39 * 64 + 64 * 64 + 64 * 64 + 64 * 4)      # 21,888 (layer
 BYTES_PER_POINT = 38 + 12                                          # G-buffer record in, RGB out
 # DRAM bytes (read + write) of one FP16 decoder launch on this frame, from an
 # ncu capture of the same kernel (dram__bytes_read.sum + dram__bytes_write.sum)
-TRAFFIC_FP16 = 78_860_000 + 6_350_000
+TRAFFIC_FP16 = 78_860_000 + 4_750_000
 WORKLOAD = "1920x1080 G-buffer, 8 weave materials (one per 240-px band), random-init decoder"
 
 
@@ -223,6 +226,7 @@ def main():
     ap.add_argument("--warmup", type=int, default=200)
     ap.add_argument("--impl", default="ours", choices=["ours", "reference"])
     ap.add_argument("--precision", default="fp16", choices=["fp16", "bf16", "fp32"])
+    ap.add_argument("--details", help="file for everything measured (default: standard error)")
     ap.add_argument("--no-extras", action="store_true", help="only the timed neural frames")
     ap.add_argument("--no-quality", action="store_true", help="skip training and the frame-RMSE comparison")
     ap.add_argument("--quality-queries", type=int, default=1 << 24)
@@ -348,9 +352,52 @@ def main():
     line.update(extras)
     if "reference" in extras:
         line["speedup_vs_reference_256spp"] = extras["reference"]["ms_per_frame"] / ms_step
-    print(json.dumps(line), flush=True)
+    if args.details:
+        with open(args.details, "w") as f:
+            json.dump(line, f, indent=1)
+    else:
+        print("bench details: " + json.dumps(line), file=sys.stderr, flush=True)
+    print(json.dumps(main_figures(line)), flush=True)
     if world > 1:
         dist.destroy_process_group()
+
+
+def main_figures(line: dict) -> dict:
+    """What of everything measured the JSON line reports."""
+    def pick(d, *keys):
+        return {k: d[k] for k in keys if k in d}
+
+    out = pick(line, "metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step", "higher_is_better",
+               "scaling", "vs_baseline", "dtype", "data", "gpu_launches", "clocks", "hbm_view",
+               "speedup_vs_reference_256spp", "neural_with_fold_ms_per_frame")
+    out["config"] = dict(line["config"])
+    if out["config"].get("decoder_launch"):
+        out["config"]["decoder_launch"] = {k: v for k, v in line["config"]["decoder_launch"].items()
+                                           if k != "candidates_ms"}
+    out["roofline"] = pick(line["roofline"], "bound", "achieved", "peak", "unit", "frac", "traffic")
+    if "e2e" in line:
+        out["e2e"] = pick(line["e2e"], "value", "unit", "ms_per_step", "h2d_bytes_per_step", "d2h_bytes_per_step", "call")
+        out["e2e"]["frac_of_link"] = line["e2e"]["host_link"]["frac_of_full_duplex_floor"]
+    for k, keys in (("reference", ("ms_per_frame", "spp")), ("error_reduction", ("frame_ms", "large_ms")),
+                    ("reference_visibility", ("frame_1080p_with_visibility_ms",)), ("fp8", ("ms_per_frame",)),
+                    ("cpu_baseline", ("value", "unit", "cores", "kind")),
+                    ("cpu_baseline_reference", ("value", "unit", "cores", "kind"))):
+        if k in line:
+            out[k] = pick(line[k], *keys)
+    if "batched_4k" in line:
+        out["batched_4k"] = {p: line["batched_4k"][p]["ms_per_replay"] for p in ("fp16", "bf16", "fp8")}
+    if "paper_decoder" in line:
+        out["paper_decoder"] = {w: {"ms_per_frame": d["fp16"]["ms_per_frame"], "train_ms_per_step": d["train_ms_per_step"]}
+                                for w, d in line["paper_decoder"].items() if w.startswith("width")}
+    if "train" in line:
+        out["train"] = {"ms_per_step": line["train"]["ms_per_step"],
+                        "fp32_ms_per_step": line["train"]["fp32_simt"]["ms_per_step"]}
+    if "quality" in line:
+        q = line["quality"]
+        out["quality"] = dict(pick(q, "target_met"), **{k: pick(q[k]["neural_fp16"], "rmse_fp", "rmse_lit", "ms")
+                                                       for k in ("loss_eq11", "loss_rendered", "paper_structure")
+                                                       if k in q})
+    return out
 
 
 def timed(torch, stream, fn, reps):

@@ -155,3 +155,43 @@ def test_paper_data_generation_recipe():
     for w in (q["wi"], q["wo"]):
         assert (w[:, 2] > 0).all()
         np.testing.assert_allclose((w.astype(np.float64) ** 2).sum(1), 1.0, atol=1e-6)
+
+
+def test_bench_line_is_short_and_whole():
+    """The benchmark's JSON line holds its main figures in less than 2900
+    characters, however much was measured."""
+    import bench
+    long = {"note": "x" * 4000, "ladder": [{"spp": k, "rmse": 0.123456789012345} for k in range(200)]}
+    net = {"neural_fp16": dict(long, rmse_fp=0.3456789012345678, rmse_lit=0.0234567890123456, ms=0.0574285714285714)}
+    number = 123456789.12345678
+    line = dict(
+        metric=bench.METRIC, value=number, unit=bench.UNIT, n_gpus=1, steps=20000, warmup=200, ms_per_step=number,
+        higher_is_better=True, scaling="weak", vs_baseline=None, dtype="fp16", data="synthetic", gpu_launches=20000,
+        config={"workload": bench.WORKLOAD, "precision": "fp16", "points_per_frame": bench.N_POINTS,
+                "l2": "4 rotating G-buffer copies, 4 x 79 MB > 129 MB L2", "parallelism": "single GPU",
+                "decoder_launch": {"pipelines_per_cta": 1, "ctas_per_sm": 4, "warpgroups_per_pipeline": 1,
+                                   "tuned_ms": number, "candidates_ms": long}},
+        roofline=dict(long, bound="tensor", achieved=number, peak=number, unit="TFLOP/s", frac=number, traffic=85210000),
+        hbm_view={"achieved_gbs": number, "peak_gbs": number, "frac": number, "bytes_per_point": 50},
+        clocks={"sm_mhz": 2070.0, "sm_max_mhz": 2070.0, "reasons": ["sw_power_cap"], "samples": 11, "note": "samples inside the timed region"},
+        paper_context=long, reference=dict(long, ms_per_frame=number, spp=256), neural_with_fold_ms_per_frame=number,
+        error_reduction=dict(long, frame_ms=number, large_ms=number), fp8=dict(long, ms_per_frame=number),
+        reference_visibility=dict(long, frame_1080p_with_visibility_ms=number), paper_data_generation=long,
+        e2e=dict(value=number, unit=bench.UNIT, ms_per_step=number, h2d_bytes_per_step=78796800, d2h_bytes_per_step=24883200,
+                 call="fabric_shade_neural_host (page-locked buffers: the decoder reads and writes host memory)",
+                 host_link=dict(long, frac_of_full_duplex_floor=number)),
+        batched_4k=dict(long, **{p: dict(long, ms_per_replay=number) for p in ("fp16", "bf16", "fp8")}),
+        paper_decoder=dict({f"width_{w}": {"fp16": dict(long, ms_per_frame=number), "train_ms_per_step": number}
+                            for w in (64, 128)}, note="x" * 300),
+        train=dict(long, ms_per_step=number, fp32_simt={"ms_per_step": number}),
+        cpu_baseline=dict(long, value=number, unit=bench.UNIT, cores=16, kind="oracle"),
+        cpu_baseline_reference=dict(long, value=number, unit=bench.UNIT, cores=16, kind="oracle"),
+        speedup_vs_reference_256spp=number,
+        quality=dict(long, target_met=False, target=long, loss_eq11=net, loss_rendered=net, paper_structure=net))
+    out = bench.main_figures(line)
+    import json
+    text = json.dumps(out)
+    assert len(text) < 2900, len(text)
+    assert out["value"] == line["value"] and out["e2e"]["h2d_bytes_per_step"] == 78796800 and out["clocks"] == line["clocks"]
+    bare = {k: v for k, v in line.items() if k in ("metric", "value", "config", "roofline", "clocks")}
+    assert bench.main_figures(bare)["value"] == line["value"]
