@@ -397,7 +397,12 @@ def main_figures(line: dict) -> dict:
         out["quality"] = dict(pick(q, "target_met"), **{k: pick(q[k]["neural_fp16"], "rmse_fp", "rmse_lit", "ms")
                                                        for k in ("loss_eq11", "loss_rendered", "paper_structure")
                                                        if k in q})
-    return out
+
+    def short(x):
+        if isinstance(x, dict):
+            return {k: short(v) for k, v in x.items()}
+        return float(f"{x:.8g}") if isinstance(x, float) else x
+    return short(out)
 
 
 def timed(torch, stream, fn, reps):

@@ -29,14 +29,15 @@
 // per-layer power-of-two scale, and the unscaling and their biases are one
 // FP32 FMA per value in the epilogue instead of a constant-one column.
 // Bound by the latency of its own instruction stream at 4 warps per scheduler
-// (tensor memory holds no more tiles): issue 58 %, tensor pipe 42 %, ALU 46 %.
+// (tensor memory holds no more tiles): issue 61 %, tensor pipe 44 %, ALU 47 %.
 // A tile's serial chain is therefore what counts, and per tile of a 1080p
 // FP16 frame (4900 cycles at 71.4 us) it lost: 270 to issuing by an elected
 // thread (65.4 us), and to encoding ahead and writing out late what the
 // products' latency hides, unrolled issue, octaves without the conversion
 // unit and loads a whole tile ahead, another 500 (59.5 us; 8.3 M points 267 ->
-// 242, step by step 260, 248, 242).  A fifth warp per CTA that only issues
-// measured 245 against 248 and costs registers the batched kernel needs.
+// 242, step by step 260, 248, 242; 57.4 with shared memory by offset).  A fifth
+// warp per CTA that only issues measured 245 against 248 and costs registers the
+// batched kernel needs.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <cuda_fp8.h>

@@ -260,8 +260,10 @@ __device__ __forceinline__ float2 unpack2(uint32_t w) {
 // a layer's conversion (665 cycles) and its products (1090 with their issue)
 // took turns; with the next layer's first products under the second half of
 // the conversion, the next tile's encoding under the head and packed
-// multiplies for the leaky ReLU: 1080p, 8 materials, width 128 363 -> 302 us
-// (tensor pipe 43 -> 60 %, issue 60 %), width 64 158 -> 155 us (issue-bound).
+// multiplies for the leaky ReLU: 1080p, 8 materials, width 128 363 -> 302 us,
+// width 64 158 -> 155 us (issue-bound); with shared memory by offset and, at width
+// 64, the leaky ReLU below 290 and 146 us (tensor pipe 62 and 36 %, issue 60 and
+// 67 %).
 template <int W, bool F16, int WG, int H>
 __global__ void __launch_bounds__(kTile * WG * H, W == 64 ? 2 : 1) pn_decoder_kernel(const PnArgs a) {
   static_assert(W == 64 * H, "two chunks per thread");

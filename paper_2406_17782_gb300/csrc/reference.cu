@@ -6,9 +6,9 @@
 // Work mapping: L lanes (L = 1..32, a power of two) share one shading point;
 // each lane takes samples lane, lane + L, ... and the five running sums are
 // combined with warp shuffles.  The kernel is bound by the issue slots (83 %
-// busy; no pipe above 57 %), so its design is about instructions: 178 for
+// busy; no pipe above 53 %), so its design is about instructions: 181 for
 // each sample of a warp at 256 spp, where the first form took 275 (1080p
-// frame 4.42 -> 2.89 ms).  Every discrete decision (cell, gap, visible
+// frame 4.42 -> 2.94 ms).  Every discrete decision (cell, gap, visible
 // yarn) is taken in 0.32 fixed-point integers from a SplitMix64 jitter
 // (Steele, Lea and Flood 2014) so that it is exactly reproducible; the
 // shading itself runs in FP32.
@@ -744,7 +744,7 @@ void launch_lanes(const RefArgs &a, unsigned blocks, bool visibility, cudaStream
 // A whole warp for large sample counts: its lanes' samples are neighbouring
 // strata, which mostly fall into the same cell and yarn, so the branches stay
 // together (1080p frame, 1024 spp: 10.8 ms with 32 lanes, 11.7 with 8, 12.4
-// with one; 256 spp: 2.89, 2.99, 3.11 ms).  With fewer samples the reduction and
+// with one; 256 spp: 2.91, 3.00, 3.11 ms).  With fewer samples the reduction and
 // the warp's rounds outweigh that (64 spp: 0.79 ms with 4 lanes, 0.80 with 8,
 // 0.84 with 16, 0.92 with 32; 16 spp: 0.22 ms with one, 0.26 with 8; 4 spp:
 // 0.076 with one, 0.105 with 4), but the lines lie where a lane's chain of

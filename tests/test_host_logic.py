@@ -192,6 +192,6 @@ def test_bench_line_is_short_and_whole():
     import json
     text = json.dumps(out)
     assert len(text) < 2900, len(text)
-    assert out["value"] == line["value"] and out["e2e"]["h2d_bytes_per_step"] == 78796800 and out["clocks"] == line["clocks"]
+    assert abs(out["value"] / line["value"] - 1.0) < 1e-7 and out["e2e"]["h2d_bytes_per_step"] == 78796800 and out["clocks"] == line["clocks"]
     bare = {k: v for k, v in line.items() if k in ("metric", "value", "config", "roofline", "clocks")}
-    assert bench.main_figures(bare)["value"] == line["value"]
+    assert bench.main_figures(bare)["value"] == out["value"]
